@@ -32,6 +32,7 @@
 #include <type_traits>
 
 #include "kernels_common.cuh"
+#include "sep_common.cuh"
 
 namespace idg {
 
@@ -112,6 +113,85 @@ __global__ void __launch_bounds__(256) stage_records_kernel(const StageArgs a, i
   }
 }
 
+// Staging for the separable-phasor gridder: one block per subgrid writes its segments' records, 16 visibilities per chunk (the last padded
+// with zeros): float4 [0..15] = (a fix, b fix, delta, 1 / scale), [16 + 2 k], [17 + 2 k] = the 4 values times
+// the segment's scale, a power of two that puts the largest component in [512, 1024) so that hi + lo
+// halves keep 22 bits down to 2^-9 of it.
+__global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float* w_ref,
+                                                        int L) {
+  const SubgridDesc sd = a.sg[blockIdx.x];
+  const int nc = sd.c1 - sd.c0;
+  const bool mirror = (sd.flags & kSubgridMirrored) != 0;
+  const double wr = double(w_ref[blockIdx.x]) + subgrid_w0(a.g, sd);
+  const double inv_l = 1.0 / double(L), sgn = subgrid_sign(sd);
+  const double off_x = double(sd.x0 + L / 2 - a.g.N / 2), off_y = double(sd.y0 + L / 2 - a.g.N / 2);
+  float4* base = a.records + size_t(sd.rec_offset) * kRecordFloat4;
+  __shared__ float s_max[8];
+  // a warp per segment where there are enough segments, else the whole block per segment
+  const bool by_warp = sd.seg_count >= 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t0 = by_warp ? lane : int(threadIdx.x), nt = by_warp ? 32 : 256;
+  int chunk0 = 0;
+  for (int s = 0; s < sd.seg_count; ++s) {
+    const SegmentDesc sg = seg[sd.seg_begin + s];
+    const int n = sg.k_end - sg.k_begin, chunks = (n + kSepK - 1) / kSepK;
+    if (!by_warp || (s & 7) == warp) {
+      const auto vis_index = [&](int k) {
+        const int row = k / nc;
+        return (size_t(sd.b) * a.g.n_t + sd.t0 + row) * a.g.n_ch + sd.c0 + (k - row * nc);
+      };
+      float m = 0.f;
+      for (int k = sg.k_begin + t0; k < sg.k_end; k += nt) {
+        const size_t v = vis_index(k);
+        const float4 v0 = a.vis[2 * v], v1 = a.vis[2 * v + 1];
+        m = fmaxf(fmaxf(fmaxf(fmaxf(m, fabsf(v0.x)), fmaxf(fabsf(v0.y), fabsf(v0.z))), fmaxf(fabsf(v0.w), fabsf(v1.x))),
+                  fmaxf(fmaxf(fabsf(v1.y), fabsf(v1.z)), fabsf(v1.w)));
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (!by_warp) {
+        if (lane == 0) s_max[warp] = m;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < 8; ++w) m = fmaxf(m, s_max[w]);
+        __syncthreads();
+      }
+      const float scale = sep_scale(m), inv = 1.f / scale;  // powers of two: exact
+      float4* dst = base + size_t(chunk0) * kGsepChunkFloat4;
+      for (int k = t0; k < chunks * kSepK; k += nt) {
+        float4* c = dst + size_t(k / kSepK) * kGsepChunkFloat4;
+        const int q = k & (kSepK - 1);
+        float4 prm = make_float4(0.f, 0.f, 0.f, inv), v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
+        if (k < n) {
+          const int row = (sg.k_begin + k) / nc, ch = sd.c0 + (sg.k_begin + k - row * nc);
+          const double* r = a.uvw + (size_t(sd.b) * a.g.n_t + sd.t0 + row) * 3;
+          const double fs = sgn * a.fscale[ch];
+          prm.x = __int_as_float(sep_fix(((r[0] * fs) * a.g.fov - off_x) * inv_l));
+          prm.y = __int_as_float(sep_fix(((r[1] * fs) * a.g.fov - off_y) * inv_l));
+          prm.z = float(r[2] * fs - wr);
+          const size_t v = vis_index(sg.k_begin + k);
+          v0 = a.vis[2 * v];
+          v1 = a.vis[2 * v + 1];
+          if (mirror) mirror_values(v0, v1);
+          v0 = make_float4(v0.x * scale, v0.y * scale, v0.z * scale, v0.w * scale);
+          v1 = make_float4(v1.x * scale, v1.y * scale, v1.z * scale, v1.w * scale);
+        }
+        c[q] = prm;
+        c[kSepK + 2 * q] = v0;
+        c[kSepK + 2 * q + 1] = v1;
+      }
+    }
+    chunk0 += chunks;
+  }
+}
+
+int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids,
+                     void* stream) {
+  if (n_subgrids <= 0) return 0;
+  stage_sep_kernel<<<n_subgrids, 256, 0, cudaStream_t(stream)>>>(a, seg, w_ref, L);
+  return int(cudaGetLastError());
+}
+
 // one warp per (interval, station): are all off-diagonal node entries zero?
 __global__ void aterm_flags_kernel(const float2* aterms, uint8_t* flags, int n_pairs, int nodes) {
   const int pair = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -182,6 +262,23 @@ IDG_GRID_TC_EXTERN(96)
 IDG_GRID_TC_EXTERN(128)
 #undef IDG_GRID_TC_EXTERN
 
+// the separable-phasor gridder lives in gridder_sep_kernels.cuh, instantiated in gridder_sep_lNN.cu
+template <int L>
+int configure_gridder_sep_l(int* persistent_blocks);
+template <int L>
+int launch_gridder_sep_l(const GridArgs& a, int n_items, int persistent_blocks, void* stream);
+template <int L>
+int launch_gridder_sep_multi_l(const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
+#define IDG_GRID_SEP_EXTERN(L)                                                                                   \
+  extern template int configure_gridder_sep_l<L>(int*);                                                         \
+  extern template int launch_gridder_sep_l<L>(const GridArgs&, int, int, void*);                                \
+  extern template int launch_gridder_sep_multi_l<L>(const GridArgs*, const int2*, int, int, void*);
+IDG_GRID_SEP_EXTERN(32)
+IDG_GRID_SEP_EXTERN(64)
+IDG_GRID_SEP_EXTERN(96)
+IDG_GRID_SEP_EXTERN(128)
+#undef IDG_GRID_SEP_EXTERN
+
 #define IDG_SWITCH_L(CALL)                 \
   switch (L) {                             \
     case 32: return CALL(32);              \
@@ -208,6 +305,22 @@ int launch_gridder_tc_multi(int L, const GridArgs* args, const int2* items, int 
 }
 int launch_stage_tc(int L, const StageArgs& a, const SegmentDesc* seg, int n_subgrids, void* stream) {
 #define C_(X) launch_stage_tc_l<X>(a, seg, n_subgrids, stream)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int configure_gridder_sep(int L, int* persistent_blocks) {
+#define C_(X) configure_gridder_sep_l<X>(persistent_blocks)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, void* stream) {
+#define C_(X) launch_gridder_sep_l<X>(a, n_items, persistent_blocks, stream)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int n_items, int max_nodes,
+                             void* stream) {
+#define C_(X) launch_gridder_sep_multi_l<X>(args, items, n_items, max_nodes, stream)
   IDG_SWITCH_L(C_)
 #undef C_
 }

@@ -52,7 +52,9 @@ struct idg_plan {
   int32_t degrid_channels = 1;       // channels per degridder lane
   int32_t grid_chunk = kDefaultGridChunk;  // staged records per gridder chunk
   int32_t mac = IDG_MAC_FP32;        // multiply-accumulate unit of the degridder
-  bool grid_tc = false;              // gridder on the tensor cores (mac, uniform channels, no A-term normalisation)
+  bool uniform = true;               // channels uniformly spaced
+  bool grid_sep = false;             // separable-phasor gridder (sep_common.cuh)
+  bool grid_tc = false;              // gridder on the tensor cores without it (mac, uniform channels, no A-term normalisation)
   cudaStream_t stream = nullptr;
   bool host_only = false;
   Partition part;
@@ -82,6 +84,9 @@ struct idg_plan {
   int* d_status = nullptr;      // kernel status word (timeouts)
   int* d_queue = nullptr;       // work-queue counters, 2 per batch (gridder, degridder)
   uint8_t* d_adiag = nullptr;   // [n_int][n_st] diagonal-A-term flags of the current call
+  float* d_sep = nullptr;       // [4][L] separable-phasor tables a, b, p, q
+  float2* d_n1 = nullptr;       // [L*L] n' as two floats
+  float* d_wref = nullptr;      // [exec subgrids] reference w
   double* d_aweights = nullptr; // [L*L + 1] A-term power weights (IDG_NORMALIZE_ATERM)
   // image-domain wrapper, made at its first use
   cufftHandle fft = 0;
@@ -172,7 +177,7 @@ void free_device(idg_plan* p) {
   p->graph_degrid = {};
   void* ptrs[] = {p->d_uvw,    p->d_fscale, p->d_taper,   p->d_blk,     p->d_twiddle, p->d_sg,     p->d_seg,
                   p->d_gitems, p->d_ditems, p->d_scratch, p->d_records, p->d_status,  p->d_queue,
-                  p->d_adiag,  p->d_blk16, p->d_inv_t, p->d_aweights};
+                  p->d_adiag,  p->d_blk16, p->d_inv_t, p->d_aweights, p->d_sep, p->d_n1, p->d_wref};
   // stream-ordered frees: no device-wide synchronisation, so plans of other
   // streams keep running while this one is released
   for (void* q : ptrs)
@@ -194,6 +199,9 @@ void free_device(idg_plan* p) {
   p->d_queue = nullptr;
   p->d_adiag = nullptr;
   p->d_aweights = nullptr;
+  p->d_sep = nullptr;
+  p->d_n1 = nullptr;
+  p->d_wref = nullptr;
 }
 
 // Block geometry table, FP64 -> FP32: for each row j and block ib of 8
@@ -242,6 +250,84 @@ std::vector<float4> block_geometry16(int L, double fov) {
       for (int q = 0; q < 4; ++q) g[1 + q] = make_float4(dn[4 * q], dn[4 * q + 1], dn[4 * q + 2], dn[4 * q + 3]);
     }
   return t;
+}
+
+// The separable form of n' over the subgrid (sep_common.cuh): n'(i,j) = A_i + B_j
+// + p_i q_j + rest, fitted with the taper as weight (A and B weighted means,
+// p q the leading singular pair of the weighted remainder).  e1 and e2 bound
+// what it neglects: max over pixels of T |rest| and of T |n' - A - B|^2 / 2, T
+// the taper product relative to its maximum.
+struct SepFit {
+  std::vector<float> tab;   // [4][L]: 2 pi A, 2 pi B, 2 pi p, q
+  std::vector<float2> n1;   // [j][i]
+  double e1 = 0.0, e2 = 0.0;
+};
+
+SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
+  SepFit f;
+  std::vector<double> w(L), c(size_t(L) * L), A(L), B(L), p(L), q(L, 1.0);
+  double wmax = 0.0, ww = 0.0;
+  for (int i = 0; i < L; ++i) wmax = std::max(wmax, std::fabs(taper[i]));
+  if (!(wmax > 0.0)) wmax = 1.0;
+  for (int i = 0; i < L; ++i) {
+    w[i] = std::max(std::fabs(taper[i]) / wmax, 1e-8);
+    ww += w[i] * w[i];
+  }
+  f.n1.resize(size_t(L) * L);
+  for (int j = 0; j < L; ++j)
+    for (int i = 0; i < L; ++i) {
+      const double l = double(i - L / 2) * fov / double(L), m = double(j - L / 2) * fov / double(L);
+      const double n = std::sqrt(1.0 - l * l - m * m) - 1.0;
+      c[size_t(j) * L + i] = n;
+      f.n1[size_t(j) * L + i] = make_float2(float(n), float(n - double(float(n))));
+    }
+  for (int i = 0; i < L; ++i) {
+    for (int j = 0; j < L; ++j) A[i] += w[j] * w[j] * c[size_t(j) * L + i];
+    A[i] /= ww;
+  }
+  for (int j = 0; j < L; ++j) {
+    for (int i = 0; i < L; ++i) B[j] += w[i] * w[i] * (c[size_t(j) * L + i] - A[i]);
+    B[j] /= ww;
+  }
+  for (int j = 0; j < L; ++j)
+    for (int i = 0; i < L; ++i) c[size_t(j) * L + i] -= A[i] + B[j];
+  // leading pair of the weighted remainder by alternating least squares
+  for (int j = 0; j < L; ++j) q[j] = B[j] - B[L / 2];
+  for (int it = 0; it < 24; ++it) {
+    double qq = 0.0, pp = 0.0;
+    for (int j = 0; j < L; ++j) qq += w[j] * w[j] * q[j] * q[j];
+    for (int i = 0; i < L; ++i) {
+      p[i] = 0.0;
+      for (int j = 0; j < L; ++j) p[i] += w[j] * w[j] * c[size_t(j) * L + i] * q[j];
+      p[i] = qq > 0.0 ? p[i] / qq : 0.0;
+      pp += w[i] * w[i] * p[i] * p[i];
+    }
+    for (int j = 0; j < L; ++j) {
+      q[j] = 0.0;
+      for (int i = 0; i < L; ++i) q[j] += w[i] * w[i] * c[size_t(j) * L + i] * p[i];
+      q[j] = pp > 0.0 ? q[j] / pp : 0.0;
+    }
+  }
+  double qm = 0.0;
+  for (double v : q) qm = std::max(qm, std::fabs(v));
+  for (int i = 0; i < L && qm > 0.0; ++i) {
+    q[i] /= qm;
+    p[i] *= qm;
+  }
+  for (int j = 0; j < L; ++j)
+    for (int i = 0; i < L; ++i) {
+      const double t = std::fabs(taper[i] * taper[j]) / (wmax * wmax), x = c[size_t(j) * L + i];
+      f.e1 = std::max(f.e1, t * std::fabs(x - p[i] * q[j]));
+      f.e2 = std::max(f.e2, t * 0.5 * x * x);
+    }
+  f.tab.resize(size_t(4) * L);
+  for (int i = 0; i < L; ++i) {
+    f.tab[i] = float(2.0 * kPi * A[i]);
+    f.tab[L + i] = float(2.0 * kPi * B[i]);
+    f.tab[2 * L + i] = float(2.0 * kPi * p[i]);
+    f.tab[3 * L + i] = float(q[i]);
+  }
+  return f;
 }
 
 size_t scratch_budget_bytes() {
@@ -383,6 +469,38 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     const int want = g->degrid_channels > 0 ? g->degrid_channels : kDefaultDegridChannels;
     p->degrid_channels = uniform ? want : 1;
   }
+  std::vector<double> taper_d;
+  if (g->taper_kind == IDG_TAPER_USER)
+    taper_d.assign(g->taper_user, g->taper_user + L);
+  else
+    taper_d = kaiser_bessel_taper(L, g->taper_beta > 0.0 ? g->taper_beta : 0.35 * kPi * g->kernel_padding);
+  // reference w of every kept subgrid (the middle of its members' w - w0) and whether the separable form
+  // holds for the largest distance from it
+  SepFit sep;
+  std::vector<float> w_ref;
+  bool sep_ok = false;
+  if (!host_only) {
+    sep = sep_fit(L, g->image_size, taper_d);
+    double delta = 0.0;
+    w_ref.reserve(p->exec.size());
+    for (SubgridDesc& d : p->exec) {
+      const double sgn = subgrid_sign(d), w0 = (double(d.layer) + 0.5) * p->part.w_step;
+      double lo = 0.0, hi = 0.0;
+      for (int t = d.t0; t < d.t1; ++t)
+        for (int e = 0; e < 2; ++e) {
+          const double w = sgn * uvw_m[(size_t(d.b) * n_timesteps + t) * 3 + 2] *
+                               (freqs_hz[e ? d.c1 - 1 : d.c0] / kSpeedOfLight) - w0;
+          lo = (t == d.t0 && !e) ? w : std::min(lo, w);
+          hi = (t == d.t0 && !e) ? w : std::max(hi, w);
+        }
+      const float mid = float(0.5 * (lo + hi));
+      delta = std::max(delta, std::max(hi - double(mid), double(mid) - lo));
+      d.rec_offset = int32_t(w_ref.size());
+      w_ref.push_back(mid);
+    }
+    const double x = 2.0 * kPi * delta;
+    sep_ok = x * sep.e1 + x * x * sep.e2 <= kSepTolerance;  // false for a NaN
+  }
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
   // cannot run); both on FP32 when channel groups were asked for, and for Stokes I (the FP32 kernels' sums
   // over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four correlations)
@@ -396,8 +514,10 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       const double s1 = freqs_hz[1] - freqs_hz[0], sc = freqs_hz[c] - freqs_hz[c - 1];
       uniform = std::fabs(sc - s1) <= 1e-12 * std::fabs(s1);
     }
-    p->grid_tc = p->mac == IDG_MAC_TENSOR && uniform && !(g->flags & IDG_NORMALIZE_ATERM);
-    if (p->mac == IDG_MAC_TENSOR && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
+    p->uniform = uniform;
+    p->grid_sep = p->mac == IDG_MAC_TENSOR && sep_ok && !(g->flags & IDG_NORMALIZE_ATERM);
+    p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && uniform && !(g->flags & IDG_NORMALIZE_ATERM);
+    if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
   }
   p->grid_chunk = g->grid_chunk > 0 ? g->grid_chunk : kDefaultGridChunk;
   for (SubgridDesc& d : p->exec) d.layer -= k_lo;  // device tables hold the grid plane set
@@ -411,6 +531,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     if (x.y0 != y.y0) return x.y0 < y.y0;
     return x.x0 < y.x0;
   });
+  {
+    // into execution order (rec_offset held each subgrid's place in w_ref)
+    const std::vector<float> src = w_ref;
+    for (size_t s = 0; s < p->exec.size(); ++s) w_ref[s] = src[p->exec[s].rec_offset];
+  }
   const size_t per_sg = size_t(4) * L * L * sizeof(float2);
   const size_t cap = std::max<size_t>(1, scratch_budget_bytes() / per_sg);
   p->batch_cap = int32_t(std::min<size_t>(cap, std::max<size_t>(1, p->exec.size())));
@@ -427,7 +552,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       SubgridDesc& d = p->exec[s0 + o];
       d.rec_offset = int32_t(recs);
       const int nc = d.c1 - d.c0;
-      recs += p->grid_tc ? tc_records(tc_row_groups(p->part.segments.data(), d.seg_begin, d.seg_count, nc), nc)
+      if (p->grid_sep)
+        for (int s = 0; s < d.seg_count; ++s) {
+          const SegmentDesc& sg = p->part.segments[d.seg_begin + s];
+          recs += (sg.k_end - sg.k_begin + kGsepChunkVis - 1) / kGsepChunkVis * (kGsepChunkFloat4 / kRecordFloat4);
+        }
+      else
+        recs += p->grid_tc ? tc_records(tc_row_groups(p->part.segments.data(), d.seg_begin, d.seg_count, nc), nc)
                          : d.n_vis;
     }
     p->max_batch_vis = std::max(p->max_batch_vis, recs);
@@ -439,7 +570,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       return p->exec[s0 + x].n_vis > p->exec[s0 + y].n_vis;
     });
     for (int32_t o : order)
-      for (int t = 0; t < (p->grid_tc ? L * L / kGtcPixels : tiles); ++t) gitems.push_back(GridItem{o, t});
+      for (int t = 0; t < (p->grid_sep ? L / kGsepColumns : p->grid_tc ? L * L / kGtcPixels : tiles); ++t) gitems.push_back(GridItem{o, t});
     // degridder items: pieces of <= `lanes` channel groups of one segment
     // (a segment's rows times G groups per row); a piece that ends its
     // segment shares its item with the first piece of the next segment when
@@ -494,11 +625,6 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   // device tables
   std::vector<double> fscale(n_channels);
   for (int c = 0; c < n_channels; ++c) fscale[c] = freqs_hz[c] / kSpeedOfLight;
-  std::vector<double> taper_d;
-  if (g->taper_kind == IDG_TAPER_USER)
-    taper_d.assign(g->taper_user, g->taper_user + L);
-  else
-    taper_d = kaiser_bessel_taper(L, g->taper_beta > 0.0 ? g->taper_beta : 0.35 * kPi * g->kernel_padding);
   std::vector<float> taper_f(taper_d.begin(), taper_d.end());
   std::vector<float4> blk = block_geometry(L, g->image_size);
   std::vector<float4> blk16 = block_geometry16(L, g->image_size);
@@ -511,6 +637,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   int e = configure_kernels(L);
   if (!e) e = configure_gridder(L, p->grid_chunk, &pg);
   if (!e && p->grid_tc) e = configure_gridder_tc(L, &pg);
+  if (!e && p->grid_sep) e = configure_gridder_sep(L, &pg);
   // the FP32 kernels serve the items of few visibilities in either mode
   if (!e) e = configure_degridder(L, g->aterm_nodes, p->degrid_channels, &pd);
   if (!e && p->mac != IDG_MAC_FP32) e = configure_degridder_tc(L, g->aterm_nodes, &pd);
@@ -524,6 +651,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   if (!e) e = upload(p, &p->d_blk, blk.data(), blk.size());
   if (!e) e = upload(p, &p->d_blk16, blk16.data(), blk16.size());
   if (!e) e = upload(p, &p->d_twiddle, tw.data(), tw.size());
+  if (!e && p->grid_sep) {
+    e = upload(p, &p->d_sep, sep.tab.data(), sep.tab.size());
+    if (!e) e = upload(p, &p->d_n1, sep.n1.data(), sep.n1.size());
+    if (!e) e = upload(p, &p->d_wref, w_ref.data(), w_ref.size());
+  }
   if (!e) e = upload(p, &p->d_sg, p->exec.data(), p->exec.size());
   if (!e) e = upload(p, &p->d_seg, p->part.segments.data(), p->part.segments.size());
   if (!e) e = upload(p, &p->d_gitems, gitems.data(), gitems.size());
@@ -598,6 +730,11 @@ static StageArgs stage_args(const idg_plan* p, const Batch& b, const void* vis) 
   return sa;
 }
 
+static SepTables sep_tables(const idg_plan* p) {
+  const int L = p->L;
+  return SepTables{p->d_sep, p->d_sep + L, p->d_sep + 2 * L, p->d_sep + 3 * L, p->d_n1};
+}
+
 static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, const void* aterms) {
   GridArgs ga{};
   ga.adiag = p->d_adiag;
@@ -615,17 +752,24 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
   ga.scratch = p->d_scratch;
   ga.aweights = p->d_aweights;
   ga.vc = p->grid_chunk;
+  if (p->grid_sep) {
+    ga.w_ref = p->d_wref + b.sg_offset;
+    ga.sep = sep_tables(p);
+  }
   ga.g = kgeom(p);
   return ga;
 }
 
 // record staging and the gridder of the plan's kind (FP32 pipe or tensor cores)
 static int stage_any(const idg_plan* p, const Batch& b, const void* vis, cudaStream_t strm) {
+  if (p->grid_sep)
+    return launch_stage_sep(p->L, stage_args(p, b, vis), p->d_seg, p->d_wref + b.sg_offset, b.sg_count, strm);
   return p->grid_tc ? launch_stage_tc(p->L, stage_args(p, b, vis), p->d_seg, b.sg_count, strm)
                     : launch_stage_records(p->L, stage_args(p, b, vis), b.sg_count, strm);
 }
 
 static int gridder_any(const idg_plan* p, const GridArgs& ga, int n_items, int persistent_blocks, cudaStream_t strm) {
+  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, persistent_blocks, strm);
   return p->grid_tc ? launch_gridder_tc(p->L, ga, n_items, persistent_blocks, strm)
                     : launch_gridder(p->L, ga, n_items, persistent_blocks, strm);
 }
@@ -840,7 +984,7 @@ idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, c
     const idg_plan* p0 = plans[0];
     if (p->L != p0->L || p->npol != p0->npol || (p->d_aweights != nullptr) != (p0->d_aweights != nullptr) ||
         p->degrid_channels != p0->degrid_channels || p->grid_chunk != p0->grid_chunk || p->mac != p0->mac ||
-        p->grid_tc != p0->grid_tc)
+        (p->mac == IDG_MAC_TENSOR && p->uniform != p0->uniform))
       return set_err(p, IDG_ERR_INVALID_ARG,
                      "plans of one call must share subgrid size, Stokes-I mode, normalisation, grid_chunk, "
                      "degrid_channels, mac_unit and the gridder kind");
@@ -890,9 +1034,11 @@ idg_status idg_grid_many(int32_t n, idg_plan* const* plans, const void* const* v
   cudaStream_t strm = cudaStream_t(cuda_stream);
   const int L = plans[0]->L;
   size_t n_waves = 0;
+  int max_nodes = 2;
   for (int32_t k = 0; k < n; ++k) {
     idg_plan* p = plans[k];
     n_waves = std::max(n_waves, p->batches.size());
+    max_nodes = std::max(max_nodes, int(p->geom.aterm_nodes));
     const int e = launch_aterm_flags(static_cast<const float2*>(aterms_c64[k]), p->d_adiag, p->n_int, p->n_st,
                                      p->geom.aterm_nodes, strm);
     if (e) return cuda_err(p, e, "A-term flag launch");
@@ -915,14 +1061,21 @@ idg_status idg_grid_many(int32_t n, idg_plan* const* plans, const void* const* v
       count.push_back(b.gi_count);
       slot_plan.push_back(k);
     }
-    const std::vector<int2> items = merge_items(cost, count);
+    // plans with and without the separable form take a launch each, their items in one list
+    std::vector<int32_t> count_sep = count;
+    for (size_t s = 0; s < count.size(); ++s) (plans[slot_plan[s]]->grid_sep ? count : count_sep)[s] = 0;
+    std::vector<int2> items = merge_items(cost, count_sep);
+    const size_t n_sep = items.size();
+    for (int2 it : merge_items(cost, count)) items.push_back(it);
     GridArgs* d_args = nullptr;
     int2* d_items = nullptr;
     int e = upload_wave(strm, args, items, &d_args, &d_items);
+    if (!e) e = launch_gridder_sep_multi(L, d_args, d_items, int(n_sep), max_nodes, strm);
     if (!e)
-      e = plans[0]->grid_tc ? launch_gridder_tc_multi(L, d_args, d_items, int(items.size()), strm)
-                            : launch_gridder_multi(L, d_args, d_items, int(items.size()),
-                                                   plans[0]->d_aweights != nullptr, plans[0]->grid_chunk, strm);
+      e = plans[0]->mac == IDG_MAC_TENSOR
+              ? launch_gridder_tc_multi(L, d_args, d_items + n_sep, int(items.size() - n_sep), strm)
+              : launch_gridder_multi(L, d_args, d_items + n_sep, int(items.size() - n_sep),
+                                     plans[0]->d_aweights != nullptr, plans[0]->grid_chunk, strm);
     if (d_args) cudaFreeAsync(d_args, strm);
     if (d_items) cudaFreeAsync(d_items, strm);
     if (e) return cuda_err(plans[0], e, "gridder launch (several plans)");

@@ -128,6 +128,28 @@ __host__ __device__ inline int64_t tc_records(int n_groups, int nc) {
   return int64_t(n_groups) * tc_group_float4(nc) / 8;
 }
 
+// Separable-phasor kernels (sep_common.cuh): the staged records of a subgrid
+// are chunks of 16 visibilities of one segment (the last chunk of a segment
+// padded with zeros), 48 float4 each
+constexpr int kGsepChunkFloat4 = 48;
+constexpr int kGsepChunkVis = 16;
+constexpr int kGsepColumns = 32;    // pixel columns per gridder work item
+// dynamic shared memory limit of those kernels (227 KB per block less their static part)
+constexpr int kSepSmemLimit = 231424;
+// largest taper-weighted error of the separable form, relative to the centre
+// pixel's weight: below the rounding of the FP32 kernels' phases
+constexpr double kSepTolerance = 3e-7;
+
+// Tables of the separable form, n'(i,j) = A_i + B_j + p_i q_j + rest: a = 2 pi A,
+// b = 2 pi B, p = 2 pi p (scaled so that max |q| = 1), and n' as two floats
+struct SepTables {
+  const float* a = nullptr;
+  const float* b = nullptr;
+  const float* p = nullptr;
+  const float* q = nullptr;
+  const float2* n1 = nullptr;  // [L (j)][L (i)]
+};
+
 
 // ---------------------------------------------------------------- planner
 
@@ -213,6 +235,8 @@ struct GridArgs {
   float2* scratch;            // [batch][4][L][L]
   double* aweights;           // A-term power weights [L*L + 1] (IDG_NORMALIZE_ATERM), else NULL
   int vc = kDefaultGridChunk;  // staged records per chunk: 32, 48 or 64
+  const float* w_ref = nullptr;  // [batch subgrids] reference w (separable-phasor gridder)
+  SepTables sep;
   KernelGeom g;
 };
 
@@ -282,6 +306,11 @@ int launch_stage_tc(int L, const StageArgs& a, const SegmentDesc* seg, int n_sub
 int launch_gridder_tc(int L, const GridArgs& a, int n_items, int persistent_blocks, void* stream);
 int configure_gridder_tc(int L, int* persistent_blocks);
 int launch_gridder_tc_multi(int L, const GridArgs* args, const int2* items, int n_items, void* stream);
+// the separable-phasor gridder (records staged by launch_stage_sep; any channel spacing)
+int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids, void* stream);
+int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, void* stream);
+int configure_gridder_sep(int L, int* persistent_blocks);
+int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
 int configure_degridder_tc(int L, int nodes, int* persistent_blocks);
 int launch_degridder_tc_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
                               void* stream);

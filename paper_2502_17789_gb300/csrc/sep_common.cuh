@@ -1,0 +1,149 @@
+// Shared device code of the separable-phasor gridder and degridder
+// (gridder_sep_kernels.cuh, degridder_sep_kernels.cuh).
+//
+// The phase of Eq. 7 over a subgrid, phi_k(i,j) = a_k i' + b_k j' + w_k n'(i,j)
+// (turns; i' = i - L/2, j' = j - L/2), is separable but for the w term, and
+// that term nearly so.  With w_ref the middle of the subgrid's w range,
+// delta_k = w_k - w_ref, and the fit n'(i,j) = A_i + B_j + p_i q_j + r_ij
+// (taper-weighted, SepTables),
+//   e^{2 pi i phi_k} = e^{2 pi i w_ref n'(i,j)} E_k(i) F_k(j) (1 + 2 pi i delta_k p_i q_j) + O(r, p^2 q^2)
+//   E_k(i) = e^{2 pi i (a_k i' + delta_k A_i)},  F_k(j) = e^{2 pi i (b_k j' + delta_k B_j)}.
+// The first factor is the same for every visibility of the subgrid and is
+// applied once per pixel; the sums over visibilities (gridder) or pixels
+// (degridder) become real matrix products of an E side and an F side, so a
+// visibility needs 2 L sines and cosines instead of L^2 and the
+// multiply-accumulate runs on the tensor cores at full tile sizes.  The plan
+// takes this path only where the neglected terms, weighted with the taper,
+// stay below kSepTolerance (sep_tables).
+//
+// Products: tcgen05.mma kind::f16 with FP32 accumulation in tensor memory.
+// Every FP32 operand is split into two halves hi + lo (22 bits), and the
+// product taken as hi hi + lo hi + hi lo; the first-order term is about 1e-3
+// of the sum and takes one more product of rounded halves.
+#pragma once
+
+#include <cuda_fp16.h>
+
+#include "kernels_common.cuh"
+
+namespace idg {
+
+constexpr int kSepThreads = 512;
+constexpr int kSepK = 16;                       // contraction length of one chunk (one MMA step)
+constexpr float kTurnsToRad = 1.4629180792671596e-9f;  // 2 pi / 2^32
+
+// ---------------------------------------------------------------- tcgen05
+
+// Shared-memory matrix descriptor, K-major without swizzle: 8-row x 16-byte
+// core matrices, `k_stride` bytes between core matrices along K and 128
+// bytes between those along M or N (consecutive rows 16 bytes apart).
+__device__ __forceinline__ uint64_t sep_desc(uint32_t addr, uint32_t k_stride) {
+  return uint64_t((addr >> 4) & 0x3fff) | (uint64_t(k_stride >> 4) << 16) | (uint64_t(128 >> 4) << 32) |
+         (uint64_t(1) << 46);
+}
+// kind::f16 instruction descriptor: FP32 accumulator, f16 A and B, both K-major, M = 128
+__host__ __device__ constexpr uint32_t sep_idesc(int n) {
+  return (1u << 4) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
+}
+__device__ __forceinline__ void sep_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// arrive on `bar` when every MMA issued so far by this thread has completed
+__device__ __forceinline__ void sep_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(cols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t cols) {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld4(float (&v)[4], uint32_t addr) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = __uint_as_float(r[k]);
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ---------------------------------------------------------------- operands
+
+// phase (radians, about [-pi, pi]) of slope `fix` (turns per pixel in units
+// of 2^-32, so the product wraps exactly) at pixel offset `off`, plus the
+// small w part `delta_k` x `fit` (fit carries 2 pi)
+__device__ __forceinline__ float sep_phase(int fix, int off, float delta, float fit) {
+  return fmaf(float(int(unsigned(fix) * unsigned(off))), kTurnsToRad, delta * fit);
+}
+
+// slope in turns per pixel as a multiple of 2^-32 (whole turns wrap away)
+__device__ __forceinline__ int sep_fix(double turns) { return int(unsigned(__double2ll_rn(turns * 4294967296.0))); }
+
+// power of two that brings `m` into [512, 1024); 1 for 0, infinity and NaN
+__device__ __forceinline__ float sep_scale(float m) {
+  if (!(m > 0.f) || m > 3.4e38f) return 1.f;
+  const int e = 9 - ilogbf(m);
+  return ldexpf(1.f, e > 126 ? 126 : e);
+}
+
+__device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
+
+// (hi, lo) halves of the pair (x0, x1): hi = x rounded to half, lo = (x - hi) rounded to half
+__device__ __forceinline__ __half2 sep_split(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(x0, x1);
+  const float2 f = __half22float2(h);
+  hi = h2_bits(h);
+  lo = h2_bits(__floats2half2_rn(x0 - f.x, x1 - f.y));
+  return h;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, const uint32_t (&v)[4]) {
+  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+
+// the F side of one column index for 8 consecutive contraction indices: rows
+// of the blocks (-Im, Re, Im) at dst, dst + block, dst + 2 block, the levels
+// (hi, lo, first order) `level` bytes apart.  SIGN = -1 takes conj(F).
+struct SepF {
+  uint32_t r_hi[4], i_hi[4], r_lo[4], i_lo[4], r_c[4], i_c[4];
+};
+__device__ __forceinline__ void sep_store_f(const SepF& f, uint32_t dst, uint32_t block, uint32_t level) {
+  uint32_t m[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) m[k] = f.i_hi[k] ^ 0x80008000u;
+  sts128(dst, m);
+  sts128(dst + block, f.r_hi);
+  sts128(dst + 2 * block, f.i_hi);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) m[k] = f.i_lo[k] ^ 0x80008000u;
+  sts128(dst + level, m);
+  sts128(dst + level + block, f.r_lo);
+  sts128(dst + level + 2 * block, f.i_lo);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) m[k] = f.i_c[k] ^ 0x80008000u;
+  sts128(dst + 2 * level, m);
+  sts128(dst + 2 * level + block, f.r_c);
+  sts128(dst + 2 * level + 2 * block, f.i_c);
+}
+
+// (cos, sin)(2 pi w_ref n') from the two-float n' (exact range reduction)
+__device__ __forceinline__ float2 sep_w_phasor(float w_ref, float2 n1) {
+  const float t = w_ref * n1.x;
+  const float lo = fmaf(w_ref, n1.y, fmaf(w_ref, n1.x, -t));
+  const float ang = ((t - rintf(t)) + lo) * kTwoPiF;
+  float s, c;
+  __sincosf(ang, &s, &c);
+  return make_float2(c, s);
+}
+
+}  // namespace idg
