@@ -19,9 +19,10 @@ SOURCES = (["planner.cpp", "gridder.cu", "fft.cu", "degridder.cu", "idg_api.cu",
            + [f"gridder_l{L}.cu" for L in (32, 64, 96, 128)] + [f"degridder_l{L}.cu" for L in (32, 64, 96, 128)]
            + [f"degridder_tc_l{L}.cu" for L in (32, 64, 96, 128)]
            + [f"gridder_tc_l{L}.cu" for L in (32, 64, 96, 128)]
-           + [f"gridder_sep_l{L}.cu" for L in (32, 64, 96, 128)])
+           + [f"{k}_sep_l{L}.cu" for k in ("gridder", "degridder") for L in (32, 64, 96, 128)])
 HEADERS = ["idg_internal.h", "kernels_common.cuh", "gridder_kernels.cuh", "degridder_kernels.cuh",
-           "degridder_tc_kernels.cuh", "gridder_tc_kernels.cuh", "sep_common.cuh", "gridder_sep_kernels.cuh"]
+           "degridder_tc_kernels.cuh", "gridder_tc_kernels.cuh", "sep_common.cuh", "gridder_sep_kernels.cuh",
+           "degridder_sep_kernels.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else "nvcc")
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=off,-fno-fast-math",

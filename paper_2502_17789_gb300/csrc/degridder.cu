@@ -67,6 +67,57 @@ IDG_DEGRID_TC_EXTERN(96)
 IDG_DEGRID_TC_EXTERN(128)
 #undef IDG_DEGRID_TC_EXTERN
 
+template <int L>
+int degridder_sep_vis_l(int nodes);
+template <int L>
+int configure_degridder_sep_l(int* persistent_blocks);
+template <int L>
+int launch_degridder_sep_l(const DegridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
+template <int L>
+int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
+#define IDG_DEGRID_SEP_EXTERN(L)                                                                                 \
+  extern template int degridder_sep_vis_l<L>(int);                                                              \
+  extern template int configure_degridder_sep_l<L>(int*);                                                       \
+  extern template int launch_degridder_sep_l<L>(const DegridArgs&, int, int, int, void*);                       \
+  extern template int launch_degridder_sep_multi_l<L>(const DegridArgs*, const int2*, int, int, void*);
+IDG_DEGRID_SEP_EXTERN(32)
+IDG_DEGRID_SEP_EXTERN(64)
+IDG_DEGRID_SEP_EXTERN(96)
+IDG_DEGRID_SEP_EXTERN(128)
+#undef IDG_DEGRID_SEP_EXTERN
+
+#define IDG_SWITCH_L(CALL)                 \
+  switch (L) {                             \
+    case 32: return CALL(32);              \
+    case 64: return CALL(64);              \
+    case 96: return CALL(96);              \
+    case 128: return CALL(128);            \
+    default: return int(cudaErrorInvalidValue); \
+  }
+
+int degridder_sep_vis(int L, int nodes) {
+#define C_(X) degridder_sep_vis_l<X>(nodes)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int configure_degridder_sep(int L, int* persistent_blocks) {
+#define C_(X) configure_degridder_sep_l<X>(persistent_blocks)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream) {
+#define C_(X) launch_degridder_sep_l<X>(a, n_items, persistent_blocks, bundle, stream)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
+                               void* stream) {
+#define C_(X) launch_degridder_sep_multi_l<X>(args, items, n_items, max_nodes, stream)
+  IDG_SWITCH_L(C_)
+#undef C_
+}
+#undef IDG_SWITCH_L
+
 int launch_degridder_tc(int L, const DegridArgs& a, int n_items, int persistent_blocks, void* stream) {
   switch (L) {
     case 32: return launch_degridder_tc_l<32>(a, n_items, persistent_blocks, stream);

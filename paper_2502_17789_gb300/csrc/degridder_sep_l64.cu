@@ -1,0 +1,11 @@
+// Separable-phasor degridder kernels for subgrid size 64 (templates in degridder_sep_kernels.cuh).
+#include "degridder_sep_kernels.cuh"
+
+namespace idg {
+
+template int configure_degridder_sep_l<64>(int*);
+template int degridder_sep_vis_l<64>(int);
+template int launch_degridder_sep_l<64>(const DegridArgs&, int, int, int, void*);
+template int launch_degridder_sep_multi_l<64>(const DegridArgs*, const int2*, int, int, void*);
+
+}  // namespace idg

@@ -13,7 +13,7 @@
 // Stockham autosort sequence of radix-4/2/3 stages.  Every stage reads its
 // butterflies into registers, synchronises, and writes them back, so one
 // L x L buffer suffices.
-#include "kernels_common.cuh"
+#include "sep_common.cuh"
 
 namespace idg {
 
@@ -206,7 +206,33 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_blocks(L)) splitter_ifft_
   fft2d<L, +1>(buf, tw);
   float4* dst = reinterpret_cast<float4*>(a.scratch + (size_t(sgi) * 4 + pol) * L * L);
   const float4* b4 = reinterpret_cast<const float4*>(buf);
-  for (int e = threadIdx.x; e < L * L / 2; e += kFftThreads) dst[e] = b4[e];
+  if (!a.ymax) {
+    for (int e = threadIdx.x; e < L * L / 2; e += kFftThreads) dst[e] = b4[e];
+    return;
+  }
+  // what every visibility of the subgrid shares (sep_common.cuh), once per pixel here instead of once per segment
+  const float w_ref = a.w_ref[sgi];
+  float m = 0.f;
+  for (int e = threadIdx.x; e < L * L / 2; e += kFftThreads) {
+    const int j = 2 * e / L, i = 2 * e - j * L;
+    float4 v = b4[e];
+    const float4 n = __ldg(reinterpret_cast<const float4*>(a.n1) + e);
+    const float tj = a.taper[j] * ((j & 1) ? -1.f : 1.f), t0 = tj * a.taper[i], t1 = -tj * a.taper[i + 1];
+    const float2 p0 = sep_w_phasor(w_ref, make_float2(n.x, n.y)), p1 = sep_w_phasor(w_ref, make_float2(n.z, n.w));
+    v = make_float4(t0 * (v.x * p0.x + v.y * p0.y), t0 * (v.y * p0.x - v.x * p0.y), t1 * (v.z * p1.x + v.w * p1.y),
+                    t1 * (v.w * p1.x - v.z * p1.y));
+    m = fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+    dst[e] = v;
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  float* part = reinterpret_cast<float*>(tw);  // the twiddles are done with
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kFftThreads / 32; ++w) m = fmaxf(m, part[w]);
+    a.ymax[sgi * 4 + pol] = m;
+  }
 }
 
 // plan-order export of subgrid images for inspection, undoing (-1)^(x+y)

@@ -192,25 +192,33 @@ int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const fl
   return int(cudaGetLastError());
 }
 
-// one warp per (interval, station): are all off-diagonal node entries zero?
-__global__ void aterm_flags_kernel(const float2* aterms, uint8_t* flags, int n_pairs, int nodes) {
+// one warp per (interval, station): are all off-diagonal node entries zero, and the largest component
+__global__ void aterm_flags_kernel(const float2* aterms, uint8_t* flags, float* amax, int n_pairs, int nodes) {
   const int pair = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (pair >= n_pairs) return;
-  const float2* A = aterms + size_t(pair) * nodes * nodes * 4;
+  const float4* A = reinterpret_cast<const float4*>(aterms + size_t(pair) * nodes * nodes * 4);
   bool diag = true;
+  float m = 0.f;
   for (int n = lane; n < nodes * nodes; n += 32) {
-    const float2 b = A[n * 4 + 1], c = A[n * 4 + 2];
-    diag = diag && b.x == 0.f && b.y == 0.f && c.x == 0.f && c.y == 0.f;
+    const float4 a = A[2 * n], b = A[2 * n + 1];  // (00, 01) (10, 11)
+    diag = diag && a.z == 0.f && a.w == 0.f && b.x == 0.f && b.y == 0.f;
+    m = fmaxf(fmaxf(fmaxf(m, fabsf(a.x)), fmaxf(fabsf(a.y), fabsf(a.z))),
+              fmaxf(fmaxf(fabsf(a.w), fabsf(b.x)), fmaxf(fmaxf(fabsf(b.y), fabsf(b.z)), fabsf(b.w))));
   }
   diag = __all_sync(0xffffffffu, diag);
-  if (lane == 0) flags[pair] = diag ? 1 : 0;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) {
+    flags[pair] = diag ? 1 : 0;
+    if (amax) amax[pair] = m;
+  }
 }
 
-int launch_aterm_flags(const float2* aterms, uint8_t* flags, int n_int, int n_st, int nodes, void* stream) {
+int launch_aterm_flags(const float2* aterms, uint8_t* flags, float* amax, int n_int, int n_st, int nodes, void* stream) {
   const int n = n_int * n_st;
   if (n <= 0) return 0;
-  aterm_flags_kernel<<<(n + 7) / 8, 256, 0, cudaStream_t(stream)>>>(aterms, flags, n, nodes);
+  aterm_flags_kernel<<<(n + 7) / 8, 256, 0, cudaStream_t(stream)>>>(aterms, flags, amax, n, nodes);
   return int(cudaGetLastError());
 }
 

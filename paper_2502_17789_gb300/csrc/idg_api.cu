@@ -54,6 +54,9 @@ struct idg_plan {
   int32_t mac = IDG_MAC_FP32;        // multiply-accumulate unit of the degridder
   bool uniform = true;               // channels uniformly spaced
   bool grid_sep = false;             // separable-phasor gridder (sep_common.cuh)
+  bool degrid_sep = false;           // and degridder
+  int32_t degrid_vis = 0;            // its visibilities per item
+  int32_t sms = 1;
   bool grid_tc = false;              // gridder on the tensor cores without it (mac, uniform channels, no A-term normalisation)
   cudaStream_t stream = nullptr;
   bool host_only = false;
@@ -87,6 +90,8 @@ struct idg_plan {
   float* d_sep = nullptr;       // [4][L] separable-phasor tables a, b, p, q
   float2* d_n1 = nullptr;       // [L*L] n' as two floats
   float* d_wref = nullptr;      // [exec subgrids] reference w
+  float* d_amax = nullptr;      // [n_int][n_st] largest A-term component of the current call (degrid_sep)
+  float* d_ymax = nullptr;      // [batch capacity][4] largest component of the split subgrid planes (degrid_sep)
   double* d_aweights = nullptr; // [L*L + 1] A-term power weights (IDG_NORMALIZE_ATERM)
   // image-domain wrapper, made at its first use
   cufftHandle fft = 0;
@@ -177,7 +182,8 @@ void free_device(idg_plan* p) {
   p->graph_degrid = {};
   void* ptrs[] = {p->d_uvw,    p->d_fscale, p->d_taper,   p->d_blk,     p->d_twiddle, p->d_sg,     p->d_seg,
                   p->d_gitems, p->d_ditems, p->d_scratch, p->d_records, p->d_status,  p->d_queue,
-                  p->d_adiag,  p->d_blk16, p->d_inv_t, p->d_aweights, p->d_sep, p->d_n1, p->d_wref};
+                  p->d_adiag,  p->d_blk16, p->d_inv_t, p->d_aweights, p->d_sep, p->d_n1, p->d_wref,
+                  p->d_amax,   p->d_ymax};
   // stream-ordered frees: no device-wide synchronisation, so plans of other
   // streams keep running while this one is released
   for (void* q : ptrs)
@@ -202,6 +208,8 @@ void free_device(idg_plan* p) {
   p->d_sep = nullptr;
   p->d_n1 = nullptr;
   p->d_wref = nullptr;
+  p->d_amax = nullptr;
+  p->d_ymax = nullptr;
 }
 
 // Block geometry table, FP64 -> FP32: for each row j and block ib of 8
@@ -515,6 +523,8 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       uniform = std::fabs(sc - s1) <= 1e-12 * std::fabs(s1);
     }
     p->uniform = uniform;
+    p->degrid_sep = p->mac != IDG_MAC_FP32 && sep_ok;
+    if (p->degrid_sep) p->degrid_vis = degridder_sep_vis(L, g->aterm_nodes);
     p->grid_sep = p->mac == IDG_MAC_TENSOR && sep_ok && !(g->flags & IDG_NORMALIZE_ATERM);
     p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && uniform && !(g->flags & IDG_NORMALIZE_ATERM);
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
@@ -579,6 +589,19 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     const size_t d_first = ditems.size();
     for (int32_t o : order) {
       const SubgridDesc& d = p->exec[s0 + o];
+      if (p->degrid_sep) {
+        // equal pieces of each segment, each a multiple of 8 visibilities but for the last
+        for (int gidx = d.seg_begin; gidx < d.seg_begin + d.seg_count; ++gidx) {
+          const SegmentDesc& sgd = p->part.segments[gidx];
+          const int n = sgd.k_end - sgd.k_begin, pieces = (n + p->degrid_vis - 1) / p->degrid_vis;
+          const int len = ((n + pieces - 1) / pieces + 7) / 8 * 8;
+          for (int k = sgd.k_begin; k < sgd.k_end; k += len) {
+            const int ke = std::min(k + len, sgd.k_end);
+            ditems.push_back(DegridItem{o, gidx, k, ke, ke, 0});
+          }
+        }
+        continue;
+      }
       const int width = d.c1 - d.c0;
       const int G = (width + p->degrid_channels - 1) / p->degrid_channels;
       bool open = false;  // the last item can take a piece of the next segment
@@ -602,10 +625,9 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     }
     // items of at most kSplitLanes lanes go last, for the kernel that spreads a visibility over
     // several lanes; both parts keep the longest-first order
-    std::stable_partition(ditems.begin() + d_first, ditems.end(),
-                          [](const DegridItem& it) { return it.k_end - it.k_begin > kSplitLanes; });
-    size_t n_small = 0;
-    for (size_t i = d_first; i < ditems.size(); ++i) n_small += ditems[i].k_end - ditems[i].k_begin <= kSplitLanes;
+    const auto few = [&](const DegridItem& it) { return !p->degrid_sep && it.k_end - it.k_begin <= kSplitLanes; };
+    std::stable_partition(ditems.begin() + d_first, ditems.end(), [&](const DegridItem& it) { return !few(it); });
+    const size_t n_small = size_t(std::count_if(ditems.begin() + d_first, ditems.end(), few));
     b.gi_count = int32_t(gitems.size()) - b.gi_offset;
     b.ds_count = int32_t(n_small);
     b.di_count = int32_t(ditems.size()) - b.di_offset - b.ds_count;
@@ -640,7 +662,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   if (!e && p->grid_sep) e = configure_gridder_sep(L, &pg);
   // the FP32 kernels serve the items of few visibilities in either mode
   if (!e) e = configure_degridder(L, g->aterm_nodes, p->degrid_channels, &pd);
-  if (!e && p->mac != IDG_MAC_FP32) e = configure_degridder_tc(L, g->aterm_nodes, &pd);
+  if (!e && p->mac != IDG_MAC_FP32 && !p->degrid_sep) e = configure_degridder_tc(L, g->aterm_nodes, &pd);
+  if (!e && p->degrid_sep) {
+    int dev = 0;
+    e = configure_degridder_sep(L, &pd);
+    if (!e) e = int(cudaGetDevice(&dev));
+    if (!e) e = int(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev));
+  }
   if (g->flags & IDG_PERSISTENT) {
     p->persistent_grid_blocks = pg;
     p->persistent_degrid_blocks = pd;
@@ -651,7 +679,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   if (!e) e = upload(p, &p->d_blk, blk.data(), blk.size());
   if (!e) e = upload(p, &p->d_blk16, blk16.data(), blk16.size());
   if (!e) e = upload(p, &p->d_twiddle, tw.data(), tw.size());
-  if (!e && p->grid_sep) {
+  if (!e && p->degrid_sep) {
+    const size_t na = size_t(n_intervals) * std::max(1, n_stations), ny = size_t(4) * p->batch_cap;
+    e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_amax), na * sizeof(float), p->stream));
+    if (!e) e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_ymax), ny * sizeof(float), p->stream));
+    if (!e) p->device_bytes += int64_t((na + ny) * sizeof(float));
+  }
+  if (!e && (p->grid_sep || p->degrid_sep)) {
     e = upload(p, &p->d_sep, sep.tab.data(), sep.tab.size());
     if (!e) e = upload(p, &p->d_n1, sep.n1.data(), sep.n1.size());
     if (!e) e = upload(p, &p->d_wref, w_ref.data(), w_ref.size());
@@ -784,7 +818,7 @@ idg_status idg_grid(idg_plan* plan, const void* vis_c64, const void* aterms_c64,
   const int L = plan->L;
   {
     const int e = timed(plan, kFlags, [&] {
-      return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->n_int, plan->n_st,
+      return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->d_amax, plan->n_int, plan->n_st,
                                 plan->geom.aterm_nodes, plan->stream);
     });
     if (e) return cuda_err(plan, e, "A-term flag launch");
@@ -812,6 +846,50 @@ idg_status idg_grid(idg_plan* plan, const void* vis_c64, const void* aterms_c64,
   return IDG_OK;
 }
 
+static FftArgs splitter_args(const idg_plan* p, const Batch& b, const void* grid_c128) {
+  FftArgs fa{p->d_sg + b.sg_offset, p->d_scratch, const_cast<double2*>(static_cast<const double2*>(grid_c128)),
+             p->d_twiddle, p->N, p->npol};
+  if (p->degrid_sep) {
+    fa.ymax = p->d_ymax;
+    fa.w_ref = p->d_wref + b.sg_offset;
+    fa.taper = p->d_taper;
+    fa.n1 = p->d_n1;
+  }
+  return fa;
+}
+
+static DegridArgs degrid_args(const idg_plan* p, const Batch& b, const void* aterms, void* vis) {
+  DegridArgs da{};
+  da.adiag = p->d_adiag;
+  da.n_items = b.di_count;
+  da.vis = static_cast<float4*>(vis);
+  da.uvw = p->d_uvw;
+  da.fscale = p->d_fscale;
+  da.aterms = static_cast<const float2*>(aterms);
+  da.sg = p->d_sg + b.sg_offset;
+  da.seg = p->d_seg;
+  da.items = p->d_ditems + b.di_offset;
+  da.taper = p->d_taper;
+  da.blk16 = p->d_blk16;
+  da.scratch = p->d_scratch;
+  da.g = kgeom(p);
+  if (p->degrid_sep) {
+    da.status = p->d_status;
+    da.amax = p->d_amax;
+    da.ymax = p->d_ymax;
+    da.w_ref = p->d_wref + b.sg_offset;
+    da.kv = p->degrid_vis;
+    da.sep = sep_tables(p);
+  }
+  return da;
+}
+
+// items per block of the separable-phasor degridder: some blocks per SM must remain to even out the load, and
+// more items per block than that spread the block's set-up
+static int degrid_bundle(const idg_plan* p, int n_items) {
+  return std::max(1, std::min(8, n_items / (8 * std::max(1, int(p->sms)))));
+}
+
 idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_c64, void* vis_c64) {
   if (!plan) return set_err(nullptr, IDG_ERR_INVALID_ARG, "plan is NULL");
   if (plan->host_only) return set_err(plan, IDG_ERR_INVALID_ARG, "plan was created with IDG_HOST_ONLY");
@@ -827,7 +905,7 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
   }
   {
     const int e = timed(plan, kFlags, [&] {
-      return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->n_int, plan->n_st,
+      return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->d_amax, plan->n_int, plan->n_st,
                                 plan->geom.aterm_nodes, plan->stream);
     });
     if (e) return cuda_err(plan, e, "A-term flag launch");
@@ -838,26 +916,15 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
   }
   for (size_t bi = 0; bi < plan->batches.size(); ++bi) {
     const Batch& b = plan->batches[bi];
-    FftArgs fa{plan->d_sg + b.sg_offset, plan->d_scratch, const_cast<double2*>(static_cast<const double2*>(grid_c128)),
-               plan->d_twiddle, plan->N, plan->npol};
+    const FftArgs fa = splitter_args(plan, b, grid_c128);
     int e = timed(plan, kSplitter, [&] { return launch_splitter_ifft(L, fa, b.sg_count, plan->stream); });
     if (e) return cuda_err(plan, e, "splitter/ifft launch");
-    DegridArgs da{};
-    da.adiag = plan->d_adiag;
+    DegridArgs da = degrid_args(plan, b, aterms_c64, vis_c64);
     da.queue = plan->d_queue + 2 * bi + 1;
-    da.n_items = b.di_count;
-    da.vis = static_cast<float4*>(vis_c64);
-    da.uvw = plan->d_uvw;
-    da.fscale = plan->d_fscale;
-    da.aterms = static_cast<const float2*>(aterms_c64);
-    da.sg = plan->d_sg + b.sg_offset;
-    da.seg = plan->d_seg;
-    da.items = plan->d_ditems + b.di_offset;
-    da.taper = plan->d_taper;
-    da.blk16 = plan->d_blk16;
-    da.scratch = plan->d_scratch;
-    da.g = kgeom(plan);
     e = timed(plan, kDegridder, [&] {
+      if (plan->degrid_sep)
+        return launch_degridder_sep(L, da, b.di_count, plan->persistent_degrid_blocks,
+                                    degrid_bundle(plan, b.di_count), plan->stream);
       if (plan->mac != IDG_MAC_FP32)
         return launch_degridder_tc(L, da, b.di_count, plan->persistent_degrid_blocks, plan->stream);
       return launch_degridder(L, plan->degrid_channels, da, b.di_count, plan->persistent_degrid_blocks,
@@ -891,7 +958,7 @@ idg_status idg_subgrid_images(idg_plan* plan, const void* vis_c64, const void* a
   int e = int(cudaMemsetAsync(out_c64, 0, total, plan->stream));
   if (e) return cuda_err(plan, e, "zeroing output");
   e = timed(plan, kFlags, [&] {
-    return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->n_int, plan->n_st,
+    return launch_aterm_flags(static_cast<const float2*>(aterms_c64), plan->d_adiag, plan->d_amax, plan->n_int, plan->n_st,
                               plan->geom.aterm_nodes, plan->stream);
   });
   if (e) return cuda_err(plan, e, "A-term flag launch");
@@ -1039,7 +1106,7 @@ idg_status idg_grid_many(int32_t n, idg_plan* const* plans, const void* const* v
     idg_plan* p = plans[k];
     n_waves = std::max(n_waves, p->batches.size());
     max_nodes = std::max(max_nodes, int(p->geom.aterm_nodes));
-    const int e = launch_aterm_flags(static_cast<const float2*>(aterms_c64[k]), p->d_adiag, p->n_int, p->n_st,
+    const int e = launch_aterm_flags(static_cast<const float2*>(aterms_c64[k]), p->d_adiag, p->d_amax, p->n_int, p->n_st,
                                      p->geom.aterm_nodes, strm);
     if (e) return cuda_err(p, e, "A-term flag launch");
   }
@@ -1109,7 +1176,7 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
       const int e = int(cudaMemsetAsync(vis_c64[k], 0, bytes, strm));
       if (e) return cuda_err(p, e, "zeroing dropped visibilities");
     }
-    const int e = launch_aterm_flags(static_cast<const float2*>(aterms_c64[k]), p->d_adiag, p->n_int, p->n_st,
+    const int e = launch_aterm_flags(static_cast<const float2*>(aterms_c64[k]), p->d_adiag, p->d_amax, p->n_int, p->n_st,
                                      p->geom.aterm_nodes, strm);
     if (e) return cuda_err(p, e, "A-term flag launch");
   }
@@ -1117,50 +1184,43 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
     std::vector<DegridArgs> args;
     std::vector<const int32_t*> cost, cost_s;
     std::vector<int32_t> count, count_s;
+    std::vector<char> slot_sep;
     for (int32_t k = 0; k < n; ++k) {
       idg_plan* p = plans[k];
       if (w >= p->batches.size()) continue;
       const Batch& b = p->batches[w];
-      FftArgs fa{p->d_sg + b.sg_offset, p->d_scratch,
-                 const_cast<double2*>(static_cast<const double2*>(grid_c128[k])), p->d_twiddle, p->N, p->npol};
+      const FftArgs fa = splitter_args(p, b, grid_c128[k]);
       const int e = launch_splitter_ifft(L, fa, b.sg_count, strm);
       if (e) return cuda_err(p, e, "splitter/ifft launch");
-      DegridArgs da{};
-      da.adiag = p->d_adiag;
-      da.n_items = b.di_count;
-      da.vis = static_cast<float4*>(vis_c64[k]);
-      da.uvw = p->d_uvw;
-      da.fscale = p->d_fscale;
-      da.aterms = static_cast<const float2*>(aterms_c64[k]);
-      da.sg = p->d_sg + b.sg_offset;
-      da.seg = p->d_seg;
-      da.items = p->d_ditems + b.di_offset;
-      da.taper = p->d_taper;
-      da.blk16 = p->d_blk16;
-      da.scratch = p->d_scratch;
-      da.g = kgeom(p);
+      const DegridArgs da = degrid_args(p, b, aterms_c64[k], vis_c64[k]);
+      slot_sep.push_back(p->degrid_sep);
       args.push_back(da);
       cost.push_back(p->dcost.data() + b.di_offset);
       count.push_back(b.di_count);
       cost_s.push_back(p->dcost.data() + b.di_offset + b.di_count);
       count_s.push_back(b.ds_count);
     }
-    // regular items, then the items of few lanes; the latter index their plan's item table past
-    // the regular ones
-    std::vector<int2> items = merge_items(cost, count);
-    const size_t n_regular = items.size();
+    // items of the plans with the separable form, regular items of the others, then the items of few lanes;
+    // the latter index their plan's item table past the regular ones
+    std::vector<int32_t> count_sep = count, count_r = count;
+    for (size_t s = 0; s < count.size(); ++s) (slot_sep[s] ? count_r : count_sep)[s] = 0;
+    std::vector<int2> items = merge_items(cost, count_sep);
+    const size_t n_sep = items.size();
+    for (int2 it : merge_items(cost, count_r)) items.push_back(it);
+    const size_t n_regular = items.size() - n_sep;
     for (int2 it : merge_items(cost_s, count_s)) items.push_back(make_int2(it.x, count[it.x] + it.y));
     DegridArgs* d_args = nullptr;
     int2* d_items = nullptr;
     int e = upload_wave(strm, args, items, &d_args, &d_items);
+    if (!e) e = launch_degridder_sep_multi(L, d_args, d_items, int(n_sep), max_nodes, strm);
     if (!e)
       e = plans[0]->mac != IDG_MAC_FP32
-              ? launch_degridder_tc_multi(L, d_args, d_items, int(n_regular), max_nodes, strm)
-              : launch_degridder_multi(L, plans[0]->degrid_channels, false, d_args, d_items, int(n_regular),
+              ? launch_degridder_tc_multi(L, d_args, d_items + n_sep, int(n_regular), max_nodes, strm)
+              : launch_degridder_multi(L, plans[0]->degrid_channels, false, d_args, d_items + n_sep, int(n_regular),
                                        max_nodes, strm);
-    if (!e && items.size() > n_regular)
-      e = launch_degridder_multi(L, plans[0]->degrid_channels, true, d_args, d_items + n_regular,
-                                 int(items.size() - n_regular), max_nodes, strm);
+    if (!e && items.size() > n_sep + n_regular)
+      e = launch_degridder_multi(L, plans[0]->degrid_channels, true, d_args, d_items + n_sep + n_regular,
+                                 int(items.size() - n_sep - n_regular), max_nodes, strm);
     if (d_args) cudaFreeAsync(d_args, strm);
     if (d_items) cudaFreeAsync(d_items, strm);
     if (e) return cuda_err(plans[0], e, "degridder launch (several plans)");

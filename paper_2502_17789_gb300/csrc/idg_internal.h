@@ -254,6 +254,13 @@ struct DegridArgs {
   const float* taper;
   const float4* blk16;        // [L][L/16][5] 16-pixel block geometry (n0, anchor offsets) (dn[0..15])
   const float2* scratch;      // [batch][4][L][L] subgrid images Y
+  // separable-phasor degridder
+  int* status = nullptr;          // device status word (kStatusTimeout)
+  const float* amax = nullptr;    // [n_int][n_st] largest component of the A-term's nodes
+  const float* ymax = nullptr;    // [batch subgrids][4] largest component of the subgrid's planes
+  const float* w_ref = nullptr;   // [batch subgrids] reference w
+  int kv = 0;                     // visibilities per item
+  SepTables sep;
   KernelGeom g;
 };
 
@@ -264,6 +271,12 @@ struct FftArgs {
   const float2* twiddle;   // [L] e^{-2 pi i m / L}
   int32_t N;
   int32_t npol = 4;        // planes per subgrid transformed and added / split (4, or 1 for Stokes I)
+  // splitter of separable-phasor plans (ymax set): the image times taper, centring sign and
+  // e^{-2 pi i w_ref n'}, and each plane's largest component
+  float* ymax = nullptr;   // [batch subgrids][4]
+  const float* w_ref = nullptr;
+  const float* taper = nullptr;
+  const float2* n1 = nullptr;
 };
 
 // Launchers (return cudaError_t as int).  `n` is the item or subgrid count.
@@ -290,8 +303,9 @@ int launch_image_pass(int npol, const double2* in, double2* out, const double* w
                       int flags, void* stream);
 // one warp waits, bounded by limit_ns, on an mbarrier nothing completes; sets kStatusTimeout bit in *status
 int launch_wait_selftest(int* status, int64_t limit_ns, void* stream);
-// flags[i][s] = 1 when every node of A-term (interval i, station s) has zero off-diagonal entries
-int launch_aterm_flags(const float2* aterms, uint8_t* flags, int n_int, int n_st, int nodes, void* stream);
+// flags[i][s] = 1 when every node of A-term (interval i, station s) has zero off-diagonal entries;
+// amax[i][s] (may be null) its largest component
+int launch_aterm_flags(const float2* aterms, uint8_t* flags, float* amax, int n_int, int n_st, int nodes, void* stream);
 // split: the items are of at most kSplitLanes lanes and run in the kernel that spreads each
 // visibility's pixels over several lanes (one block per item; persistent_blocks is ignored)
 int launch_degridder(int L, int channels, const DegridArgs& a, int n_items, int persistent_blocks, void* stream,
@@ -314,6 +328,12 @@ int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int
 int configure_degridder_tc(int L, int nodes, int* persistent_blocks);
 int launch_degridder_tc_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
                               void* stream);
+// the separable-phasor degridder: items of up to degridder_sep_vis visibilities of one segment, `bundle` of them per block
+int degridder_sep_vis(int L, int nodes);
+int configure_degridder_sep(int L, int* persistent_blocks);
+int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
+int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
+                               void* stream);
 // mode 0: FFT + add into grid; mode 1: FFT in place in scratch (inspection)
 int launch_fft_adder(int L, const FftArgs& a, int n_subgrids, int mode, void* stream);
 int launch_splitter_ifft(int L, const FftArgs& a, int n_subgrids, void* stream);
