@@ -663,10 +663,10 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   // the FP32 kernels serve the items of few visibilities in either mode
   if (!e) e = configure_degridder(L, g->aterm_nodes, p->degrid_channels, &pd);
   if (!e && p->mac != IDG_MAC_FP32 && !p->degrid_sep) e = configure_degridder_tc(L, g->aterm_nodes, &pd);
-  if (!e && p->degrid_sep) {
+  if (!e && p->degrid_sep) e = configure_degridder_sep(L, &pd);
+  if (!e && (p->grid_sep || p->degrid_sep)) {
     int dev = 0;
-    e = configure_degridder_sep(L, &pd);
-    if (!e) e = int(cudaGetDevice(&dev));
+    e = int(cudaGetDevice(&dev));
     if (!e) e = int(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev));
   }
   if (g->flags & IDG_PERSISTENT) {
@@ -794,6 +794,12 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
   return ga;
 }
 
+// items per block of the separable-phasor kernels: some blocks per SM must remain to even out the load, and
+// more items per block than that spread the block's set-up
+static int sep_bundle(const idg_plan* p, int n_items) {
+  return std::max(1, std::min(8, n_items / (8 * std::max(1, int(p->sms)))));
+}
+
 // record staging and the gridder of the plan's kind (FP32 pipe or tensor cores)
 static int stage_any(const idg_plan* p, const Batch& b, const void* vis, cudaStream_t strm) {
   if (p->grid_sep)
@@ -803,7 +809,7 @@ static int stage_any(const idg_plan* p, const Batch& b, const void* vis, cudaStr
 }
 
 static int gridder_any(const idg_plan* p, const GridArgs& ga, int n_items, int persistent_blocks, cudaStream_t strm) {
-  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, persistent_blocks, strm);
+  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, persistent_blocks, sep_bundle(p, n_items), strm);
   return p->grid_tc ? launch_gridder_tc(p->L, ga, n_items, persistent_blocks, strm)
                     : launch_gridder(p->L, ga, n_items, persistent_blocks, strm);
 }
@@ -884,12 +890,6 @@ static DegridArgs degrid_args(const idg_plan* p, const Batch& b, const void* ate
   return da;
 }
 
-// items per block of the separable-phasor degridder: some blocks per SM must remain to even out the load, and
-// more items per block than that spread the block's set-up
-static int degrid_bundle(const idg_plan* p, int n_items) {
-  return std::max(1, std::min(8, n_items / (8 * std::max(1, int(p->sms)))));
-}
-
 idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_c64, void* vis_c64) {
   if (!plan) return set_err(nullptr, IDG_ERR_INVALID_ARG, "plan is NULL");
   if (plan->host_only) return set_err(plan, IDG_ERR_INVALID_ARG, "plan was created with IDG_HOST_ONLY");
@@ -924,7 +924,7 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
     e = timed(plan, kDegridder, [&] {
       if (plan->degrid_sep)
         return launch_degridder_sep(L, da, b.di_count, plan->persistent_degrid_blocks,
-                                    degrid_bundle(plan, b.di_count), plan->stream);
+                                    sep_bundle(plan, b.di_count), plan->stream);
       if (plan->mac != IDG_MAC_FP32)
         return launch_degridder_tc(L, da, b.di_count, plan->persistent_degrid_blocks, plan->stream);
       return launch_degridder(L, plan->degrid_channels, da, b.di_count, plan->persistent_degrid_blocks,

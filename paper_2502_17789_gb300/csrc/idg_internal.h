@@ -322,7 +322,7 @@ int configure_gridder_tc(int L, int* persistent_blocks);
 int launch_gridder_tc_multi(int L, const GridArgs* args, const int2* items, int n_items, void* stream);
 // the separable-phasor gridder (records staged by launch_stage_sep; any channel spacing)
 int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids, void* stream);
-int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, void* stream);
+int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
 int configure_gridder_sep(int L, int* persistent_blocks);
 int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
 int configure_degridder_tc(int L, int nodes, int* persistent_blocks);

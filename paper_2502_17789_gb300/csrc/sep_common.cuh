@@ -67,15 +67,52 @@ __device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t cols) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld4(float (&v)[4], uint32_t addr) {
-  uint32_t r[4];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+__device__ __forceinline__ void tmem_ld8(float (&v)[8], uint32_t addr) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(addr));
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = __uint_as_float(r[k]);
+  for (int k = 0; k < 8; ++k) v[k] = __uint_as_float(r[k]);
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ---------------------------------------------------------------- roles
+
+// The block's first 256 threads (producers) write operands and issue MMAs, the
+// others (consumers) read the accumulators; each half has its own barrier.
+constexpr int kSepHalf = 256;
+constexpr int kSepProducerBar = 1, kSepConsumerBar = 2;
+__device__ __forceinline__ void half_sync(int bar) {
+  asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// the 65536 registers of the launch (512 threads x 128) split between the halves: REGS + 256 - REGS
+template <int REGS>
+__device__ __forceinline__ void regs_take() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+template <int REGS>
+__device__ __forceinline__ void regs_give() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+
+// bounded wait that reports a timeout once and then lets every later wait of the block pass
+__device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, int* status) {
+  if (mbar_try_wait(bar, parity)) return;
+  if (*reinterpret_cast<volatile int*>(fail)) return;
+  if (!mbar_wait_bounded(bar, parity)) {
+    atomicOr(status, kStatusTimeout);
+    *reinterpret_cast<volatile int*>(fail) = 1;
+  }
+}
+
+// complex numbers of two pixels, for packed f32x2 arithmetic
+struct c2 {
+  float2 re, im;
+};
 
 // ---------------------------------------------------------------- operands
 
