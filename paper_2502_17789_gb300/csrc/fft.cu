@@ -210,19 +210,22 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_blocks(L)) splitter_ifft_
     for (int e = threadIdx.x; e < L * L / 2; e += kFftThreads) dst[e] = b4[e];
     return;
   }
-  // what every visibility of the subgrid shares (sep_common.cuh), once per pixel here instead of once per segment
+  // what every visibility of the subgrid shares (sep_common.cuh), once per pixel here instead of once per segment;
+  // written as the degridder reads it, [row pair][re, im][column] of the values at both rows
   const float w_ref = a.w_ref[sgi];
+  float2* pairs = a.scratch + (size_t(sgi) * 4 + pol) * L * L;
   float m = 0.f;
   for (int e = threadIdx.x; e < L * L / 2; e += kFftThreads) {
-    const int j = 2 * e / L, i = 2 * e - j * L;
-    float4 v = b4[e];
-    const float4 n = __ldg(reinterpret_cast<const float4*>(a.n1) + e);
-    const float tj = a.taper[j] * ((j & 1) ? -1.f : 1.f), t0 = tj * a.taper[i], t1 = -tj * a.taper[i + 1];
-    const float2 p0 = sep_w_phasor(w_ref, make_float2(n.x, n.y)), p1 = sep_w_phasor(w_ref, make_float2(n.z, n.w));
-    v = make_float4(t0 * (v.x * p0.x + v.y * p0.y), t0 * (v.y * p0.x - v.x * p0.y), t1 * (v.z * p1.x + v.w * p1.y),
-                    t1 * (v.w * p1.x - v.z * p1.y));
-    m = fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
-    dst[e] = v;
+    const int jp = e / L, i = e - jp * L;
+    const float2 v0 = buf[2 * jp * L + i], v1 = buf[(2 * jp + 1) * L + i];
+    const float ti = a.taper[i] * ((i & 1) ? -1.f : 1.f), t0 = ti * a.taper[2 * jp], t1 = -ti * a.taper[2 * jp + 1];
+    const float2 p0 = sep_w_phasor(w_ref, __ldg(a.n1 + 2 * jp * L + i));
+    const float2 p1 = sep_w_phasor(w_ref, __ldg(a.n1 + (2 * jp + 1) * L + i));
+    const float2 re = make_float2(t0 * (v0.x * p0.x + v0.y * p0.y), t1 * (v1.x * p1.x + v1.y * p1.y));
+    const float2 im = make_float2(t0 * (v0.y * p0.x - v0.x * p0.y), t1 * (v1.y * p1.x - v1.x * p1.y));
+    m = fmaxf(fmaxf(fmaxf(m, fabsf(re.x)), fabsf(re.y)), fmaxf(fabsf(im.x), fabsf(im.y)));
+    pairs[(size_t(jp) * 2) * L + i] = re;
+    pairs[(size_t(jp) * 2 + 1) * L + i] = im;
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));

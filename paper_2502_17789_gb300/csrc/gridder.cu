@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(256) stage_records_kernel(const StageArgs a, i
 }
 
 // Staging for the separable-phasor gridder: one block per subgrid writes its segments' records, 16 visibilities per chunk (the last padded
-// with zeros): float4 [0..15] = (a fix, b fix, delta, 1 / scale), [16 + 2 k], [17 + 2 k] = the 4 values times
-// the segment's scale, a power of two that puts the largest component in [512, 1024) so that hi + lo
-// halves keep 22 bits down to 2^-9 of it.
+// with zeros; kGsepChunkFloat4): a fix, b fix, delta, 1 / scale and the 4 values times the segment's scale, a
+// power of two that puts the largest component in [512, 1024) so that hi + lo halves keep 22 bits down to
+// 2^-9 of it.
 __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float* w_ref,
                                                         int L) {
   const SubgridDesc sd = a.sg[blockIdx.x];
@@ -159,8 +159,7 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
       const float scale = sep_scale(m), inv = 1.f / scale;  // powers of two: exact
       float4* dst = base + size_t(chunk0) * kGsepChunkFloat4;
       for (int k = t0; k < chunks * kSepK; k += nt) {
-        float4* c = dst + size_t(k / kSepK) * kGsepChunkFloat4;
-        const int q = k & (kSepK - 1);
+        float* c = reinterpret_cast<float*>(dst + size_t(k / kSepK) * kGsepChunkFloat4) + (k & (kSepK - 1));
         float4 prm = make_float4(0.f, 0.f, 0.f, inv), v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
         if (k < n) {
           const int row = (sg.k_begin + k) / nc, ch = sd.c0 + (sg.k_begin + k - row * nc);
@@ -176,9 +175,17 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
           v0 = make_float4(v0.x * scale, v0.y * scale, v0.z * scale, v0.w * scale);
           v1 = make_float4(v1.x * scale, v1.y * scale, v1.z * scale, v1.w * scale);
         }
-        c[q] = prm;
-        c[kSepK + 2 * q] = v0;
-        c[kSepK + 2 * q + 1] = v1;
+        c[0] = prm.x;
+        c[16] = prm.y;
+        c[32] = prm.z;
+        c[48] = prm.w;
+        const float re[4] = {v0.x, v0.z, v1.x, v1.z}, im[4] = {v0.y, v0.w, v1.y, v1.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          c[64 + 48 * p] = re[p];
+          c[80 + 48 * p] = im[p];
+          c[96 + 48 * p] = -im[p];
+        }
       }
     }
     chunk0 += chunks;

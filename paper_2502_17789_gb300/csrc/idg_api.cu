@@ -580,7 +580,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       return p->exec[s0 + x].n_vis > p->exec[s0 + y].n_vis;
     });
     for (int32_t o : order)
-      for (int t = 0; t < (p->grid_sep ? L / kGsepColumns : p->grid_tc ? L * L / kGtcPixels : tiles); ++t) gitems.push_back(GridItem{o, t});
+      for (int t = 0; t < (p->grid_sep ? gsep_tiles(L) : p->grid_tc ? L * L / kGtcPixels : tiles); ++t) gitems.push_back(GridItem{o, t});
     // degridder items: pieces of <= `lanes` channel groups of one segment
     // (a segment's rows times G groups per row); a piece that ends its
     // segment shares its item with the first piece of the next segment when
@@ -590,11 +590,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     for (int32_t o : order) {
       const SubgridDesc& d = p->exec[s0 + o];
       if (p->degrid_sep) {
-        // equal pieces of each segment, each a multiple of 8 visibilities but for the last
+        // equal pieces of each segment, each a multiple of 16 visibilities but for the last
         for (int gidx = d.seg_begin; gidx < d.seg_begin + d.seg_count; ++gidx) {
           const SegmentDesc& sgd = p->part.segments[gidx];
           const int n = sgd.k_end - sgd.k_begin, pieces = (n + p->degrid_vis - 1) / p->degrid_vis;
-          const int len = ((n + pieces - 1) / pieces + 7) / 8 * 8;
+          const int len = ((n + pieces - 1) / pieces + 15) / 16 * 16;
           for (int k = sgd.k_begin; k < sgd.k_end; k += len) {
             const int ke = std::min(k + len, sgd.k_end);
             ditems.push_back(DegridItem{o, gidx, k, ke, ke, 0});

@@ -41,15 +41,16 @@ __device__ __forceinline__ uint64_t sep_desc(uint32_t addr, uint32_t k_stride) {
   return uint64_t((addr >> 4) & 0x3fff) | (uint64_t(k_stride >> 4) << 16) | (uint64_t(128 >> 4) << 32) |
          (uint64_t(1) << 46);
 }
-// kind::f16 instruction descriptor: FP32 accumulator, f16 A and B, both K-major, M = 128
-__host__ __device__ constexpr uint32_t sep_idesc(int n) {
-  return (1u << 4) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
+// kind::f16 instruction descriptor: FP32 accumulator, f16 A and B, both K-major, M = 128; negate: D -= A B
+__host__ __device__ constexpr uint32_t sep_idesc(int n, bool negate = false) {
+  return (1u << 4) | (uint32_t(negate) << 13) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
 }
-__device__ __forceinline__ void sep_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// D (+)= A B with A in tensor memory (row = lane, two halves per column) and B in shared memory
+__device__ __forceinline__ void sep_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // arrive on `bar` when every MMA issued so far by this thread has completed
@@ -67,14 +68,22 @@ __device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t cols) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld8(float (&v)[8], uint32_t addr) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(addr));
+__device__ __forceinline__ void tmem_ld16(float (&v)[16], uint32_t addr) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
 #pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = __uint_as_float(r[k]);
+  for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
 }
+__device__ __forceinline__ void tmem_st4(uint32_t addr, const uint32_t (&v)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v[0]), "r"(v[1]),
+               "r"(v[2]), "r"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------- roles
@@ -109,10 +118,30 @@ __device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fa
   }
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest N groups of this thread have landed
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // complex numbers of two pixels, for packed f32x2 arithmetic
 struct c2 {
   float2 re, im;
 };
+
+// one lane of the (converged) warp: code under it may use the uniform datapath that MMA operands come from
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
+}
+// the thread's warp as a value the compiler knows to be the same for the whole warp, so that a role taken by one
+// warp is a branch for the others and not predicated through
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0); }
 
 // ---------------------------------------------------------------- operands
 
@@ -135,42 +164,60 @@ __device__ __forceinline__ float sep_scale(float m) {
 
 __device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
 
-// (hi, lo) halves of the pair (x0, x1): hi = x rounded to half, lo = (x - hi) rounded to half
-__device__ __forceinline__ __half2 sep_split(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(x0, x1);
-  const float2 f = __half22float2(h);
+// (hi, lo) halves of a pair: hi = x rounded to half, lo = (x - hi) rounded to half; returns hi
+__device__ __forceinline__ __half2 sep_split(float2 x, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(x.x, x.y);
   hi = h2_bits(h);
-  lo = h2_bits(__floats2half2_rn(x0 - f.x, x1 - f.y));
+  const float2 r = ffma2(__half22float2(h), make_float2(-1.f, -1.f), x);
+  lo = h2_bits(__floats2half2_rn(r.x, r.y));
   return h;
+}
+// e^{i phase} of two contraction indices: slopes in units of 2^-32 turns, deltas
+__device__ __forceinline__ void sep_phasor2(int fix0, int fix1, int off, float2 delta, float fit, float2& c,
+                                            float2& s) {
+  const float2 ph = make_float2(float(int(unsigned(fix0) * unsigned(off))), float(int(unsigned(fix1) * unsigned(off))));
+  const float2 x = ffma2(ph, make_float2(kTurnsToRad, kTurnsToRad), fmul2(delta, make_float2(fit, fit)));
+  __sincosf(x.x, &s.x, &c.x);
+  __sincosf(x.y, &s.y, &c.y);
+}
+__device__ __forceinline__ float2 pair_of(const float4& v, int h) {
+  return h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
 }
 __device__ __forceinline__ void sts128(uint32_t addr, const uint32_t (&v)[4]) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
                : "memory");
 }
 
-// the F side of one column index for 8 consecutive contraction indices: rows
-// of the blocks (-Im, Re, Im) at dst, dst + block, dst + 2 block, the levels
-// (hi, lo, first order) `level` bytes apart.  SIGN = -1 takes conj(F).
+// the F side of one column index for 8 consecutive contraction indices: Re and Im rows at dst and dst + block,
+// the levels (hi, lo, first order) `level` bytes apart
 struct SepF {
   uint32_t r_hi[4], i_hi[4], r_lo[4], i_lo[4], r_c[4], i_c[4];
 };
 __device__ __forceinline__ void sep_store_f(const SepF& f, uint32_t dst, uint32_t block, uint32_t level) {
-  uint32_t m[4];
+  sts128(dst, f.r_hi);
+  sts128(dst + block, f.i_hi);
+  sts128(dst + level, f.r_lo);
+  sts128(dst + level + block, f.i_lo);
+  sts128(dst + 2 * level, f.r_c);
+  sts128(dst + 2 * level + block, f.i_c);
+}
+// D (+)= E F for one contraction step of 16: the E side in tensor memory at column `e` as (Re hi, Im hi, Re lo, Im lo,
+// Re first order, Im first order) of 8 columns each, the F side in shared memory (sep_store_f, k groups `group`
+// bytes apart), D = re at column d and im at d + n, n columns each.  Products lo hi, hi lo, first order, hi hi; all
+// MMAs on one accumulator have the same shape, so they run in the order of issue.
+__device__ __forceinline__ void sep_product(uint32_t d, uint32_t e, uint32_t f, int n, uint32_t block, uint32_t group,
+                                            uint32_t level, bool first) {
+  const uint32_t add = sep_idesc(n), sub = sep_idesc(n, true);
+  const uint32_t el[4] = {1, 0, 2, 0}, fl[4] = {0, 1, 2, 0};
 #pragma unroll
-  for (int k = 0; k < 4; ++k) m[k] = f.i_hi[k] ^ 0x80008000u;
-  sts128(dst, m);
-  sts128(dst + block, f.r_hi);
-  sts128(dst + 2 * block, f.i_hi);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) m[k] = f.i_lo[k] ^ 0x80008000u;
-  sts128(dst + level, m);
-  sts128(dst + level + block, f.r_lo);
-  sts128(dst + level + 2 * block, f.i_lo);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) m[k] = f.i_c[k] ^ 0x80008000u;
-  sts128(dst + 2 * level, m);
-  sts128(dst + 2 * level + block, f.r_c);
-  sts128(dst + 2 * level + 2 * block, f.i_c);
+  for (int t = 0; t < 4; ++t) {
+    const uint32_t ea = e + el[t] * 16, fa = f + fl[t] * level, acc = (first && t == 0) ? 0u : 1u;
+    const uint64_t fr = sep_desc(fa, group), fi = sep_desc(fa + block, group);
+    sep_mma(d, ea, fr, add, acc);           // re += Re E Re F
+    sep_mma(d + n, ea, fi, add, acc);       // im += Re E Im F
+    sep_mma(d, ea + 8, fi, sub, 1u);        // re -= Im E Im F
+    sep_mma(d + n, ea + 8, fr, add, 1u);    // im += Im E Re F
+  }
 }
 
 // (cos, sin)(2 pi w_ref n') from the two-float n' (exact range reduction)
