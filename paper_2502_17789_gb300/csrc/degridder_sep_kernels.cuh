@@ -101,108 +101,93 @@ struct Dsep {
     cp_async_commit();
   }
 
-  // Z of rows 16 jc .. for column block ib: thread = (p, i) x 8 rows j
-  template <bool DIAG>
-  __device__ __forceinline__ void produce(uint32_t e_col, int buf, const float4* samples, float scale, NodeWeight wx,
-                                          int jc, __half2 fit_p) {
+  // Z of rows 16 jc .. for column block ib: thread = (p, i) x 8 rows j.  QUAD: node cells start at multiples of four
+  // rows, so the cell can change only half way and not at every row.
+  template <bool DIAG, bool QUAD>
+  __device__ __forceinline__ void produce(uint32_t e_col, const float2* yb, const float4* samples, float scale,
+                                          NodeWeight wx, int jc, __half2 fit_p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = warp & 3, g = warp >> 2, pa = p >> 1, pb = p & 1;
     const int nodes = a.g.nodes, step = nodes - 1;
     const bool stokes = a.g.npol == 1;
     constexpr int NE = DIAG ? 1 : 2;  // entries of each station's matrix that this correlation needs
-    // node row r interpolated along i: p_aa, q_bb (diagonal) or p_a0, p_a1, q_b0, q_b1
+    // an off-diagonal correlation of a Stokes-I model with diagonal matrices is zero
+    const float kp = (DIAG && stokes && pa != pb) ? 0.f : scale;
+    const float k1[2] = {wx.f * kp, wx.f}, k0[2] = {(1.f - wx.f) * kp, 1.f - wx.f};
+    const float2* smp[2];
+#pragma unroll
+    for (int st = 0; st < 2; ++st)
+      smp[st] = reinterpret_cast<const float2*>(samples + st * nodes * nodes * 2) + wx.a * 4 +
+                (DIAG ? 3 * (st ? pb : pa) : 2 * (st ? pb : pa));
+    // node row r interpolated along i, p_aa, q_bb (diagonal) or p_a0, p_a1, q_b0, q_b1, and the step to the next
     cf u[2][NE], d[2][NE];
-    auto row = [&](int r, cf (&v)[2][NE]) {
-#pragma unroll
-      for (int st = 0; st < 2; ++st) {
-        const float2* n0 = reinterpret_cast<const float2*>(samples + st * nodes * nodes * 2) + (r * nodes + wx.a) * 4 +
-                           (DIAG ? 3 * (st ? pb : pa) : 2 * (st ? pb : pa));
-        const float k1 = st ? wx.f : wx.f * scale, k0 = st ? 1.f - wx.f : (1.f - wx.f) * scale;
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-          const float2 x = n0[e], y = n0[4 + e];
-          v[st][e] = {k0 * x.x + k1 * y.x, k0 * x.y + k1 * y.y};
-        }
-      }
-    };
-    const int j0 = 16 * jc + 8 * g;
-    int at = step * j0 / L, rem = step * j0 - at * L, node = -1;
-    auto cell = [&]() {  // the same for the whole warp
-      if (at == node) return;
-      node = at;
-      row(at, u);
-      row(at + 1, d);
+    auto load_cell = [&](int r) {
 #pragma unroll
       for (int st = 0; st < 2; ++st)
 #pragma unroll
-        for (int e = 0; e < NE; ++e) d[st][e] = {d[st][e].re - u[st][e].re, d[st][e].im - u[st][e].im};
+        for (int e = 0; e < NE; ++e) {
+          const float2* n0 = smp[st] + r * nodes * 4 + e;
+          const float2 x0 = n0[0], y0 = n0[4], x1 = n0[nodes * 4], y1 = n0[nodes * 4 + 4];
+          u[st][e] = {k0[st] * x0.x + k1[st] * y0.x, k0[st] * x0.y + k1[st] * y0.y};
+          d[st][e] = {fmaf(k0[st], x1.x, fmaf(k1[st], y1.x, -u[st][e].re)),
+                      fmaf(k0[st], x1.y, fmaf(k1[st], y1.y, -u[st][e].im))};
+        }
     };
+    // row q of the octet lies at (rem + step q) / L of the cell that starts at node row `at`
+    int at = step * (16 * jc + 8 * g) / L, rem = step * (16 * jc + 8 * g) - at * L;
+    load_cell(at);
+    float f0 = float(rem) * (1.f / float(L));
+    const float df = float(step) * (1.f / float(L));
+    const float2* y0 = yb + (4 * g) * 64 + lane;  // [pol][row pair][re, im][column]
     uint32_t re_hi[4], re_lo[4], re_c[4], im_hi[4], im_lo[4], im_c[4];
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-      c2 m[2][NE];      // the entries at both rows
-      float2 n[2][NE];  // minus their imaginary parts
+      float2 yr[DIAG ? 1 : 4], yi[DIAG ? 1 : 4];  // Y at both rows of the pair
+#pragma unroll
+      for (int k = 0; k < (DIAG ? 1 : 4); ++k) {
+        const float2* y = y0 + (stokes ? 0 : DIAG ? p : k) * 512 + w * 64;
+        yr[k] = y[0];
+        yi[k] = y[32];
+      }
+      float2 zr, zi;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        cell();
-        const float f = float(rem) * (1.f / float(L));
+        const int q = 2 * w + h;
+        if (QUAD ? q == 4 : q > 0) {
+          if (rem + step * q >= L) {  // the same for the whole warp
+            rem -= L;
+            f0 -= 1.f;
+            load_cell(++at);
+          }
+        }
+        const float f = fmaf(float(q), df, f0);
+        cf m[2][NE];  // the entries at this row
 #pragma unroll
         for (int st = 0; st < 2; ++st)
 #pragma unroll
-          for (int e = 0; e < NE; ++e) {
-            const float re = fmaf(f, d[st][e].re, u[st][e].re), im = fmaf(f, d[st][e].im, u[st][e].im);
-            const float ni = fmaf(-f, d[st][e].im, -u[st][e].im);
-            if (h) {
-              m[st][e].re.y = re;
-              m[st][e].im.y = im;
-              n[st][e].y = ni;
-            } else {
-              m[st][e].re.x = re;
-              m[st][e].im.x = im;
-              n[st][e].x = ni;
-            }
-          }
-        rem += step;
-        if (rem >= L) {
-          rem -= L;
-          ++at;
-        }
-      }
-      auto load = [&](int pol) { return c2{S.y[buf][pol][4 * g + w][0][lane], S.y[buf][pol][4 * g + w][1][lane]}; };
-      // x y, t += x y;  t conj(q), z += t conj(q)
-      auto mul = [](const c2& x, float2 nx, const c2& y) {
-        return c2{ffma2(nx, y.im, fmul2(x.re, y.re)), ffma2(x.im, y.re, fmul2(x.re, y.im))};
-      };
-      auto mul_add = [](const c2& x, float2 nx, const c2& y, c2& t) {
-        t.re = ffma2(nx, y.im, ffma2(x.re, y.re, t.re));
-        t.im = ffma2(x.im, y.re, ffma2(x.re, y.im, t.im));
-      };
-      auto mul_conj = [](const c2& t, const c2& q, float2 nq) {
-        return c2{ffma2(t.im, q.im, fmul2(t.re, q.re)), ffma2(nq, t.re, fmul2(t.im, q.re))};
-      };
-      c2 z;
-      if constexpr (DIAG) {
-        z = mul_conj(mul(m[0][0], n[0][0], load(stokes ? 0 : p)), m[1][0], n[1][0]);
-        if (stokes && pa != pb) z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      } else {
-        c2 t0, t1;
-        if (stokes) {
-          const c2 y = load(0);
-          t0 = mul(m[0][0], n[0][0], y);
-          t1 = mul(m[0][1], n[0][1], y);
+          for (int e = 0; e < NE; ++e) m[st][e] = {fmaf(f, d[st][e].re, u[st][e].re), fmaf(f, d[st][e].im, u[st][e].im)};
+        cf y[DIAG ? 1 : 4];
+#pragma unroll
+        for (int k = 0; k < (DIAG ? 1 : 4); ++k) y[k] = h ? cf{yr[k].y, yi[k].y} : cf{yr[k].x, yi[k].x};
+        cf z;
+        if constexpr (DIAG) {
+          z = cmulc(m[1][0], cmul(m[0][0], y[0]));
+        } else if (stokes) {
+          z = cadd(cmulc(m[1][0], cmul(m[0][0], y[0])), cmulc(m[1][1], cmul(m[0][1], y[0])));
         } else {
-          t0 = mul(m[0][0], n[0][0], load(0));
-          t1 = mul(m[0][0], n[0][0], load(1));
-          mul_add(m[0][1], n[0][1], load(2), t0);
-          mul_add(m[0][1], n[0][1], load(3), t1);
+          z = cadd(cmulc(m[1][0], cadd(cmul(m[0][0], y[0]), cmul(m[0][1], y[2]))),
+                   cmulc(m[1][1], cadd(cmul(m[0][0], y[1]), cmul(m[0][1], y[3]))));
         }
-        z = mul_conj(t0, m[1][0], n[1][0]);
-        const c2 z1 = mul_conj(t1, m[1][1], n[1][1]);
-        z.re = ffma2(z1.re, make_float2(1.f, 1.f), z.re);
-        z.im = ffma2(z1.im, make_float2(1.f, 1.f), z.im);
+        if (h) {
+          zr.y = z.re;
+          zi.y = z.im;
+        } else {
+          zr.x = z.re;
+          zi.x = z.im;
+        }
       }
-      re_c[w] = h2_bits(__hmul2(sep_split(z.re, re_hi[w], re_lo[w]), fit_p));
-      im_c[w] = h2_bits(__hmul2(sep_split(z.im, im_hi[w], im_lo[w]), fit_p));
+      re_c[w] = h2_bits(__hmul2(sep_split(zr, re_hi[w], re_lo[w]), fit_p));
+      im_c[w] = h2_bits(__hmul2(sep_split(zi, im_hi[w], im_lo[w]), fit_p));
     }
     const uint32_t dst = e_col + (uint32_t(p * 32) << 16) + 4 * g;
     tmem_st4(dst, re_hi);
@@ -216,12 +201,22 @@ struct Dsep {
   __device__ __forceinline__ void producer() {
     const int lane = threadIdx.x & 31, nodes = a.g.nodes;
     const bool issuer = uniform_warp() == 0;
+    const bool quad = L % (nodes - 1) == 0 && L / (nodes - 1) % 4 == 0;
     const uint32_t tm = S.tmem;
     uint32_t pg = 0, dg = 0, n = 0;  // pieces, accumulators and items of this block so far
+    int yb = 0;                      // pg % kDsepYRing
     if (first >= last) return;
     wait(&S.ready[0], 0);
-    fetch_y(0, S.info[0].sg, 0, 0);
-    fetch_y(1, S.info[0].sg, 0, 1);
+    int y_sg = S.info[0].sg, y_ib = 0, y_jc = 0;  // the piece of Y to fetch next
+    auto fetch_next = [&](int buf) {
+      fetch_y(buf, y_sg, y_ib, y_jc);
+      if (++y_jc == kPieces) {
+        y_jc = 0;
+        ++y_ib;
+      }
+    };
+    fetch_next(0);
+    fetch_next(1);
     cp_async_wait<1>();
     half_sync(kSepProducerBar);
     for (int idx = first; idx < last; idx += stride, ++n) {
@@ -238,26 +233,34 @@ struct Dsep {
 #pragma unroll 1
         for (int jc = 0; jc < kPieces; ++jc, ++pg) {
           // two pieces ahead, in the next item past this one's end
-          const int t = ib * kPieces + jc + 2;
-          if (t < kBlocks * kPieces) {
-            fetch_y((pg + 2) % kDsepYRing, info.sg, t / kPieces, t % kPieces);
-          } else if (more) {
-            if (t == kBlocks * kPieces) wait(&S.ready[(n + 1) & 1], ((n + 1) >> 1) & 1);
-            const int r = t - kBlocks * kPieces;
-            fetch_y((pg + 2) % kDsepYRing, S.info[(n + 1) & 1].sg, r / kPieces, r % kPieces);
-          } else {
-            cp_async_commit();  // keeps the count of groups
+          if (y_ib == kBlocks && more) {
+            wait(&S.ready[(n + 1) & 1], ((n + 1) >> 1) & 1);
+            y_sg = S.info[(n + 1) & 1].sg;
+            y_ib = 0;
           }
+          const int buf = yb;
+          if (++yb == kDsepYRing) yb = 0;
+          if (y_ib < kBlocks)
+            fetch_next(buf == 0 ? 2 : buf - 1);
+          else
+            cp_async_commit();  // keeps the count of groups
           const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
           if (turn > 0) {
             wait(&S.empty[slot], (turn - 1) & 1);
             tc_fence_after();
           }
           const uint32_t e_col = tm + kDsepZCol + slot * 48;
-          if (info.diag)
-            produce<true>(e_col, pg % kDsepYRing, samples, info.scale, wx, jc, fit_p);
-          else
-            produce<false>(e_col, pg % kDsepYRing, samples, info.scale, wx, jc, fit_p);
+          const float2* y = &S.y[buf][0][0][0][0];
+          if (quad) {
+            if (info.diag)
+              produce<true, true>(e_col, y, samples, info.scale, wx, jc, fit_p);
+            else
+              produce<false, true>(e_col, y, samples, info.scale, wx, jc, fit_p);
+          } else if (info.diag) {
+            produce<true, false>(e_col, y, samples, info.scale, wx, jc, fit_p);
+          } else {
+            produce<false, false>(e_col, y, samples, info.scale, wx, jc, fit_p);
+          }
           cp_async_wait<1>();
           tmem_wait_st();
           tc_fence_before();
@@ -331,14 +334,11 @@ struct Dsep {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int w = 2 * u + h, off = 8 * o + 2 * w - L / 2;
-          const float2 ph = make_float2(float(int(unsigned(fix) * unsigned(off))),
-                                        float(int(unsigned(fix) * unsigned(off + 1))));
-          const float2 x = ffma2(ph, make_float2(kTurnsToRad, kTurnsToRad), fmul2(make_float2(dl, dl), pair_of(b4, h)));
+          const float2 fb = pair_of(b4, h), fq = pair_of(q4, h);
           float2 c, s;
-          __sincosf(x.x, &s.x, &c.x);
-          __sincosf(x.y, &s.y, &c.y);
-          const float2 dq = fmul2(make_float2(-dl, -dl), pair_of(q4, h));
-          const __half2 d2 = __floats2half2_rn(dq.x, dq.y);
+          __sincosf(sep_phase(fix, off, dl, fb.x), &s.x, &c.x);
+          __sincosf(sep_phase(fix, off + 1, dl, fb.y), &s.y, &c.y);
+          const __half2 d2 = __floats2half2_rn(-dl * fq.x, -dl * fq.y);
           const __half2 hc = sep_split(c, f.r_hi[w], f.r_lo[w]);
           const __half2 hs = sep_split(s, f.i_hi[w], f.i_lo[w]);
           // conj(F) = (c, -s); -i delta q conj(F) = (-delta q s, -delta q c)
@@ -358,6 +358,7 @@ struct Dsep {
 
   __device__ __forceinline__ void consumer() {
     const int tid = threadIdx.x - kSepHalf, warp = tid >> 5, lane = tid & 31;
+    const bool poller = uniform_warp() == kSepHalf / 32;
     uint32_t dg = 0, n = 0;  // accumulators and items of this block so far
     if (first >= last) return;
     prepare(first, 0);
@@ -376,7 +377,8 @@ struct Dsep {
       for (int ib = 0; ib < kBlocks; ++ib, ++dg) {
         const int i = ib * 32 + lane;
         const float fit_a = __ldg(a.sep.a + i);
-        wait(&S.full[dg & 1], (dg >> 1) & 1);
+        if (poller) wait(&S.full[dg & 1], (dg >> 1) & 1);
+        half_sync(kSepConsumerBar);
         tc_fence_after();
         const uint32_t d = S.tmem + (uint32_t((warp & 3) * 32) << 16) + (dg & 1) * kDsepColStride;
 #pragma unroll
@@ -395,8 +397,10 @@ struct Dsep {
               float2 c, s;
               sep_phasor2(__float_as_int(f.x), __float_as_int(f.y), i - L / 2, pair_of(dl[k >> 1], k & 1), fit_a, c, s);
               const float2 r = make_float2(dr[2 * k], dr[2 * k + 1]), m = make_float2(di[2 * k], di[2 * k + 1]);
-              re[h][k] = ffma2(r, c, ffma2(m, s, re[h][k]));
-              im[h][k] = ffma2(m, c, ffma2(make_float2(-r.x, -r.y), s, im[h][k]));
+              re[h][k].x = fmaf(r.x, c.x, fmaf(m.x, s.x, re[h][k].x));
+              re[h][k].y = fmaf(r.y, c.y, fmaf(m.y, s.y, re[h][k].y));
+              im[h][k].x = fmaf(m.x, c.x, fmaf(-r.x, s.x, im[h][k].x));
+              im[h][k].y = fmaf(m.y, c.y, fmaf(-r.y, s.y, im[h][k].y));
             }
           }
         }

@@ -85,18 +85,17 @@ __device__ __forceinline__ void gsep_produce(uint32_t e_col, uint32_t buf, const
     uint32_t re_hi[4], re_lo[4], re_c[4], im_hi[4], im_lo[4], im_c[4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const float4 fx = rec[2 * g + u], dl = rec[8 + 2 * g + u], vr = val[u], vi = val[4 + u], vn = val[8 + u];
+      const float4 fx = rec[2 * g + u], dl = rec[8 + 2 * g + u], vr = val[u], vi = val[4 + u];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int h = 2 * u + e;
         const float2 f = pair_of(fx, e), d = pair_of(dl, e);
         float2 c, s;
         sep_phasor2(__float_as_int(f.x), __float_as_int(f.y), i_off, d, fit_a, c, s);
-        const float2 dp = fmul2(d, make_float2(fit_p, fit_p));
-        const __half2 d2 = __floats2half2_rn(dp.x, dp.y);
-        const float2 r = pair_of(vr, e);
-        re_c[h] = h2_bits(__hmul2(sep_split(ffma2(pair_of(vn, e), s, fmul2(r, c)), re_hi[h], re_lo[h]), d2));
-        im_c[h] = h2_bits(__hmul2(sep_split(ffma2(pair_of(vi, e), c, fmul2(r, s)), im_hi[h], im_lo[h]), d2));
+        const __half2 d2 = __floats2half2_rn(d.x * fit_p, d.y * fit_p);
+        const float2 r = pair_of(vr, e), m = pair_of(vi, e);
+        re_c[h] = h2_bits(__hmul2(sep_split(make_float2(r.x * c.x - m.x * s.x, r.y * c.y - m.y * s.y), re_hi[h], re_lo[h]), d2));
+        im_c[h] = h2_bits(__hmul2(sep_split(make_float2(r.x * s.x + m.x * c.x, r.y * s.y + m.y * c.y), im_hi[h], im_lo[h]), d2));
       }
     }
     const uint32_t dst = e_col + (uint32_t(p * 32) << 16) + 4 * g;
@@ -203,6 +202,9 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
   using C = Gsep<L>;
   const int warp = (threadIdx.x >> 5) - kSepHalf / 32, lane = threadIdx.x & 31;
   const int nodes = a.g.nodes, n4 = nodes * nodes * 2;  // float4s of one station's samples
+  const bool poller = uniform_warp() == kSepHalf / 32;
+  // rows of a thread within one node cell: every cell starts at a multiple of kSpan rows
+  const bool one_cell = L % (nodes - 1) == 0 && L / (nodes - 1) % C::kSpan == 0;
   uint32_t sc = 0;  // segments of this block so far
   for (int idx = first; idx < last; idx += stride) {
     const GridItem item = a.items[idx];
@@ -211,11 +213,11 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
     const int i = org.x + lane, j0 = org.y + warp * C::kSpan;
     const NodeWeight wx = node_weight(i, nodes, L);
     const float4* rec = a.records + size_t(sd.rec_offset) * kRecordFloat4;  // first chunk of the next segment
-    c2 acc[C::kPairs][4];
+    cf acc[C::kSpan][4];
 #pragma unroll
-    for (int st = 0; st < C::kPairs; ++st)
+    for (int r = 0; r < C::kSpan; ++r)
 #pragma unroll
-      for (int p = 0; p < 4; ++p) acc[st][p] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int p = 0; p < 4; ++p) acc[r][p] = {0.f, 0.f};
 
     // A-term samples of segment s of the item (the block's segment number c), on their way while another is worked on
     int diag_next = 0;
@@ -224,9 +226,12 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
     auto fetch = [&](int s, uint32_t c) {
       const int sp = seg.interval * a.g.n_st + sd.p, sq = seg.interval * a.g.n_st + sd.q;
       float4* dst = raw + (c & 1) * 2 * n4;
-      const float4* src = reinterpret_cast<const float4*>(a.aterms);
-      for (int e = threadIdx.x - kSepHalf; e < 2 * n4; e += kSepHalf)
-        cp_async16(dst + e, src + (e < n4 ? size_t(sp) * n4 + e : size_t(sq) * n4 + e - n4));
+      const float4* pp = reinterpret_cast<const float4*>(a.aterms) + size_t(sp) * n4;
+      const float4* qq = reinterpret_cast<const float4*>(a.aterms) + size_t(sq) * n4;
+      for (int e = threadIdx.x - kSepHalf; e < n4; e += kSepHalf) {
+        cp_async16(dst + e, pp + e);
+        cp_async16(dst + n4 + e, qq + e);
+      }
       cp_async_commit();
       diag_next = a.adiag[sp] & a.adiag[sq];
       inv_next = __ldg(&rec[12].x);  // 1 / scale of the segment's values, undone on the p side
@@ -238,12 +243,12 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
     for (int s = 0; s < sd.seg_count; ++s, ++sc) {
       const bool diag = diag_next != 0;
       const float inv = inv_next;
-      half_sync(kSepConsumerBar);  // S.x and the other samples free
+      if (poller) sep_wait(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
+      half_sync(kSepConsumerBar);  // the segment's sums complete; S.x and the other samples free
+      tc_fence_after();
       const bool more = s + 1 < sd.seg_count;
       if (more) fetch(s + 1, sc + 1);
       // sums of the segment: tensor memory -> S.x; warp = correlation, half of the rows
-      sep_wait(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
-      tc_fence_after();
       {
         const int pol = warp & 3, r0 = (warp >> 2) * (C::kRows / 2);
         const uint32_t d = S.tmem + (uint32_t(pol * 32) << 16) + (sc & 1) * C::kColStride + r0;
@@ -288,20 +293,30 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
       auto diff = [](const float4& v, const float4& u) {
         return make_float4(v.x - u.x, v.y - u.y, v.z - u.z, v.w - u.w);
       };
-      auto pixels = [&](auto dtag) {
+      // one_cell: the thread's rows lie in one node cell, so its rows are read once; otherwise the cell is followed
+      // from row to row
+      auto pixels = [&](auto dtag, auto one_cell) {
         constexpr int NV = decltype(dtag)::value ? 2 : 4;
+        constexpr bool ONE = decltype(one_cell)::value;
         float4 u[4], dl[4];  // the node row below the pixel row and the step to the next
-        int node = -1;
+        auto load_cell = [&](int node) {
+#pragma unroll
+          for (int w = 0; w < NV; ++w) {
+            u[w] = row(node, w, dtag);
+            dl[w] = diff(row(node + 1, w, dtag), u[w]);
+          }
+        };
         // node cell and position of the next row; kept opaque so that the rows' values are not all held over the
         // segments (registers)
         const int step = nodes - 1;
         int jn = step * j0;
         asm volatile("" : "+r"(jn));
-        int at = jn / L, rem = jn - at * L;
+        int at = jn / L, rem = jn - at * L, node = -1;
+        if (ONE) load_cell(at);
         auto next_row = [&]() {
           const NodeWeight w = {at, float(rem) * (1.f / float(L))};
           rem += step;
-          if (rem >= L) {
+          if (!ONE && rem >= L) {
             rem -= L;
             ++at;
           }
@@ -310,116 +325,97 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
 #pragma unroll
         for (int st = 0; st < C::kPairs; ++st) {
           const NodeWeight w0 = next_row(), w1 = next_row();
-          if (w0.a != node) {  // the same for the whole warp, every L / (nodes - 1) rows
+          if (!ONE && w0.a != node) {  // the same for the whole warp
             node = w0.a;
-#pragma unroll
-            for (int w = 0; w < NV; ++w) {
-              u[w] = row(node, w, dtag);
-              dl[w] = diff(row(node + 1, w, dtag), u[w]);
-            }
+            load_cell(node);
           }
-          c2 X[4];
+          float2 xr[4], xi[4];
 #pragma unroll
-          for (int p = 0; p < 4; ++p)
-            X[p] = {S.x[p][0][warp * C::kPairs + st][lane], S.x[p][1][warp * C::kPairs + st][lane]};
-          c2 e[2];      // the two entries of vector w at both rows of the pair
-          float2 n[2];  // minus their imaginary parts
-          auto lerp = [&](int w) {
-            float4 v = u[w], d = dl[w];
-            e[0].re.x = fmaf(w0.f, d.x, v.x);
-            e[0].im.x = fmaf(w0.f, d.y, v.y);
-            n[0].x = fmaf(-w0.f, d.y, -v.y);
-            e[1].re.x = fmaf(w0.f, d.z, v.z);
-            e[1].im.x = fmaf(w0.f, d.w, v.w);
-            n[1].x = fmaf(-w0.f, d.w, -v.w);
-            if (w1.a != w0.a) {  // a node row between the two (only where nodes - 1 does not divide L / 2)
-              v = row(w1.a, w, dtag);
-              d = diff(row(w1.a + 1, w, dtag), v);
-            }
-            e[0].re.y = fmaf(w1.f, d.x, v.x);
-            e[0].im.y = fmaf(w1.f, d.y, v.y);
-            n[0].y = fmaf(-w1.f, d.y, -v.y);
-            e[1].re.y = fmaf(w1.f, d.z, v.z);
-            e[1].im.y = fmaf(w1.f, d.w, v.w);
-            n[1].y = fmaf(-w1.f, d.w, -v.w);
-          };
-          // conj(x) y and t += x y, t += conj(x) y, with nx = -Im x
-          auto conj_mul = [](const c2& x, float2 nx, const c2& y) {
-            return c2{ffma2(x.im, y.im, fmul2(x.re, y.re)), ffma2(nx, y.re, fmul2(x.re, y.im))};
-          };
-          auto mul = [](const c2& x, float2 nx, const c2& y) {
-            return c2{ffma2(nx, y.im, fmul2(x.re, y.re)), ffma2(x.im, y.re, fmul2(x.re, y.im))};
-          };
-          auto mul_add = [](const c2& x, float2 nx, const c2& y, c2& t) {
-            t.re = ffma2(nx, y.im, ffma2(x.re, y.re, t.re));
-            t.im = ffma2(x.im, y.re, ffma2(x.re, y.im, t.im));
-          };
-          auto conj_mul_add = [](const c2& x, float2 nx, const c2& y, c2& t) {
-            t.re = ffma2(x.im, y.im, ffma2(x.re, y.re, t.re));
-            t.im = ffma2(nx, y.re, ffma2(x.re, y.im, t.im));
-          };
-          if constexpr (decltype(dtag)::value) {  // conj(p_a) X_ab q_b
-            c2 t[4];
-            lerp(0);
+          for (int p = 0; p < 4; ++p) {
+            xr[p] = S.x[p][0][warp * C::kPairs + st][lane];
+            xi[p] = S.x[p][1][warp * C::kPairs + st][lane];
+          }
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-              t[b] = conj_mul(e[0], n[0], X[b]);
-              t[2 + b] = conj_mul(e[1], n[1], X[2 + b]);
-            }
-            lerp(1);
+          for (int h = 0; h < 2; ++h) {
+            const NodeWeight wn = h ? w1 : w0;
+            cf X[4];
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              mul_add(e[0], n[0], t[2 * r], acc[st][2 * r]);
-              mul_add(e[1], n[1], t[2 * r + 1], acc[st][2 * r + 1]);
-            }
-          } else {  // A_p^H (X A_q): by the rows of A_q, then of A_p
-            c2 m[4];
-            lerp(2);
+            for (int p = 0; p < 4; ++p) X[p] = h ? cf{xr[p].y, xi[p].y} : cf{xr[p].x, xi[p].x};
+            cf e[2];  // the two entries of vector w
+            auto lerp = [&](int w) {
+              float4 v = u[w], d = dl[w];
+              if (!ONE && h == 1 && w1.a != w0.a) {  // a node row between the two
+                v = row(w1.a, w, dtag);
+                d = diff(row(w1.a + 1, w, dtag), v);
+              }
+              e[0] = {fmaf(wn.f, d.x, v.x), fmaf(wn.f, d.y, v.y)};
+              e[1] = {fmaf(wn.f, d.z, v.z), fmaf(wn.f, d.w, v.w)};
+            };
+            auto mul_add = [](cf x, cf y, cf& t) {  // t += x y
+              t.re = fmaf(-x.im, y.im, fmaf(x.re, y.re, t.re));
+              t.im = fmaf(x.im, y.re, fmaf(x.re, y.im, t.im));
+            };
+            auto conj_mul_add = [](cf x, cf y, cf& t) {  // t += conj(x) y
+              t.re = fmaf(x.im, y.im, fmaf(x.re, y.re, t.re));
+              t.im = fmaf(-x.im, y.re, fmaf(x.re, y.im, t.im));
+            };
+            cf* o = acc[2 * st + h];
+            if constexpr (decltype(dtag)::value) {  // conj(p_a) X_ab q_b
+              cf t[4];
+              lerp(0);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) m[k] = mul(e[k & 1], n[k & 1], X[k & 2]);
-            lerp(3);
+              for (int k = 0; k < 4; ++k) t[k] = cmulc(e[k >> 1], X[k]);
+              lerp(1);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) mul_add(e[k & 1], n[k & 1], X[(k & 2) + 1], m[k]);
+              for (int k = 0; k < 4; ++k) mul_add(t[k], e[k & 1], o[k]);
+            } else {  // A_p^H (X A_q): by the rows of A_q, then of A_p
+              cf m[4];
+              lerp(2);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              lerp(h);
+              for (int k = 0; k < 4; ++k) m[k] = cmul(X[k & 2], e[k & 1]);
+              lerp(3);
 #pragma unroll
-              for (int k = 0; k < 4; ++k) conj_mul_add(e[k >> 1], n[k >> 1], m[2 * h + (k & 1)], acc[st][k]);
+              for (int k = 0; k < 4; ++k) mul_add(X[(k & 2) + 1], e[k & 1], m[k]);
+#pragma unroll
+              for (int r = 0; r < 2; ++r) {
+                lerp(r);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) conj_mul_add(e[k >> 1], m[2 * r + (k & 1)], o[k]);
+              }
             }
           }
         }
       };
-      if (diag)
-        pixels(std::true_type{});
-      else
-        pixels(std::false_type{});
+      if (one_cell) {
+        if (diag)
+          pixels(std::true_type{}, std::true_type{});
+        else
+          pixels(std::false_type{}, std::true_type{});
+      } else if (diag) {
+        pixels(std::true_type{}, std::false_type{});
+      } else {
+        pixels(std::false_type{}, std::false_type{});
+      }
     }
 
     // ---- pixels of the item: w_ref, taper, centring sign; [sg][pol][j][i]; Stokes I: plane 0, (XX + YY) / 2
     const float w_ref = a.w_ref[item.sg];
     const float ti = a.taper[i];
 #pragma unroll
-    for (int st = 0; st < C::kPairs; ++st) {
+    for (int r = 0; r < C::kSpan; ++r) {
+      const int j = j0 + r;
+      const float2 ph = sep_w_phasor(w_ref, __ldg(a.sep.n1 + j * L + i));
+      const float wgt = ti * a.taper[j] * (((i + j) & 1) ? -1.f : 1.f);
+      const cf rot = {wgt * ph.x, wgt * ph.y};
+      float2* dst = a.scratch + size_t(item.sg) * 4 * L * L + j * L + i;
+      if (a.g.npol == 1) {
+        const cf x = cmul(rot, cf{0.5f * (acc[r][0].re + acc[r][3].re), 0.5f * (acc[r][0].im + acc[r][3].im)});
+        dst[0] = make_float2(x.re, x.im);
+      } else {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = j0 + 2 * st + h;
-        const float2 ph = sep_w_phasor(w_ref, __ldg(a.sep.n1 + j * L + i));
-        const float wgt = ti * a.taper[j] * (((i + j) & 1) ? -1.f : 1.f);
-        const cf rot = {wgt * ph.x, wgt * ph.y};
-        float2* dst = a.scratch + size_t(item.sg) * 4 * L * L + j * L + i;
-        cf v[4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-          v[p] = h ? cf{acc[st][p].re.y, acc[st][p].im.y} : cf{acc[st][p].re.x, acc[st][p].im.x};
-        if (a.g.npol == 1) {
-          const cf x = cmul(rot, cf{0.5f * (v[0].re + v[3].re), 0.5f * (v[0].im + v[3].im)});
-          dst[0] = make_float2(x.re, x.im);
-        } else {
-#pragma unroll
-          for (int p = 0; p < 4; ++p) {
-            const cf x = cmul(rot, v[p]);
-            dst[size_t(p) * L * L] = make_float2(x.re, x.im);
-          }
+        for (int p = 0; p < 4; ++p) {
+          const cf x = cmul(rot, acc[r][p]);
+          dst[size_t(p) * L * L] = make_float2(x.re, x.im);
         }
       }
     }

@@ -108,13 +108,19 @@ __device__ __forceinline__ void regs_give() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
 }
 
-// bounded wait that reports a timeout once and then lets every later wait of the block pass
+// bounded wait that reports a timeout once and then lets every later wait of the block pass.  Where many warps wait
+// for long, one polls and the others stand at a named barrier: polling takes issue slots from the working warps.
 __device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, int* status) {
   if (mbar_try_wait(bar, parity)) return;
   if (*reinterpret_cast<volatile int*>(fail)) return;
-  if (!mbar_wait_bounded(bar, parity)) {
-    atomicOr(status, kStatusTimeout);
-    *reinterpret_cast<volatile int*>(fail) = 1;
+  const uint64_t t0 = global_ns();
+  while (!mbar_try_wait(bar, parity)) {
+    if (global_ns() - t0 > kWaitLimitNs) {
+      atomicOr(status, kStatusTimeout);
+      *reinterpret_cast<volatile int*>(fail) = 1;
+      return;
+    }
+    __nanosleep(40);
   }
 }
 
@@ -168,17 +174,15 @@ __device__ __forceinline__ uint32_t h2_bits(__half2 h) { return *reinterpret_cas
 __device__ __forceinline__ __half2 sep_split(float2 x, uint32_t& hi, uint32_t& lo) {
   const __half2 h = __floats2half2_rn(x.x, x.y);
   hi = h2_bits(h);
-  const float2 r = ffma2(__half22float2(h), make_float2(-1.f, -1.f), x);
-  lo = h2_bits(__floats2half2_rn(r.x, r.y));
+  const float2 f = __half22float2(h);
+  lo = h2_bits(__floats2half2_rn(x.x - f.x, x.y - f.y));
   return h;
 }
 // e^{i phase} of two contraction indices: slopes in units of 2^-32 turns, deltas
 __device__ __forceinline__ void sep_phasor2(int fix0, int fix1, int off, float2 delta, float fit, float2& c,
                                             float2& s) {
-  const float2 ph = make_float2(float(int(unsigned(fix0) * unsigned(off))), float(int(unsigned(fix1) * unsigned(off))));
-  const float2 x = ffma2(ph, make_float2(kTurnsToRad, kTurnsToRad), fmul2(delta, make_float2(fit, fit)));
-  __sincosf(x.x, &s.x, &c.x);
-  __sincosf(x.y, &s.y, &c.y);
+  __sincosf(sep_phase(fix0, off, delta.x, fit), &s.x, &c.x);
+  __sincosf(sep_phase(fix1, off, delta.y, fit), &s.y, &c.y);
 }
 __device__ __forceinline__ float2 pair_of(const float4& v, int h) {
   return h ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
