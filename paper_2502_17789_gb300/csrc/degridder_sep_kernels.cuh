@@ -13,22 +13,22 @@
 // sum over i takes one complex multiply-add per (visibility, column), 1/L of
 // the direct sum.
 //
-// One block of 512 threads per bundle of items (an item is up to kv
-// visibilities of one segment), split into two halves that run side by side.
-// Producers: per piece of 16 rows j of a block of 32 columns, thread = row
-// (p, i) x 8 rows j writes Z to tensor memory (two rows at a time in packed f32x2),
-// from Y pieces copied to shared memory two pieces ahead; one of them issues the
-// piece's 16 MMAs, whose commit frees it.  Consumers: while an item runs they
-// prepare the next one (phase slopes, the F side of all L rows, A-term samples;
-// double buffers), and take the accumulators, which alternate between two
-// column ranges of tensor memory from column block to column block, through
-// the sum over i; a transposing butterfly per item adds the 32 columns of a
-// warp.
+// One block of 24 warps per bundle of items (an item is up to kv
+// visibilities of one segment), whose warps have roles that run side by side.
+// Producers (two groups of 8 warps, every other piece each): per piece of 16 rows j of a block of 32 columns, thread = row
+// (p, i) x 8 rows j writes Z to tensor memory, from Y pieces that a loading warp
+// copies to shared memory up to four pieces ahead; an issuing warp starts the piece's
+// 16 MMAs, whose commit frees it.  Consumers take the accumulators, which alternate
+// between two column ranges of tensor memory from column block to column
+// block, through the sum over i: a transposing butterfly adds the 32 columns of a
+// warp.  Preparing warps write the next item's phase slopes, F side of all L
+// rows and A-term samples (double buffers) while one runs.
 //
-// Measured (GB300, MWA-like workload, 96 x 96 subgrids, segments of about 60
-// visibilities, per degrid call): 38.4 ms, against 46.8 ms with all threads
-// doing each step in turn and Z in shared memory, and 78.4 ms of the kernel
-// with one phasor per visibility and pixel (degridder_tc_kernels.cuh).
+// What bounds it: issue slots.  With all threads doing each step in turn and Z in
+// shared memory it took 46.8 ms (MWA-like workload, 96 x 96 subgrids, segments
+// of about 60 visibilities, per degrid call on GB300), with a half of producers
+// in step and a half of consumers 31.4 ms, with these roles 21.0 ms; the kernel with
+// one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.
 #pragma once
 
 #include "sep_common.cuh"
@@ -36,15 +36,23 @@
 namespace idg {
 
 constexpr int kDsepMaxVis = 64;   // visibilities per item at most
-constexpr int kDsepRing = 4;      // Z pieces in tensor memory
-constexpr int kDsepYRing = 3;     // Y pieces in shared memory
+constexpr int kDsepRing = 4;      // Y pieces in shared memory, Z pieces in tensor memory
+// roles: two producer groups of 8 warps, 4 consumer warps, the issuing warp, the loading warp, 2 preparing warps
+constexpr int kDsepThreads = 768, kDsepConsumer = 512, kDsepIssuer = 640, kDsepLoader = 672, kDsepPreparer = 704;
+constexpr int kDsepPreparers = 64;
+static_assert(kDsepMaxVis <= kDsepPreparers, "a visibility per preparing thread");
+constexpr int kDsepPreparerBar = 4;
+// registers per thread: 80 at launch, then by role
+constexpr int kDsepLaunchRegs = 80, kDsepProducerRegs = 72, kDsepConsumerRegs = 120, kDsepOtherRegs = 72;
+static_assert(512 * kDsepProducerRegs + 128 * (kDsepConsumerRegs + kDsepOtherRegs) <= kDsepThreads * kDsepLaunchRegs,
+              "registers");
 constexpr int kDsepColStride = 2 * kDsepMaxVis;       // between the two accumulators (re, im)
 constexpr int kDsepZCol = 2 * kDsepColStride;         // first column of the Z ring
 constexpr uint32_t kDsepTmemCols = 512;
 static_assert(kDsepZCol + kDsepRing * 48 <= int(kDsepTmemCols), "tensor memory");
 
 struct alignas(128) DsepShared {
-  float2 y[kDsepYRing][4][8][2][32];  // [piece][pol][row pair][re, im][column]
+  float2 y[kDsepRing][4][8][2][32];  // [piece][pol][row pair][re, im][column]
   float fix_a[2][kDsepMaxVis], fix_b[2][kDsepMaxVis], delta[2][kDsepMaxVis];  // [item parity][visibility]
   float out[kDsepMaxVis][8];
   // the producers' part of an item, by item parity
@@ -52,10 +60,13 @@ struct alignas(128) DsepShared {
     float scale;   // of Z, a power of two
     int sg, n_pad, diag;
   } info[2];
-  uint64_t ready[2];        // item prepared (8 consumer warps)
+  uint64_t ready[2];        // item prepared (2 preparing warps)
+  uint64_t loaded[kDsepRing]; // Y piece copied
+  uint64_t done[2];         // item's visibilities written, its operands read (4 consumer warps)
+  uint64_t filled[kDsepRing]; // Z piece written (8 producer warps)
   uint64_t empty[kDsepRing];  // Z piece read by its MMAs
   uint64_t full[2];         // accumulator complete
-  uint64_t drained[2];      // accumulator read (8 consumer warps)
+  uint64_t drained[2];      // accumulator read (4 consumer warps)
   uint32_t tmem;
   int fail;
 };
@@ -84,22 +95,12 @@ struct Dsep {
 
   static constexpr int kBlocks = L / 32, kPieces = L / 16;
 
-  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) { sep_wait(bar, parity, &S.fail, a.status); }
+  template <int SLEEP = 32>
+  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) {
+    sep_wait<SLEEP>(bar, parity, &S.fail, a.status);
+  }
 
   // ---------------------------------------------------------------- producers
-
-  // Y rows 16 jc .. of column block ib of batch subgrid sg, on their way to buffer y
-  __device__ __forceinline__ void fetch_y(int buf, int sg, int ib, int jc) {
-    const int pol = threadIdx.x >> 6, u = threadIdx.x & 63;  // 64 threads per correlation
-    if (pol < a.g.npol) {
-      // [pol][row pair][re, im][column]: 16 runs of 256 bytes
-      const float2* src = a.scratch + size_t(sg) * 4 * L * L + (size_t(pol) * (L / 2) + 8 * jc) * 2 * L + 32 * ib;
-      float2* dst = &S.y[buf][pol][0][0][0];
-#pragma unroll
-      for (int e = u; e < 256; e += 64) cp_async16(dst + 2 * e, src + (e >> 4) * L + 2 * (e & 15));
-    }
-    cp_async_commit();
-  }
 
   // Z of rows 16 jc .. for column block ib: thread = (p, i) x 8 rows j.  QUAD: node cells start at multiples of four
   // rows, so the cell can change only half way and not at every row.
@@ -107,7 +108,7 @@ struct Dsep {
   __device__ __forceinline__ void produce(uint32_t e_col, const float2* yb, const float4* samples, float scale,
                                           NodeWeight wx, int jc, __half2 fit_p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int p = warp & 3, g = warp >> 2, pa = p >> 1, pb = p & 1;
+    const int p = warp & 3, g = (warp >> 2) & 1, pa = p >> 1, pb = p & 1;
     const int nodes = a.g.nodes, step = nodes - 1;
     const bool stokes = a.g.npol == 1;
     constexpr int NE = DIAG ? 1 : 2;  // entries of each station's matrix that this correlation needs
@@ -139,7 +140,8 @@ struct Dsep {
     float f0 = float(rem) * (1.f / float(L));
     const float df = float(step) * (1.f / float(L));
     const float2* y0 = yb + (4 * g) * 64 + lane;  // [pol][row pair][re, im][column]
-    uint32_t re_hi[4], re_lo[4], re_c[4], im_hi[4], im_lo[4], im_c[4];
+    uint32_t re_hi[2], re_lo[2], re_c[2], im_hi[2], im_lo[2], im_c[2];
+    const uint32_t dst = e_col + (uint32_t(p * 32) << 16) + 4 * g;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       float2 yr[DIAG ? 1 : 4], yi[DIAG ? 1 : 4];  // Y at both rows of the pair
@@ -186,142 +188,166 @@ struct Dsep {
           zi.x = z.im;
         }
       }
-      re_c[w] = h2_bits(__hmul2(sep_split(zr, re_hi[w], re_lo[w]), fit_p));
-      im_c[w] = h2_bits(__hmul2(sep_split(zi, im_hi[w], im_lo[w]), fit_p));
+      const int o = w & 1;
+      re_c[o] = h2_bits(__hmul2(sep_split(zr, re_hi[o], re_lo[o]), fit_p));
+      im_c[o] = h2_bits(__hmul2(sep_split(zi, im_hi[o], im_lo[o]), fit_p));
+      if (o) {  // four rows at a time: the block's registers are spread over many producers
+        const uint32_t to = dst + (w & 2);
+        tmem_st2(to, re_hi[0], re_hi[1]);
+        tmem_st2(to + 8, im_hi[0], im_hi[1]);
+        tmem_st2(to + 16, re_lo[0], re_lo[1]);
+        tmem_st2(to + 24, im_lo[0], im_lo[1]);
+        tmem_st2(to + 32, re_c[0], re_c[1]);
+        tmem_st2(to + 40, im_c[0], im_c[1]);
+      }
     }
-    const uint32_t dst = e_col + (uint32_t(p * 32) << 16) + 4 * g;
-    tmem_st4(dst, re_hi);
-    tmem_st4(dst + 8, im_hi);
-    tmem_st4(dst + 16, re_lo);
-    tmem_st4(dst + 24, im_lo);
-    tmem_st4(dst + 32, re_c);
-    tmem_st4(dst + 40, im_c);
   }
 
+  // group 0 takes the even pieces of every item, group 1 the odd ones (an item has an even number); the warps of
+  // a group go their own way between the rings' barriers
   __device__ __forceinline__ void producer() {
-    const int lane = threadIdx.x & 31, nodes = a.g.nodes;
-    const bool issuer = uniform_warp() == 0;
+    const int lane = threadIdx.x & 31, nodes = a.g.nodes, grp = uniform_warp() >> 3;
     const bool quad = L % (nodes - 1) == 0 && L / (nodes - 1) % 4 == 0;
     const uint32_t tm = S.tmem;
-    uint32_t pg = 0, dg = 0, n = 0;  // pieces, accumulators and items of this block so far
-    int yb = 0;                      // pg % kDsepYRing
-    if (first >= last) return;
-    wait(&S.ready[0], 0);
-    int y_sg = S.info[0].sg, y_ib = 0, y_jc = 0;  // the piece of Y to fetch next
-    auto fetch_next = [&](int buf) {
-      fetch_y(buf, y_sg, y_ib, y_jc);
-      if (++y_jc == kPieces) {
-        y_jc = 0;
-        ++y_ib;
-      }
-    };
-    fetch_next(0);
-    fetch_next(1);
-    cp_async_wait<1>();
-    half_sync(kSepProducerBar);
+    uint32_t n = 0, pg = grp;  // items and (both groups') pieces of this block so far
     for (int idx = first; idx < last; idx += stride, ++n) {
-      const DsepShared::Info info = S.info[n & 1];
-      const bool more = idx + stride < last;
+      wait(&S.ready[n & 1], (n >> 1) & 1);
+      const float scale = S.info[n & 1].scale;
+      const bool diag = S.info[n & 1].diag != 0;
       const float4* samples = raw + (n & 1) * 4 * nodes * nodes;
-      const uint32_t block = uint32_t(info.n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
-      const uint32_t f0 = smem_u32(fside) + (n & 1) * uint32_t(a.kv) * L * 12;
 #pragma unroll 1
-      for (int ib = 0; ib < kBlocks; ++ib, ++dg) {
+      for (int ib = 0; ib < kBlocks; ++ib) {
         const int i = ib * 32 + lane;
         const NodeWeight wx = node_weight(i, nodes, L);
         const __half2 fit_p = __float2half2_rn(__ldg(a.sep.p + i));
 #pragma unroll 1
-        for (int jc = 0; jc < kPieces; ++jc, ++pg) {
-          // two pieces ahead, in the next item past this one's end
-          if (y_ib == kBlocks && more) {
-            wait(&S.ready[(n + 1) & 1], ((n + 1) >> 1) & 1);
-            y_sg = S.info[(n + 1) & 1].sg;
-            y_ib = 0;
-          }
-          const int buf = yb;
-          if (++yb == kDsepYRing) yb = 0;
-          if (y_ib < kBlocks)
-            fetch_next(buf == 0 ? 2 : buf - 1);
-          else
-            cp_async_commit();  // keeps the count of groups
+        for (int jc = grp; jc < kPieces; jc += 2, pg += 2) {
           const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
+          wait(&S.loaded[slot], turn & 1);
           if (turn > 0) {
             wait(&S.empty[slot], (turn - 1) & 1);
             tc_fence_after();
           }
           const uint32_t e_col = tm + kDsepZCol + slot * 48;
-          const float2* y = &S.y[buf][0][0][0][0];
+          const float2* y = &S.y[slot][0][0][0][0];
           if (quad) {
-            if (info.diag)
-              produce<true, true>(e_col, y, samples, info.scale, wx, jc, fit_p);
+            if (diag)
+              produce<true, true>(e_col, y, samples, scale, wx, jc, fit_p);
             else
-              produce<false, true>(e_col, y, samples, info.scale, wx, jc, fit_p);
-          } else if (info.diag) {
-            produce<true, false>(e_col, y, samples, info.scale, wx, jc, fit_p);
+              produce<false, true>(e_col, y, samples, scale, wx, jc, fit_p);
+          } else if (diag) {
+            produce<true, false>(e_col, y, samples, scale, wx, jc, fit_p);
           } else {
-            produce<false, false>(e_col, y, samples, info.scale, wx, jc, fit_p);
+            produce<false, false>(e_col, y, samples, scale, wx, jc, fit_p);
           }
-          cp_async_wait<1>();
           tmem_wait_st();
           tc_fence_before();
-          half_sync(kSepProducerBar);
-          if (issuer && elect_one()) {
-            // the accumulator's previous column block (two back) has been read
-            if (jc == 0 && dg >= 2) wait(&S.drained[dg & 1], ((dg >> 1) - 1) & 1);
-            tc_fence_after();
-            sep_product(tm + (dg & 1) * kDsepColStride, e_col, f0 + jc * chunk, info.n_pad, block, group, level, jc == 0);
-            sep_commit(&S.empty[slot]);
-            if (jc + 1 == kPieces) sep_commit(&S.full[dg & 1]);
-          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&S.filled[slot]);
         }
       }
     }
-    cp_async_wait<0>();
   }
 
-  // ---------------------------------------------------------------- consumers
+  // ---------------------------------------------------------------- loader (one warp)
+
+  // Y in scratch: [pol][column block][row pair][re, im][32 columns], so a piece is one run of 4 KB per plane
+  __device__ __forceinline__ void loader() {
+    uint32_t n = 0, pg = 0;  // items and pieces of this block so far
+    for (int idx = first; idx < last; idx += stride, ++n) {
+      wait<64>(&S.ready[n & 1], (n >> 1) & 1);
+      const float2* Y = a.scratch + size_t(S.info[n & 1].sg) * 4 * L * L;
+#pragma unroll 1
+      for (int t = 0; t < kBlocks * kPieces; ++t, ++pg) {
+        const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
+        if (turn > 0) wait(&S.filled[slot], (turn - 1) & 1);  // the ring's previous piece has been read
+        __syncwarp();
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&S.loaded[slot], 4096 * a.g.npol);
+          for (int pol = 0; pol < a.g.npol; ++pol)
+            bulk_copy_g2s(&S.y[slot][pol][0][0][0], Y + size_t(pol) * L * L + t * 512, 4096, &S.loaded[slot]);
+        }
+        __syncwarp();
+      }
+    }
+  }
+
+  // ---------------------------------------------------------------- issuer (one warp)
+
+  __device__ __forceinline__ void issuer() {
+    const uint32_t tm = S.tmem;
+    uint32_t n = 0, pg = 0, dg = 0;  // items, pieces and accumulators of this block so far
+    for (int idx = first; idx < last; idx += stride, ++n) {
+      wait(&S.ready[n & 1], (n >> 1) & 1);
+      const int n_pad = S.info[n & 1].n_pad;
+      const uint32_t block = uint32_t(n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
+      const uint32_t f0 = smem_u32(fside) + (n & 1) * uint32_t(a.kv) * L * 12;
+#pragma unroll 1
+      for (int ib = 0; ib < kBlocks; ++ib, ++dg) {
+        // the accumulator's previous column block (two back) has been read
+        if (dg >= 2) wait(&S.drained[dg & 1], ((dg >> 1) - 1) & 1);
+#pragma unroll 1
+        for (int jc = 0; jc < kPieces; ++jc, ++pg) {
+          const uint32_t slot = pg % kDsepRing;
+          wait(&S.filled[slot], (pg / kDsepRing) & 1);
+          tc_fence_after();
+          __syncwarp();
+          if (elect_one()) {
+            sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block, group,
+                        level, jc == 0);
+            sep_commit(&S.empty[slot]);
+            if (jc + 1 == kPieces) sep_commit(&S.full[dg & 1]);
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+
+  // ---------------------------------------------------------------- preparers
 
   // item idx, number n of the block: phase slopes, A-term samples, conj(F) at all rows, the producers' part
   __device__ __forceinline__ void prepare(int idx, uint32_t n) {
-    const int tid = threadIdx.x - kSepHalf, lane = tid & 31;
+    const int tid = threadIdx.x - kDsepPreparer, lane = tid & 31;
     const DegridItem item = a.items[idx];
     const SubgridDesc sd = a.sg[item.sg];
     const SegmentDesc seg = a.seg[item.segment];
     const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
     const int nodes = a.g.nodes, n4 = nodes * nodes * 2;
     const int sp = seg.interval * a.g.n_st + sd.p, sq = seg.interval * a.g.n_st + sd.q;
+    // what comes from global memory, before the buffers are free
+    int fa = 0, fb = 0;
+    float dl = 0.f;
+    if (tid < nv) {
+      const int nc = sd.c1 - sd.c0, k = item.k_begin + tid, row = k / nc, ch = sd.c0 + (k - row * nc);
+      const double* r = a.uvw + (size_t(sd.b) * a.g.n_t + sd.t0 + row) * 3;
+      const double fs = subgrid_sign(sd) * a.fscale[ch], inv_l = 1.0 / double(L);
+      fa = sep_fix(((r[0] * fs) * a.g.fov - double(sd.x0 + L / 2 - a.g.N / 2)) * inv_l);
+      fb = sep_fix(((r[1] * fs) * a.g.fov - double(sd.y0 + L / 2 - a.g.N / 2)) * inv_l);
+      dl = float(r[2] * fs - (double(a.w_ref[item.sg]) + subgrid_w0(a.g, sd)));
+    }
+    // scale of Z from the largest components of Y and of the A-terms' nodes
+    float ym = 0.f;
+    for (int k = 0; k < a.g.npol; ++k) ym = fmaxf(ym, a.ymax[item.sg * 4 + k]);
+    const DsepShared::Info info = {sep_scale(ym * a.amax[sp] * a.amax[sq]), item.sg, n_pad, a.adiag[sp] & a.adiag[sq]};
+    if (n >= 2) wait<100>(&S.done[b], ((n >> 1) - 1) & 1);  // the buffers' previous item (two back) is done
     {
       const float4* src = reinterpret_cast<const float4*>(a.aterms);
       float4* dst = raw + size_t(b) * 2 * n4;
-      for (int e = tid; e < 2 * n4; e += kSepHalf)
+      for (int e = tid; e < 2 * n4; e += kDsepPreparers)
         cp_async16(dst + e, src + (e < n4 ? size_t(sp) * n4 + e : size_t(sq) * n4 + e - n4));
       cp_async_commit();
     }
     if (tid < n_pad) {
-      int fa = 0, fb = 0;
-      float dl = 0.f;
-      if (tid < nv) {
-        const int nc = sd.c1 - sd.c0, k = item.k_begin + tid, row = k / nc, ch = sd.c0 + (k - row * nc);
-        const double* r = a.uvw + (size_t(sd.b) * a.g.n_t + sd.t0 + row) * 3;
-        const double fs = subgrid_sign(sd) * a.fscale[ch], inv_l = 1.0 / double(L);
-        fa = sep_fix(((r[0] * fs) * a.g.fov - double(sd.x0 + L / 2 - a.g.N / 2)) * inv_l);
-        fb = sep_fix(((r[1] * fs) * a.g.fov - double(sd.y0 + L / 2 - a.g.N / 2)) * inv_l);
-        dl = float(r[2] * fs - (double(a.w_ref[item.sg]) + subgrid_w0(a.g, sd)));
-      }
       S.fix_a[b][tid] = __int_as_float(fa);
       S.fix_b[b][tid] = __int_as_float(fb);
       S.delta[b][tid] = dl;
     }
-    if (tid == 0) {
-      // scale of Z from the largest components of Y and of the A-terms' nodes
-      float ym = 0.f;
-      for (int k = 0; k < a.g.npol; ++k) ym = fmaxf(ym, a.ymax[item.sg * 4 + k]);
-      S.info[b] = {sep_scale(ym * a.amax[sp] * a.amax[sq]), item.sg, n_pad, a.adiag[sp] && a.adiag[sq]};
-    }
-    half_sync(kSepConsumerBar);
+    if (tid == 0) S.info[b] = info;
+    asm volatile("bar.sync %0, %1;" ::"n"(kDsepPreparerBar), "n"(kDsepPreparers) : "memory");
     const uint32_t block = uint32_t(n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
     const uint32_t base = smem_u32(fside) + b * uint32_t(a.kv) * L * 12;
-    for (int e = tid; e < n_pad * (L / 8); e += kSepHalf) {
+    for (int e = tid; e < n_pad * (L / 8); e += kDsepPreparers) {
       const int o = e / n_pad, k = e - o * n_pad;
       const int fix = __float_as_int(S.fix_b[b][k]);
       const float dl = S.delta[b][k];
@@ -356,84 +382,76 @@ struct Dsep {
     if (lane == 0) mbar_arrive(&S.ready[b]);
   }
 
+  __device__ __forceinline__ void preparer() {
+    uint32_t n = 0;
+    for (int idx = first; idx < last; idx += stride, ++n) prepare(idx, n);
+  }
+
+  // ---------------------------------------------------------------- consumers
+
+  // thread = row (p, i) of the column block
   __device__ __forceinline__ void consumer() {
-    const int tid = threadIdx.x - kSepHalf, warp = tid >> 5, lane = tid & 31;
-    const bool poller = uniform_warp() == kSepHalf / 32;
+    const int tid = threadIdx.x - kDsepConsumer, pol = tid >> 5, lane = tid & 31;
     uint32_t dg = 0, n = 0;  // accumulators and items of this block so far
-    if (first >= last) return;
-    prepare(first, 0);
     for (int idx = first; idx < last; idx += stride, ++n) {
-      if (idx + stride < last) prepare(idx + stride, n + 1);
       const DegridItem item = a.items[idx];
       const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
+      wait(&S.ready[b], (n >> 1) & 1);
       const float inv = 1.f / S.info[b].scale;
-      // thread = row (p, i), 16-visibility blocks warp / 4 and warp / 4 + 2
-      float2 re[2][8], im[2][8];  // visibility pairs
+      float sum[kDsepMaxVis / 16];  // component lane & 1 of visibility 16 h + lane / 2
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) re[h][k] = im[h][k] = make_float2(0.f, 0.f);
+      for (int h = 0; h < kDsepMaxVis / 16; ++h) sum[h] = 0.f;
 #pragma unroll 1
       for (int ib = 0; ib < kBlocks; ++ib, ++dg) {
         const int i = ib * 32 + lane;
         const float fit_a = __ldg(a.sep.a + i);
-        if (poller) wait(&S.full[dg & 1], (dg >> 1) & 1);
-        half_sync(kSepConsumerBar);
+        wait<250>(&S.full[dg & 1], (dg >> 1) & 1);
         tc_fence_after();
-        const uint32_t d = S.tmem + (uint32_t((warp & 3) * 32) << 16) + (dg & 1) * kDsepColStride;
+        const uint32_t d = S.tmem + (uint32_t(pol * 32) << 16) + (dg & 1) * kDsepColStride;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k0 = 16 * ((warp >> 2) + 2 * h);
+        for (int h = 0; h < kDsepMaxVis / 16; ++h) {
+          const int k0 = 16 * h;
           if (k0 < n_pad) {
-            float dr[16], di[16];
-            tmem_ld16(dr, d + k0);
-            tmem_ld16(di, d + n_pad + k0);
-            tmem_wait_ld();
-            const float4* fx = reinterpret_cast<const float4*>(&S.fix_a[b][k0]);
-            const float4* dl = reinterpret_cast<const float4*>(&S.delta[b][k0]);
+            float v[32];  // (re, im) of 16 visibilities
+            {
+              float dr[16], di[16];
+              tmem_ld16(dr, d + k0);
+              tmem_ld16(di, d + n_pad + k0);
+              tmem_wait_ld();
+              const float4* fx = reinterpret_cast<const float4*>(&S.fix_a[b][k0]);
+              const float4* dl = reinterpret_cast<const float4*>(&S.delta[b][k0]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const float2 f = pair_of(fx[k >> 1], k & 1);
-              float2 c, s;
-              sep_phasor2(__float_as_int(f.x), __float_as_int(f.y), i - L / 2, pair_of(dl[k >> 1], k & 1), fit_a, c, s);
-              const float2 r = make_float2(dr[2 * k], dr[2 * k + 1]), m = make_float2(di[2 * k], di[2 * k + 1]);
-              re[h][k].x = fmaf(r.x, c.x, fmaf(m.x, s.x, re[h][k].x));
-              re[h][k].y = fmaf(r.y, c.y, fmaf(m.y, s.y, re[h][k].y));
-              im[h][k].x = fmaf(m.x, c.x, fmaf(-r.x, s.x, im[h][k].x));
-              im[h][k].y = fmaf(m.y, c.y, fmaf(-r.y, s.y, im[h][k].y));
+              for (int k = 0; k < 16; ++k) {
+                const float4 f4 = fx[k >> 2], d4 = dl[k >> 2];
+                const float f = (k & 3) == 0 ? f4.x : (k & 3) == 1 ? f4.y : (k & 3) == 2 ? f4.z : f4.w;
+                const float dk = (k & 3) == 0 ? d4.x : (k & 3) == 1 ? d4.y : (k & 3) == 2 ? d4.z : d4.w;
+                float c, s;
+                __sincosf(sep_phase(__float_as_int(f), i - L / 2, dk, fit_a), &s, &c);
+                v[2 * k] = fmaf(dr[k], c, di[k] * s);
+                v[2 * k + 1] = fmaf(di[k], c, -dr[k] * s);
+              }
             }
+            // sum over the 32 columns of the warp, lane l ending with value l
+#pragma unroll
+            for (int w = 16; w; w >>= 1) {
+              const bool up = lane & w;
+#pragma unroll
+              for (int k = 0; k < w; ++k) {
+                const float keep = up ? v[k + w] : v[k], give = up ? v[k] : v[k + w];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+              }
+            }
+            sum[h] += v[0];
           }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.drained[dg & 1]);
       }
-      // sums over the 32 columns of the warp: lane l ends with component l & 1 of visibility l / 2 of the block
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k0 = 16 * ((warp >> 2) + 2 * h);
-        if (k0 < n_pad) {
-          float v[32];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            v[4 * k] = re[h][k].x;
-            v[4 * k + 1] = im[h][k].x;
-            v[4 * k + 2] = re[h][k].y;
-            v[4 * k + 3] = im[h][k].y;
-          }
-#pragma unroll
-          for (int w = 16; w; w >>= 1) {
-            const bool up = lane & w;
-#pragma unroll
-            for (int k = 0; k < w; ++k) {
-              const float keep = up ? v[k + w] : v[k], give = up ? v[k] : v[k + w];
-              v[k] = keep + __shfl_xor_sync(0xffffffffu, give, w);
-            }
-          }
-          S.out[k0 + (lane >> 1)][2 * (warp & 3) + (lane & 1)] = inv * v[0];
-        }
-      }
-      half_sync(kSepConsumerBar);
+      for (int h = 0; h < kDsepMaxVis / 16; ++h)
+        if (16 * h < n_pad) S.out[16 * h + (lane >> 1)][2 * pol + (lane & 1)] = inv * sum[h];
+      asm volatile("bar.sync %0, 128;" ::"n"(kSepConsumerBar) : "memory");
       if (tid < nv) {
         const SubgridDesc sd = a.sg[item.sg];
         const int nc = sd.c1 - sd.c0, k = item.k_begin + tid, row = k / nc;
@@ -444,7 +462,8 @@ struct Dsep {
         a.vis[2 * vrow] = v0;
         a.vis[2 * vrow + 1] = v1;
       }
-      half_sync(kSepConsumerBar);  // S.out free
+      if (lane == 0) mbar_arrive(&S.done[b]);
+      asm volatile("bar.sync %0, 128;" ::"n"(kSepConsumerBar) : "memory");  // S.out free
     }
   }
 };
@@ -456,11 +475,16 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
   DsepShared& S = *reinterpret_cast<DsepShared*>(smem);
   unsigned char* fside = reinterpret_cast<unsigned char*>(&S + 1);
   if (threadIdx.x == 0) {
-    for (int k = 0; k < kDsepRing; ++k) mbar_init(&S.empty[k], 1);
+    for (int k = 0; k < kDsepRing; ++k) {
+      mbar_init(&S.empty[k], 1);
+      mbar_init(&S.filled[k], 8);
+      mbar_init(&S.loaded[k], 1);
+    }
     for (int k = 0; k < 2; ++k) {
       mbar_init(&S.full[k], 1);
-      mbar_init(&S.drained[k], kSepHalf / 32);
-      mbar_init(&S.ready[k], kSepHalf / 32);
+      mbar_init(&S.drained[k], 4);
+      mbar_init(&S.ready[k], kDsepPreparers / 32);
+      mbar_init(&S.done[k], 4);
     }
     fence_mbar_init();
     S.fail = 0;
@@ -470,15 +494,27 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
   __syncthreads();
   tc_fence_after();
   Dsep<L> it{a, S, fside, reinterpret_cast<float4*>(fside + size_t(2) * a.kv * L * 12), first, last, stride};
-  if (threadIdx.x < kSepHalf)
+  if (threadIdx.x < kDsepConsumer) {
+    regs_give<kDsepProducerRegs>();
     it.producer();
-  else
+  } else if (threadIdx.x < kDsepIssuer) {
+    regs_take<kDsepConsumerRegs>();
     it.consumer();
-  // after a wait that gave up: one more bounded wait for MMAs that may still run before their memory goes
+  } else {
+    regs_give<kDsepOtherRegs>();
+    if (threadIdx.x < kDsepLoader)
+      it.issuer();
+    else if (threadIdx.x < kDsepPreparer)
+      it.loader();
+    else
+      it.preparer();
+  }
+  // after a wait that gave up: one more bounded wait for copies and MMAs that may still run before their memory goes
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x < 32) {
     if (*reinterpret_cast<volatile int*>(&S.fail) && threadIdx.x == 0) {
+      for (int k = 0; k < kDsepRing; ++k) mbar_wait_bounded(&S.loaded[k], 0, kWaitLimitNs / 8);
       sep_commit(&S.full[0]);
       mbar_wait_bounded(&S.full[0], 0);
     }
@@ -489,7 +525,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
 }
 
 template <int L>
-__global__ void __launch_bounds__(kSepThreads, 1) degridder_sep_kernel(const DegridArgs a, int bundle) {
+__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_kernel(const DegridArgs a, int bundle) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
   const int b = blockIdx.x;
   if (bundle > 0)  // neighbouring items (segments of one subgrid)
@@ -500,7 +536,7 @@ __global__ void __launch_bounds__(kSepThreads, 1) degridder_sep_kernel(const Deg
 
 // One launch over the items of several plans (items = (plan slot, item index))
 template <int L>
-__global__ void __launch_bounds__(kSepThreads, 1) degridder_sep_multi_kernel(const DegridArgs* args,
+__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_multi_kernel(const DegridArgs* args,
                                                                             const int2* items) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
   __shared__ __align__(16) unsigned char s_args_raw[sizeof(DegridArgs)];
@@ -512,14 +548,17 @@ __global__ void __launch_bounds__(kSepThreads, 1) degridder_sep_multi_kernel(con
 
 template <int L>
 int configure_degridder_sep_l(int* persistent_blocks) {
-  cudaError_t e = cudaFuncSetAttribute(degridder_sep_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  // the roles' register split is of the registers the block is launched with
+  cudaError_t e = sep_check_regs(degridder_sep_kernel<L>, kDsepLaunchRegs);
+  if (e == cudaSuccess) e = sep_check_regs(degridder_sep_multi_kernel<L>, kDsepLaunchRegs);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(degridder_sep_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kSepSmemLimit);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(degridder_sep_multi_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSepSmemLimit);
   int dev = 0, sms = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  *persistent_blocks = sms;  // 512 threads of up to 128 registers: one block per SM
+  *persistent_blocks = sms;  // one block per SM (registers, tensor memory)
   return int(e);
 }
 
@@ -529,11 +568,13 @@ int degridder_sep_vis_l(int nodes) {
 }
 
 template <int L>
-int launch_degridder_sep_l(const DegridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream) {
+int launch_degridder_sep_l(const DegridArgs& args, int n_items, int persistent_blocks, int bundle, void* stream) {
   if (n_items <= 0) return 0;
+  DegridArgs a = args;
+  a.n_items = n_items;
   const int blocks = persistent_blocks > 0 ? (persistent_blocks < n_items ? persistent_blocks : n_items)
                                            : (n_items + bundle - 1) / bundle;
-  degridder_sep_kernel<L><<<blocks, kSepThreads, dsep_smem<L>(a.kv, a.g.nodes), cudaStream_t(stream)>>>(
+  degridder_sep_kernel<L><<<blocks, kDsepThreads, dsep_smem<L>(a.kv, a.g.nodes), cudaStream_t(stream)>>>(
       a, persistent_blocks > 0 ? 0 : bundle);
   return int(cudaGetLastError());
 }
@@ -547,7 +588,7 @@ int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* items, int 
     const size_t s = dsep_smem<L>(dsep_vis<L>(n), n);
     smem = s > smem ? s : smem;
   }
-  degridder_sep_multi_kernel<L><<<n_items, kSepThreads, smem, cudaStream_t(stream)>>>(args, items);
+  degridder_sep_multi_kernel<L><<<n_items, kDsepThreads, smem, cudaStream_t(stream)>>>(args, items);
   return int(cudaGetLastError());
 }
 

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_blocks(L)) splitter_ifft_
     return;
   }
   // what every visibility of the subgrid shares (sep_common.cuh), once per pixel here instead of once per segment;
-  // written as the degridder reads it, [row pair][re, im][column] of the values at both rows
+  // written as the degridder reads it, [32 columns][row pair][re, im][column] of the values at both rows
   const float w_ref = a.w_ref[sgi];
   float2* pairs = a.scratch + (size_t(sgi) * 4 + pol) * L * L;
   float m = 0.f;
@@ -224,8 +224,9 @@ __global__ void __launch_bounds__(kFftThreads, fft_min_blocks(L)) splitter_ifft_
     const float2 re = make_float2(t0 * (v0.x * p0.x + v0.y * p0.y), t1 * (v1.x * p1.x + v1.y * p1.y));
     const float2 im = make_float2(t0 * (v0.y * p0.x - v0.x * p0.y), t1 * (v1.y * p1.x - v1.x * p1.y));
     m = fmaxf(fmaxf(fmaxf(m, fabsf(re.x)), fabsf(re.y)), fmaxf(fabsf(im.x), fabsf(im.y)));
-    pairs[(size_t(jp) * 2) * L + i] = re;
-    pairs[(size_t(jp) * 2 + 1) * L + i] = im;
+    float2* dst = pairs + (size_t(i >> 5) * (L / 2) + jp) * 64 + (i & 31);
+    dst[0] = re;
+    dst[32] = im;
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));

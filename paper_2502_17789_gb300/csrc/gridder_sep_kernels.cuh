@@ -25,9 +25,9 @@
 //
 // What bounds it: issue slots, then shared memory.  With the E side in
 // shared memory too, operands, their reads by the MMAs and a transpose per 16 rows kept
-// shared memory 80 % busy (21.2 ms where this takes 17.6); the E side in tensor
+// shared memory 80 % busy (21.2 ms where this takes 17.0); the E side in tensor
 // memory costs none.  Measured (GB300, MWA-like workload, 96 x 96 subgrids,
-// segments of about 60 visibilities, per grid call): 17.6 ms, against 81.7 ms of the
+// segments of about 60 visibilities, per grid call): 17.0 ms, against 81.7 ms of the
 // kernel with one phasor per visibility and pixel (gridder_tc_kernels.cuh);
 // grid error 9e-7 against 2.2e-6.
 #pragma once
@@ -243,7 +243,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
     for (int s = 0; s < sd.seg_count; ++s, ++sc) {
       const bool diag = diag_next != 0;
       const float inv = inv_next;
-      if (poller) sep_wait(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
+      if (poller) sep_wait<100>(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
       half_sync(kSepConsumerBar);  // the segment's sums complete; S.x and the other samples free
       tc_fence_after();
       const bool more = s + 1 < sd.seg_count;
@@ -484,7 +484,10 @@ __global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_multi_kernel(const
 
 template <int L>
 int configure_gridder_sep_l(int* persistent_blocks) {
-  cudaError_t e = cudaFuncSetAttribute(gridder_sep_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  // the halves' register split is of the registers the block is launched with
+  cudaError_t e = sep_check_regs(gridder_sep_kernel<L>, 128);
+  if (e == cudaSuccess) e = sep_check_regs(gridder_sep_multi_kernel<L>, 128);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gridder_sep_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kSepSmemLimit);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gridder_sep_multi_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSepSmemLimit);
@@ -496,8 +499,10 @@ int configure_gridder_sep_l(int* persistent_blocks) {
 }
 
 template <int L>
-int launch_gridder_sep_l(const GridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream) {
+int launch_gridder_sep_l(const GridArgs& args, int n_items, int persistent_blocks, int bundle, void* stream) {
   if (n_items <= 0) return 0;
+  GridArgs a = args;
+  a.n_items = n_items;
   const int blocks = persistent_blocks > 0 ? (persistent_blocks < n_items ? persistent_blocks : n_items)
                                            : (n_items + bundle - 1) / bundle;
   gridder_sep_kernel<L><<<blocks, kSepThreads, gsep_smem<L>(a.g.nodes), cudaStream_t(stream)>>>(

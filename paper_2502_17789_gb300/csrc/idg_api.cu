@@ -797,7 +797,7 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
 // items per block of the separable-phasor kernels: some blocks per SM must remain to even out the load, and
 // more items per block than that spread the block's set-up
 static int sep_bundle(const idg_plan* p, int n_items) {
-  return std::max(1, std::min(8, n_items / (8 * std::max(1, int(p->sms)))));
+  return std::max(1, std::min(24, n_items / (8 * std::max(1, int(p->sms)))));
 }
 
 // record staging and the gridder of the plan's kind (FP32 pipe or tensor cores)

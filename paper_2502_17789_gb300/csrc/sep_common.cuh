@@ -83,6 +83,9 @@ __device__ __forceinline__ void tmem_st4(uint32_t addr, const uint32_t (&v)[4]) 
                "r"(v[2]), "r"(v[3])
                : "memory");
 }
+__device__ __forceinline__ void tmem_st2(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -91,7 +94,7 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 // The block's first 256 threads (producers) write operands and issue MMAs, the
 // others (consumers) read the accumulators; each half has its own barrier.
 constexpr int kSepHalf = 256;
-constexpr int kSepProducerBar = 1, kSepConsumerBar = 2;
+constexpr int kSepProducerBar = 1, kSepConsumerBar = 2;  // + 2 for a second producer group
 __device__ __forceinline__ void half_sync(int bar) {
   asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory");
 }
@@ -108,20 +111,32 @@ __device__ __forceinline__ void regs_give() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
 }
 
-// bounded wait that reports a timeout once and then lets every later wait of the block pass.  Where many warps wait
-// for long, one polls and the others stand at a named barrier: polling takes issue slots from the working warps.
+// host: whether the kernel was built with the registers per thread that its roles divide among them (a block whose
+// roles ask for more than it was launched with would wait for them forever)
+template <typename K>
+cudaError_t sep_check_regs(K kernel, int regs) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  return e != cudaSuccess ? e : at.numRegs == regs ? cudaSuccess : cudaErrorInvalidConfiguration;
+}
+
+// bounded wait that reports a timeout once and then lets every later wait of the block pass.  It sleeps between
+// polls, SLEEP ns where the wait is expected to be long: polling takes issue slots from the working warps (with 40 ns
+// throughout, a quarter of the degridder's instructions were polls).
+template <int SLEEP = 32>
 __device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, int* status) {
   if (mbar_try_wait(bar, parity)) return;
   if (*reinterpret_cast<volatile int*>(fail)) return;
   const uint64_t t0 = global_ns();
-  while (!mbar_try_wait(bar, parity)) {
-    if (global_ns() - t0 > kWaitLimitNs) {
-      atomicOr(status, kStatusTimeout);
-      *reinterpret_cast<volatile int*>(fail) = 1;
-      return;
+  do {
+#pragma unroll 1
+    for (int k = 0; k < 64; ++k) {
+      __nanosleep(SLEEP);
+      if (mbar_try_wait(bar, parity)) return;
     }
-    __nanosleep(40);
-  }
+  } while (global_ns() - t0 <= kWaitLimitNs);
+  atomicOr(status, kStatusTimeout);
+  *reinterpret_cast<volatile int*>(fail) = 1;
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
