@@ -13,8 +13,8 @@
 // sum over i takes one complex multiply-add per (visibility, column), 1/L of
 // the direct sum.
 //
-// One block of 24 warps per bundle of items (an item is up to kv
-// visibilities of one segment), whose warps have roles that run side by side.
+// A block of 24 warps works through a share of the items (an item is up to kv
+// visibilities of one segment); its warps have roles that run side by side.
 // Producers (two groups of 8 warps, every other piece each): per piece of 16 rows j of a block of 32 columns, thread = row
 // (p, i) x 8 rows j writes Z to tensor memory, from Y pieces that a loading warp
 // copies to shared memory up to four pieces ahead; an issuing warp starts the piece's
@@ -397,7 +397,7 @@ struct Dsep {
       const DegridItem item = a.items[idx];
       const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
       wait(&S.ready[b], (n >> 1) & 1);
-      const float inv = 1.f / S.info[b].scale;
+      const float inv = sep_unbias(kPieces) / S.info[b].scale;
       float sum[kDsepMaxVis / 16];  // component lane & 1 of visibility 16 h + lane / 2
 #pragma unroll
       for (int h = 0; h < kDsepMaxVis / 16; ++h) sum[h] = 0.f;
@@ -524,26 +524,26 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
   }
 }
 
+// Blocks take every gridDim-th item of the longest-first list: an even share of long and short items each, the
+// neighbouring items of a subgrid at the same time on neighbouring SMs, and one set-up per block
 template <int L>
-__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_kernel(const DegridArgs a, int bundle) {
+__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_kernel(const DegridArgs a) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
-  const int b = blockIdx.x;
-  if (bundle > 0)  // neighbouring items (segments of one subgrid)
-    degridder_sep_block<L>(a, b * bundle, imin((b + 1) * bundle, a.n_items), 1, sep_smem);
-  else             // persistent: every gridDim-th item of the longest-first list
-    degridder_sep_block<L>(a, b, a.n_items, gridDim.x, sep_smem);
+  degridder_sep_block<L>(a, blockIdx.x, a.n_items, gridDim.x, sep_smem);
 }
 
-// One launch over the items of several plans (items = (plan slot, item index))
+// One launch over the items of several plans: blocks = (plan slot, first item), each taking every `stride`-th item of
+// its plan from there
 template <int L>
 __global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_multi_kernel(const DegridArgs* args,
-                                                                            const int2* items) {
+                                                                            const int2* blocks) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
   __shared__ __align__(16) unsigned char s_args_raw[sizeof(DegridArgs)];
-  const int2 it = items[blockIdx.x];
+  const int2 it = blocks[blockIdx.x];
   if (threadIdx.x == 0) memcpy(s_args_raw, args + it.x, sizeof(DegridArgs));
   __syncthreads();
-  degridder_sep_block<L>(*reinterpret_cast<const DegridArgs*>(s_args_raw), it.y, it.y + 1, 1, sep_smem);
+  const DegridArgs& a = *reinterpret_cast<const DegridArgs*>(s_args_raw);
+  degridder_sep_block<L>(a, it.y, a.n_items, a.stride, sep_smem);
 }
 
 template <int L>
@@ -568,27 +568,24 @@ int degridder_sep_vis_l(int nodes) {
 }
 
 template <int L>
-int launch_degridder_sep_l(const DegridArgs& args, int n_items, int persistent_blocks, int bundle, void* stream) {
+int launch_degridder_sep_l(const DegridArgs& args, int n_items, int blocks, void* stream) {
   if (n_items <= 0) return 0;
   DegridArgs a = args;
   a.n_items = n_items;
-  const int blocks = persistent_blocks > 0 ? (persistent_blocks < n_items ? persistent_blocks : n_items)
-                                           : (n_items + bundle - 1) / bundle;
-  degridder_sep_kernel<L><<<blocks, kDsepThreads, dsep_smem<L>(a.kv, a.g.nodes), cudaStream_t(stream)>>>(
-      a, persistent_blocks > 0 ? 0 : bundle);
+  degridder_sep_kernel<L><<<blocks, kDsepThreads, dsep_smem<L>(a.kv, a.g.nodes), cudaStream_t(stream)>>>(a);
   return int(cudaGetLastError());
 }
 
 template <int L>
-int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* items, int n_items, int max_nodes,
+int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
                                  void* stream) {
-  if (n_items <= 0) return 0;
+  if (n_blocks <= 0) return 0;
   size_t smem = 0;  // the largest layout of any plan of up to max_nodes (a plan's items are cut to its own)
   for (int n = 2; n <= max_nodes; ++n) {
     const size_t s = dsep_smem<L>(dsep_vis<L>(n), n);
     smem = s > smem ? s : smem;
   }
-  degridder_sep_multi_kernel<L><<<n_items, kDsepThreads, smem, cudaStream_t(stream)>>>(args, items);
+  degridder_sep_multi_kernel<L><<<n_blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(args, blocks);
   return int(cudaGetLastError());
 }
 

@@ -281,12 +281,12 @@ IDG_GRID_TC_EXTERN(128)
 template <int L>
 int configure_gridder_sep_l(int* persistent_blocks);
 template <int L>
-int launch_gridder_sep_l(const GridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
+int launch_gridder_sep_l(const GridArgs& a, int n_items, int blocks, void* stream);
 template <int L>
 int launch_gridder_sep_multi_l(const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
 #define IDG_GRID_SEP_EXTERN(L)                                                                                   \
   extern template int configure_gridder_sep_l<L>(int*);                                                         \
-  extern template int launch_gridder_sep_l<L>(const GridArgs&, int, int, int, void*);                           \
+  extern template int launch_gridder_sep_l<L>(const GridArgs&, int, int, void*);                                \
   extern template int launch_gridder_sep_multi_l<L>(const GridArgs*, const int2*, int, int, void*);
 IDG_GRID_SEP_EXTERN(32)
 IDG_GRID_SEP_EXTERN(64)
@@ -328,14 +328,14 @@ int configure_gridder_sep(int L, int* persistent_blocks) {
   IDG_SWITCH_L(C_)
 #undef C_
 }
-int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream) {
-#define C_(X) launch_gridder_sep_l<X>(a, n_items, persistent_blocks, bundle, stream)
+int launch_gridder_sep(int L, const GridArgs& a, int n_items, int blocks, void* stream) {
+#define C_(X) launch_gridder_sep_l<X>(a, n_items, blocks, stream)
   IDG_SWITCH_L(C_)
 #undef C_
 }
-int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int n_items, int max_nodes,
+int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
                              void* stream) {
-#define C_(X) launch_gridder_sep_multi_l<X>(args, items, n_items, max_nodes, stream)
+#define C_(X) launch_gridder_sep_multi_l<X>(args, blocks, n_blocks, max_nodes, stream)
   IDG_SWITCH_L(C_)
 #undef C_
 }

@@ -9,8 +9,8 @@
 // rows (p, i), 4 x 32 = 128, the height of one tcgen05 tile at every L;
 // columns j, real and imaginary sums as two accumulators of J columns.
 //
-// One block of 512 threads per bundle of items (subgrid, tile), split into
-// two halves that run side by side.  Producers: per chunk of 16 visibilities
+// A block of 512 threads works through a share of the items (subgrid, tile),
+// split into two halves that run side by side.  Producers: per chunk of 16 visibilities
 // every thread writes one row (p, i) x 8 visibilities of the E side to tensor
 // memory and, of the F side, one row j x 8 visibilities to shared memory, in
 // a ring of 2-4 chunks; one of them issues the chunk's 16 MMAs, whose commit
@@ -130,6 +130,12 @@ __device__ __forceinline__ void gsep_produce(uint32_t e_col, uint32_t buf, const
 }
 
 __device__ __forceinline__ int gsep_chunks(const SegmentDesc& d) { return (d.k_end - d.k_begin + kSepK - 1) / kSepK; }
+// A segment is summed in parts of up to kSepMaxChain chunks, each with its own accumulation and correction: chunks of
+// the next part when `left` remain
+__device__ __forceinline__ int gsep_part(int left) {
+  const int parts = (left + kSepMaxChain - 1) / kSepMaxChain;
+  return parts <= 1 ? left : (left + parts - 1) / parts;
+}
 
 // first column and row of an item's tile
 template <int L>
@@ -145,7 +151,7 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, int first, int 
   const int tid = threadIdx.x, lane = tid & 31;
   const bool issuer = uniform_warp() == kSepHalf / 32 - 1;  // the producer warp with the least to write
   const uint32_t ring0 = smem_u32(S.ring), tm = S.tmem;
-  uint32_t cg = 0, sc = 0;  // chunks and segments of this block so far
+  uint32_t cg = 0, sc = 0;  // chunks and segment parts of this block so far
   for (int idx = first; idx < last; idx += stride) {
     const GridItem item = a.items[idx];
     const SubgridDesc sd = a.sg[item.sg];
@@ -155,7 +161,8 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, int first, int 
     const float4* recs = a.records + size_t(sd.rec_offset) * kRecordFloat4;
     int total = 0;
     for (int s = 0; s < sd.seg_count; ++s) total += gsep_chunks(a.seg[sd.seg_begin + s]);
-    int s = 0, c_in = 0, n_in = gsep_chunks(a.seg[sd.seg_begin]);
+    int s = 0, left = gsep_chunks(a.seg[sd.seg_begin]);  // segment, its chunks not yet in a finished part
+    int c_in = 0, n_in = gsep_part(left);                 // chunk of the part, its length
     if (tid < kGsepChunkFloat4) S.rec[cg & 1][tid] = __ldg(recs + tid);
     half_sync(kSepProducerBar);
     for (int c = 0; c < total; ++c) {
@@ -187,9 +194,10 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, int first, int 
       ++c_in;
       if (last_c) {
         ++sc;
-        ++s;
+        left -= n_in;
         c_in = 0;
-        if (c + 1 < total) n_in = gsep_chunks(a.seg[sd.seg_begin + s]);
+        if (left == 0 && c + 1 < total) left = gsep_chunks(a.seg[sd.seg_begin + ++s]);
+        n_in = gsep_part(left);
       }
     }
   }
@@ -205,7 +213,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
   const bool poller = uniform_warp() == kSepHalf / 32;
   // rows of a thread within one node cell: every cell starts at a multiple of kSpan rows
   const bool one_cell = L % (nodes - 1) == 0 && L / (nodes - 1) % C::kSpan == 0;
-  uint32_t sc = 0;  // segments of this block so far
+  uint32_t sc = 0;  // segment parts of this block so far
   for (int idx = first; idx < last; idx += stride) {
     const GridItem item = a.items[idx];
     const SubgridDesc sd = a.sg[item.sg];
@@ -219,11 +227,12 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
 #pragma unroll
       for (int p = 0; p < 4; ++p) acc[r][p] = {0.f, 0.f};
 
-    // A-term samples of segment s of the item (the block's segment number c), on their way while another is worked on
+    // A-term samples of the item's next part (the block's part number c), on their way while another is worked on
     int diag_next = 0;
     float inv_next = 0.f;
-    SegmentDesc seg = a.seg[sd.seg_begin];  // of the segment fetched next
-    auto fetch = [&](int s, uint32_t c) {
+    int s = 0, left = 0;                    // segments fetched, chunks of the last one not yet in a part
+    SegmentDesc seg = a.seg[sd.seg_begin];  // of the part fetched next
+    auto fetch = [&](uint32_t c) {
       const int sp = seg.interval * a.g.n_st + sd.p, sq = seg.interval * a.g.n_st + sd.q;
       float4* dst = raw + (c & 1) * 2 * n4;
       const float4* pp = reinterpret_cast<const float4*>(a.aterms) + size_t(sp) * n4;
@@ -233,22 +242,26 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
         cp_async16(dst + n4 + e, qq + e);
       }
       cp_async_commit();
+      if (left == 0) left = gsep_chunks(seg);
+      const int n = gsep_part(left);
       diag_next = a.adiag[sp] & a.adiag[sq];
-      inv_next = __ldg(&rec[12].x);  // 1 / scale of the segment's values, undone on the p side
-      rec += size_t(gsep_chunks(seg)) * kGsepChunkFloat4;
-      if (s + 1 < sd.seg_count) seg = a.seg[sd.seg_begin + s + 1];
+      // 1 / scale of the segment's values (undone on the p side) and the accumulation's bias
+      inv_next = __ldg(&rec[12].x) * sep_unbias(n);
+      rec += size_t(n) * kGsepChunkFloat4;
+      left -= n;
+      if (left == 0 && ++s < sd.seg_count) seg = a.seg[sd.seg_begin + s];
     };
     half_sync(kSepConsumerBar);  // every thread is done with the previous item's samples
-    fetch(0, sc);
-    for (int s = 0; s < sd.seg_count; ++s, ++sc) {
+    fetch(sc);
+    for (bool more = true; more; ++sc) {
       const bool diag = diag_next != 0;
       const float inv = inv_next;
       if (poller) sep_wait<100>(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
       half_sync(kSepConsumerBar);  // the segment's sums complete; S.x and the other samples free
       tc_fence_after();
-      const bool more = s + 1 < sd.seg_count;
-      if (more) fetch(s + 1, sc + 1);
-      // sums of the segment: tensor memory -> S.x; warp = correlation, half of the rows
+      more = s < sd.seg_count;
+      if (more) fetch(sc + 1);
+      // sums of the part: tensor memory -> S.x; warp = correlation, half of the rows
       {
         const int pol = warp & 3, r0 = (warp >> 2) * (C::kRows / 2);
         const uint32_t d = S.tmem + (uint32_t(pol * 32) << 16) + (sc & 1) * C::kColStride + r0;
@@ -461,25 +474,24 @@ __device__ __forceinline__ void gridder_sep_block(const GridArgs& a, int first, 
   }
 }
 
+// Blocks take every gridDim-th item of the longest-first list (as in the degridder)
 template <int L>
-__global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_kernel(const GridArgs a, int bundle) {
+__global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_kernel(const GridArgs a) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
-  const int b = blockIdx.x;
-  if (bundle > 0)  // neighbouring items (tiles of one subgrid)
-    gridder_sep_block<L>(a, b * bundle, imin((b + 1) * bundle, a.n_items), 1, sep_smem);
-  else             // persistent: every gridDim-th item of the longest-first list
-    gridder_sep_block<L>(a, b, a.n_items, gridDim.x, sep_smem);
+  gridder_sep_block<L>(a, blockIdx.x, a.n_items, gridDim.x, sep_smem);
 }
 
-// One launch over the items of several plans (items = (plan slot, item index))
+// One launch over the items of several plans: blocks = (plan slot, first item), each taking every `stride`-th item of
+// its plan from there
 template <int L>
-__global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_multi_kernel(const GridArgs* args, const int2* items) {
+__global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_multi_kernel(const GridArgs* args, const int2* blocks) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
   __shared__ __align__(16) unsigned char s_args_raw[sizeof(GridArgs)];
-  const int2 it = items[blockIdx.x];
+  const int2 it = blocks[blockIdx.x];
   if (threadIdx.x == 0) memcpy(s_args_raw, args + it.x, sizeof(GridArgs));
   __syncthreads();
-  gridder_sep_block<L>(*reinterpret_cast<const GridArgs*>(s_args_raw), it.y, it.y + 1, 1, sep_smem);
+  const GridArgs& a = *reinterpret_cast<const GridArgs*>(s_args_raw);
+  gridder_sep_block<L>(a, it.y, a.n_items, a.stride, sep_smem);
 }
 
 template <int L>
@@ -499,21 +511,18 @@ int configure_gridder_sep_l(int* persistent_blocks) {
 }
 
 template <int L>
-int launch_gridder_sep_l(const GridArgs& args, int n_items, int persistent_blocks, int bundle, void* stream) {
+int launch_gridder_sep_l(const GridArgs& args, int n_items, int blocks, void* stream) {
   if (n_items <= 0) return 0;
   GridArgs a = args;
   a.n_items = n_items;
-  const int blocks = persistent_blocks > 0 ? (persistent_blocks < n_items ? persistent_blocks : n_items)
-                                           : (n_items + bundle - 1) / bundle;
-  gridder_sep_kernel<L><<<blocks, kSepThreads, gsep_smem<L>(a.g.nodes), cudaStream_t(stream)>>>(
-      a, persistent_blocks > 0 ? 0 : bundle);
+  gridder_sep_kernel<L><<<blocks, kSepThreads, gsep_smem<L>(a.g.nodes), cudaStream_t(stream)>>>(a);
   return int(cudaGetLastError());
 }
 
 template <int L>
-int launch_gridder_sep_multi_l(const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream) {
-  if (n_items <= 0) return 0;
-  gridder_sep_multi_kernel<L><<<n_items, kSepThreads, gsep_smem<L>(max_nodes), cudaStream_t(stream)>>>(args, items);
+int launch_gridder_sep_multi_l(const GridArgs* args, const int2* blocks, int n_blocks, int max_nodes, void* stream) {
+  if (n_blocks <= 0) return 0;
+  gridder_sep_multi_kernel<L><<<n_blocks, kSepThreads, gsep_smem<L>(max_nodes), cudaStream_t(stream)>>>(args, blocks);
   return int(cudaGetLastError());
 }
 

@@ -4,7 +4,7 @@
 namespace idg {
 
 template int configure_gridder_sep_l<32>(int*);
-template int launch_gridder_sep_l<32>(const GridArgs&, int, int, int, void*);
+template int launch_gridder_sep_l<32>(const GridArgs&, int, int, void*);
 template int launch_gridder_sep_multi_l<32>(const GridArgs*, const int2*, int, int, void*);
 
 }  // namespace idg

@@ -4,7 +4,7 @@
 namespace idg {
 
 template int configure_gridder_sep_l<96>(int*);
-template int launch_gridder_sep_l<96>(const GridArgs&, int, int, int, void*);
+template int launch_gridder_sep_l<96>(const GridArgs&, int, int, void*);
 template int launch_gridder_sep_multi_l<96>(const GridArgs*, const int2*, int, int, void*);
 
 }  // namespace idg

@@ -510,10 +510,12 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     sep_ok = x * sep.e1 + x * x * sep.e2 <= kSepTolerance;  // false for a NaN
   }
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
-  // cannot run); both on FP32 when channel groups were asked for, and for Stokes I (the FP32 kernels' sums
-  // over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four correlations)
+  // cannot run); both on FP32 when channel groups were asked for, and for Stokes I without the separable form
+  // (the FP32 kernels' sums over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four
+  // correlations: an 80-station predict-and-grid cycle takes 10.7 ms on them, and @@ ms on the separable kernels,
+  // which sum all four)
   p->mac = g->mac_unit != IDG_MAC_DEFAULT ? g->mac_unit
-           : (g->degrid_channels > 1 || (g->flags & IDG_STOKES_I)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
+           : (g->degrid_channels > 1 || ((g->flags & IDG_STOKES_I) && !sep_ok)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
   if (p->mac != IDG_MAC_FP32) p->degrid_channels = 1;  // one visibility per row of the tensor-core product
   {
     // the tensor-core gridder rotates phasors by one channel step along each row
@@ -794,10 +796,12 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
   return ga;
 }
 
-// items per block of the separable-phasor kernels: some blocks per SM must remain to even out the load, and
-// more items per block than that spread the block's set-up
-static int sep_bundle(const idg_plan* p, int n_items) {
-  return std::max(1, std::min(24, n_items / (8 * std::max(1, int(p->sms)))));
+// Blocks of the separable-phasor kernels for n items: one per SM (all that fit), so that a block's set-up and the
+// latency of its first item are paid once and its roles run ahead from item to item; more only where a block would
+// hold more than 512 items, so that a launch leaves SMs to other streams within a few milliseconds.
+static int sep_blocks(const idg_plan* p, int n) {
+  const int sms = std::max(1, int(p->sms));
+  return std::min(std::max(n, 1), sms * std::max(1, n / (512 * sms)));
 }
 
 // record staging and the gridder of the plan's kind (FP32 pipe or tensor cores)
@@ -809,7 +813,7 @@ static int stage_any(const idg_plan* p, const Batch& b, const void* vis, cudaStr
 }
 
 static int gridder_any(const idg_plan* p, const GridArgs& ga, int n_items, int persistent_blocks, cudaStream_t strm) {
-  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, persistent_blocks, sep_bundle(p, n_items), strm);
+  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, sep_blocks(p, n_items), strm);
   return p->grid_tc ? launch_gridder_tc(p->L, ga, n_items, persistent_blocks, strm)
                     : launch_gridder(p->L, ga, n_items, persistent_blocks, strm);
 }
@@ -923,8 +927,7 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
     da.queue = plan->d_queue + 2 * bi + 1;
     e = timed(plan, kDegridder, [&] {
       if (plan->degrid_sep)
-        return launch_degridder_sep(L, da, b.di_count, plan->persistent_degrid_blocks,
-                                    sep_bundle(plan, b.di_count), plan->stream);
+        return launch_degridder_sep(L, da, b.di_count, sep_blocks(plan, b.di_count), plan->stream);
       if (plan->mac != IDG_MAC_FP32)
         return launch_degridder_tc(L, da, b.di_count, plan->persistent_degrid_blocks, plan->stream);
       return launch_degridder(L, plan->degrid_channels, da, b.di_count, plan->persistent_degrid_blocks,
@@ -1078,6 +1081,29 @@ std::vector<int2> merge_items(const std::vector<const int32_t*>& cost, const std
   return out;
 }
 
+// Blocks of one separable-phasor launch over several plans: sep_blocks of all items together, shared out by the slots'
+// item counts; block (slot, first item) takes every strides[slot]-th item of its slot
+std::vector<int2> share_blocks(const idg_plan* p, const std::vector<int32_t>& count, std::vector<int32_t>* strides) {
+  int64_t total = 0;
+  for (int32_t c : count) total += c;
+  std::vector<int2> out;
+  strides->assign(count.size(), 1);
+  if (total == 0) return out;
+  // items per block: the least that needs no more blocks than that (a few more would be a wave of their own)
+  const int64_t most = sep_blocks(p, int(total));
+  for (int64_t each = (total + most - 1) / most;; each += std::max<int64_t>(1, each / 32)) {
+    int64_t n = 0;
+    for (size_t s = 0; s < count.size(); ++s) {
+      (*strides)[s] = std::max<int32_t>(1, int32_t((count[s] + each - 1) / each));
+      n += std::min((*strides)[s], count[s]);
+    }
+    if (n <= most || each >= total) break;
+  }
+  for (size_t s = 0; s < count.size(); ++s)
+    for (int32_t k = 0; k < std::min((*strides)[s], count[s]); ++k) out.push_back(make_int2(int(s), k));
+  return out;
+}
+
 // device copies of the wave's argument table and item list (stream-ordered, freed after the launch)
 template <typename A>
 int upload_wave(cudaStream_t st, const std::vector<A>& args, const std::vector<int2>& items, A** d_args,
@@ -1131,7 +1157,9 @@ idg_status idg_grid_many(int32_t n, idg_plan* const* plans, const void* const* v
     // plans with and without the separable form take a launch each, their items in one list
     std::vector<int32_t> count_sep = count;
     for (size_t s = 0; s < count.size(); ++s) (plans[slot_plan[s]]->grid_sep ? count : count_sep)[s] = 0;
-    std::vector<int2> items = merge_items(cost, count_sep);
+    std::vector<int32_t> strides;
+    std::vector<int2> items = share_blocks(plans[0], count_sep, &strides);
+    for (size_t s = 0; s < args.size(); ++s) args[s].stride = strides[s];
     const size_t n_sep = items.size();
     for (int2 it : merge_items(cost, count)) items.push_back(it);
     GridArgs* d_args = nullptr;
@@ -1204,7 +1232,9 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
     // the latter index their plan's item table past the regular ones
     std::vector<int32_t> count_sep = count, count_r = count;
     for (size_t s = 0; s < count.size(); ++s) (slot_sep[s] ? count_r : count_sep)[s] = 0;
-    std::vector<int2> items = merge_items(cost, count_sep);
+    std::vector<int32_t> strides;
+    std::vector<int2> items = share_blocks(plans[0], count_sep, &strides);
+    for (size_t s = 0; s < args.size(); ++s) args[s].stride = strides[s];
     const size_t n_sep = items.size();
     for (int2 it : merge_items(cost, count_r)) items.push_back(it);
     const size_t n_regular = items.size() - n_sep;

@@ -241,6 +241,7 @@ struct GridArgs {
   int vc = kDefaultGridChunk;  // staged records per chunk: 32, 48 or 64
   const float* w_ref = nullptr;  // [batch subgrids] reference w (separable-phasor gridder)
   SepTables sep;
+  int stride = 1;             // items between a block's items (one launch over several plans)
   KernelGeom g;
 };
 
@@ -264,6 +265,7 @@ struct DegridArgs {
   const float* ymax = nullptr;    // [batch subgrids][4] largest component of the subgrid's planes
   const float* w_ref = nullptr;   // [batch subgrids] reference w
   int kv = 0;                     // visibilities per item
+  int stride = 1;                 // items between a block's items (one launch over several plans)
   SepTables sep;
   KernelGeom g;
 };
@@ -326,17 +328,17 @@ int configure_gridder_tc(int L, int* persistent_blocks);
 int launch_gridder_tc_multi(int L, const GridArgs* args, const int2* items, int n_items, void* stream);
 // the separable-phasor gridder (records staged by launch_stage_sep; any channel spacing)
 int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids, void* stream);
-int launch_gridder_sep(int L, const GridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
+int launch_gridder_sep(int L, const GridArgs& a, int n_items, int blocks, void* stream);
 int configure_gridder_sep(int L, int* persistent_blocks);
-int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
+int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* blocks, int n_blocks, int max_nodes, void* stream);
 int configure_degridder_tc(int L, int nodes, int* persistent_blocks);
 int launch_degridder_tc_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
                               void* stream);
-// the separable-phasor degridder: items of up to degridder_sep_vis visibilities of one segment, `bundle` of them per block
+// the separable-phasor degridder: items of up to degridder_sep_vis visibilities of one segment
 int degridder_sep_vis(int L, int nodes);
 int configure_degridder_sep(int L, int* persistent_blocks);
-int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int persistent_blocks, int bundle, void* stream);
-int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
+int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int blocks, void* stream);
+int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
                                void* stream);
 // mode 0: FFT + add into grid; mode 1: FFT in place in scratch (inspection)
 int launch_fft_adder(int L, const FftArgs& a, int n_subgrids, int mode, void* stream);

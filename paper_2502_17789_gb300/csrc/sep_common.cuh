@@ -53,6 +53,13 @@ __device__ __forceinline__ void sep_mma(uint32_t d, uint32_t a, uint64_t b, uint
       "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// The tensor core adds each MMA to the FP32 accumulator with truncation: measured against 64 bits, sums shrink by
+// 1.7e-8 per MMA (1.4 .. 2.1e-8 over chains of 16 to 120 MMAs and all subgrid sizes).  Results are scaled back by the
+// mean, and chains are kept short (kSepMaxChain chunks of 8 MMAs in the gridder, L / 16 in the degridder): the grid's
+// error against 64 bits at L = 96 falls from 9.7e-7 to 5e-7, and does not grow with the length of a segment.
+constexpr int kSepMaxChain = 8;
+__device__ __forceinline__ float sep_unbias(int chunks) { return fmaf(1.7e-8f * 8.f, float(chunks), 1.f); }
+
 // arrive on `bar` when every MMA issued so far by this thread has completed
 __device__ __forceinline__ void sep_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
