@@ -91,7 +91,7 @@ struct Dsep {
   DsepShared& S;
   unsigned char* fside;   // [item parity][level][16 rows][k group][Re, Im][visibility] rows of 16 bytes
   float4* raw;            // [item parity][station][nodes][nodes][2]
-  const int first, last, stride;
+  const SepShare share;
 
   static constexpr int kBlocks = L / 32, kPieces = L / 16;
 
@@ -210,7 +210,7 @@ struct Dsep {
     const bool quad = L % (nodes - 1) == 0 && L / (nodes - 1) % 4 == 0;
     const uint32_t tm = S.tmem;
     uint32_t n = 0, pg = grp;  // items and (both groups') pieces of this block so far
-    for (int idx = first; idx < last; idx += stride, ++n) {
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       wait(&S.ready[n & 1], (n >> 1) & 1);
       const float scale = S.info[n & 1].scale;
       const bool diag = S.info[n & 1].diag != 0;
@@ -254,7 +254,7 @@ struct Dsep {
   // Y in scratch: [pol][column block][row pair][re, im][32 columns], so a piece is one run of 4 KB per plane
   __device__ __forceinline__ void loader() {
     uint32_t n = 0, pg = 0;  // items and pieces of this block so far
-    for (int idx = first; idx < last; idx += stride, ++n) {
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       wait<64>(&S.ready[n & 1], (n >> 1) & 1);
       const float2* Y = a.scratch + size_t(S.info[n & 1].sg) * 4 * L * L;
 #pragma unroll 1
@@ -277,7 +277,7 @@ struct Dsep {
   __device__ __forceinline__ void issuer() {
     const uint32_t tm = S.tmem;
     uint32_t n = 0, pg = 0, dg = 0;  // items, pieces and accumulators of this block so far
-    for (int idx = first; idx < last; idx += stride, ++n) {
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       wait(&S.ready[n & 1], (n >> 1) & 1);
       const int n_pad = S.info[n & 1].n_pad;
       const uint32_t block = uint32_t(n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
@@ -384,7 +384,7 @@ struct Dsep {
 
   __device__ __forceinline__ void preparer() {
     uint32_t n = 0;
-    for (int idx = first; idx < last; idx += stride, ++n) prepare(idx, n);
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) prepare(idx, n);
   }
 
   // ---------------------------------------------------------------- consumers
@@ -393,7 +393,7 @@ struct Dsep {
   __device__ __forceinline__ void consumer() {
     const int tid = threadIdx.x - kDsepConsumer, pol = tid >> 5, lane = tid & 31;
     uint32_t dg = 0, n = 0;  // accumulators and items of this block so far
-    for (int idx = first; idx < last; idx += stride, ++n) {
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       const DegridItem item = a.items[idx];
       const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
       wait(&S.ready[b], (n >> 1) & 1);
@@ -468,10 +468,8 @@ struct Dsep {
   }
 };
 
-// items first, first + stride, ... below last
 template <int L>
-__device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int first, int last, int stride,
-                                                    unsigned char* smem) {
+__device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShare share, unsigned char* smem) {
   DsepShared& S = *reinterpret_cast<DsepShared*>(smem);
   unsigned char* fside = reinterpret_cast<unsigned char*>(&S + 1);
   if (threadIdx.x == 0) {
@@ -493,7 +491,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  Dsep<L> it{a, S, fside, reinterpret_cast<float4*>(fside + size_t(2) * a.kv * L * 12), first, last, stride};
+  Dsep<L> it{a, S, fside, reinterpret_cast<float4*>(fside + size_t(2) * a.kv * L * 12), share};
   if (threadIdx.x < kDsepConsumer) {
     regs_give<kDsepProducerRegs>();
     it.producer();
@@ -524,16 +522,14 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, int fir
   }
 }
 
-// Blocks take every gridDim-th item of the longest-first list: an even share of long and short items each, the
-// neighbouring items of a subgrid at the same time on neighbouring SMs, and one set-up per block
 template <int L>
 __global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_kernel(const DegridArgs a) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
-  degridder_sep_block<L>(a, blockIdx.x, a.n_items, gridDim.x, sep_smem);
+  degridder_sep_block<L>(a, SepShare{int(blockIdx.x) * a.run, a.n_items, int(gridDim.x), a.run}, sep_smem);
 }
 
-// One launch over the items of several plans: blocks = (plan slot, first item), each taking every `stride`-th item of
-// its plan from there
+// One launch over the items of several plans: blocks = (plan slot, first run), each taking every `stride`-th run of its
+// plan from there
 template <int L>
 __global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_multi_kernel(const DegridArgs* args,
                                                                             const int2* blocks) {
@@ -543,7 +539,7 @@ __global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_multi_kernel(co
   if (threadIdx.x == 0) memcpy(s_args_raw, args + it.x, sizeof(DegridArgs));
   __syncthreads();
   const DegridArgs& a = *reinterpret_cast<const DegridArgs*>(s_args_raw);
-  degridder_sep_block<L>(a, it.y, a.n_items, a.stride, sep_smem);
+  degridder_sep_block<L>(a, SepShare{it.y * a.run, a.n_items, a.stride, a.run}, sep_smem);
 }
 
 template <int L>

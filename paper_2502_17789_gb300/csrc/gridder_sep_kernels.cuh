@@ -144,15 +144,15 @@ __device__ __forceinline__ int2 gsep_origin(const GridItem& item) {
   return make_int2(item.tile / n * kGsepColumns, item.tile % n * Gsep<L>::kRows);
 }
 
-// items first, first + stride, ... below last, producers' side
+// producers' side
 template <int L>
-__device__ __forceinline__ void gsep_producer(const GridArgs& a, int first, int last, int stride, GsepShared<L>& S) {
+__device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share, GsepShared<L>& S) {
   using C = Gsep<L>;
   const int tid = threadIdx.x, lane = tid & 31;
   const bool issuer = uniform_warp() == kSepHalf / 32 - 1;  // the producer warp with the least to write
   const uint32_t ring0 = smem_u32(S.ring), tm = S.tmem;
   uint32_t cg = 0, sc = 0;  // chunks and segment parts of this block so far
-  for (int idx = first; idx < last; idx += stride) {
+  for (int idx = share.first; idx < share.last; idx = share.next(idx)) {
     const GridItem item = a.items[idx];
     const SubgridDesc sd = a.sg[item.sg];
     const int2 org = gsep_origin<L>(item);
@@ -205,8 +205,7 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, int first, int 
 
 // consumers' side: thread = column i of the tile x kSpan neighbouring rows
 template <int L>
-__device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int last, int stride, GsepShared<L>& S,
-                                              float4* raw) {
+__device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share, GsepShared<L>& S, float4* raw) {
   using C = Gsep<L>;
   const int warp = (threadIdx.x >> 5) - kSepHalf / 32, lane = threadIdx.x & 31;
   const int nodes = a.g.nodes, n4 = nodes * nodes * 2;  // float4s of one station's samples
@@ -214,7 +213,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
   // rows of a thread within one node cell: every cell starts at a multiple of kSpan rows
   const bool one_cell = L % (nodes - 1) == 0 && L / (nodes - 1) % C::kSpan == 0;
   uint32_t sc = 0;  // segment parts of this block so far
-  for (int idx = first; idx < last; idx += stride) {
+  for (int idx = share.first; idx < share.last; idx = share.next(idx)) {
     const GridItem item = a.items[idx];
     const SubgridDesc sd = a.sg[item.sg];
     const int2 org = gsep_origin<L>(item);
@@ -436,8 +435,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, int first, int 
 }
 
 template <int L>
-__device__ __forceinline__ void gridder_sep_block(const GridArgs& a, int first, int last, int stride,
-                                                  unsigned char* smem) {
+__device__ __forceinline__ void gridder_sep_block(const GridArgs& a, SepShare share, unsigned char* smem) {
   using C = Gsep<L>;
   GsepShared<L>& S = *reinterpret_cast<GsepShared<L>*>(smem);
   if (threadIdx.x == 0) {
@@ -455,10 +453,10 @@ __device__ __forceinline__ void gridder_sep_block(const GridArgs& a, int first, 
   tc_fence_after();
   if (threadIdx.x < kSepHalf) {
     regs_give<256 - C::kConsumerRegs>();
-    gsep_producer<L>(a, first, last, stride, S);
+    gsep_producer<L>(a, share, S);
   } else {
     regs_take<C::kConsumerRegs>();
-    gsep_consumer<L>(a, first, last, stride, S, reinterpret_cast<float4*>(&S + 1));
+    gsep_consumer<L>(a, share, S, reinterpret_cast<float4*>(&S + 1));
   }
   // after a wait that gave up: one more bounded wait for MMAs that may still run before their memory goes
   tc_fence_before();
@@ -474,15 +472,14 @@ __device__ __forceinline__ void gridder_sep_block(const GridArgs& a, int first, 
   }
 }
 
-// Blocks take every gridDim-th item of the longest-first list (as in the degridder)
 template <int L>
 __global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_kernel(const GridArgs a) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
-  gridder_sep_block<L>(a, blockIdx.x, a.n_items, gridDim.x, sep_smem);
+  gridder_sep_block<L>(a, SepShare{int(blockIdx.x) * a.run, a.n_items, int(gridDim.x), a.run}, sep_smem);
 }
 
-// One launch over the items of several plans: blocks = (plan slot, first item), each taking every `stride`-th item of
-// its plan from there
+// One launch over the items of several plans: blocks = (plan slot, first run), each taking every `stride`-th run of its
+// plan from there
 template <int L>
 __global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_multi_kernel(const GridArgs* args, const int2* blocks) {
   extern __shared__ __align__(128) unsigned char sep_smem[];
@@ -491,7 +488,7 @@ __global__ void __launch_bounds__(kSepThreads, 1) gridder_sep_multi_kernel(const
   if (threadIdx.x == 0) memcpy(s_args_raw, args + it.x, sizeof(GridArgs));
   __syncthreads();
   const GridArgs& a = *reinterpret_cast<const GridArgs*>(s_args_raw);
-  gridder_sep_block<L>(a, it.y, a.n_items, a.stride, sep_smem);
+  gridder_sep_block<L>(a, SepShare{it.y * a.run, a.n_items, a.stride, a.run}, sep_smem);
 }
 
 template <int L>

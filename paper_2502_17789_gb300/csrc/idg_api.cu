@@ -512,7 +512,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
   // cannot run); both on FP32 when channel groups were asked for, and for Stokes I without the separable form
   // (the FP32 kernels' sums over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four
-  // correlations: an 80-station predict-and-grid cycle takes 10.7 ms on them, and @@ ms on the separable kernels,
+  // correlations: an 80-station predict-and-grid cycle takes 10.7 ms on them, and 4.1 ms on the separable kernels,
   // which sum all four)
   p->mac = g->mac_unit != IDG_MAC_DEFAULT ? g->mac_unit
            : (g->degrid_channels > 1 || ((g->flags & IDG_STOKES_I) && !sep_ok)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
@@ -796,12 +796,15 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
   return ga;
 }
 
-// Blocks of the separable-phasor kernels for n items: one per SM (all that fit), so that a block's set-up and the
-// latency of its first item are paid once and its roles run ahead from item to item; more only where a block would
-// hold more than 512 items, so that a launch leaves SMs to other streams within a few milliseconds.
-static int sep_blocks(const idg_plan* p, int n) {
+// Items per run (SepShare) of the degridder and blocks of the separable-phasor kernels for n items.  Runs where every
+// block still gets eight of them (the gridder reads nothing but its own records: single items, 16.7 ms on the
+// MWA-like workload against 17.4 in runs of 12); one block per SM (all that fit), so that a block's set-up and the latency of its first item are
+// paid once and its roles run ahead from item to item; more only where a block would hold more than 512 items, so
+// that a launch leaves SMs to other streams within a few milliseconds.
+static int sep_run(const idg_plan* p, int n) { return std::max(1, std::min(12, n / (8 * std::max(1, int(p->sms))))); }
+static int sep_blocks(const idg_plan* p, int n, int run) {
   const int sms = std::max(1, int(p->sms));
-  return std::min(std::max(n, 1), sms * std::max(1, n / (512 * sms)));
+  return std::min(std::max(1, (n + run - 1) / run), sms * std::max(1, n / (512 * sms)));
 }
 
 // record staging and the gridder of the plan's kind (FP32 pipe or tensor cores)
@@ -813,7 +816,7 @@ static int stage_any(const idg_plan* p, const Batch& b, const void* vis, cudaStr
 }
 
 static int gridder_any(const idg_plan* p, const GridArgs& ga, int n_items, int persistent_blocks, cudaStream_t strm) {
-  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, sep_blocks(p, n_items), strm);
+  if (p->grid_sep) return launch_gridder_sep(p->L, ga, n_items, sep_blocks(p, n_items, 1), strm);
   return p->grid_tc ? launch_gridder_tc(p->L, ga, n_items, persistent_blocks, strm)
                     : launch_gridder(p->L, ga, n_items, persistent_blocks, strm);
 }
@@ -925,9 +928,10 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
     if (e) return cuda_err(plan, e, "splitter/ifft launch");
     DegridArgs da = degrid_args(plan, b, aterms_c64, vis_c64);
     da.queue = plan->d_queue + 2 * bi + 1;
+    da.run = sep_run(plan, b.di_count);
     e = timed(plan, kDegridder, [&] {
       if (plan->degrid_sep)
-        return launch_degridder_sep(L, da, b.di_count, sep_blocks(plan, b.di_count), plan->stream);
+        return launch_degridder_sep(L, da, b.di_count, sep_blocks(plan, b.di_count, da.run), plan->stream);
       if (plan->mac != IDG_MAC_FP32)
         return launch_degridder_tc(L, da, b.di_count, plan->persistent_degrid_blocks, plan->stream);
       return launch_degridder(L, plan->degrid_channels, da, b.di_count, plan->persistent_degrid_blocks,
@@ -1090,7 +1094,7 @@ std::vector<int2> share_blocks(const idg_plan* p, const std::vector<int32_t>& co
   strides->assign(count.size(), 1);
   if (total == 0) return out;
   // items per block: the least that needs no more blocks than that (a few more would be a wave of their own)
-  const int64_t most = sep_blocks(p, int(total));
+  const int64_t most = sep_blocks(p, int(total), 1);
   for (int64_t each = (total + most - 1) / most;; each += std::max<int64_t>(1, each / 32)) {
     int64_t n = 0;
     for (size_t s = 0; s < count.size(); ++s) {

@@ -241,7 +241,7 @@ struct GridArgs {
   int vc = kDefaultGridChunk;  // staged records per chunk: 32, 48 or 64
   const float* w_ref = nullptr;  // [batch subgrids] reference w (separable-phasor gridder)
   SepTables sep;
-  int stride = 1;             // items between a block's items (one launch over several plans)
+  int run = 1, stride = 1;    // a block's items (SepShare); stride: one launch over several plans
   KernelGeom g;
 };
 
@@ -265,7 +265,7 @@ struct DegridArgs {
   const float* ymax = nullptr;    // [batch subgrids][4] largest component of the subgrid's planes
   const float* w_ref = nullptr;   // [batch subgrids] reference w
   int kv = 0;                     // visibilities per item
-  int stride = 1;                 // items between a block's items (one launch over several plans)
+  int run = 1, stride = 1;        // a block's items (SepShare); stride: one launch over several plans
   SepTables sep;
   KernelGeom g;
 };

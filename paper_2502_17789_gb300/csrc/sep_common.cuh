@@ -171,6 +171,15 @@ __device__ __forceinline__ bool elect_one() {
 // warp is a branch for the others and not predicated through
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0); }
 
+// The items of a block: runs of `run` neighbouring items of the longest-first list, every `stride`-th run.  A run
+// re-reads the subgrid it belongs to from L2 at its own time (with single items as many SMs as a subgrid has items
+// read the same lines at once: 5.5 instead of 4.9 ms in the degridder of the uneven array), and the stride gives every
+// block an even share of long and short items.
+struct SepShare {
+  int first, last, stride, run;
+  __device__ __forceinline__ int next(int idx) const { return (idx + 1) % run ? idx + 1 : idx + 1 + (stride - 1) * run; }
+};
+
 // ---------------------------------------------------------------- operands
 
 // phase (radians, about [-pi, pi]) of slope `fix` (turns per pixel in units
