@@ -1318,34 +1318,20 @@ idg_status idg_invert(idg_plan* plan, const void* vis_c64, const void* aterms_c6
   };
   double2* img = static_cast<double2*>(image_c128);
   double2* grid = static_cast<double2*>(grid_c128);
-  auto inverse = [&](double2* x) {
-    return cufftExecZ2Z(plan->fft, reinterpret_cast<cufftDoubleComplex*>(x), reinterpret_cast<cufftDoubleComplex*>(x),
-                        CUFFT_INVERSE);
-  };
   const bool single = (plan->geom.flags & IDG_W_LAYERS) == 0;
-  if (single) {
-    // one layer at w0 = 0: transform a signed copy, the gridded plane stays in `grid`
-    e = launch_image_pass(plan->npol, grid, img, nullptr, 1.0, 0.0, fov, N, kPassSign, plan->stream);
-    if (e) return cuda_err(plan, e, "centring signs");
-    const cufftResult r = inverse(img);
-    if (r != CUFFT_SUCCESS) return fft_err(plan, r, "cufftExecZ2Z");
-    e = launch_image_pass(plan->npol, img, img, plan->d_inv_t, inv_l2, 0.0, fov, N, kPassSign, plan->stream);
-    if (e) return cuda_err(plan, e, "taper correction");
-    return weight_correction();
-  }
-  // w-stacking (Eq. 11): transform every layer in place, shift it from w0 to w = 0, sum
+  // w-stacking (Eq. 11): transform every layer, shift it from w0 to w = 0 and correct the taper in
+  // one pass, sum.  A single layer is at w0 = 0 and stays in `grid`: its transform goes to `image`.
   for (int li = 0; li < plan->n_layers; ++li) {
     double2* gl = grid + plane_set * li;
-    const double w0 = (double(plan->k_min + li) + 0.5) * plan->part.w_step;
-    e = launch_image_pass(plan->npol, gl, gl, nullptr, 1.0, 0.0, fov, N, kPassSign, plan->stream);
-    if (e) return cuda_err(plan, e, "centring signs");
-    const cufftResult r = inverse(gl);
+    double2* out = single ? img : gl;
+    const double w0 = single ? 0.0 : (double(plan->k_min + li) + 0.5) * plan->part.w_step;
+    const cufftResult r = cufftExecZ2Z(plan->fft, reinterpret_cast<cufftDoubleComplex*>(gl),
+                                       reinterpret_cast<cufftDoubleComplex*>(out), CUFFT_INVERSE);
     if (r != CUFFT_SUCCESS) return fft_err(plan, r, "cufftExecZ2Z");
-    e = launch_image_pass(plan->npol, gl, img, nullptr, 1.0, w0, fov, N, kPassSign | (li ? kPassAccumulate : 0), plan->stream);
-    if (e) return cuda_err(plan, e, "w-stacking");
+    e = launch_image_pass(plan->npol, out, img, plan->d_inv_t, inv_l2, w0, fov, N,
+                          kPassToImage | (li ? kPassAccumulate : 0), plan->stream);
+    if (e) return cuda_err(plan, e, "w-stacking and taper correction");
   }
-  e = launch_image_pass(plan->npol, img, img, plan->d_inv_t, inv_l2, 0.0, fov, N, 0, plan->stream);
-  if (e) return cuda_err(plan, e, "taper correction");
   return weight_correction();
 }
 
@@ -1366,13 +1352,11 @@ idg_status idg_predict(idg_plan* plan, const void* image_c128, const void* aterm
   for (int li = 0; li < plan->n_layers; ++li) {
     double2* gl = grid + plane_set * li;
     const double w0 = (double(plan->k_min + li) + 0.5) * plan->part.w_step;
-    int e = launch_image_pass(plan->npol, img, gl, plan->d_inv_t, inv_l2, -w0, fov, N, kPassSign, plan->stream);
+    const int e = launch_image_pass(plan->npol, img, gl, plan->d_inv_t, inv_l2, -w0, fov, N, 0, plan->stream);
     if (e) return cuda_err(plan, e, "taper correction");
     const cufftResult r = cufftExecZ2Z(plan->fft, reinterpret_cast<cufftDoubleComplex*>(gl),
                                        reinterpret_cast<cufftDoubleComplex*>(gl), CUFFT_FORWARD);
     if (r != CUFFT_SUCCESS) return fft_err(plan, r, "cufftExecZ2Z");
-    e = launch_image_pass(plan->npol, gl, gl, nullptr, 1.0, 0.0, fov, N, kPassSign, plan->stream);
-    if (e) return cuda_err(plan, e, "centring signs");
   }
   return idg_degrid(plan, grid_c128, aterms_c64, vis_c64);
 }

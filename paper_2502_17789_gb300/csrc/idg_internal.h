@@ -298,10 +298,11 @@ int configure_gridder(int L, int vc, int* persistent_blocks);   // attributes + 
 int configure_degridder(int L, int nodes, int channels, int* persistent_blocks);
 bool supported_degrid_channels(int channels);
 int launch_stage_records(int L, const StageArgs& a, int n_subgrids, void* stream);
-// element-wise pass over the 4 N x N complex128 planes of one w layer (image-domain wrapper):
-// out (+)= in * c * w[x] w[y] * (-1)^(x+y) * e^{i 2 pi w0 n'(x,y)}; w may be null
-constexpr int kPassSign = 1;        // apply (-1)^(x+y)
-constexpr int kPassAccumulate = 2;  // add into out
+// element-wise pass over the npol N x N complex128 planes of one w layer (image-domain wrapper),
+// f(x, y) = c * w[x] w[y] * (-1)^(x+y) * e^{i 2 pi w0 n'(x, y)}:
+// out(x + N/2, y + N/2) = in(x, y) f(x, y) ahead of a transform to the grid; N even, in == out allowed
+constexpr int kPassToImage = 1;     // after a transform from it: out(x, y) = in(x + N/2, y + N/2) f(x, y)
+constexpr int kPassAccumulate = 2;  // with kPassToImage: add into out
 // image /= W(p, q) with W the A-term weight map [L*L + 1] (sum n_seg / f,
 // then sum n_seg) averaged and interpolated bilinearly from the subgrid lattice
 int launch_weight_correction(int npol, double2* image, const double* aweights, int N, int L, void* stream);
