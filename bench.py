@@ -63,7 +63,8 @@ MAC_NAMES = {1: "FP32 pipe (gridder and degridder)", 2: "tensor cores (gridder a
 
 
 def ncu_traffic_command(kern: str) -> str:
-    mac = {"gridder": " --mac-unit 3", "gridder_tc": " --mac-unit 2", "degridder": " --mac-unit 1"}.get(kern, "")
+    mac = {"gridder": " --mac-unit 3", "gridder_tc": " --mac-unit 2", "gridder_sep": " --mac-unit 2",
+           "degridder": " --mac-unit 1"}.get(kern, "")
     return (f'ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none '
             f'--kernel-name-base demangled -k regex:"idg::{kern}_kernel<" -c 2 --csv '
             f'--log-file traffic_{kern}.csv {BENCH_SHORT} --stations {TRAFFIC_STATIONS}{mac}')
@@ -71,15 +72,31 @@ KERNEL_SOURCES = {"gridder": ["gridder.cu", "gridder_kernels.cuh", "kernels_comm
                   "degridder": ["degridder.cu", "degridder_kernels.cuh", "kernels_common.cuh", "idg_internal.h"],
                   "degridder_tc": ["degridder.cu", "degridder_tc_kernels.cuh", "degridder_kernels.cuh",
                                    "kernels_common.cuh", "idg_internal.h"],
-                  "gridder_tc": ["gridder.cu", "gridder_tc_kernels.cuh", "kernels_common.cuh", "idg_internal.h"]}
+                  "gridder_tc": ["gridder.cu", "gridder_tc_kernels.cuh", "kernels_common.cuh", "idg_internal.h"],
+                  "gridder_sep": ["gridder.cu", "gridder_sep_kernels.cuh", "sep_common.cuh", "kernels_common.cuh",
+                                  "idg_internal.h"],
+                  "degridder_sep": ["degridder.cu", "degridder_sep_kernels.cuh", "sep_common.cuh",
+                                    "kernels_common.cuh", "idg_internal.h"]}
+# tensor-core operations of the separable kernels: 16 real multiply-adds per visibility-pixel (4-pol complex
+# product) in three f16 products (hi hi + hi lo + lo hi)
+SEP_FLOP_PER_VISPX = 96.0
 
 
-def kernel_of(kind: str, mac_unit: int) -> str:
+def kernel_of(kind: str, mac_unit: int, separable: bool = False) -> str:
     """The kernel (ncu name prefix, traffic key) a plan with `mac_unit` in use
-    runs for the timing class `kind` (gridder or degridder)."""
+    runs for the timing class `kind` (gridder or degridder); `separable`: the
+    plan's w terms are small enough for the separable-phasor kernels."""
     if kind == "gridder":
-        return "gridder_tc" if mac_unit == 2 else "gridder"
-    return "degridder" if mac_unit == 1 else "degridder_tc"
+        return "gridder" if mac_unit != 2 else "gridder_sep" if separable else "gridder_tc"
+    return "degridder" if mac_unit == 1 else "degridder_sep" if separable else "degridder_tc"
+
+
+def separable_plan(stats, L: int) -> bool:
+    """Whether a plan of the tensor cores runs the separable-phasor kernels:
+    their gridder items are L/32 column strips of a subgrid (two halves each
+    for L = 128), the others 512-pixel tiles."""
+    n_sg = int(stats.n_subgrids) - int(stats.n_subgrids_dropped)
+    return int(stats.mac_unit) == 2 and int(stats.n_grid_items) == n_sg * (L // 32) * (2 if L == 128 else 1)
 
 
 def _env_int(name, default):
@@ -325,9 +342,10 @@ def recorded_traffic(kern: str, workload: str):
 
 def algorithmic_bytes_per_launch(kern: str, obs, L: int) -> float:
     """DRAM bytes a launch must move, averaged over the plan's batches:
-    gridder 128 B staged record read per visibility + 32 B subgrid image
-    written per pixel; degridder 32 B image read per pixel + 32 B per
-    visibility written (host-only plan, no device work)."""
+    gridder 128 B staged record (48 B for the separable kernel) read per
+    visibility + 32 B subgrid image written per pixel; degridder 32 B image
+    read per pixel + 32 B per visibility written (host-only plan, no device
+    work)."""
     from paper_2502_17789_gb300 import idg
 
     g, keep = idg.make_geometry(obs.grid_size, L, obs.kernel_padding, obs.image_size, aterm_nodes=obs.aterm_nodes,
@@ -343,7 +361,8 @@ def algorithmic_bytes_per_launch(kern: str, obs, L: int) -> float:
     per_sg = 4 * L * L * 8
     n_batches = max(1, -(-n_sg // max(1, (1 << 30) // per_sg)))
     pix = n_sg * L * L * 32.0
-    total = (128.0 * n_vis + pix) if kern.startswith("gridder") else (pix + 32.0 * n_vis)
+    record = 48.0 if kern == "gridder_sep" else 128.0
+    total = (record * n_vis + pix) if kern.startswith("gridder") else (pix + 32.0 * n_vis)
     return total / n_batches
 
 
@@ -569,13 +588,20 @@ def run_native(args):
     peak_tflops = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     achieved_vispx = vispx / (k_ms * 1e-3)
     achieved = achieved_vispx * FLOP_PER_VISPX / 1e12
-    kern_name = kernel_of(kern, int(st.mac_unit))
+    separable = separable_plan(st, obs_r.subgrid_size)
+    kern_name = kernel_of(kern, int(st.mac_unit), separable)
     traffic = recorded_traffic(kern_name, desc)
     roofline = {"bound": "alu", "kernel": kern_name, "achieved": round(achieved, 3), "peak": round(peak_tflops, 3),
                 "unit": "TFLOP/s", "frac": round(achieved / peak_tflops, 4), "traffic": traffic,
                 "peak_basis": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 FMA lanes x 2 flop x {sm_max:.0f} MHz (max SM clock)",
                 "achieved_vispx_per_s": achieved_vispx, "flop_per_vispx": FLOP_PER_VISPX,
                 "launches": k_launches, "avg_launch_ms": k_ms / max(k_launches, 1)}
+    if separable and peaks.get("bf16_tflops"):
+        # the separable kernels replace the direct sum's FP32 operations (`frac` above is against those and
+        # may pass 1) by f16 products on the tensor cores, at the measured rate of a 16-bit GEMM
+        t = achieved_vispx * SEP_FLOP_PER_VISPX / 1e12
+        roofline["tensor"] = {"achieved": round(t, 1), "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+                              "frac": round(t / peaks["bf16_tflops"], 4), "flop_per_vispx": SEP_FLOP_PER_VISPX}
     if clocks.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = round(achieved / (peak_tflops * clocks["sm_mhz"] / sm_max), 4)
     # the same fractions against the rates the library's probe kernels measure on this device (FP32

@@ -83,7 +83,8 @@ enum {
   IDG_DROP_OUT_OF_GRID = 1,         /* drop subgrids that leave the grid instead of failing */
   IDG_SPLIT_AT_ATERM_INTERVALS = 2, /* never let a subgrid span two A-term intervals (Section 3.3 as written) */
   IDG_HOST_ONLY = 4,                /* plan on the host only: no device memory, grid/degrid refused */
-  IDG_PERSISTENT = 8,               /* persistent launches: #SMs x occupancy blocks drain a work queue */
+  IDG_PERSISTENT = 8,               /* persistent launches: #SMs x occupancy blocks drain a work queue (the kernels
+                                       with factored phasors always share their items out over the SMs) */
   IDG_W_LAYERS = 16,                /* w layers (Section 2.4): rows (baseline, timestep) with w < 0 are taken
                                        as their mirrors V^H of baseline (q, p) at (-u, -v, -w) (the footnote's
                                        V(u,v,w) = V(-u,-v,-w)^H), and each subgrid sits on one layer
@@ -127,7 +128,7 @@ typedef struct {
   int64_t n_vis_dropped;      /* visibilities of dropped subgrids */
   int64_t n_subgrids_dropped;
   int64_t n_grid_items;       /* gridder work items (subgrid, pixel tile) */
-  int64_t n_degrid_items;     /* degridder work items (<= 256 visibilities of one or two segments) */
+  int64_t n_degrid_items;     /* degridder work items (visibilities of one or two segments) */
   int64_t n_batches;          /* device batches the subgrids are processed in */
   int64_t occupancy_hist[16]; /* subgrids with visibility count in [2^k, 2^(k+1)), last bin open */
   int64_t device_bytes;       /* device memory held by the plan */

@@ -113,10 +113,11 @@ __global__ void __launch_bounds__(256) stage_records_kernel(const StageArgs a, i
   }
 }
 
-// Staging for the separable-phasor gridder: one block per subgrid writes its segments' records, 16 visibilities per chunk (the last padded
-// with zeros; kGsepChunkFloat4): a fix, b fix, delta, 1 / scale and the 4 values times the segment's scale, a
-// power of two that puts the largest component in [512, 1024) so that hi + lo halves keep 22 bits down to
-// 2^-9 of it.
+// Staging for the separable-phasor gridder: one block per subgrid writes its segments' records, 16 visibilities per
+// chunk (the last padded with zeros; kGsepChunkFloat4): a fix, b fix, delta, 1 / scale and the 4 values times the
+// segment's scale, a power of two that puts the largest component in [512, 1024) so that hi + lo halves keep 22 bits
+// down to 2^-9 of it.  Bound by latency, not bytes: a pass over a segment's values for the scale, then one that reads
+// them again (from L1 or L2) and writes.
 __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float* w_ref,
                                                         int L) {
   const SubgridDesc sd = a.sg[blockIdx.x];
@@ -182,9 +183,8 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
         const float re[4] = {v0.x, v0.z, v1.x, v1.z}, im[4] = {v0.y, v0.w, v1.y, v1.w};
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-          c[64 + 48 * p] = re[p];
-          c[80 + 48 * p] = im[p];
-          c[96 + 48 * p] = -im[p];
+          c[64 + 32 * p] = re[p];
+          c[80 + 32 * p] = im[p];
         }
       }
     }

@@ -23,13 +23,17 @@
 // written.  The pixel sums need J registers of a consumer, so the halves
 // split the block's registers unevenly.
 //
-// What bounds it: issue slots, then shared memory.  With the E side in
-// shared memory too, operands, their reads by the MMAs and a transpose per 16 rows kept
-// shared memory 80 % busy (21.2 ms where this takes 17.0); the E side in tensor
-// memory costs none.  Measured (GB300, MWA-like workload, 96 x 96 subgrids,
-// segments of about 60 visibilities, per grid call): 17.0 ms, against 81.7 ms of the
-// kernel with one phasor per visibility and pixel (gridder_tc_kernels.cuh);
-// grid error 9e-7 against 2.2e-6.
+// What bounds it: the latency of a chunk's chain (phasors, splits, the stores to
+// tensor memory, a barrier, the MMAs) at 4 warps a scheduler, which the pixel sums'
+// registers allow: 55 % of the issue slots, tensor pipe 34 % and shared memory 53 %
+// busy.  With the E side in shared memory too, operands, their reads by the MMAs
+// and a transpose per 16 rows kept shared memory 80 % busy (21.2 ms where this takes
+// 16.8); the E side in tensor memory costs none.  E's phasors computed once for the
+// 4 correlations and passed through shared memory lengthen the chain (17.6 ms).
+// Measured (GB300, MWA-like workload, 96 x 96 subgrids, segments of about 60
+// visibilities, per grid call): 16.8 ms, against 81.7 ms of the kernel with one
+// phasor per visibility and pixel (gridder_tc_kernels.cuh); grid error 5e-7
+// against 2.2e-6.
 #pragma once
 
 #include <type_traits>
@@ -81,7 +85,7 @@ __device__ __forceinline__ void gsep_produce(uint32_t e_col, uint32_t buf, const
   const int tid = threadIdx.x, warp = tid >> 5;
   {
     const int p = warp & 3, g = warp >> 2;
-    const float4* val = rec + 16 + 12 * p + 2 * g;
+    const float4* val = rec + 16 + 8 * p + 2 * g;
     uint32_t re_hi[4], re_lo[4], re_c[4], im_hi[4], im_lo[4], im_c[4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {

@@ -487,7 +487,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   SepFit sep;
   std::vector<float> w_ref;
   bool sep_ok = false;
-  if (!host_only) {
+  if (supported_subgrid_size(L)) {  // host-only plans take other sizes too
     sep = sep_fit(L, g->image_size, taper_d);
     double delta = 0.0;
     w_ref.reserve(p->exec.size());
@@ -512,7 +512,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
   // cannot run); both on FP32 when channel groups were asked for, and for Stokes I without the separable form
   // (the FP32 kernels' sums over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four
-  // correlations: an 80-station predict-and-grid cycle takes 10.7 ms on them, and 4.1 ms on the separable kernels,
+  // correlations: an 80-station predict-and-grid cycle takes 10.8 ms on them, and 3.9 ms on the separable kernels,
   // which sum all four)
   p->mac = g->mac_unit != IDG_MAC_DEFAULT ? g->mac_unit
            : (g->degrid_channels > 1 || ((g->flags & IDG_STOKES_I) && !sep_ok)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
@@ -797,10 +797,10 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
 }
 
 // Items per run (SepShare) of the degridder and blocks of the separable-phasor kernels for n items.  Runs where every
-// block still gets eight of them (the gridder reads nothing but its own records: single items, 16.7 ms on the
-// MWA-like workload against 17.4 in runs of 12); one block per SM (all that fit), so that a block's set-up and the latency of its first item are
-// paid once and its roles run ahead from item to item; more only where a block would hold more than 512 items, so
-// that a launch leaves SMs to other streams within a few milliseconds.
+// block still gets eight of them (the gridder reads nothing but its own records: single items, 16.8 ms on the
+// MWA-like workload against 17.4 in runs of 12); one block per SM (all that fit), so that a block's set-up and the
+// latency of its first item are paid once and its roles run ahead from item to item; more only where a block would
+// hold more than 512 items, so that a launch leaves SMs to other streams within a few milliseconds.
 static int sep_run(const idg_plan* p, int n) { return std::max(1, std::min(12, n / (8 * std::max(1, int(p->sms))))); }
 static int sep_blocks(const idg_plan* p, int n, int run) {
   const int sms = std::max(1, int(p->sms));

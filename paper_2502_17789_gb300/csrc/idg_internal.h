@@ -131,9 +131,9 @@ __host__ __device__ inline int64_t tc_records(int n_groups, int nc) {
 // Separable-phasor kernels (sep_common.cuh): the staged records of a subgrid
 // are chunks of 16 visibilities of one segment (the last chunk of a segment
 // padded with zeros): 16 floats each of a fix, b fix, delta (sep_common.cuh) and
-// 1 / scale, then per correlation 16 each of Re, Im and -Im
+// 1 / scale, then per correlation 16 each of Re and Im (48 bytes a visibility)
 constexpr int kGsepChunkVis = 16;
-constexpr int kGsepChunkFloat4 = 64;
+constexpr int kGsepChunkFloat4 = 48;
 // gridder work item: 32 pixel columns x gsep_rows(L) rows
 constexpr int kGsepColumns = 32;
 __host__ __device__ constexpr int gsep_rows(int L) { return L == 128 ? 64 : L; }

@@ -14,7 +14,7 @@
 // visibility needs 2 L sines and cosines instead of L^2 and the
 // multiply-accumulate runs on the tensor cores at full tile sizes.  The plan
 // takes this path only where the neglected terms, weighted with the taper,
-// stay below kSepTolerance (sep_tables).
+// stay below kSepTolerance (sep_fit).
 //
 // Products: tcgen05.mma kind::f16 with FP32 accumulation in tensor memory.
 // Every FP32 operand is split into two halves hi + lo (22 bits), and the

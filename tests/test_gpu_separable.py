@@ -31,7 +31,7 @@ def _check(c, seed):
 
 
 # segments of 1, 15, 16, 17 and several hundred visibilities (chunks of 16, rings of 2 to 4 chunks,
-# items of 64 and 128 visibilities), the largest A-term tables
+# items of at most 64 visibilities), the largest A-term tables
 @pytest.mark.parametrize("L,n_ch,n_t,steps,nodes", [(32, 1, 3, 1, 2), (64, 5, 6, 3, 9), (96, 4, 8, 4, 25),
                                                     (128, 17, 4, 1, 25), (64, 31, 20, 20, 9), (32, 33, 9, 5, 25),
                                                     (96, 43, 7, 7, 9), (128, 3, 50, 43, 9)])
