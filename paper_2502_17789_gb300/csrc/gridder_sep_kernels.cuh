@@ -24,14 +24,14 @@
 // split the block's registers unevenly.
 //
 // What bounds it: the latency of a chunk's chain (phasors, splits, the stores to
-// tensor memory, a barrier, the MMAs) at 4 warps a scheduler, which the pixel sums'
-// registers allow: 55 % of the issue slots, tensor pipe 34 % and shared memory 53 %
-// busy.  With the E side in shared memory too, operands, their reads by the MMAs
-// and a transpose per 16 rows kept shared memory 80 % busy (21.2 ms where this takes
-// 16.8); the E side in tensor memory costs none.  E's phasors computed once for the
-// 4 correlations and passed through shared memory lengthen the chain (17.6 ms).
+// tensor memory, a barrier) at 4 warps a scheduler, which the pixel sums'
+// registers allow: about 60 % of the issue slots, tensor pipe 37 % and shared
+// memory 59 % busy.  With the E side in shared memory too, operands, their reads by the MMAs
+// and a transpose per 16 rows kept shared memory 80 % busy (21.2 ms where that took
+// 17.6); the E side in tensor memory costs none.  E's phasors computed once for the
+// 4 correlations and passed through shared memory lengthen the chain (16.0 ms).
 // Measured (GB300, MWA-like workload, 96 x 96 subgrids, segments of about 60
-// visibilities, per grid call): 16.8 ms, against 81.7 ms of the kernel with one
+// visibilities, per grid call): 15.2 ms, against 81.7 ms of the kernel with one
 // phasor per visibility and pixel (gridder_tc_kernels.cuh); grid error 5e-7
 // against 2.2e-6.
 #pragma once
@@ -56,6 +56,9 @@ struct Gsep {
   static constexpr int kSpan = kRows / 8;                        // rows of a consumer thread
   static constexpr int kPairs = kSpan / 2;
   static constexpr int kConsumerRegs = kRows > 64 ? 184 : 160;   // the producers keep 256 less
+  // How a producer gets the next chunk's record: with 72 registers by cp.async (a register held for it is spilled at
+  // once, and the spill waits for the load: 16.0 -> 15.2 ms at L = 96), with 96 through registers (3.9 -> 3.8 ms at 64)
+  static constexpr bool kAsyncRecord = kRows > 64;
   static_assert(kECol + kRing * 48 <= int(kTmemCols), "tensor memory");
 };
 
@@ -65,6 +68,7 @@ struct GsepShared {
   unsigned char ring[Gsep<L>::kRing * Gsep<L>::kBufBytes];
   float2 x[4][2][Gsep<L>::kRows / 2][32];  // [pol][re, im][row pair][column] of a segment's sums
   float4 rec[2][kGsepChunkFloat4];
+  int part[2];               // [chunk parity] its place in its part: 1 first, 2 last
   uint64_t empty[4];         // chunk read by its MMAs
   uint64_t full[2];          // accumulator complete
   uint64_t drained[2];       // accumulator read by the 8 consumer warps
@@ -148,12 +152,16 @@ __device__ __forceinline__ int2 gsep_origin(const GridItem& item) {
   return make_int2(item.tile / n * kGsepColumns, item.tile % n * Gsep<L>::kRows);
 }
 
-// producers' side
+// Producers' side.  What stands between two chunks is kept off their path: of the two warps without a part of F one
+// issues the MMAs, the other keeps the segments (whose lengths come from global memory) and waits for the next
+// chunk's place in the ring, which the barrier passes on to the others (per chunk at L = 96 some 150 and 100 of 2350
+// clocks when every warp did both; 16.8 -> 16.0 ms, at L = 64 4.3 -> 3.8).
 template <int L>
 __device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share, GsepShared<L>& S) {
   using C = Gsep<L>;
   const int tid = threadIdx.x, lane = tid & 31;
-  const bool issuer = uniform_warp() == kSepHalf / 32 - 1;  // the producer warp with the least to write
+  // the producer warps with the least to write: one issues, one waits for places of the ring
+  const bool issuer = uniform_warp() == kSepHalf / 32 - 1, waiter = uniform_warp() == kSepHalf / 32 - 2;
   const uint32_t ring0 = smem_u32(S.ring), tm = S.tmem;
   uint32_t cg = 0, sc = 0;  // chunks and segment parts of this block so far
   for (int idx = share.first; idx < share.last; idx = share.next(idx)) {
@@ -170,39 +178,53 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share,
     if (tid < kGsepChunkFloat4) S.rec[cg & 1][tid] = __ldg(recs + tid);
     half_sync(kSepProducerBar);
     for (int c = 0; c < total; ++c) {
+      // the next chunk's record
       float4 nxt;
       const bool more = c + 1 < total && tid < kGsepChunkFloat4;
-      if (more) nxt = __ldg(recs + size_t(c + 1) * kGsepChunkFloat4 + tid);
-      const uint32_t slot = cg % C::kRing, turn = cg / C::kRing;
-      if (turn > 0) {
-        sep_wait(&S.empty[slot], (turn - 1) & 1, &S.fail, a.status);
-        tc_fence_after();
+      if (more) {
+        const float4* src = recs + size_t(c + 1) * kGsepChunkFloat4 + tid;
+        if (C::kAsyncRecord)
+          cp_async16(&S.rec[(cg + 1) & 1][tid], src);
+        else
+          nxt = __ldg(src);
       }
+      if (C::kAsyncRecord) cp_async_commit();
+      const uint32_t slot = cg % C::kRing, turn = cg / C::kRing;
+      if (turn > 0) tc_fence_after();
       const uint32_t buf = ring0 + slot * C::kBufBytes, e_col = tm + C::kECol + slot * 48;
       gsep_produce<L>(e_col, buf, S.rec[cg & 1], i - L / 2, fit_a, fit_p, j - L / 2, fit_b, fit_q);
-      if (more) S.rec[(cg + 1) & 1][tid] = nxt;
+      if (!C::kAsyncRecord && more) S.rec[(cg + 1) & 1][tid] = nxt;
+      if (waiter) {
+        const bool last_c = c_in + 1 == n_in;
+        if (lane == 0) S.part[cg & 1] = int(c_in == 0) | int(last_c) << 1;
+        ++c_in;
+        if (last_c) {
+          left -= n_in;
+          c_in = 0;
+          if (left == 0 && c + 1 < total) left = gsep_chunks(a.seg[sd.seg_begin + ++s]);
+          n_in = gsep_part(left);
+        }
+        if (cg + 1 >= uint32_t(C::kRing))
+          sep_wait(&S.empty[(cg + 1) % C::kRing], ((cg + 1) / C::kRing - 1) & 1, &S.fail, a.status);
+      }
+      if (C::kAsyncRecord) cp_async_wait<0>();
       tmem_wait_st();
       tc_fence_before();
       fence_proxy_async();
       half_sync(kSepProducerBar);
-      const bool last_c = c_in + 1 == n_in;
-      if (issuer && elect_one()) {
-        // the accumulator's previous segment (two back) has been read
-        if (c_in == 0 && sc >= 2) sep_wait(&S.drained[sc & 1], ((sc >> 1) - 1) & 1, &S.fail, a.status);
-        tc_fence_after();
-        sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, c_in == 0);
-        sep_commit(&S.empty[slot]);
-        if (last_c) sep_commit(&S.full[sc & 1]);
+      if (issuer) {
+        const int part = S.part[cg & 1];
+        if (elect_one()) {
+          // the accumulator's previous segment (two back) has been read
+          if ((part & 1) && sc >= 2) sep_wait(&S.drained[sc & 1], ((sc >> 1) - 1) & 1, &S.fail, a.status);
+          tc_fence_after();
+          sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, part & 1);
+          sep_commit(&S.empty[slot]);
+          if (part & 2) sep_commit(&S.full[sc & 1]);
+        }
+        sc += part >> 1;
       }
       ++cg;
-      ++c_in;
-      if (last_c) {
-        ++sc;
-        left -= n_in;
-        c_in = 0;
-        if (left == 0 && c + 1 < total) left = gsep_chunks(a.seg[sd.seg_begin + ++s]);
-        n_in = gsep_part(left);
-      }
     }
   }
 }

@@ -797,8 +797,8 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
 }
 
 // Items per run (SepShare) of the degridder and blocks of the separable-phasor kernels for n items.  Runs where every
-// block still gets eight of them (the gridder reads nothing but its own records: single items, 16.8 ms on the
-// MWA-like workload against 17.4 in runs of 12); one block per SM (all that fit), so that a block's set-up and the
+// block still gets eight of them (the gridder reads nothing but its own records: single items, 15.2 ms on the
+// MWA-like workload, 4 % more in runs of 12); one block per SM (all that fit), so that a block's set-up and the
 // latency of its first item are paid once and its roles run ahead from item to item; more only where a block would
 // hold more than 512 items, so that a launch leaves SMs to other streams within a few milliseconds.
 static int sep_run(const idg_plan* p, int n) { return std::max(1, std::min(12, n / (8 * std::max(1, int(p->sms))))); }
