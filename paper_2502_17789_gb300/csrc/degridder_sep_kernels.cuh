@@ -27,7 +27,7 @@
 // What bounds it: issue slots (83 % taken; tensor pipe 29 %).  With all threads doing each step in turn and Z in
 // shared memory it took 46.8 ms (MWA-like workload, 96 x 96 subgrids, segments
 // of about 60 visibilities, per degrid call on GB300), with a half of producers
-// in step and a half of consumers 31.4 ms, with these roles 20.1 ms; the kernel with
+// in step and a half of consumers 31.4 ms, with these roles 19.7 ms; the kernel with
 // one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.
 #pragma once
 
@@ -224,10 +224,7 @@ struct Dsep {
         for (int jc = grp; jc < kPieces; jc += 2, pg += 2) {
           const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
           wait(&S.loaded[slot], turn & 1);
-          if (turn > 0) {
-            wait(&S.empty[slot], (turn - 1) & 1);
-            tc_fence_after();
-          }
+          if (turn > 0) tc_fence_after();  // the loader has seen the slot's last MMAs complete
           const uint32_t e_col = tm + kDsepZCol + slot * 48;
           const float2* y = &S.y[slot][0][0][0][0];
           if (quad) {
@@ -260,7 +257,8 @@ struct Dsep {
 #pragma unroll 1
       for (int t = 0; t < kBlocks * kPieces; ++t, ++pg) {
         const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
-        if (turn > 0) wait(&S.filled[slot], (turn - 1) & 1);  // the ring's previous piece has been read
+        // the slot's previous piece of Y has been read and its Z multiplied: one wait less for every producer
+        if (turn > 0) wait(&S.empty[slot], (turn - 1) & 1);
         __syncwarp();
         if (elect_one()) {
           mbar_arrive_expect_tx(&S.loaded[slot], 4096 * a.g.npol);
