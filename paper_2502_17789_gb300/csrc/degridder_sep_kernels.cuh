@@ -13,10 +13,10 @@
 // sum over i takes one complex multiply-add per (visibility, column), 1/L of
 // the direct sum.
 //
-// A block of 24 warps works through a share of the items (an item is up to kv
+// A block of 20 warps works through a share of the items (an item is up to kv
 // visibilities of one segment); its warps have roles that run side by side.
-// Producers (two groups of 8 warps, every other piece each): per piece of 16 rows j of a block of 32 columns, thread = row
-// (p, i) x 8 rows j writes Z to tensor memory, from Y pieces that a loading warp
+// Producers (three groups of 4 warps, pieces in turn): per piece of 16 rows j of a block of 32 columns, thread = row
+// (p, i) x 16 rows j writes Z to tensor memory, from Y pieces that a loading warp
 // copies to shared memory up to four pieces ahead; an issuing warp starts the piece's
 // 16 MMAs, whose commit frees it.  Consumers take the accumulators, which alternate
 // between two column ranges of tensor memory from column block to column
@@ -24,11 +24,14 @@
 // warp.  Preparing warps write the next item's phase slopes, F side of all L
 // rows and A-term samples (double buffers) while one runs.
 //
-// What bounds it: issue slots (83 % taken; tensor pipe 29 %).  With all threads doing each step in turn and Z in
-// shared memory it took 46.8 ms (MWA-like workload, 96 x 96 subgrids, segments
-// of about 60 visibilities, per degrid call on GB300), with a half of producers
-// in step and a half of consumers 31.4 ms, with these roles 19.7 ms; the kernel with
-// one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.
+// What bounds it: the producers' issue slots and instruction supply.  With all threads
+// doing each step in turn and Z in shared memory it took 46.8 ms (MWA-like workload, 96 x
+// 96 subgrids, segments of about 60 visibilities, per degrid call on GB300), with a half
+// of producers in step and a half of consumers 31.4 ms, with roles and a thread's 8 rows
+// of a piece written out 19.7 ms; 16 rows per thread pay a piece's waits and set-up for
+// twice the rows, and four rows at a time in a loop keep the code small (18.2 ms; full
+// Jones matrices, 64 stations: 1.43 -> 1.16; written out 16 times 20.6 and 1.65).  The
+// kernel with one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.
 #pragma once
 
 #include "sep_common.cuh"
@@ -37,14 +40,15 @@ namespace idg {
 
 constexpr int kDsepMaxVis = 64;   // visibilities per item at most
 constexpr int kDsepRing = 4;      // Y pieces in shared memory, Z pieces in tensor memory
-// roles: two producer groups of 8 warps, 4 consumer warps, the issuing warp, the loading warp, 2 preparing warps
-constexpr int kDsepThreads = 768, kDsepConsumer = 512, kDsepIssuer = 640, kDsepLoader = 672, kDsepPreparer = 704;
+// roles: three producer groups of 4 warps, 4 consumer warps, the issuing warp, the loading warp, 2 preparing warps
+constexpr int kDsepGroups = 3;
+constexpr int kDsepThreads = 640, kDsepConsumer = 384, kDsepIssuer = 512, kDsepLoader = 544, kDsepPreparer = 576;
 constexpr int kDsepPreparers = 64;
 static_assert(kDsepMaxVis <= kDsepPreparers, "a visibility per preparing thread");
 constexpr int kDsepPreparerBar = 4;
-// registers per thread: 80 at launch, then by role
-constexpr int kDsepLaunchRegs = 80, kDsepProducerRegs = 72, kDsepConsumerRegs = 120, kDsepOtherRegs = 72;
-static_assert(512 * kDsepProducerRegs + 128 * (kDsepConsumerRegs + kDsepOtherRegs) <= kDsepThreads * kDsepLaunchRegs,
+// registers per thread: 96 at launch, then by role
+constexpr int kDsepLaunchRegs = 96, kDsepProducerRegs = 88, kDsepConsumerRegs = 136, kDsepOtherRegs = 80;
+static_assert(kDsepConsumer * kDsepProducerRegs + 128 * (kDsepConsumerRegs + kDsepOtherRegs) <= kDsepThreads * kDsepLaunchRegs,
               "registers");
 constexpr int kDsepColStride = 2 * kDsepMaxVis;       // between the two accumulators (re, im)
 constexpr int kDsepZCol = 2 * kDsepColStride;         // first column of the Z ring
@@ -63,7 +67,7 @@ struct alignas(128) DsepShared {
   uint64_t ready[2];        // item prepared (2 preparing warps)
   uint64_t loaded[kDsepRing]; // Y piece copied
   uint64_t done[2];         // item's visibilities written, its operands read (4 consumer warps)
-  uint64_t filled[kDsepRing]; // Z piece written (8 producer warps)
+  uint64_t filled[kDsepRing]; // Z piece written (4 producer warps)
   uint64_t empty[kDsepRing];  // Z piece read by its MMAs
   uint64_t full[2];         // accumulator complete
   uint64_t drained[2];      // accumulator read (4 consumer warps)
@@ -102,13 +106,13 @@ struct Dsep {
 
   // ---------------------------------------------------------------- producers
 
-  // Z of rows 16 jc .. for column block ib: thread = (p, i) x 8 rows j.  QUAD: node cells start at multiples of four
-  // rows, so the cell can change only half way and not at every row.
+  // Z of rows 16 jc .. for column block ib: thread = (p, i) x 16 rows j.  QUAD: node cells start at multiples of four
+  // rows, so the cell can change only there and not at every row.
   template <bool DIAG, bool QUAD>
   __device__ __forceinline__ void produce(uint32_t e_col, const float2* yb, const float4* samples, float scale,
                                           NodeWeight wx, int jc, __half2 fit_p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int p = warp & 3, g = (warp >> 2) & 1, pa = p >> 1, pb = p & 1;
+    const int p = warp & 3, pa = p >> 1, pb = p & 1;
     const int nodes = a.g.nodes, step = nodes - 1;
     const bool stokes = a.g.npol == 1;
     constexpr int NE = DIAG ? 1 : 2;  // entries of each station's matrix that this correlation needs
@@ -134,114 +138,113 @@ struct Dsep {
                       fmaf(k0[st], x1.y, fmaf(k1[st], y1.y, -u[st][e].im))};
         }
     };
-    // row q of the octet lies at (rem + step q) / L of the cell that starts at node row `at`
-    int at = step * (16 * jc + 8 * g) / L, rem = step * (16 * jc + 8 * g) - at * L;
+    // row r of the piece lies at (rem + step r) / L of the cell that starts at node row `at`; four rows at a time, in
+    // a loop that stays small: with the rows written out 16 times the warps wait for instructions
+    int at = step * 16 * jc / L, rem = step * 16 * jc - at * L;
     load_cell(at);
-    float f0 = float(rem) * (1.f / float(L));
     const float df = float(step) * (1.f / float(L));
-    const float2* y0 = yb + (4 * g) * 64 + lane;  // [pol][row pair][re, im][column]
-    uint32_t re_hi[2], re_lo[2], re_c[2], im_hi[2], im_lo[2], im_c[2];
-    const uint32_t dst = e_col + (uint32_t(p * 32) << 16) + 4 * g;
+    const float2* y0 = yb + lane;  // [pol][row pair][re, im][column]
+    uint32_t dst = e_col + (uint32_t(p * 32) << 16);
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r, dst += 2, y0 += 128, rem += 4 * step) {
+      uint32_t re_hi[2], re_lo[2], re_c[2], im_hi[2], im_lo[2], im_c[2];
+      float f0 = float(rem) * (1.f / float(L));
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      float2 yr[DIAG ? 1 : 4], yi[DIAG ? 1 : 4];  // Y at both rows of the pair
+      for (int w = 0; w < 2; ++w) {
+        float2 yr[DIAG ? 1 : 4], yi[DIAG ? 1 : 4];  // Y at both rows of the pair
 #pragma unroll
-      for (int k = 0; k < (DIAG ? 1 : 4); ++k) {
-        const float2* y = y0 + (stokes ? 0 : DIAG ? p : k) * 512 + w * 64;
-        yr[k] = y[0];
-        yi[k] = y[32];
-      }
-      float2 zr, zi;
+        for (int k = 0; k < (DIAG ? 1 : 4); ++k) {
+          const float2* y = y0 + (stokes ? 0 : DIAG ? p : k) * 512 + w * 64;
+          yr[k] = y[0];
+          yi[k] = y[32];
+        }
+        float2 zr, zi;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int q = 2 * w + h;
-        if (QUAD ? q == 4 : q > 0) {
-          if (rem + step * q >= L) {  // the same for the whole warp
-            rem -= L;
-            f0 -= 1.f;
-            load_cell(++at);
+        for (int h = 0; h < 2; ++h) {
+          const int q = 2 * w + h;
+          if (!QUAD || q == 0) {
+            if (rem + step * q >= L) {  // the same for the whole warp
+              rem -= L;
+              f0 -= 1.f;
+              load_cell(++at);
+            }
+          }
+          const float f = fmaf(float(q), df, f0);
+          cf m[2][NE];  // the entries at this row
+#pragma unroll
+          for (int st = 0; st < 2; ++st)
+#pragma unroll
+            for (int e = 0; e < NE; ++e) m[st][e] = {fmaf(f, d[st][e].re, u[st][e].re), fmaf(f, d[st][e].im, u[st][e].im)};
+          cf y[DIAG ? 1 : 4];
+#pragma unroll
+          for (int k = 0; k < (DIAG ? 1 : 4); ++k) y[k] = h ? cf{yr[k].y, yi[k].y} : cf{yr[k].x, yi[k].x};
+          cf z;
+          if constexpr (DIAG) {
+            z = cmulc(m[1][0], cmul(m[0][0], y[0]));
+          } else if (stokes) {
+            z = cadd(cmulc(m[1][0], cmul(m[0][0], y[0])), cmulc(m[1][1], cmul(m[0][1], y[0])));
+          } else {
+            z = cadd(cmulc(m[1][0], cadd(cmul(m[0][0], y[0]), cmul(m[0][1], y[2]))),
+                     cmulc(m[1][1], cadd(cmul(m[0][0], y[1]), cmul(m[0][1], y[3]))));
+          }
+          if (h) {
+            zr.y = z.re;
+            zi.y = z.im;
+          } else {
+            zr.x = z.re;
+            zi.x = z.im;
           }
         }
-        const float f = fmaf(float(q), df, f0);
-        cf m[2][NE];  // the entries at this row
-#pragma unroll
-        for (int st = 0; st < 2; ++st)
-#pragma unroll
-          for (int e = 0; e < NE; ++e) m[st][e] = {fmaf(f, d[st][e].re, u[st][e].re), fmaf(f, d[st][e].im, u[st][e].im)};
-        cf y[DIAG ? 1 : 4];
-#pragma unroll
-        for (int k = 0; k < (DIAG ? 1 : 4); ++k) y[k] = h ? cf{yr[k].y, yi[k].y} : cf{yr[k].x, yi[k].x};
-        cf z;
-        if constexpr (DIAG) {
-          z = cmulc(m[1][0], cmul(m[0][0], y[0]));
-        } else if (stokes) {
-          z = cadd(cmulc(m[1][0], cmul(m[0][0], y[0])), cmulc(m[1][1], cmul(m[0][1], y[0])));
-        } else {
-          z = cadd(cmulc(m[1][0], cadd(cmul(m[0][0], y[0]), cmul(m[0][1], y[2]))),
-                   cmulc(m[1][1], cadd(cmul(m[0][0], y[1]), cmul(m[0][1], y[3]))));
-        }
-        if (h) {
-          zr.y = z.re;
-          zi.y = z.im;
-        } else {
-          zr.x = z.re;
-          zi.x = z.im;
-        }
+        re_c[w] = h2_bits(__hmul2(sep_split(zr, re_hi[w], re_lo[w]), fit_p));
+        im_c[w] = h2_bits(__hmul2(sep_split(zi, im_hi[w], im_lo[w]), fit_p));
       }
-      const int o = w & 1;
-      re_c[o] = h2_bits(__hmul2(sep_split(zr, re_hi[o], re_lo[o]), fit_p));
-      im_c[o] = h2_bits(__hmul2(sep_split(zi, im_hi[o], im_lo[o]), fit_p));
-      if (o) {  // four rows at a time: the block's registers are spread over many producers
-        const uint32_t to = dst + (w & 2);
-        tmem_st2(to, re_hi[0], re_hi[1]);
-        tmem_st2(to + 8, im_hi[0], im_hi[1]);
-        tmem_st2(to + 16, re_lo[0], re_lo[1]);
-        tmem_st2(to + 24, im_lo[0], im_lo[1]);
-        tmem_st2(to + 32, re_c[0], re_c[1]);
-        tmem_st2(to + 40, im_c[0], im_c[1]);
-      }
+      tmem_st2(dst, re_hi[0], re_hi[1]);
+      tmem_st2(dst + 8, im_hi[0], im_hi[1]);
+      tmem_st2(dst + 16, re_lo[0], re_lo[1]);
+      tmem_st2(dst + 24, im_lo[0], im_lo[1]);
+      tmem_st2(dst + 32, re_c[0], re_c[1]);
+      tmem_st2(dst + 40, im_c[0], im_c[1]);
     }
   }
 
-  // group 0 takes the even pieces of every item, group 1 the odd ones (an item has an even number); the warps of
-  // a group go their own way between the rings' barriers
+  // the groups take the block's pieces in turn; the warps of a group go their own way between the rings' barriers
   __device__ __forceinline__ void producer() {
-    const int lane = threadIdx.x & 31, nodes = a.g.nodes, grp = uniform_warp() >> 3;
+    constexpr uint32_t kItemPieces = kBlocks * kPieces;
+    const int lane = threadIdx.x & 31, nodes = a.g.nodes;
     const bool quad = L % (nodes - 1) == 0 && L / (nodes - 1) % 4 == 0;
     const uint32_t tm = S.tmem;
-    uint32_t n = 0, pg = grp;  // items and (both groups') pieces of this block so far
-    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
+    uint32_t n = 0, pg = uniform_warp() >> 2, base = 0;  // items so far, the group's next piece, the item's first
+    for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n, base += kItemPieces) {
+      // an item without a piece of this group is passed over: its barriers may be phases ahead
+      if (pg >= base + kItemPieces) continue;
       wait(&S.ready[n & 1], (n >> 1) & 1);
       const float scale = S.info[n & 1].scale;
       const bool diag = S.info[n & 1].diag != 0;
       const float4* samples = raw + (n & 1) * 4 * nodes * nodes;
 #pragma unroll 1
-      for (int ib = 0; ib < kBlocks; ++ib) {
-        const int i = ib * 32 + lane;
+      for (; pg < base + kItemPieces; pg += kDsepGroups) {
+        const int t = pg - base, ib = t / kPieces, jc = t - ib * kPieces, i = ib * 32 + lane;
         const NodeWeight wx = node_weight(i, nodes, L);
         const __half2 fit_p = __float2half2_rn(__ldg(a.sep.p + i));
-#pragma unroll 1
-        for (int jc = grp; jc < kPieces; jc += 2, pg += 2) {
-          const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
-          wait(&S.loaded[slot], turn & 1);
-          if (turn > 0) tc_fence_after();  // the loader has seen the slot's last MMAs complete
-          const uint32_t e_col = tm + kDsepZCol + slot * 48;
-          const float2* y = &S.y[slot][0][0][0][0];
-          if (quad) {
-            if (diag)
-              produce<true, true>(e_col, y, samples, scale, wx, jc, fit_p);
-            else
-              produce<false, true>(e_col, y, samples, scale, wx, jc, fit_p);
-          } else if (diag) {
-            produce<true, false>(e_col, y, samples, scale, wx, jc, fit_p);
-          } else {
-            produce<false, false>(e_col, y, samples, scale, wx, jc, fit_p);
-          }
-          tmem_wait_st();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&S.filled[slot]);
+        const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
+        wait(&S.loaded[slot], turn & 1);
+        if (turn > 0) tc_fence_after();  // the loader has seen the slot's last MMAs complete
+        const uint32_t e_col = tm + kDsepZCol + slot * 48;
+        const float2* y = &S.y[slot][0][0][0][0];
+        if (quad) {
+          if (diag)
+            produce<true, true>(e_col, y, samples, scale, wx, jc, fit_p);
+          else
+            produce<false, true>(e_col, y, samples, scale, wx, jc, fit_p);
+        } else if (diag) {
+          produce<true, false>(e_col, y, samples, scale, wx, jc, fit_p);
+        } else {
+          produce<false, false>(e_col, y, samples, scale, wx, jc, fit_p);
         }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.filled[slot]);
       }
     }
   }
@@ -473,7 +476,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
   if (threadIdx.x == 0) {
     for (int k = 0; k < kDsepRing; ++k) {
       mbar_init(&S.empty[k], 1);
-      mbar_init(&S.filled[k], 8);
+      mbar_init(&S.filled[k], 4);
       mbar_init(&S.loaded[k], 1);
     }
     for (int k = 0; k < 2; ++k) {
