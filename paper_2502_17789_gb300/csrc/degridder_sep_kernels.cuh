@@ -42,6 +42,12 @@ constexpr int kDsepMaxVis = 64;   // visibilities per item at most
 constexpr int kDsepRing = 4;      // Y pieces in shared memory, Z pieces in tensor memory
 // roles: three producer groups of 4 warps, 4 consumer warps, the issuing warp, the loading warp, 2 preparing warps
 constexpr int kDsepGroups = 3;
+// Arrivals of Y pieces have a barrier per (slot, group) pair in turn: a wait on a barrier's parity is only sound for a
+// warp that has waited for every phase before it, and a slot's pieces go to the groups in rotation, so with one barrier
+// per slot a group could take the phase of a piece that is still on its way to another group for its own.
+constexpr int kDsepLoaded = 12;
+static_assert(kDsepLoaded % kDsepGroups == 0 && kDsepLoaded % kDsepRing == 0,
+              "a barrier's pieces belong to one group and slot");
 constexpr int kDsepThreads = 640, kDsepConsumer = 384, kDsepIssuer = 512, kDsepLoader = 544, kDsepPreparer = 576;
 constexpr int kDsepPreparers = 64;
 static_assert(kDsepMaxVis <= kDsepPreparers, "a visibility per preparing thread");
@@ -65,7 +71,7 @@ struct alignas(128) DsepShared {
     int sg, n_pad, diag;
   } info[2];
   uint64_t ready[2];        // item prepared (2 preparing warps)
-  uint64_t loaded[kDsepRing]; // Y piece copied
+  uint64_t loaded[kDsepLoaded];  // Y piece copied, by piece modulo kDsepLoaded
   uint64_t done[2];         // item's visibilities written, its operands read (4 consumer warps)
   uint64_t filled[kDsepRing]; // Z piece written (4 producer warps)
   uint64_t empty[kDsepRing];  // Z piece read by its MMAs
@@ -226,9 +232,9 @@ struct Dsep {
         const int t = pg - base, ib = t / kPieces, jc = t - ib * kPieces, i = ib * 32 + lane;
         const NodeWeight wx = node_weight(i, nodes, L);
         const __half2 fit_p = __float2half2_rn(__ldg(a.sep.p + i));
-        const uint32_t slot = pg % kDsepRing, turn = pg / kDsepRing;
-        wait(&S.loaded[slot], turn & 1);
-        if (turn > 0) tc_fence_after();  // the loader has seen the slot's last MMAs complete
+        const uint32_t slot = pg % kDsepRing;
+        wait(&S.loaded[pg % kDsepLoaded], (pg / kDsepLoaded) & 1);
+        if (pg >= uint32_t(kDsepRing)) tc_fence_after();  // the loader has seen the slot's last MMAs complete
         const uint32_t e_col = tm + kDsepZCol + slot * 48;
         const float2* y = &S.y[slot][0][0][0][0];
         if (quad) {
@@ -264,9 +270,9 @@ struct Dsep {
         if (turn > 0) wait(&S.empty[slot], (turn - 1) & 1);
         __syncwarp();
         if (elect_one()) {
-          mbar_arrive_expect_tx(&S.loaded[slot], 4096 * a.g.npol);
+          mbar_arrive_expect_tx(&S.loaded[pg % kDsepLoaded], 4096 * a.g.npol);
           for (int pol = 0; pol < a.g.npol; ++pol)
-            bulk_copy_g2s(&S.y[slot][pol][0][0][0], Y + size_t(pol) * L * L + t * 512, 4096, &S.loaded[slot]);
+            bulk_copy_g2s(&S.y[slot][pol][0][0][0], Y + size_t(pol) * L * L + t * 512, 4096, &S.loaded[pg % kDsepLoaded]);
         }
         __syncwarp();
       }
@@ -477,8 +483,8 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
     for (int k = 0; k < kDsepRing; ++k) {
       mbar_init(&S.empty[k], 1);
       mbar_init(&S.filled[k], 4);
-      mbar_init(&S.loaded[k], 1);
     }
+    for (int k = 0; k < kDsepLoaded; ++k) mbar_init(&S.loaded[k], 1);
     for (int k = 0; k < 2; ++k) {
       mbar_init(&S.full[k], 1);
       mbar_init(&S.drained[k], 4);
@@ -513,7 +519,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
   __syncthreads();
   if (threadIdx.x < 32) {
     if (*reinterpret_cast<volatile int*>(&S.fail) && threadIdx.x == 0) {
-      for (int k = 0; k < kDsepRing; ++k) mbar_wait_bounded(&S.loaded[k], 0, kWaitLimitNs / 8);
+      for (int k = 0; k < kDsepLoaded; ++k) mbar_wait_bounded(&S.loaded[k], 0, kWaitLimitNs / 32);
       sep_commit(&S.full[0]);
       mbar_wait_bounded(&S.full[0], 0);
     }
