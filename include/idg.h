@@ -379,6 +379,17 @@ idg_status idg_predict(idg_plan* plan, const void* image_c128, const void* aterm
  */
 idg_status idg_wait_selftest(idg_plan* plan, int32_t limit_us);
 
+/*
+ * idg_set_wait_limit -- how long one device-side wait of the plan's kernels
+ * with factored phasors may last (nanoseconds, 0 .. 2e9, the default).  No
+ * counterpart in the paper.  A wait over the limit ends the call's work early:
+ * its outputs are undefined, the next idg_synchronize returns IDG_ERR_TIMEOUT
+ * and the context stays usable.  With 0 every wait that is not already over
+ * gives up.  Calls made from now on; IDG_ERR_INVALID_ARG for host-only plans
+ * or a limit out of range.
+ */
+idg_status idg_set_wait_limit(idg_plan* plan, int64_t limit_ns);
+
 /* Message for the last failure (never NULL; "" when none). */
 const char* idg_last_error(const idg_plan* plan);
 

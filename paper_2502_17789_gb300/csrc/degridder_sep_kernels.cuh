@@ -77,6 +77,7 @@ struct alignas(128) DsepShared {
   uint64_t empty[kDsepRing];  // Z piece read by its MMAs
   uint64_t full[2];         // accumulator complete
   uint64_t drained[2];      // accumulator read (4 consumer warps)
+  uint64_t drain;           // every MMA complete, after a wait that gave up
   uint32_t tmem;
   int fail;
 };
@@ -107,7 +108,7 @@ struct Dsep {
 
   template <int SLEEP = 32>
   __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) {
-    sep_wait<SLEEP>(bar, parity, &S.fail, a.status);
+    sep_wait<SLEEP>(bar, parity, &S.fail, a);
   }
 
   // ---------------------------------------------------------------- producers
@@ -260,6 +261,7 @@ struct Dsep {
   // Y in scratch: [pol][column block][row pair][re, im][32 columns], so a piece is one run of 4 KB per plane
   __device__ __forceinline__ void loader() {
     uint32_t n = 0, pg = 0;  // items and pieces of this block so far
+    uint32_t issued = 0;     // pieces the elected lane has started to copy: all, unless a wait gave up
     for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       wait<64>(&S.ready[n & 1], (n >> 1) & 1);
       const float2* Y = a.scratch + size_t(S.info[n & 1].sg) * 4 * L * L;
@@ -269,14 +271,19 @@ struct Dsep {
         // the slot's previous piece of Y has been read and its Z multiplied: one wait less for every producer
         if (turn > 0) wait(&S.empty[slot], (turn - 1) & 1);
         __syncwarp();
-        if (elect_one()) {
+        if (elect_one() && !sep_failed(&S.fail)) {
           mbar_arrive_expect_tx(&S.loaded[pg % kDsepLoaded], 4096 * a.g.npol);
           for (int pol = 0; pol < a.g.npol; ++pol)
             bulk_copy_g2s(&S.y[slot][pol][0][0][0], Y + size_t(pol) * L * L + t * 512, 4096, &S.loaded[pg % kDsepLoaded]);
+          ++issued;
         }
         __syncwarp();
       }
     }
+    // after a wait that gave up the producers may not have waited for these
+    if (elect_one() && issued < pg)
+      for (uint32_t k = issued > kDsepLoaded ? issued - kDsepLoaded : 0; k < issued; ++k)
+        mbar_wait_bounded(&S.loaded[k % kDsepLoaded], (k / kDsepLoaded) & 1);
   }
 
   // ---------------------------------------------------------------- issuer (one warp)
@@ -300,8 +307,9 @@ struct Dsep {
           tc_fence_after();
           __syncwarp();
           if (elect_one()) {
-            sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block, group,
-                        level, jc == 0);
+            if (!sep_failed(&S.fail))
+              sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block,
+                          group, level, jc == 0);
             sep_commit(&S.empty[slot]);
             if (jc + 1 == kPieces) sep_commit(&S.full[dg & 1]);
           }
@@ -485,6 +493,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
       mbar_init(&S.filled[k], 4);
     }
     for (int k = 0; k < kDsepLoaded; ++k) mbar_init(&S.loaded[k], 1);
+    mbar_init(&S.drain, 1);
     for (int k = 0; k < 2; ++k) {
       mbar_init(&S.full[k], 1);
       mbar_init(&S.drained[k], 4);
@@ -514,16 +523,8 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
     else
       it.preparer();
   }
-  // after a wait that gave up: one more bounded wait for copies and MMAs that may still run before their memory goes
-  tc_fence_before();
-  __syncthreads();
+  sep_drain(&S.fail, uniform_warp() == kDsepIssuer / 32, &S.drain);
   if (threadIdx.x < 32) {
-    if (*reinterpret_cast<volatile int*>(&S.fail) && threadIdx.x == 0) {
-      for (int k = 0; k < kDsepLoaded; ++k) mbar_wait_bounded(&S.loaded[k], 0, kWaitLimitNs / 32);
-      sep_commit(&S.full[0]);
-      mbar_wait_bounded(&S.full[0], 0);
-    }
-    __syncwarp();
     tc_fence_after();
     tmem_free(S.tmem, kDsepTmemCols);
   }

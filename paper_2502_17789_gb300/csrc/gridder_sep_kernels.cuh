@@ -72,6 +72,7 @@ struct GsepShared {
   uint64_t empty[4];         // chunk read by its MMAs
   uint64_t full[2];          // accumulator complete
   uint64_t drained[2];       // accumulator read by the 8 consumer warps
+  uint64_t drain;            // every MMA complete, after a wait that gave up
   uint32_t tmem;
   int fail;
 };
@@ -205,7 +206,7 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share,
           n_in = gsep_part(left);
         }
         if (cg + 1 >= uint32_t(C::kRing))
-          sep_wait(&S.empty[(cg + 1) % C::kRing], ((cg + 1) / C::kRing - 1) & 1, &S.fail, a.status);
+          sep_wait(&S.empty[(cg + 1) % C::kRing], ((cg + 1) / C::kRing - 1) & 1, &S.fail, a);
       }
       if (C::kAsyncRecord) cp_async_wait<0>();
       tmem_wait_st();
@@ -216,9 +217,10 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share,
         const int part = S.part[cg & 1];
         if (elect_one()) {
           // the accumulator's previous segment (two back) has been read
-          if ((part & 1) && sc >= 2) sep_wait(&S.drained[sc & 1], ((sc >> 1) - 1) & 1, &S.fail, a.status);
+          if ((part & 1) && sc >= 2) sep_wait(&S.drained[sc & 1], ((sc >> 1) - 1) & 1, &S.fail, a);
           tc_fence_after();
-          sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, part & 1);
+          if (!sep_failed(&S.fail))
+            sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, part & 1);
           sep_commit(&S.empty[slot]);
           if (part & 2) sep_commit(&S.full[sc & 1]);
         }
@@ -281,7 +283,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
     for (bool more = true; more; ++sc) {
       const bool diag = diag_next != 0;
       const float inv = inv_next;
-      if (poller) sep_wait<100>(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a.status);
+      if (poller) sep_wait<100>(&S.full[sc & 1], (sc >> 1) & 1, &S.fail, a);
       half_sync(kSepConsumerBar);  // the segment's sums complete; S.x and the other samples free
       tc_fence_after();
       more = s < sd.seg_count;
@@ -466,6 +468,7 @@ __device__ __forceinline__ void gridder_sep_block(const GridArgs& a, SepShare sh
   GsepShared<L>& S = *reinterpret_cast<GsepShared<L>*>(smem);
   if (threadIdx.x == 0) {
     for (int k = 0; k < C::kRing; ++k) mbar_init(&S.empty[k], 1);
+    mbar_init(&S.drain, 1);
     for (int k = 0; k < 2; ++k) {
       mbar_init(&S.full[k], 1);
       mbar_init(&S.drained[k], kSepHalf / 32);
@@ -484,15 +487,8 @@ __device__ __forceinline__ void gridder_sep_block(const GridArgs& a, SepShare sh
     regs_take<C::kConsumerRegs>();
     gsep_consumer<L>(a, share, S, reinterpret_cast<float4*>(&S + 1));
   }
-  // after a wait that gave up: one more bounded wait for MMAs that may still run before their memory goes
-  tc_fence_before();
-  __syncthreads();
+  sep_drain(&S.fail, uniform_warp() == kSepHalf / 32 - 1, &S.drain);
   if (threadIdx.x < 32) {
-    if (*reinterpret_cast<volatile int*>(&S.fail) && threadIdx.x == 0) {
-      sep_commit(&S.full[0]);
-      mbar_wait_bounded(&S.full[0], 0);
-    }
-    __syncwarp();
     tc_fence_after();
     tmem_free(S.tmem, C::kTmemCols);
   }

@@ -85,6 +85,7 @@ struct idg_plan {
   float2* d_scratch = nullptr;
   float4* d_records = nullptr;  // staged visibility records of one batch
   int* d_status = nullptr;      // kernel status word (timeouts)
+  uint64_t wait_ns = kWaitLimitNs;  // limit of a device-side wait of the separable-phasor kernels
   int* d_queue = nullptr;       // work-queue counters, 2 per batch (gridder, degridder)
   uint8_t* d_adiag = nullptr;   // [n_int][n_st] diagonal-A-term flags of the current call
   float* d_sep = nullptr;       // [4][L] separable-phasor tables a, b, p, q
@@ -789,6 +790,7 @@ static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, co
   ga.aweights = p->d_aweights;
   ga.vc = p->grid_chunk;
   if (p->grid_sep) {
+    ga.wait_ns = p->wait_ns;
     ga.w_ref = p->d_wref + b.sg_offset;
     ga.sep = sep_tables(p);
   }
@@ -888,6 +890,7 @@ static DegridArgs degrid_args(const idg_plan* p, const Batch& b, const void* ate
   da.g = kgeom(p);
   if (p->degrid_sep) {
     da.status = p->d_status;
+    da.wait_ns = p->wait_ns;
     da.amax = p->d_amax;
     da.ymax = p->d_ymax;
     da.w_ref = p->d_wref + b.sg_offset;
@@ -1387,6 +1390,20 @@ idg_status idg_synchronize(idg_plan* plan) {
     if (!e) e = int(cudaStreamSynchronize(plan->stream));
     if (e) return cuda_err(plan, e, "idg_synchronize");
     return set_err(plan, IDG_ERR_TIMEOUT, "a kernel gave up waiting for a bulk copy (bounded wait expired)");
+  }
+  return IDG_OK;
+}
+
+idg_status idg_set_wait_limit(idg_plan* plan, int64_t limit_ns) {
+  if (!plan) return set_err(nullptr, IDG_ERR_INVALID_ARG, "plan is NULL");
+  if (plan->host_only) return set_err(plan, IDG_ERR_INVALID_ARG, "plan was created with IDG_HOST_ONLY");
+  if (limit_ns < 0 || uint64_t(limit_ns) > kWaitLimitNs)
+    return set_err(plan, IDG_ERR_INVALID_ARG, "limit_ns must be in [0, 2e9]");
+  plan->wait_ns = uint64_t(limit_ns);
+  // captured calls hold the limit they were captured with
+  for (idg_plan::GraphCache* gc : {&plan->graph_grid, &plan->graph_degrid}) {
+    if (gc->exec) cudaGraphExecDestroy(gc->exec);
+    *gc = {};
   }
   return IDG_OK;
 }

@@ -242,6 +242,7 @@ struct GridArgs {
   const float* w_ref = nullptr;  // [batch subgrids] reference w (separable-phasor gridder)
   SepTables sep;
   int run = 1, stride = 1;    // a block's items (SepShare); stride: one launch over several plans
+  uint64_t wait_ns = 0;       // limit of one wait of the separable-phasor gridder
   KernelGeom g;
 };
 
@@ -266,6 +267,7 @@ struct DegridArgs {
   const float* w_ref = nullptr;   // [batch subgrids] reference w
   int kv = 0;                     // visibilities per item
   int run = 1, stride = 1;        // a block's items (SepShare); stride: one launch over several plans
+  uint64_t wait_ns = 0;           // limit of one wait
   SepTables sep;
   KernelGeom g;
 };
@@ -284,6 +286,9 @@ struct FftArgs {
   const float* taper = nullptr;
   const float2* n1 = nullptr;
 };
+
+// how long a device-side wait lasts before the kernel reports a timeout (idg_set_wait_limit)
+constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 // Launchers (return cudaError_t as int).  `n` is the item or subgrid count.
 // persistent_blocks > 0: persistent launch of that many blocks draining a.queue

@@ -240,7 +240,6 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 // Wait for phase `parity` of `bar` to complete; gives up after `limit_ns`
 // nanoseconds (returns false) so a lost transaction cannot hang the GPU.
-constexpr uint64_t kWaitLimitNs = 2000000000ull;
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_ns();

@@ -127,23 +127,51 @@ cudaError_t sep_check_regs(K kernel, int regs) {
   return e != cudaSuccess ? e : at.numRegs == regs ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-// bounded wait that reports a timeout once and then lets every later wait of the block pass.  It sleeps between
-// polls, SLEEP ns where the wait is expected to be long: polling takes issue slots from the working warps (with 40 ns
-// throughout, a quarter of the degridder's instructions were polls).
-template <int SLEEP = 32>
-__device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, int* status) {
+// one lane of the (converged) warp: code under it may use the uniform datapath that MMA operands come from
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
+}
+// whether a wait of the block has given up
+__device__ __forceinline__ bool sep_failed(const int* fail) { return *reinterpret_cast<const volatile int*>(fail) != 0; }
+
+// bounded wait (a.wait_ns) that reports a timeout once and then lets every later wait of the block pass; from then on
+// the barriers say nothing about the data behind them, so MMAs and bulk copies are no longer started (sep_failed).  It
+// sleeps between polls, SLEEP ns where the wait is expected to be long: polling takes issue slots from the working
+// warps (with 40 ns throughout, a quarter of the degridder's instructions were polls).
+template <int SLEEP = 32, typename Args>
+__device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, const Args& a) {
   if (mbar_try_wait(bar, parity)) return;
-  if (*reinterpret_cast<volatile int*>(fail)) return;
+  if (sep_failed(fail)) return;
   const uint64_t t0 = global_ns();
-  do {
+  while (global_ns() - t0 < a.wait_ns) {
 #pragma unroll 1
     for (int k = 0; k < 64; ++k) {
       __nanosleep(SLEEP);
       if (mbar_try_wait(bar, parity)) return;
     }
-  } while (global_ns() - t0 <= kWaitLimitNs);
-  atomicOr(status, kStatusTimeout);
+  }
+  atomicOr(a.status, kStatusTimeout);
   *reinterpret_cast<volatile int*>(fail) = 1;
+}
+
+// The block's end, after every role's last wait: where a wait gave up, MMAs may still run.  The lane that issued them
+// (elect.sync picks the same lane of a full warp each time; a commit tracks the MMAs of its own thread) waits for them,
+// bounded, on a barrier that nothing else uses, before the tensor memory goes.
+__device__ __forceinline__ void sep_drain(const int* fail, bool issuer_warp, uint64_t* drain) {
+  tc_fence_before();
+  __syncthreads();
+  if (sep_failed(fail)) {  // the same for the whole block: no wait is left that could set it
+    if (issuer_warp) {
+      if (elect_one()) {
+        sep_commit(drain);
+        mbar_wait_bounded(drain, 0);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  }
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -161,12 +189,6 @@ struct c2 {
   float2 re, im;
 };
 
-// one lane of the (converged) warp: code under it may use the uniform datapath that MMA operands come from
-__device__ __forceinline__ bool elect_one() {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
-  return ok != 0;
-}
 // the thread's warp as a value the compiler knows to be the same for the whole warp, so that a role taken by one
 // warp is a branch for the others and not predicated through
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, int(threadIdx.x) >> 5, 0); }

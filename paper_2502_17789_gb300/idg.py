@@ -28,7 +28,7 @@ IDG_MAC_DEFAULT, IDG_MAC_FP32, IDG_MAC_TENSOR, IDG_MAC_TENSOR_DEGRID = 0, 1, 2, 
 # every function declared in include/idg.h
 EXPORTS = ["idg_plan_create", "idg_grid", "idg_degrid", "idg_grid_graph", "idg_degrid_graph", "idg_set_stream", "idg_plan_stats", "idg_plan_subgrids",
            "idg_plan_segments", "idg_plan_layers", "idg_subgrid_images", "idg_synchronize", "idg_profile_enable", "idg_profile_read",
-           "idg_grid_noalloc", "idg_invert", "idg_predict", "idg_wait_selftest", "idg_aterm_weights", "idg_last_error",
+           "idg_grid_noalloc", "idg_invert", "idg_predict", "idg_wait_selftest", "idg_set_wait_limit", "idg_aterm_weights", "idg_last_error",
            "idg_plan_destroy", "idg_abi_version", "idg_peak_rates", "idg_grid_many", "idg_degrid_many"]
 KERNEL_CLASSES = ["gridder", "fft_adder", "splitter_ifft", "degridder", "stage", "aterm_flags"]
 
@@ -90,6 +90,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.idg_synchronize.argtypes = [P]
     lib.idg_grid_noalloc.argtypes = [P, P, P, P]
     lib.idg_wait_selftest.argtypes = [P, ctypes.c_int32]
+    lib.idg_set_wait_limit.argtypes = [P, i64]
     lib.idg_aterm_weights.argtypes = [P, P, i32]
     lib.idg_invert.argtypes = [P, P, P, P, P]
     lib.idg_predict.argtypes = [P, P, P, P, P]
@@ -159,6 +160,10 @@ def idg_predict(plan, image_ptr, aterms_ptr, grid_ptr, vis_ptr):
 
 def idg_wait_selftest(plan, limit_us: int):
     _check(load().idg_wait_selftest(plan, int(limit_us)), "idg_wait_selftest", plan)
+
+
+def idg_set_wait_limit(plan, limit_ns: int):
+    _check(load().idg_set_wait_limit(plan, int(limit_ns)), "idg_set_wait_limit", plan)
 
 
 def idg_degrid(plan, grid_ptr, aterms_ptr, vis_ptr):
@@ -388,6 +393,9 @@ class Plan:
 
     def wait_selftest(self, limit_us: int = 20000):
         idg_wait_selftest(self.handle, limit_us)
+
+    def set_wait_limit(self, limit_ns: int):
+        idg_set_wait_limit(self.handle, limit_ns)
 
     def profile(self, on: bool = True):
         idg_profile_enable(self.handle, on)
