@@ -667,7 +667,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   if (!e) e = configure_degridder(L, g->aterm_nodes, p->degrid_channels, &pd);
   if (!e && p->mac != IDG_MAC_FP32 && !p->degrid_sep) e = configure_degridder_tc(L, g->aterm_nodes, &pd);
   if (!e && p->degrid_sep) e = configure_degridder_sep(L, &pd);
-  if (!e && (p->grid_sep || p->degrid_sep)) {
+  if (!e) {  // for every plan: the first of several in one launch sizes it for all
     int dev = 0;
     e = int(cudaGetDevice(&dev));
     if (!e) e = int(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev));
