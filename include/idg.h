@@ -79,6 +79,13 @@ enum {
   IDG_MAC_TENSOR_DEGRID = 3  /* degridder on the tensor cores, gridder on the FP32 pipe */
 };
 
+/* Kernels of a plan (idg_plan_kernels) */
+enum {
+  IDG_KERNEL_FP32 = 1,      /* FP32 FMA pipe, a phasor per visibility and pixel */
+  IDG_KERNEL_TENSOR = 2,    /* tensor cores, a phasor per visibility and pixel */
+  IDG_KERNEL_FACTORED = 3   /* tensor cores, factored phasors */
+};
+
 enum {
   IDG_DROP_OUT_OF_GRID = 1,         /* drop subgrids that leave the grid instead of failing */
   IDG_SPLIT_AT_ATERM_INTERVALS = 2, /* never let a subgrid span two A-term intervals (Section 3.3 as written) */
@@ -220,6 +227,12 @@ idg_status idg_set_stream(idg_plan* plan, void* cuda_stream);
 
 /* Plan statistics (host only, no device work). */
 idg_status idg_plan_stats(const idg_plan* plan, idg_plan_stats_t* out);
+
+/*
+ * idg_plan_kernels -- the kernels the plan's gridding and degridding run on,
+ * IDG_KERNEL_FP32, IDG_KERNEL_TENSOR or IDG_KERNEL_FACTORED each.
+ */
+idg_status idg_plan_kernels(const idg_plan* plan, int32_t* gridder, int32_t* degridder);
 
 /*
  * idg_plan_subgrids -- copy the partition, in plan order, to host memory.
@@ -409,7 +422,9 @@ idg_status idg_plan_destroy(idg_plan* plan);
  *   n            number of plans, >= 1
  *   plans        [n] device plans, distinct, sharing the subgrid size, the
  *                Stokes-I flag, the A-term normalisation flag, grid_chunk,
- *                degrid_channels and mac_unit (IDG_ERR_INVALID_ARG otherwise)
+ *                degrid_channels and mac_unit (IDG_ERR_INVALID_ARG otherwise):
+ *                the unit in use, or the one used where the phasors are not
+ *                factored; plans of different kernels take a launch each
  *   vis_c64, aterms_c64, grid_c128
  *                [n] device buffers, per plan as for idg_grid / idg_degrid
  *   cuda_stream  the stream every launch of the call goes to (the plans' own

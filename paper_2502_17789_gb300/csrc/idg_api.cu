@@ -52,7 +52,7 @@ struct idg_plan {
   int32_t degrid_channels = 1;       // channels per degridder lane
   int32_t grid_chunk = kDefaultGridChunk;  // staged records per gridder chunk
   int32_t mac = IDG_MAC_FP32;        // multiply-accumulate unit of the degridder
-  bool uniform = true;               // channels uniformly spaced
+  int32_t mac_general = IDG_MAC_FP32;  // the unit without the separable kernels
   bool grid_sep = false;             // separable-phasor gridder (sep_common.cuh)
   bool degrid_sep = false;           // and degridder
   int32_t degrid_vis = 0;            // its visibilities per item
@@ -358,6 +358,13 @@ idg_status check_buffer(idg_plan* p, const void* ptr, const char* name) {
 
 namespace idg {
 
+static int kernel_of_gridder(const idg_plan* p) {
+  return p->grid_sep ? IDG_KERNEL_FACTORED : p->grid_tc ? IDG_KERNEL_TENSOR : IDG_KERNEL_FP32;
+}
+static int kernel_of_degridder(const idg_plan* p) {
+  return p->degrid_sep ? IDG_KERNEL_FACTORED : p->mac != IDG_MAC_FP32 ? IDG_KERNEL_TENSOR : IDG_KERNEL_FP32;
+}
+
 bool plan_device_view(const idg_plan* p, PlanDeviceView* v) {
   if (!p || p->host_only || !v) return false;
   v->g = KernelGeom{p->N, p->L, p->n_t, p->n_ch, p->n_st, p->geom.aterm_nodes, p->geom.image_size,
@@ -515,8 +522,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   // (the FP32 kernels' sums over XX and YY alone, with diagonal A-terms, do half the multiply-adds of the four
   // correlations: an 80-station predict-and-grid cycle takes 10.8 ms on them, and 3.9 ms on the separable kernels,
   // which sum all four)
-  p->mac = g->mac_unit != IDG_MAC_DEFAULT ? g->mac_unit
-           : (g->degrid_channels > 1 || ((g->flags & IDG_STOKES_I) && !sep_ok)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
+  const auto unit = [&](bool sep) {
+    return g->mac_unit != IDG_MAC_DEFAULT ? g->mac_unit
+           : (g->degrid_channels > 1 || ((g->flags & IDG_STOKES_I) && !sep)) ? IDG_MAC_FP32 : IDG_MAC_TENSOR;
+  };
+  p->mac = unit(sep_ok);
   if (p->mac != IDG_MAC_FP32) p->degrid_channels = 1;  // one visibility per row of the tensor-core product
   {
     // the tensor-core gridder rotates phasors by one channel step along each row
@@ -525,11 +535,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       const double s1 = freqs_hz[1] - freqs_hz[0], sc = freqs_hz[c] - freqs_hz[c - 1];
       uniform = std::fabs(sc - s1) <= 1e-12 * std::fabs(s1);
     }
-    p->uniform = uniform;
+    // the unit in use: both on the tensor cores only where one of their gridders runs
+    const bool tc_ok = uniform && !(g->flags & IDG_NORMALIZE_ATERM);
+    p->mac_general = unit(false) == IDG_MAC_TENSOR && !tc_ok ? IDG_MAC_TENSOR_DEGRID : unit(false);
     p->degrid_sep = p->mac != IDG_MAC_FP32 && sep_ok;
     if (p->degrid_sep) p->degrid_vis = degridder_sep_vis(L, g->aterm_nodes);
     p->grid_sep = p->mac == IDG_MAC_TENSOR && sep_ok && !(g->flags & IDG_NORMALIZE_ATERM);
-    p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && uniform && !(g->flags & IDG_NORMALIZE_ATERM);
+    p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && tc_ok;
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
   }
   p->grid_chunk = g->grid_chunk > 0 ? g->grid_chunk : kDefaultGridChunk;
@@ -1045,9 +1057,12 @@ idg_status idg_degrid_graph(idg_plan* plan, const void* grid_c128, const void* a
 
 namespace {
 
-// The plans of one grid_many / degrid_many call must share the kernel
-// instantiation: subgrid size, planes per layer, normalisation, degridder
-// channels per lane.
+// The plans of one grid_many / degrid_many call must share subgrid size,
+// planes per layer, normalisation, degridder channels per lane and the
+// multiply-accumulate unit: the one in use, or the one that is used where the
+// separable form does not hold.  Whether it holds follows from the uvw data, and
+// neither a plan's neighbours nor the caller should have to know: plans of the
+// separable kernels and of the general ones run side by side, a launch each.
 idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, const void* const* b,
                       void* const* c, const char* an, const char* bn, const char* cn) {
   if (n < 1 || !plans || !a || !b || !c) return set_err(nullptr, IDG_ERR_INVALID_ARG, "NULL array or n < 1");
@@ -1060,15 +1075,22 @@ idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, c
       return st;
     const idg_plan* p0 = plans[0];
     if (p->L != p0->L || p->npol != p0->npol || (p->d_aweights != nullptr) != (p0->d_aweights != nullptr) ||
-        p->degrid_channels != p0->degrid_channels || p->grid_chunk != p0->grid_chunk || p->mac != p0->mac ||
-        (p->mac == IDG_MAC_TENSOR && p->uniform != p0->uniform))
+        p->degrid_channels != p0->degrid_channels || p->grid_chunk != p0->grid_chunk ||
+        (p->mac != p0->mac && p->mac_general != p0->mac_general))
       return set_err(p, IDG_ERR_INVALID_ARG,
                      "plans of one call must share subgrid size, Stokes-I mode, normalisation, grid_chunk, "
-                     "degrid_channels, mac_unit and the gridder kind");
+                     "degrid_channels and mac_unit");
     for (int32_t j = 0; j < k; ++j)
       if (plans[j] == p) return set_err(p, IDG_ERR_INVALID_ARG, "a plan appears twice");
   }
   return IDG_OK;
+}
+
+// The counts of the slots whose kernel is `kind`, 0 for the others
+std::vector<int32_t> of_kind(const std::vector<int32_t>& count, const std::vector<int>& slot_kind, int kind) {
+  std::vector<int32_t> out(count.size());
+  for (size_t s = 0; s < count.size(); ++s) out[s] = slot_kind[s] == kind ? count[s] : 0;
+  return out;
 }
 
 // Items of several plans' batches merged longest first (each plan's batch is
@@ -1161,23 +1183,24 @@ idg_status idg_grid_many(int32_t n, idg_plan* const* plans, const void* const* v
       count.push_back(b.gi_count);
       slot_plan.push_back(k);
     }
-    // plans with and without the separable form take a launch each, their items in one list
-    std::vector<int32_t> count_sep = count;
-    for (size_t s = 0; s < count.size(); ++s) (plans[slot_plan[s]]->grid_sep ? count : count_sep)[s] = 0;
+    // a launch per kernel that these plans use, their items in one list
+    std::vector<int> kind;
+    for (int32_t k : slot_plan) kind.push_back(kernel_of_gridder(plans[k]));
     std::vector<int32_t> strides;
-    std::vector<int2> items = share_blocks(plans[0], count_sep, &strides);
+    std::vector<int2> items = share_blocks(plans[0], of_kind(count, kind, IDG_KERNEL_FACTORED), &strides);
     for (size_t s = 0; s < args.size(); ++s) args[s].stride = strides[s];
     const size_t n_sep = items.size();
-    for (int2 it : merge_items(cost, count)) items.push_back(it);
+    for (int2 it : merge_items(cost, of_kind(count, kind, IDG_KERNEL_TENSOR))) items.push_back(it);
+    const size_t n_tc = items.size() - n_sep;
+    for (int2 it : merge_items(cost, of_kind(count, kind, IDG_KERNEL_FP32))) items.push_back(it);
     GridArgs* d_args = nullptr;
     int2* d_items = nullptr;
     int e = upload_wave(strm, args, items, &d_args, &d_items);
     if (!e) e = launch_gridder_sep_multi(L, d_args, d_items, int(n_sep), max_nodes, strm);
+    if (!e) e = launch_gridder_tc_multi(L, d_args, d_items + n_sep, int(n_tc), strm);
     if (!e)
-      e = plans[0]->mac == IDG_MAC_TENSOR
-              ? launch_gridder_tc_multi(L, d_args, d_items + n_sep, int(items.size() - n_sep), strm)
-              : launch_gridder_multi(L, d_args, d_items + n_sep, int(items.size() - n_sep),
-                                     plans[0]->d_aweights != nullptr, plans[0]->grid_chunk, strm);
+      e = launch_gridder_multi(L, d_args, d_items + n_sep + n_tc, int(items.size() - n_sep - n_tc),
+                               plans[0]->d_aweights != nullptr, plans[0]->grid_chunk, strm);
     if (d_args) cudaFreeAsync(d_args, strm);
     if (d_items) cudaFreeAsync(d_items, strm);
     if (e) return cuda_err(plans[0], e, "gridder launch (several plans)");
@@ -1219,7 +1242,7 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
     std::vector<DegridArgs> args;
     std::vector<const int32_t*> cost, cost_s;
     std::vector<int32_t> count, count_s;
-    std::vector<char> slot_sep;
+    std::vector<int> kind;
     for (int32_t k = 0; k < n; ++k) {
       idg_plan* p = plans[k];
       if (w >= p->batches.size()) continue;
@@ -1228,33 +1251,32 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
       const int e = launch_splitter_ifft(L, fa, b.sg_count, strm);
       if (e) return cuda_err(p, e, "splitter/ifft launch");
       const DegridArgs da = degrid_args(p, b, aterms_c64[k], vis_c64[k]);
-      slot_sep.push_back(p->degrid_sep);
+      kind.push_back(kernel_of_degridder(p));
       args.push_back(da);
       cost.push_back(p->dcost.data() + b.di_offset);
       count.push_back(b.di_count);
       cost_s.push_back(p->dcost.data() + b.di_offset + b.di_count);
       count_s.push_back(b.ds_count);
     }
-    // items of the plans with the separable form, regular items of the others, then the items of few lanes;
-    // the latter index their plan's item table past the regular ones
-    std::vector<int32_t> count_sep = count, count_r = count;
-    for (size_t s = 0; s < count.size(); ++s) (slot_sep[s] ? count_r : count_sep)[s] = 0;
+    // a launch per kernel that these plans use; then the items of few lanes (the general kernels' plans), which
+    // index their plan's item table past the regular ones
     std::vector<int32_t> strides;
-    std::vector<int2> items = share_blocks(plans[0], count_sep, &strides);
+    std::vector<int2> items = share_blocks(plans[0], of_kind(count, kind, IDG_KERNEL_FACTORED), &strides);
     for (size_t s = 0; s < args.size(); ++s) args[s].stride = strides[s];
     const size_t n_sep = items.size();
-    for (int2 it : merge_items(cost, count_r)) items.push_back(it);
+    for (int2 it : merge_items(cost, of_kind(count, kind, IDG_KERNEL_TENSOR))) items.push_back(it);
+    const size_t n_tc = items.size() - n_sep;
+    for (int2 it : merge_items(cost, of_kind(count, kind, IDG_KERNEL_FP32))) items.push_back(it);
     const size_t n_regular = items.size() - n_sep;
     for (int2 it : merge_items(cost_s, count_s)) items.push_back(make_int2(it.x, count[it.x] + it.y));
     DegridArgs* d_args = nullptr;
     int2* d_items = nullptr;
     int e = upload_wave(strm, args, items, &d_args, &d_items);
     if (!e) e = launch_degridder_sep_multi(L, d_args, d_items, int(n_sep), max_nodes, strm);
+    if (!e) e = launch_degridder_tc_multi(L, d_args, d_items + n_sep, int(n_tc), max_nodes, strm);
     if (!e)
-      e = plans[0]->mac != IDG_MAC_FP32
-              ? launch_degridder_tc_multi(L, d_args, d_items + n_sep, int(n_regular), max_nodes, strm)
-              : launch_degridder_multi(L, plans[0]->degrid_channels, false, d_args, d_items + n_sep, int(n_regular),
-                                       max_nodes, strm);
+      e = launch_degridder_multi(L, plans[0]->degrid_channels, false, d_args, d_items + n_sep + n_tc,
+                                 int(n_regular - n_tc), max_nodes, strm);
     if (!e && items.size() > n_sep + n_regular)
       e = launch_degridder_multi(L, plans[0]->degrid_channels, true, d_args, d_items + n_sep + n_regular,
                                  int(items.size() - n_sep - n_regular), max_nodes, strm);
@@ -1470,6 +1492,13 @@ idg_status idg_plan_stats(const idg_plan* plan, idg_plan_stats_t* out) {
   out->degrid_channels = plan->degrid_channels;
   out->grid_chunk = plan->grid_chunk;
   out->mac_unit = plan->mac;
+  return IDG_OK;
+}
+
+idg_status idg_plan_kernels(const idg_plan* plan, int32_t* gridder, int32_t* degridder) {
+  if (!plan || !gridder || !degridder) return set_err(nullptr, IDG_ERR_INVALID_ARG, "NULL argument");
+  *gridder = kernel_of_gridder(plan);
+  *degridder = kernel_of_degridder(plan);
   return IDG_OK;
 }
 

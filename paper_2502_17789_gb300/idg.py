@@ -23,11 +23,12 @@ STATUS_NAMES = {0: "IDG_OK", 1: "IDG_ERR_INVALID_ARG", 2: "IDG_ERR_UNSORTED_FREQ
 IDG_TAPER_KB, IDG_TAPER_USER = 0, 1
 IDG_DROP_OUT_OF_GRID, IDG_SPLIT_AT_ATERM_INTERVALS, IDG_HOST_ONLY, IDG_PERSISTENT, IDG_W_LAYERS = 1, 2, 4, 8, 16
 IDG_NORMALIZE_ATERM, IDG_STOKES_I = 32, 64
+IDG_KERNEL_FP32, IDG_KERNEL_TENSOR, IDG_KERNEL_FACTORED = 1, 2, 3
 IDG_MAC_DEFAULT, IDG_MAC_FP32, IDG_MAC_TENSOR, IDG_MAC_TENSOR_DEGRID = 0, 1, 2, 3
 
 # every function declared in include/idg.h
 EXPORTS = ["idg_plan_create", "idg_grid", "idg_degrid", "idg_grid_graph", "idg_degrid_graph", "idg_set_stream", "idg_plan_stats", "idg_plan_subgrids",
-           "idg_plan_segments", "idg_plan_layers", "idg_subgrid_images", "idg_synchronize", "idg_profile_enable", "idg_profile_read",
+           "idg_plan_segments", "idg_plan_layers", "idg_plan_kernels", "idg_subgrid_images", "idg_synchronize", "idg_profile_enable", "idg_profile_read",
            "idg_grid_noalloc", "idg_invert", "idg_predict", "idg_wait_selftest", "idg_set_wait_limit", "idg_aterm_weights", "idg_last_error",
            "idg_plan_destroy", "idg_abi_version", "idg_peak_rates", "idg_grid_many", "idg_degrid_many"]
 KERNEL_CLASSES = ["gridder", "fft_adder", "splitter_ifft", "degridder", "stage", "aterm_flags"]
@@ -86,6 +87,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.idg_plan_subgrids.argtypes = [P, P, i64, ctypes.POINTER(i64)]
     lib.idg_plan_segments.argtypes = [P, P, i64, ctypes.POINTER(i64)]
     lib.idg_plan_layers.argtypes = [P, P, i64, ctypes.POINTER(i64)]
+    lib.idg_plan_kernels.argtypes = [P, ctypes.POINTER(i32), ctypes.POINTER(i32)]
     lib.idg_subgrid_images.argtypes = [P, P, P, i32, P]
     lib.idg_synchronize.argtypes = [P]
     lib.idg_grid_noalloc.argtypes = [P, P, P, P]
@@ -206,6 +208,13 @@ def idg_plan_layers(plan) -> np.ndarray:
     out = np.zeros((max(n.value, 1), 2), np.int32)
     _check(lib.idg_plan_layers(plan, _np_ptr(out), n.value, ctypes.byref(n)), "idg_plan_layers", plan)
     return out[: n.value]
+
+
+def idg_plan_kernels(plan) -> tuple[int, int]:
+    """(gridder, degridder) of the plan: IDG_KERNEL_FP32, IDG_KERNEL_TENSOR or IDG_KERNEL_FACTORED."""
+    g, d = ctypes.c_int32(0), ctypes.c_int32(0)
+    _check(load().idg_plan_kernels(plan, ctypes.byref(g), ctypes.byref(d)), "idg_plan_kernels", plan)
+    return int(g.value), int(d.value)
 
 
 def idg_plan_segments(plan) -> np.ndarray:
@@ -414,6 +423,9 @@ class Plan:
 
     def layers(self) -> np.ndarray:
         return idg_plan_layers(self.handle)
+
+    def kernels(self) -> tuple[int, int]:
+        return idg_plan_kernels(self.handle)
 
     def grid_shape(self) -> tuple:
         """Shape of the master grid this plan grids into: [n_w_layers, n_pol, N, N],

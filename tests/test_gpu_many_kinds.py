@@ -61,3 +61,76 @@ def test_order_of_plans_does_not_size_the_launch(idg_mod, cuda_device):
     finally:
         for p in plans:
             p.close()
+
+
+def _same_as_alone(idg_mod, plans, obs_list, stokes_i=False):
+    import torch
+    A, V, G = _inputs(plans, obs_list)
+    idg_mod.grid_many(plans, V, A, G)
+    outs = [torch.full_like(v, 7.0 + 7.0j) for v in V]
+    idg_mod.degrid_many(plans, G, A, outs)
+    torch.cuda.synchronize()
+    for p, v, a, g, o in zip(plans, V, A, G, outs):
+        ref, out = torch.zeros_like(g), torch.full_like(v, 7.0 + 7.0j)
+        p.grid(v, a, ref)
+        p.degrid(g, a, out)
+        p.synchronize()
+        # the same kernels: only the order of FP64 and of shared-memory additions differs
+        assert float(torch.linalg.vector_norm(g - ref) / torch.linalg.vector_norm(ref)) < 1e-12
+        assert float((o - out).abs().max() / out.abs().max()) < 1e-6
+
+
+FACTORED, GENERAL = dict(), dict(fov=0.8, heights=300.0)
+
+
+@pytest.mark.parametrize("order", [(0, 1, 0), (1, 0, 1)])
+@pytest.mark.parametrize("L", [32, 64, 96, 128])
+@pytest.mark.parametrize("kind", ["tensor", "stokes", "irregular"])
+def test_plans_of_one_geometry_share_a_call(idg_mod, cuda_device, L, kind, order):
+    """Plans inside and outside the bound of the factored phasors, in both orders: four correlations (the tensor-core
+    kernels beside the factored ones), Stokes I (the FP32 kernels) and irregularly spaced channels (the FP32 gridder
+    and the tensor-core degridder)."""
+    F, T, P = idg_mod.IDG_KERNEL_FACTORED, idg_mod.IDG_KERNEL_TENSOR, idg_mod.IDG_KERNEL_FP32
+    general = {"tensor": (T, T), "stokes": (P, P), "irregular": (P, T)}[kind]
+    obs_list, plans = [], []
+    try:
+        for s, k in enumerate(order):
+            obs = _obs(L=L, seed=5 + s, n_ch=7 + s, N=4096, **(GENERAL if k else FACTORED))
+            if L == 32:
+                obs.kernel_padding = 12
+            if kind == "irregular":
+                obs.freqs = obs.freqs + np.linspace(0.0, 1.0, obs.n_channels) ** 2 * 2e5
+            obs_list.append(obs)
+            plans.append(idg_mod.Plan(obs, flags=idg_mod.IDG_W_LAYERS | (idg_mod.IDG_STOKES_I if kind == "stokes" else 0)))
+            assert plans[-1].kernels() == (general if k else (F, F))
+        _same_as_alone(idg_mod, plans, obs_list)
+    finally:
+        for p in plans:
+            p.close()
+
+
+def test_uniform_and_irregular_channels_share_a_call(idg_mod, cuda_device):
+    """Both run the factored kernels and report one unit."""
+    obs_list = [_obs(seed=9), _obs(seed=10)]
+    obs_list[1].freqs = obs_list[1].freqs + np.linspace(0.0, 1.0, obs_list[1].n_channels) ** 2 * 2e5
+    plans = [idg_mod.Plan(o) for o in obs_list]
+    try:
+        assert plans[0].kernels() == plans[1].kernels() and plans[0].stats().mac_unit == plans[1].stats().mac_unit
+        _same_as_alone(idg_mod, plans, obs_list)
+    finally:
+        for p in plans:
+            p.close()
+
+
+def test_other_units_are_still_refused(idg_mod, cuda_device):
+    obs = _obs(seed=9)
+    plans = [idg_mod.Plan(obs, mac_unit=m) for m in (idg_mod.IDG_MAC_TENSOR, idg_mod.IDG_MAC_FP32)]
+    try:
+        A, V, G = _inputs(plans, [obs, obs])
+        for call, args in ((idg_mod.grid_many, (plans, V, A, G)), (idg_mod.degrid_many, (plans, G, A, V))):
+            with pytest.raises(idg_mod.IdgError) as e:
+                call(*args)
+            assert e.value.status == 1
+    finally:
+        for p in plans:
+            p.close()
