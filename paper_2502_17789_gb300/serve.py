@@ -82,6 +82,32 @@ class Result:
         return self.finished - self.arrival
 
 
+def record_bytes(obs: synth.Observation) -> int:
+    """Upper bound of the staged records of a plan: 128 bytes a visibility, or
+    with factored phasors 768 bytes per started chunk of 16 visibilities of a
+    segment (a subgrid's part in one A-term interval).
+
+    Segments are bounded per baseline from the partition's rules: the channels
+    of a timestep are cut into runs that leave Sc = 3/4 S pixels along u or v
+    with the next channel, so two neighbouring runs together pass Sc on one
+    axis; a run's timesteps are cut where they leave S, so each cut takes a
+    move of at least S - Sc, and every A-term interval starts a segment."""
+    if obs.n_vis == 0:
+        return 0
+    S = max(1, obs.subgrid_size - obs.kernel_padding - 4)
+    margin = max(2, S // 4)
+    Sc = max(1, S - margin)
+    px = obs.uvw[:, :, :2] * (obs.image_size / 299792458.0)          # pixels per hertz
+    band = float(obs.freqs[-1] - obs.freqs[0])
+    span = np.abs(px).max(1) * band                                  # [bl, axis]
+    runs = np.minimum(1 + np.ceil(2 * span / Sc).sum(-1), obs.n_channels)
+    path = np.abs(np.diff(px, axis=1)).sum(1) * float(obs.freqs[-1])  # [bl, axis]
+    cuts = np.minimum(obs.n_intervals + np.ceil(path / margin).sum(-1), obs.n_timesteps)
+    segments = float((runs * cuts).sum())
+    chunks = min(float(obs.n_vis), obs.n_vis / 16 + segments)
+    return int(max(128 * obs.n_vis, 768 * chunks))
+
+
 def footprint_bytes(req: Request) -> int:
     """Device memory a request holds while resident: its input and output
     arrays, the plan's subgrid scratch (bounded by the 1 GiB batch budget),
@@ -92,7 +118,7 @@ def footprint_bytes(req: Request) -> int:
     per_sg = 4 * o.subgrid_size ** 2 * 8
     # subgrids <= visibilities; the plan's scratch holds at most 1 GiB of images
     scratch = min(1 << 30, max(1, o.n_vis) * per_sg)
-    records = o.n_vis * 128
+    records = record_bytes(o)
     tables = o.uvw.nbytes + (64 << 20)
     return int(vis + grid + scratch + records + tables + req.aterms.nbytes)
 
