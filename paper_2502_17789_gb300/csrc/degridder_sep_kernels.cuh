@@ -68,7 +68,7 @@ struct alignas(128) DsepShared {
   // the producers' part of an item, by item parity
   struct Info {
     float scale;   // of Z, a power of two
-    int sg, n_pad, diag;
+    int sg, diag;
   } info[2];
   uint64_t ready[2];        // item prepared (2 preparing warps)
   uint64_t loaded[kDsepLoaded];  // Y piece copied, by piece modulo kDsepLoaded
@@ -261,7 +261,7 @@ struct Dsep {
   // Y in scratch: [pol][column block][row pair][re, im][32 columns], so a piece is one run of 4 KB per plane
   __device__ __forceinline__ void loader() {
     uint32_t n = 0, pg = 0;  // items and pieces of this block so far
-    uint32_t issued = 0;     // pieces the elected lane has started to copy: all, unless a wait gave up
+    uint32_t issued = 0;     // pieces the elected lane has started to copy
     for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
       wait<64>(&S.ready[n & 1], (n >> 1) & 1);
       const float2* Y = a.scratch + size_t(S.info[n & 1].sg) * 4 * L * L;
@@ -271,6 +271,7 @@ struct Dsep {
         // the slot's previous piece of Y has been read and its Z multiplied: one wait less for every producer
         if (turn > 0) wait(&S.empty[slot], (turn - 1) & 1);
         __syncwarp();
+        // none after a wait that gave up: the subgrid, and the barrier's phase, may then be anything
         if (elect_one() && !sep_failed(&S.fail)) {
           mbar_arrive_expect_tx(&S.loaded[pg % kDsepLoaded], 4096 * a.g.npol);
           for (int pol = 0; pol < a.g.npol; ++pol)
@@ -280,8 +281,8 @@ struct Dsep {
         __syncwarp();
       }
     }
-    // after a wait that gave up the producers may not have waited for these
-    if (elect_one() && issued < pg)
+    // the producers wait for every piece, but not once a wait of theirs has given up
+    if (elect_one())
       for (uint32_t k = issued > kDsepLoaded ? issued - kDsepLoaded : 0; k < issued; ++k)
         mbar_wait_bounded(&S.loaded[k % kDsepLoaded], (k / kDsepLoaded) & 1);
   }
@@ -291,9 +292,16 @@ struct Dsep {
   __device__ __forceinline__ void issuer() {
     const uint32_t tm = S.tmem;
     uint32_t n = 0, pg = 0, dg = 0;  // items, pieces and accumulators of this block so far
+    // columns of an item: from the item itself, a step ahead, so that the MMAs' shapes and operands are the block's own
+    // also after a wait that gave up (their sums are lost then, and sep_drain waits for them)
+    const auto columns = [&](int idx) {
+      return idx < share.last ? (a.items[idx].k_end - a.items[idx].k_begin + 15) & ~15 : 16;
+    };
+    int n_next = columns(share.first);
     for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n) {
+      const int n_pad = n_next;
+      n_next = columns(share.next(idx));
       wait(&S.ready[n & 1], (n >> 1) & 1);
-      const int n_pad = S.info[n & 1].n_pad;
       const uint32_t block = uint32_t(n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
       const uint32_t f0 = smem_u32(fside) + (n & 1) * uint32_t(a.kv) * L * 12;
 #pragma unroll 1
@@ -307,9 +315,8 @@ struct Dsep {
           tc_fence_after();
           __syncwarp();
           if (elect_one()) {
-            if (!sep_failed(&S.fail))
-              sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block,
-                          group, level, jc == 0);
+            sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block, group,
+                        level, jc == 0);
             sep_commit(&S.empty[slot]);
             if (jc + 1 == kPieces) sep_commit(&S.full[dg & 1]);
           }
@@ -344,7 +351,7 @@ struct Dsep {
     // scale of Z from the largest components of Y and of the A-terms' nodes
     float ym = 0.f;
     for (int k = 0; k < a.g.npol; ++k) ym = fmaxf(ym, a.ymax[item.sg * 4 + k]);
-    const DsepShared::Info info = {sep_scale(ym * a.amax[sp] * a.amax[sq]), item.sg, n_pad, a.adiag[sp] & a.adiag[sq]};
+    const DsepShared::Info info = {sep_scale(ym * a.amax[sp] * a.amax[sq]), item.sg, a.adiag[sp] & a.adiag[sq]};
     if (n >= 2) wait<100>(&S.done[b], ((n >> 1) - 1) & 1);  // the buffers' previous item (two back) is done
     {
       const float4* src = reinterpret_cast<const float4*>(a.aterms);

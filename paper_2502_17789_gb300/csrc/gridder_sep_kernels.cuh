@@ -219,8 +219,9 @@ __device__ __forceinline__ void gsep_producer(const GridArgs& a, SepShare share,
           // the accumulator's previous segment (two back) has been read
           if ((part & 1) && sc >= 2) sep_wait(&S.drained[sc & 1], ((sc >> 1) - 1) & 1, &S.fail, a);
           tc_fence_after();
-          if (!sep_failed(&S.fail))
-            sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, part & 1);
+          // also after a wait that gave up (the sums are lost then, but operands and accumulator are the block's own, and
+          // sep_drain waits): a look at S.fail here costs 2 % at L = 64
+          sep_product(tm + (sc & 1) * C::kColStride, e_col, buf, C::kRows, C::kFBlock, C::kFGroup, C::kFLevel, part & 1);
           sep_commit(&S.empty[slot]);
           if (part & 2) sep_commit(&S.full[sc & 1]);
         }

@@ -137,20 +137,22 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ bool sep_failed(const int* fail) { return *reinterpret_cast<const volatile int*>(fail) != 0; }
 
 // bounded wait (a.wait_ns) that reports a timeout once and then lets every later wait of the block pass; from then on
-// the barriers say nothing about the data behind them, so MMAs and bulk copies are no longer started (sep_failed).  It
-// sleeps between polls, SLEEP ns where the wait is expected to be long: polling takes issue slots from the working
+// the barriers say nothing about the data behind them, so nothing whose addresses come from such data may be started
+// (sep_failed).  It sleeps between polls, SLEEP ns where the wait is expected to be long: polling takes issue slots from the working
 // warps (with 40 ns throughout, a quarter of the degridder's instructions were polls).
 template <int SLEEP = 32, typename Args>
 __device__ __forceinline__ void sep_wait(uint64_t* bar, uint32_t parity, int* fail, const Args& a) {
   if (mbar_try_wait(bar, parity)) return;
   if (sep_failed(fail)) return;
-  const uint64_t t0 = global_ns();
-  while (global_ns() - t0 < a.wait_ns) {
+  if (a.wait_ns) {  // 0: no wait at all
+    const uint64_t t0 = global_ns();
+    do {
 #pragma unroll 1
-    for (int k = 0; k < 64; ++k) {
-      __nanosleep(SLEEP);
-      if (mbar_try_wait(bar, parity)) return;
-    }
+      for (int k = 0; k < 64; ++k) {
+        __nanosleep(SLEEP);
+        if (mbar_try_wait(bar, parity)) return;
+      }
+    } while (global_ns() - t0 <= a.wait_ns);
   }
   atomicOr(a.status, kStatusTimeout);
   *reinterpret_cast<volatile int*>(fail) = 1;
