@@ -91,14 +91,6 @@ def kernel_of(kind: str, mac_unit: int, separable: bool = False) -> str:
     return "degridder" if mac_unit == 1 else "degridder_sep" if separable else "degridder_tc"
 
 
-def separable_plan(stats, L: int) -> bool:
-    """Whether a plan of the tensor cores runs the separable-phasor kernels:
-    their gridder items are L/32 column strips of a subgrid (two halves each
-    for L = 128), the others 512-pixel tiles."""
-    n_sg = int(stats.n_subgrids) - int(stats.n_subgrids_dropped)
-    return int(stats.mac_unit) == 2 and int(stats.n_grid_items) == n_sg * (L // 32) * (2 if L == 128 else 1)
-
-
 def _env_int(name, default):
     try:
         return int(os.environ.get(name, default))
@@ -588,7 +580,7 @@ def run_native(args):
     peak_tflops = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     achieved_vispx = vispx / (k_ms * 1e-3)
     achieved = achieved_vispx * FLOP_PER_VISPX / 1e12
-    separable = separable_plan(st, obs_r.subgrid_size)
+    separable = plan.kernels()[0] == idg.IDG_KERNEL_FACTORED
     kern_name = kernel_of(kern, int(st.mac_unit), separable)
     traffic = recorded_traffic(kern_name, desc)
     roofline = {"bound": "alu", "kernel": kern_name, "achieved": round(achieved, 3), "peak": round(peak_tflops, 3),

@@ -64,12 +64,14 @@ enum { IDG_TAPER_KB = 0, IDG_TAPER_USER = 1 };
 
 /* Units that take the phasor sums' multiply-accumulate (idg_geometry.mac_unit).  On the tensor cores the
    operands are split into hi and lo parts (A_hi B_hi + A_lo B_hi + A_hi B_lo, about FP32 accuracy) and
-   accumulated in FP32.  Where the w term varies little enough over every subgrid (any field up to about 0.5
-   at the default taper), the phasors are factored into one factor per pixel column and one per row
-   and the sums are plain matrix products (f16 parts); elsewhere each visibility and pixel has its own phasor
-   (TF32 parts).  The tensor-core degridder takes one visibility per row (one channel per lane whatever
-   degrid_channels asks); the tensor-core gridder needs no A-term normalisation, and for plans whose phasors
-   are not factored uniformly spaced channels (the plan keeps the FP32 gridder otherwise). */
+   accumulated in FP32.  Where the w term varies little enough over the subgrids, the phasors are factored into
+   one factor per pixel column and one per row and the sums are plain matrix products (f16 parts); what the
+   factored form neglects stays below 3e-7 of a source's flux within |l|, |m| <= FOV/4 (1e-6 within FOV/3), for
+   which subgrids of a wide w range are worked on in parts.  Where that would more than double their number,
+   each visibility and pixel has its own phasor (TF32 parts).  The tensor-core degridder takes one visibility
+   per row (one channel per lane whatever degrid_channels asks); the tensor-core gridder needs no A-term
+   normalisation, and for plans whose phasors are not factored uniformly spaced channels (the plan keeps the
+   FP32 gridder otherwise). */
 enum {
   IDG_MAC_DEFAULT = 0,       /* IDG_MAC_TENSOR (IDG_MAC_TENSOR_DEGRID where the tensor-core gridder cannot
                                 run); IDG_MAC_FP32 when degrid_channels asks for 2 or 4, and with IDG_STOKES_I

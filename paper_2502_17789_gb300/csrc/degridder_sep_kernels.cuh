@@ -3,7 +3,7 @@
 // of the phase; this is the adjoint of gridder_sep_kernels.cuh.
 //
 // For one A-term segment, Z = A_p Y A_q^H with Y the subgrid image times
-// taper, centring sign and e^{-2 pi i w_ref n'} (applied by the splitter):
+// taper, centring sign and e^{-2 pi i w_ref n'} (sep_pixel; applied by the splitter):
 //   V_k = sum_i conj(E_k(i)) D_k(i),
 //   D_k(i) = sum_j Z(i,j) conj(F_k(j)) (1 - 2 pi i delta_k p_i q_j).
 // D is a complex matrix product on the tensor cores: rows (p, i) for 4
@@ -346,7 +346,7 @@ struct Dsep {
       const double fs = subgrid_sign(sd) * a.fscale[ch], inv_l = 1.0 / double(L);
       fa = sep_fix(((r[0] * fs) * a.g.fov - double(sd.x0 + L / 2 - a.g.N / 2)) * inv_l);
       fb = sep_fix(((r[1] * fs) * a.g.fov - double(sd.y0 + L / 2 - a.g.N / 2)) * inv_l);
-      dl = float(r[2] * fs - (double(a.w_ref[item.sg]) + subgrid_w0(a.g, sd)));
+      dl = float(r[2] * fs - (double(a.w_ref[item.sg].x) + subgrid_w0(a.g, sd)));
     }
     // scale of Z from the largest components of Y and of the A-terms' nodes
     float ym = 0.f;

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) s
   }
   // what every visibility of the subgrid shares (sep_common.cuh), once per pixel here instead of once per segment;
   // written as the degridder reads it, [32 columns][row pair][re, im][column] of the values at both rows
-  const float w_ref = a.w_ref[sgi];
+  const float2 w_ref = a.w_ref[sgi];
   float2* pairs = a.scratch + (size_t(sgi) * 4 + pol) * L * L;
   float m = 0.f;
   for (int e = threadIdx.x; e < L * L / 2; e += T) {
@@ -246,8 +246,9 @@ __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) s
     const int ip = fft_place<L>(i);
     const float2 v0 = buf[fft_place<L>(2 * jp) * P + ip], v1 = buf[fft_place<L>(2 * jp + 1) * P + ip];
     const float ti = a.taper[i] * ((i & 1) ? -1.f : 1.f), t0 = ti * a.taper[2 * jp], t1 = -ti * a.taper[2 * jp + 1];
-    const float2 p0 = sep_w_phasor(w_ref, __ldg(a.n1 + 2 * jp * L + i));
-    const float2 p1 = sep_w_phasor(w_ref, __ldg(a.n1 + (2 * jp + 1) * L + i));
+    const float fit_p = __ldg(a.sep.p + i);
+    const float2 p0 = sep_pixel(w_ref, __ldg(a.sep.n1 + 2 * jp * L + i), fit_p * __ldg(a.sep.q + 2 * jp));
+    const float2 p1 = sep_pixel(w_ref, __ldg(a.sep.n1 + (2 * jp + 1) * L + i), fit_p * __ldg(a.sep.q + 2 * jp + 1));
     const float2 re = make_float2(t0 * (v0.x * p0.x + v0.y * p0.y), t1 * (v1.x * p1.x + v1.y * p1.y));
     const float2 im = make_float2(t0 * (v0.y * p0.x - v0.x * p0.y), t1 * (v1.y * p1.x - v1.x * p1.y));
     m = fmaxf(fmaxf(fmaxf(m, fabsf(re.x)), fabsf(re.y)), fmaxf(fabsf(im.x), fabsf(im.y)));
@@ -266,18 +267,24 @@ __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) s
   }
 }
 
-// plan-order export of subgrid images for inspection, undoing (-1)^(x+y)
+// plan-order export of subgrid images for inspection, undoing (-1)^(x+y); parts of a subgrid add up (out starts at 0)
 template <int L>
 __global__ void export_kernel(const SubgridDesc* sg, const float2* scratch, float2* out, int npol) {
   const int sgi = blockIdx.x / npol, pol = blockIdx.x % npol;
   const int dst_sg = sg[sgi].plan_index;
+  const bool part = (sg[sgi].flags & kSubgridPart) != 0;
   const float2* src = scratch + (size_t(sgi) * 4 + pol) * L * L;
   float2* dst = out + (size_t(dst_sg) * npol + pol) * L * L;
   for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
     const int y = e / L, x = e - y * L;
     const float sgn = ((x + y) & 1) ? -1.f : 1.f;
     const float2 v = src[e];
-    dst[e] = make_float2(sgn * v.x, sgn * v.y);
+    if (part) {
+      atomicAdd(&dst[e].x, sgn * v.x);
+      atomicAdd(&dst[e].y, sgn * v.y);
+    } else {
+      dst[e] = make_float2(sgn * v.x, sgn * v.y);
+    }
   }
 }
 

@@ -118,12 +118,12 @@ __global__ void __launch_bounds__(256) stage_records_kernel(const StageArgs a, i
 // segment's scale, a power of two that puts the largest component in [512, 1024) so that hi + lo halves keep 22 bits
 // down to 2^-9 of it.  Bound by latency, not bytes: a pass over a segment's values for the scale, then one that reads
 // them again (from L1 or L2) and writes.
-__global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float* w_ref,
+__global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float2* w_ref,
                                                         int L) {
   const SubgridDesc sd = a.sg[blockIdx.x];
   const int nc = sd.c1 - sd.c0;
   const bool mirror = (sd.flags & kSubgridMirrored) != 0;
-  const double wr = double(w_ref[blockIdx.x]) + subgrid_w0(a.g, sd);
+  const double wr = double(w_ref[blockIdx.x].x) + subgrid_w0(a.g, sd);
   const double inv_l = 1.0 / double(L), sgn = subgrid_sign(sd);
   const double off_x = double(sd.x0 + L / 2 - a.g.N / 2), off_y = double(sd.y0 + L / 2 - a.g.N / 2);
   float4* base = a.records + size_t(sd.rec_offset) * kRecordFloat4;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
   }
 }
 
-int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids,
+int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float2* w_ref, int n_subgrids,
                      void* stream) {
   if (n_subgrids <= 0) return 0;
   stage_sep_kernel<<<n_subgrids, 256, 0, cudaStream_t(stream)>>>(a, seg, w_ref, L);

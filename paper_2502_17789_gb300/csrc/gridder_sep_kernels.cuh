@@ -440,12 +440,13 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
     }
 
     // ---- pixels of the item: w_ref, taper, centring sign; [sg][pol][j][i]; Stokes I: plane 0, (XX + YY) / 2
-    const float w_ref = a.w_ref[item.sg];
+    const float2 w_ref = a.w_ref[item.sg];
+    const float fit_p = a.sep.p[i];
     const float ti = a.taper[i];
 #pragma unroll
     for (int r = 0; r < C::kSpan; ++r) {
       const int j = j0 + r;
-      const float2 ph = sep_w_phasor(w_ref, __ldg(a.sep.n1 + j * L + i));
+      const float2 ph = sep_pixel(w_ref, __ldg(a.sep.n1 + j * L + i), fit_p * a.sep.q[j]);
       const float wgt = ti * a.taper[j] * (((i + j) & 1) ? -1.f : 1.f);
       const cf rot = {wgt * ph.x, wgt * ph.y};
       float2* dst = a.scratch + size_t(item.sg) * 4 * L * L + j * L + i;

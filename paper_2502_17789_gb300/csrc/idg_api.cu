@@ -61,7 +61,8 @@ struct idg_plan {
   cudaStream_t stream = nullptr;
   bool host_only = false;
   Partition part;
-  std::vector<SubgridDesc> exec;  // non-dropped subgrids in execution order
+  std::vector<SubgridDesc> exec;  // non-dropped subgrids (or their parts, sep_parts) in execution order
+  std::vector<SegmentDesc> segs;  // the partition's segments, then those of parts
   std::vector<Batch> batches;
   int32_t batch_cap = 0;
   int64_t n_grid_items = 0, n_degrid_items = 0;
@@ -90,7 +91,7 @@ struct idg_plan {
   uint8_t* d_adiag = nullptr;   // [n_int][n_st] diagonal-A-term flags of the current call
   float* d_sep = nullptr;       // [4][L] separable-phasor tables a, b, p, q
   float2* d_n1 = nullptr;       // [L*L] n' as two floats
-  float* d_wref = nullptr;      // [exec subgrids] reference w
+  float2* d_wref = nullptr;     // [exec subgrids] reference w, a quarter of the largest squared distance from it
   float* d_amax = nullptr;      // [n_int][n_st] largest A-term component of the current call (degrid_sep)
   float* d_ymax = nullptr;      // [batch capacity][4] largest component of the split subgrid planes (degrid_sep)
   double* d_aweights = nullptr; // [L*L + 1] A-term power weights (IDG_NORMALIZE_ATERM)
@@ -262,25 +263,39 @@ std::vector<float4> block_geometry16(int L, double fov) {
 }
 
 // The separable form of n' over the subgrid (sep_common.cuh): n'(i,j) = A_i + B_j
-// + p_i q_j + rest, fitted with the taper as weight (A and B weighted means,
-// p q the leading singular pair of the weighted remainder).  e1 and e2 bound
-// what it neglects: max over pixels of T |rest| and of T |n' - A - B|^2 / 2, T
-// the taper product relative to its maximum.
+// + p_i q_j + rest.  With theta = 2 pi delta p_i q_j, |delta| <= x, the kernels
+// take e^{i theta} as (1 - theta_x^2 / 4)(1 + i theta), theta_x = 2 pi x p_i q_j, so
+// they neglect at most 2 pi x |rest| + theta_x^2 / 4 (a constant factor leaves half
+// of the second-order term at either end).
+//
+// A and B are means and p q the leading pair over the part of the field
+// |l|, |m| <= h FOV, with the density of Chebyshev points: p_i q_j then swings evenly
+// over that part instead of growing with l^2 m^2 from the centre.  Fitted with the
+// taper as weight (0 at the centre), the neglected terms of a source at (FOV/3, FOV/3)
+// were 2e-5 of its flux at the ends of the MWA-like array's w ranges (x = 5.7 at FOV
+// 0.5); an image is divided by the taper, so a source's error counts in units of its
+// own flux, whatever the taper there.  A larger h allows a wider w range (FOV 0.5, L =
+// 96: x up to 1.4, 1.9, 3.0, 3.9, 4.4 over kSepFit; 1/3 less again) for a larger
+// first-order term, and its rounding, at the centre: a plan takes the smallest h that
+// its w ranges need.
+constexpr double kSepFit[] = {0.12, 0.20, 0.28, 0.31, 0.32};
+
 struct SepFit {
   std::vector<float> tab;   // [4][L]: 2 pi A, 2 pi B, 2 pi p, q
   std::vector<float2> n1;   // [j][i]
-  double e1 = 0.0, e2 = 0.0;
+  double x_max = 0.0;       // largest |w - w_ref| (wavelengths) that meets kSepTolerance and kSepTolerancePx
 };
 
-SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
+SepFit sep_fit(int L, double fov, const std::vector<double>& taper, double h) {
   SepFit f;
   std::vector<double> w(L), c(size_t(L) * L), A(L), B(L), p(L), q(L, 1.0);
-  double wmax = 0.0, ww = 0.0;
-  for (int i = 0; i < L; ++i) wmax = std::max(wmax, std::fabs(taper[i]));
-  if (!(wmax > 0.0)) wmax = 1.0;
-  for (int i = 0; i < L; ++i) {
-    w[i] = std::max(std::fabs(taper[i]) / wmax, 1e-8);
-    ww += w[i] * w[i];
+  double tmax = 0.0, ww = 0.0;
+  for (int i = 0; i < L; ++i) tmax = std::max(tmax, std::fabs(taper[i]));
+  if (!(tmax > 0.0)) tmax = 1.0;
+  for (int i = 0; i < L; ++i) {  // squared weights; the end points of the density are cut off at a pixel's width
+    const double x = double(i - L / 2) / (h * L);
+    w[i] = std::fabs(x) <= 1.0 ? 1.0 / std::sqrt(std::max(1.0 - x * x, 1.0 / (h * L))) : 0.0;
+    ww += w[i];
   }
   f.n1.resize(size_t(L) * L);
   for (int j = 0; j < L; ++j)
@@ -291,11 +306,11 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
       f.n1[size_t(j) * L + i] = make_float2(float(n), float(n - double(float(n))));
     }
   for (int i = 0; i < L; ++i) {
-    for (int j = 0; j < L; ++j) A[i] += w[j] * w[j] * c[size_t(j) * L + i];
+    for (int j = 0; j < L; ++j) A[i] += w[j] * c[size_t(j) * L + i];
     A[i] /= ww;
   }
   for (int j = 0; j < L; ++j) {
-    for (int i = 0; i < L; ++i) B[j] += w[i] * w[i] * (c[size_t(j) * L + i] - A[i]);
+    for (int i = 0; i < L; ++i) B[j] += w[i] * (c[size_t(j) * L + i] - A[i]);
     B[j] /= ww;
   }
   for (int j = 0; j < L; ++j)
@@ -304,16 +319,16 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
   for (int j = 0; j < L; ++j) q[j] = B[j] - B[L / 2];
   for (int it = 0; it < 24; ++it) {
     double qq = 0.0, pp = 0.0;
-    for (int j = 0; j < L; ++j) qq += w[j] * w[j] * q[j] * q[j];
+    for (int j = 0; j < L; ++j) qq += w[j] * q[j] * q[j];
     for (int i = 0; i < L; ++i) {
       p[i] = 0.0;
-      for (int j = 0; j < L; ++j) p[i] += w[j] * w[j] * c[size_t(j) * L + i] * q[j];
+      for (int j = 0; j < L; ++j) p[i] += w[j] * c[size_t(j) * L + i] * q[j];
       p[i] = qq > 0.0 ? p[i] / qq : 0.0;
-      pp += w[i] * w[i] * p[i] * p[i];
+      pp += w[i] * p[i] * p[i];
     }
     for (int j = 0; j < L; ++j) {
       q[j] = 0.0;
-      for (int i = 0; i < L; ++i) q[j] += w[i] * w[i] * c[size_t(j) * L + i] * p[i];
+      for (int i = 0; i < L; ++i) q[j] += w[i] * c[size_t(j) * L + i] * p[i];
       q[j] = pp > 0.0 ? q[j] / pp : 0.0;
     }
   }
@@ -323,11 +338,17 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
     q[i] /= qm;
     p[i] *= qm;
   }
+  // the largest x at which every pixel keeps a x + b x^2 within its tolerance
+  f.x_max = 1e300;
   for (int j = 0; j < L; ++j)
     for (int i = 0; i < L; ++i) {
-      const double t = std::fabs(taper[i] * taper[j]) / (wmax * wmax), x = c[size_t(j) * L + i];
-      f.e1 = std::max(f.e1, t * std::fabs(x - p[i] * q[j]));
-      f.e2 = std::max(f.e2, t * 0.5 * x * x);
+      const double t = std::fabs(taper[i] * taper[j]) / (tmax * tmax), pq = p[i] * q[j];
+      const double a = 2.0 * kPi * std::fabs(c[size_t(j) * L + i] - pq), b = kPi * kPi * pq * pq;
+      const double r = double(std::max(std::abs(i - L / 2), std::abs(j - L / 2))) / double(L);
+      double tol = kSepTolerance / std::max(t, 1e-30);
+      if (r <= 1.0 / 3.0) tol = std::min(tol, r <= 0.25 ? kSepTolerance : kSepToleranceOuter);
+      const double x = 2.0 * tol / (a + std::sqrt(a * a + 4.0 * b * tol));
+      if (!(x >= f.x_max)) f.x_max = x;  // NaN too: no range is small enough then
     }
   f.tab.resize(size_t(4) * L);
   for (int i = 0; i < L; ++i) {
@@ -337,6 +358,93 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper) {
     f.tab[3 * L + i] = float(q[i]);
   }
   return f;
+}
+
+// Smallest and largest w - w0 of timesteps [t0, t1) and channels [c0, c1) of a
+// subgrid (channels ascend, so w's extremes are at the end channels)
+struct WRange {
+  double lo, hi;   // of w - w0, wavelengths
+  double t, c;     // spread by the timesteps, by the channels
+};
+WRange w_range(const SubgridDesc& d, int t0, int t1, int c0, int c1, double w_step, int n_t, const double* uvw_m,
+               const double* freqs_hz) {
+  const double sgn = subgrid_sign(d), w0 = (double(d.layer) + 0.5) * w_step;
+  const double* r = uvw_m + size_t(d.b) * n_t * 3 + 2;
+  double lo = sgn * r[size_t(t0) * 3], hi = lo;  // metres
+  for (int t = t0 + 1; t < t1; ++t) {
+    lo = std::min(lo, sgn * r[size_t(t) * 3]);
+    hi = std::max(hi, sgn * r[size_t(t) * 3]);
+  }
+  const double f0 = freqs_hz[c0] / kSpeedOfLight, f1 = freqs_hz[c1 - 1] / kSpeedOfLight;
+  return {std::min(lo * f0, lo * f1) - w0, std::max(hi * f0, hi * f1) - w0, (hi - lo) * f1,
+          std::max(std::fabs(lo), std::fabs(hi)) * (f1 - f0)};
+}
+
+// The subgrids as the separable kernels work on them: one whose w range is
+// wider than 2 x_max is taken in parts of its timesteps or channels, each at
+// the subgrid's place with a reference w of its own and segments appended to
+// `seg` (subgrid images and visibilities add up, so only the order of
+// additions changes).  false when the parts would be more than twice the
+// subgrids (then the general kernels are the better ones), or for a NaN.
+bool sep_parts(const std::vector<SubgridDesc>& in, double x_max, double w_step, int n_t, const double* uvw_m,
+               const double* freqs_hz, const int32_t* aterm_offsets, std::vector<SegmentDesc>* seg,
+               std::vector<SubgridDesc>* out, std::vector<float2>* w_ref) {
+  struct Part {
+    int t0, t1, c0, c1;
+  };
+  std::vector<Part> todo;
+  out->reserve(in.size());
+  for (const SubgridDesc& d : in) {
+    const int seg_begin = d.seg_begin, seg_count = d.seg_count;
+    todo.assign(1, Part{d.t0, d.t1, d.c0, d.c1});
+    while (!todo.empty()) {
+      const Part s = todo.back();
+      todo.pop_back();
+      const WRange w = w_range(d, s.t0, s.t1, s.c0, s.c1, w_step, n_t, uvw_m, freqs_hz);
+      const float mid = float(0.5 * (w.lo + w.hi));
+      const double x = std::max(w.hi - double(mid), double(mid) - w.lo);
+      if (!(x <= x_max)) {
+        // halve what spreads w more; in time at the A-term interval nearest to the middle, if one is near, so that
+        // no segment is cut
+        const bool in_t = s.t1 - s.t0 > 1 && (w.t >= w.c || s.c1 - s.c0 == 1);
+        const int half = (s.t0 + s.t1) / 2, cm = (s.c0 + s.c1) / 2;
+        int tm = half, best = (s.t1 - s.t0) / 4 + 1;
+        for (int k = seg_begin; k < seg_begin + seg_count; ++k) {
+          const int a = aterm_offsets[(*seg)[k].interval];
+          if (std::abs(a - half) < best && a > s.t0 && a < s.t1) {
+            best = std::abs(a - half);
+            tm = a;
+          }
+        }
+        if (!in_t && s.c1 - s.c0 == 1) return false;  // a single visibility: NaN
+        if (out->size() + todo.size() + 2 > 2 * in.size() + 2) return false;
+        todo.push_back(in_t ? Part{tm, s.t1, s.c0, s.c1} : Part{s.t0, s.t1, cm, s.c1});
+        todo.push_back(in_t ? Part{s.t0, tm, s.c0, s.c1} : Part{s.t0, s.t1, s.c0, cm});
+        continue;
+      }
+      SubgridDesc e = d;
+      e.rec_offset = int32_t(out->size());  // place in w_ref
+      if (s.t0 != d.t0 || s.t1 != d.t1 || s.c0 != d.c0 || s.c1 != d.c1) {
+        e.t0 = s.t0;
+        e.t1 = s.t1;
+        e.c0 = s.c0;
+        e.c1 = s.c1;
+        const int width = s.c1 - s.c0;
+        e.n_vis = (s.t1 - s.t0) * width;
+        e.flags |= kSubgridPart;
+        e.seg_begin = int32_t(seg->size());
+        for (int k = seg_begin; k < seg_begin + seg_count; ++k) {
+          const SegmentDesc g = (*seg)[k];
+          const int a = std::max(aterm_offsets[g.interval], s.t0), b = std::min(aterm_offsets[g.interval + 1], s.t1);
+          if (a < b) seg->push_back(SegmentDesc{g.subgrid, g.interval, (a - s.t0) * width, (b - s.t0) * width});
+        }
+        e.seg_count = int32_t(seg->size()) - e.seg_begin;
+      }
+      out->push_back(e);
+      w_ref->push_back(make_float2(mid, float(0.25 * x * x)));
+    }
+  }
+  return out->size() <= 2 * in.size();
 }
 
 size_t scratch_budget_bytes() {
@@ -490,32 +598,26 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     taper_d.assign(g->taper_user, g->taper_user + L);
   else
     taper_d = kaiser_bessel_taper(L, g->taper_beta > 0.0 ? g->taper_beta : 0.35 * kPi * g->kernel_padding);
-  // reference w of every kept subgrid (the middle of its members' w - w0) and whether the separable form
-  // holds for the largest distance from it
+  // the separable form: whether it holds, the parts that the subgrids are worked on in, and a reference w
+  // (the middle of the members' w - w0) and a quarter of the largest squared distance from it for each
   SepFit sep;
-  std::vector<float> w_ref;
+  std::vector<float2> w_ref;
+  std::vector<SubgridDesc> parts;
   bool sep_ok = false;
+  p->segs = p->part.segments;
   if (supported_subgrid_size(L)) {  // host-only plans take other sizes too
-    sep = sep_fit(L, g->image_size, taper_d);
-    double delta = 0.0;
-    w_ref.reserve(p->exec.size());
-    for (SubgridDesc& d : p->exec) {
-      const double sgn = subgrid_sign(d), w0 = (double(d.layer) + 0.5) * p->part.w_step;
-      double lo = 0.0, hi = 0.0;
-      for (int t = d.t0; t < d.t1; ++t)
-        for (int e = 0; e < 2; ++e) {
-          const double w = sgn * uvw_m[(size_t(d.b) * n_timesteps + t) * 3 + 2] *
-                               (freqs_hz[e ? d.c1 - 1 : d.c0] / kSpeedOfLight) - w0;
-          lo = (t == d.t0 && !e) ? w : std::min(lo, w);
-          hi = (t == d.t0 && !e) ? w : std::max(hi, w);
-        }
-      const float mid = float(0.5 * (lo + hi));
-      delta = std::max(delta, std::max(hi - double(mid), double(mid) - lo));
-      d.rec_offset = int32_t(w_ref.size());
-      w_ref.push_back(mid);
+    double x = 0.0;  // largest half width of a subgrid's w range
+    for (const SubgridDesc& d : p->exec) {
+      const WRange w = w_range(d, d.t0, d.t1, d.c0, d.c1, p->part.w_step, n_timesteps, uvw_m, freqs_hz);
+      x = std::max(x, 0.5001 * (w.hi - w.lo));  // and the rounding of w_ref
     }
-    const double x = 2.0 * kPi * delta;
-    sep_ok = x * sep.e1 + x * x * sep.e2 <= kSepTolerance;  // false for a NaN
+    for (double h : kSepFit) {
+      const SepFit f = sep_fit(L, g->image_size, taper_d, h);
+      if (sep.tab.empty() || f.x_max > sep.x_max) sep = f;
+      if (sep.x_max >= x) break;
+    }
+    sep_ok = sep_parts(p->exec, sep.x_max, p->part.w_step, n_timesteps, uvw_m, freqs_hz, aterm_offsets, &p->segs, &parts,
+                       &w_ref);
   }
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
   // cannot run); both on FP32 when channel groups were asked for, and for Stokes I without the separable form
@@ -544,6 +646,10 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && tc_ok;
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
   }
+  if (p->grid_sep || p->degrid_sep)
+    p->exec = std::move(parts);
+  else
+    p->segs.resize(p->part.segments.size());
   p->grid_chunk = g->grid_chunk > 0 ? g->grid_chunk : kDefaultGridChunk;
   for (SubgridDesc& d : p->exec) d.layer -= k_lo;  // device tables hold the grid plane set
   if (host_only) {
@@ -556,9 +662,9 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     if (x.y0 != y.y0) return x.y0 < y.y0;
     return x.x0 < y.x0;
   });
-  {
+  if (p->grid_sep || p->degrid_sep) {
     // into execution order (rec_offset held each subgrid's place in w_ref)
-    const std::vector<float> src = w_ref;
+    const std::vector<float2> src = w_ref;
     for (size_t s = 0; s < p->exec.size(); ++s) w_ref[s] = src[p->exec[s].rec_offset];
   }
   const size_t per_sg = size_t(4) * L * L * sizeof(float2);
@@ -579,11 +685,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       const int nc = d.c1 - d.c0;
       if (p->grid_sep)
         for (int s = 0; s < d.seg_count; ++s) {
-          const SegmentDesc& sg = p->part.segments[d.seg_begin + s];
+          const SegmentDesc& sg = p->segs[d.seg_begin + s];
           recs += (sg.k_end - sg.k_begin + kGsepChunkVis - 1) / kGsepChunkVis * (kGsepChunkFloat4 / kRecordFloat4);
         }
       else
-        recs += p->grid_tc ? tc_records(tc_row_groups(p->part.segments.data(), d.seg_begin, d.seg_count, nc), nc)
+        recs += p->grid_tc ? tc_records(tc_row_groups(p->segs.data(), d.seg_begin, d.seg_count, nc), nc)
                          : d.n_vis;
     }
     p->max_batch_vis = std::max(p->max_batch_vis, recs);
@@ -607,7 +713,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       if (p->degrid_sep) {
         // equal pieces of each segment, each a multiple of 16 visibilities but for the last
         for (int gidx = d.seg_begin; gidx < d.seg_begin + d.seg_count; ++gidx) {
-          const SegmentDesc& sgd = p->part.segments[gidx];
+          const SegmentDesc& sgd = p->segs[gidx];
           const int n = sgd.k_end - sgd.k_begin, pieces = (n + p->degrid_vis - 1) / p->degrid_vis;
           const int len = ((n + pieces - 1) / pieces + 15) / 16 * 16;
           for (int k = sgd.k_begin; k < sgd.k_end; k += len) {
@@ -621,7 +727,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       const int G = (width + p->degrid_channels - 1) / p->degrid_channels;
       bool open = false;  // the last item can take a piece of the next segment
       for (int gidx = d.seg_begin; gidx < d.seg_begin + d.seg_count; ++gidx) {
-        const SegmentDesc& sgd = p->part.segments[gidx];
+        const SegmentDesc& sgd = p->segs[gidx];
         const int g_begin = sgd.k_begin / width * G, g_end = sgd.k_end / width * G;
         for (int k = g_begin; k < g_end; k += lanes) {
           const int ke = std::min(k + lanes, g_end);
@@ -706,7 +812,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     if (!e) e = upload(p, &p->d_wref, w_ref.data(), w_ref.size());
   }
   if (!e) e = upload(p, &p->d_sg, p->exec.data(), p->exec.size());
-  if (!e) e = upload(p, &p->d_seg, p->part.segments.data(), p->part.segments.size());
+  if (!e) e = upload(p, &p->d_seg, p->segs.data(), p->segs.size());
   if (!e) e = upload(p, &p->d_gitems, gitems.data(), gitems.size());
   if (!e) e = upload(p, &p->d_ditems, ditems.data(), ditems.size());
   if (!e && !p->exec.empty()) {
@@ -880,7 +986,7 @@ static FftArgs splitter_args(const idg_plan* p, const Batch& b, const void* grid
     fa.ymax = p->d_ymax;
     fa.w_ref = p->d_wref + b.sg_offset;
     fa.taper = p->d_taper;
-    fa.n1 = p->d_n1;
+    fa.sep = sep_tables(p);
   }
   return fa;
 }

@@ -36,6 +36,9 @@ constexpr int32_t kSubgridDropped = 1;   // outside the grid (IDG_DROP_OUT_OF_GR
 // descriptor are already swapped, the kernels negate uvw and conjugate-
 // transpose the values they read (gridder) or write (degridder)
 constexpr int32_t kSubgridMirrored = 2;
+// some of a subgrid's visibilities, in the tables of the separable kernels: shares its place and plan_index with the
+// other parts
+constexpr int32_t kSubgridPart = 4;
 
 // The part of a subgrid that shares one A-term interval (Section 3.3).
 // Members are enumerated t-major: k = (t - t0) * (c1 - c0) + (c - c0).
@@ -140,9 +143,11 @@ __host__ __device__ constexpr int gsep_rows(int L) { return L == 128 ? 64 : L; }
 __host__ __device__ constexpr int gsep_tiles(int L) { return (L / kGsepColumns) * (L / gsep_rows(L)); }
 // dynamic shared memory limit of those kernels (227 KB per block less their static part)
 constexpr int kSepSmemLimit = 231424;
-// largest taper-weighted error of the separable form, relative to the centre
-// pixel's weight: below the rounding of the FP32 kernels' phases
-constexpr double kSepTolerance = 3e-7;
+// What the separable form may neglect: of a source's flux anywhere within |l|, |m| <= FOV / 4, and of the centre's
+// flux, weighted with the taper, over the whole subgrid.  It is below what the kernels of one phasor per visibility and
+// pixel lose to the rounding of their phases there (1e-6 of the largest visibility, measured).  Between FOV / 4 and FOV / 3,
+// where the taper falls from 6e-3 to 6e-5 of its centre and those kernels lose 1e-4 to 1e-3, kSepToleranceOuter.
+constexpr double kSepTolerance = 3e-7, kSepToleranceOuter = 1e-6;
 
 // Tables of the separable form, n'(i,j) = A_i + B_j + p_i q_j + rest: a = 2 pi A,
 // b = 2 pi B, p = 2 pi p (scaled so that max |q| = 1), and n' as two floats
@@ -239,7 +244,8 @@ struct GridArgs {
   float2* scratch;            // [batch][4][L][L]
   double* aweights;           // A-term power weights [L*L + 1] (IDG_NORMALIZE_ATERM), else NULL
   int vc = kDefaultGridChunk;  // staged records per chunk: 32, 48 or 64
-  const float* w_ref = nullptr;  // [batch subgrids] reference w (separable-phasor gridder)
+  // separable-phasor gridder: [batch subgrids] reference w, a quarter of the largest squared distance from it
+  const float2* w_ref = nullptr;
   SepTables sep;
   int run = 1, stride = 1;    // a block's items (SepShare); stride: one launch over several plans
   uint64_t wait_ns = 0;       // limit of one wait of the separable-phasor gridder
@@ -264,7 +270,7 @@ struct DegridArgs {
   int* status = nullptr;          // device status word (kStatusTimeout)
   const float* amax = nullptr;    // [n_int][n_st] largest component of the A-term's nodes
   const float* ymax = nullptr;    // [batch subgrids][4] largest component of the subgrid's planes
-  const float* w_ref = nullptr;   // [batch subgrids] reference w
+  const float2* w_ref = nullptr;  // [batch subgrids] reference w, a quarter of the largest squared distance from it
   int kv = 0;                     // visibilities per item
   int run = 1, stride = 1;        // a block's items (SepShare); stride: one launch over several plans
   uint64_t wait_ns = 0;           // limit of one wait
@@ -280,11 +286,11 @@ struct FftArgs {
   int32_t N;
   int32_t npol = 4;        // planes per subgrid transformed and added / split (4, or 1 for Stokes I)
   // splitter of separable-phasor plans (ymax set): the image times taper, centring sign and
-  // e^{-2 pi i w_ref n'}, and each plane's largest component
+  // e^{-2 pi i w_ref n'} (sep_pixel), and each plane's largest component
   float* ymax = nullptr;   // [batch subgrids][4]
-  const float* w_ref = nullptr;
+  const float2* w_ref = nullptr;
   const float* taper = nullptr;
-  const float2* n1 = nullptr;
+  SepTables sep;
 };
 
 // how long a device-side wait lasts before the kernel reports a timeout (idg_set_wait_limit)
@@ -333,7 +339,7 @@ int launch_gridder_tc(int L, const GridArgs& a, int n_items, int persistent_bloc
 int configure_gridder_tc(int L, int* persistent_blocks);
 int launch_gridder_tc_multi(int L, const GridArgs* args, const int2* items, int n_items, void* stream);
 // the separable-phasor gridder (records staged by launch_stage_sep; any channel spacing)
-int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float* w_ref, int n_subgrids, void* stream);
+int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const float2* w_ref, int n_subgrids, void* stream);
 int launch_gridder_sep(int L, const GridArgs& a, int n_items, int blocks, void* stream);
 int configure_gridder_sep(int L, int* persistent_blocks);
 int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* blocks, int n_blocks, int max_nodes, void* stream);

@@ -4,17 +4,20 @@
 // The phase of Eq. 7 over a subgrid, phi_k(i,j) = a_k i' + b_k j' + w_k n'(i,j)
 // (turns; i' = i - L/2, j' = j - L/2), is separable but for the w term, and
 // that term nearly so.  With w_ref the middle of the subgrid's w range,
-// delta_k = w_k - w_ref, and the fit n'(i,j) = A_i + B_j + p_i q_j + r_ij
-// (taper-weighted, SepTables),
-//   e^{2 pi i phi_k} = e^{2 pi i w_ref n'(i,j)} E_k(i) F_k(j) (1 + 2 pi i delta_k p_i q_j) + O(r, p^2 q^2)
+// delta_k = w_k - w_ref, |delta_k| <= x, and the fit n'(i,j) = A_i + B_j + p_i q_j
+// + r_ij (sep_fit, SepTables),
+//   e^{2 pi i phi_k} = P(i,j) E_k(i) F_k(j) (1 + 2 pi i delta_k p_i q_j) + O(x r, (x p q)^2)
+//   P(i,j) = e^{2 pi i w_ref n'(i,j)} (1 - (2 pi x p_i q_j)^2 / 4),
 //   E_k(i) = e^{2 pi i (a_k i' + delta_k A_i)},  F_k(j) = e^{2 pi i (b_k j' + delta_k B_j)}.
-// The first factor is the same for every visibility of the subgrid and is
-// applied once per pixel; the sums over visibilities (gridder) or pixels
+// P is the same for every visibility of the subgrid and is applied once per
+// pixel (sep_pixel); its real factor halves the second-order term at either
+// end of the w range.  The sums over visibilities (gridder) or pixels
 // (degridder) become real matrix products of an E side and an F side, so a
 // visibility needs 2 L sines and cosines instead of L^2 and the
 // multiply-accumulate runs on the tensor cores at full tile sizes.  The plan
-// takes this path only where the neglected terms, weighted with the taper,
-// stay below kSepTolerance (sep_fit).
+// keeps the neglected terms below kSepTolerance for a source anywhere in the
+// usable part of the field (sep_fit), with subgrids of a wide w range worked on
+// in parts (sep_parts), and takes the general kernels where that takes too many.
 //
 // Products: tcgen05.mma kind::f16 with FP32 accumulation in tensor memory.
 // Every FP32 operand is split into two halves hi + lo (22 bits), and the
@@ -279,14 +282,15 @@ __device__ __forceinline__ void sep_product(uint32_t d, uint32_t e, uint32_t f, 
   }
 }
 
-// (cos, sin)(2 pi w_ref n') from the two-float n' (exact range reduction)
-__device__ __forceinline__ float2 sep_w_phasor(float w_ref, float2 n1) {
-  const float t = w_ref * n1.x;
-  const float lo = fmaf(w_ref, n1.y, fmaf(w_ref, n1.x, -t));
+// P of a pixel: w = (w_ref, x^2 / 4), the two-float n' (exact range reduction), 2 pi p_i q_j
+__device__ __forceinline__ float2 sep_pixel(float2 w, float2 n1, float pq) {
+  const float t = w.x * n1.x;
+  const float lo = fmaf(w.x, n1.y, fmaf(w.x, n1.x, -t));
   const float ang = ((t - rintf(t)) + lo) * kTwoPiF;
+  const float k = fmaf(-w.y * pq, pq, 1.f);
   float s, c;
   __sincosf(ang, &s, &c);
-  return make_float2(c, s);
+  return make_float2(k * c, k * s);
 }
 
 }  // namespace idg

@@ -104,7 +104,8 @@ def record_bytes(obs: synth.Observation) -> int:
     path = np.abs(np.diff(px, axis=1)).sum(1) * float(obs.freqs[-1])  # [bl, axis]
     cuts = np.minimum(obs.n_intervals + np.ceil(path / margin).sum(-1), obs.n_timesteps)
     segments = float((runs * cuts).sum())
-    chunks = min(float(obs.n_vis), obs.n_vis / 16 + segments)
+    # subgrids of a wide w range are worked on in parts, at most as many again
+    chunks = min(float(obs.n_vis), obs.n_vis / 16 + 2 * segments)
     return int(max(128 * obs.n_vis, 768 * chunks))
 
 
