@@ -220,6 +220,7 @@ struct Dsep {
     const int lane = threadIdx.x & 31, nodes = a.g.nodes;
     const bool quad = L % (nodes - 1) == 0 && L / (nodes - 1) % 4 == 0;
     const uint32_t tm = S.tmem;
+    const float inv_p = 1.f / a.sep.p_scale;
     uint32_t n = 0, pg = uniform_warp() >> 2, base = 0;  // items so far, the group's next piece, the item's first
     for (int idx = share.first; idx < share.last; idx = share.next(idx), ++n, base += kItemPieces) {
       // an item without a piece of this group is passed over: its barriers may be phases ahead
@@ -232,7 +233,7 @@ struct Dsep {
       for (; pg < base + kItemPieces; pg += kDsepGroups) {
         const int t = pg - base, ib = t / kPieces, jc = t - ib * kPieces, i = ib * 32 + lane;
         const NodeWeight wx = node_weight(i, nodes, L);
-        const __half2 fit_p = __float2half2_rn(__ldg(a.sep.p + i));
+        const __half2 fit_p = __float2half2_rn(__ldg(a.sep.p + i) * inv_p);
         const uint32_t slot = pg % kDsepRing;
         wait(&S.loaded[pg % kDsepLoaded], (pg / kDsepLoaded) & 1);
         if (pg >= uint32_t(kDsepRing)) tc_fence_after();  // the loader has seen the slot's last MMAs complete
@@ -372,7 +373,7 @@ struct Dsep {
     for (int e = tid; e < n_pad * (L / 8); e += kDsepPreparers) {
       const int o = e / n_pad, k = e - o * n_pad;
       const int fix = __float_as_int(S.fix_b[b][k]);
-      const float dl = S.delta[b][k];
+      const float dl = S.delta[b][k], dp = dl * a.sep.p_scale;
       const float4* tb = reinterpret_cast<const float4*>(a.sep.b + 8 * o);
       const float4* tq = reinterpret_cast<const float4*>(a.sep.q + 8 * o);
       SepF f;
@@ -386,7 +387,7 @@ struct Dsep {
           float2 c, s;
           __sincosf(sep_phase(fix, off, dl, fb.x), &s.x, &c.x);
           __sincosf(sep_phase(fix, off + 1, dl, fb.y), &s.y, &c.y);
-          const __half2 d2 = __floats2half2_rn(-dl * fq.x, -dl * fq.y);
+          const __half2 d2 = __floats2half2_rn(-dp * fq.x, -dp * fq.y);
           const __half2 hc = sep_split(c, f.r_hi[w], f.r_lo[w]);
           const __half2 hs = sep_split(s, f.i_hi[w], f.i_lo[w]);
           // conj(F) = (c, -s); -i delta q conj(F) = (-delta q s, -delta q c)

@@ -90,6 +90,7 @@ struct idg_plan {
   int* d_queue = nullptr;       // work-queue counters, 2 per batch (gridder, degridder)
   uint8_t* d_adiag = nullptr;   // [n_int][n_st] diagonal-A-term flags of the current call
   float* d_sep = nullptr;       // [4][L] separable-phasor tables a, b, p, q
+  float sep_p_scale = 1.f;      // of p (SepTables)
   float2* d_n1 = nullptr;       // [L*L] n' as two floats
   float2* d_wref = nullptr;     // [exec subgrids] reference w, a quarter of the largest squared distance from it
   float* d_amax = nullptr;      // [n_int][n_st] largest A-term component of the current call (degrid_sep)
@@ -283,7 +284,8 @@ constexpr double kSepFit[] = {0.12, 0.20, 0.28, 0.31, 0.32};
 struct SepFit {
   std::vector<float> tab;   // [4][L]: 2 pi A, 2 pi B, 2 pi p, q
   std::vector<float2> n1;   // [j][i]
-  double x_max = 0.0;       // largest |w - w_ref| (wavelengths) that meets kSepTolerance and kSepTolerancePx
+  float p_scale = 1.f;      // of 2 pi p (SepTables)
+  double x_max = 0.0;       // largest |w - w_ref| (wavelengths) that meets kSepTolerance, kSepToleranceOuter and kSepPhase
 };
 
 SepFit sep_fit(int L, double fov, const std::vector<double>& taper, double h) {
@@ -338,8 +340,20 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper, double h) {
     q[i] /= qm;
     p[i] *= qm;
   }
-  // the largest x at which every pixel keeps a x + b x^2 within its tolerance
+  // power of two that brings max |2 pi p| into [1/2, 1)
+  double pm = 0.0;
+  for (double v : p) pm = std::max(pm, 2.0 * kPi * std::fabs(v));
+  int e = 0;
+  if (pm > 0.0) std::frexp(pm, &e);
+  f.p_scale = float(std::ldexp(1.0, std::max(-120, std::min(e, 120))));
+  // the largest x that keeps the phases delta A and delta B within kSepPhase in the usable part of the field...
   f.x_max = 1e300;
+  for (int i = 0; i < L; ++i)
+    if (std::abs(i - L / 2) * 3 <= L) {
+      const double a = 2.0 * kPi * std::max(std::fabs(A[i]), std::fabs(B[i]));
+      if (!(kSepPhase / a >= f.x_max)) f.x_max = kSepPhase / a;
+    }
+  // ... and at which every pixel keeps a x + b x^2 within its tolerance
   for (int j = 0; j < L; ++j)
     for (int i = 0; i < L; ++i) {
       const double t = std::fabs(taper[i] * taper[j]) / (tmax * tmax), pq = p[i] * q[j];
@@ -646,6 +660,7 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && tc_ok;
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
   }
+  p->sep_p_scale = sep.p_scale;
   if (p->grid_sep || p->degrid_sep)
     p->exec = std::move(parts);
   else
@@ -887,7 +902,7 @@ static StageArgs stage_args(const idg_plan* p, const Batch& b, const void* vis) 
 
 static SepTables sep_tables(const idg_plan* p) {
   const int L = p->L;
-  return SepTables{p->d_sep, p->d_sep + L, p->d_sep + 2 * L, p->d_sep + 3 * L, p->d_n1};
+  return SepTables{p->d_sep, p->d_sep + L, p->d_sep + 2 * L, p->d_sep + 3 * L, p->d_n1, p->sep_p_scale};
 }
 
 static GridArgs grid_args(const idg_plan* p, const Batch& b, const void* vis, const void* aterms) {

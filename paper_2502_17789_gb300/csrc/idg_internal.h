@@ -148,6 +148,9 @@ constexpr int kSepSmemLimit = 231424;
 // pixel lose to the rounding of their phases there (1e-6 of the largest visibility, measured).  Between FOV / 4 and FOV / 3,
 // where the taper falls from 6e-3 to 6e-5 of its centre and those kernels lose 1e-4 to 1e-3, kSepToleranceOuter.
 constexpr double kSepTolerance = 3e-7, kSepToleranceOuter = 1e-6;
+// largest |2 pi delta A|, |2 pi delta B| within the same part: what the phases of E and F may pass [-pi, pi] by.  Their
+// rounding in FP32 and __sincosf's error grow with the argument (at a field of 0.2 w ranges inside the bounds above reach 4 turns).
+constexpr double kSepPhase = 1.57;
 
 // Tables of the separable form, n'(i,j) = A_i + B_j + p_i q_j + rest: a = 2 pi A,
 // b = 2 pi B, p = 2 pi p (scaled so that max |q| = 1), and n' as two floats
@@ -157,6 +160,9 @@ struct SepTables {
   const float* p = nullptr;
   const float* q = nullptr;
   const float2* n1 = nullptr;  // [L (j)][L (i)]
+  // power of two with |p| < p_scale: halves hold p / p_scale and delta p_scale q, where p alone falls below their
+  // range at small fields (7e-6 at FOV 0.1) and delta q may pass it
+  float p_scale = 1.f;
 };
 
 

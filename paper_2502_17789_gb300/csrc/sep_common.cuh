@@ -209,9 +209,10 @@ struct SepShare {
 
 // ---------------------------------------------------------------- operands
 
-// phase (radians, about [-pi, pi]) of slope `fix` (turns per pixel in units
-// of 2^-32, so the product wraps exactly) at pixel offset `off`, plus the
-// small w part `delta_k` x `fit` (fit carries 2 pi)
+// phase (radians) of slope `fix` (turns per pixel in units of 2^-32, so the
+// product wraps exactly to [-pi, pi]) at pixel offset `off`, plus the w part
+// `delta_k` x `fit` (fit carries 2 pi), at most kSepPhase more in the usable
+// part of the field and about twice that at its edges
 __device__ __forceinline__ float sep_phase(int fix, int off, float delta, float fit) {
   return fmaf(float(int(unsigned(fix) * unsigned(off))), kTurnsToRad, delta * fit);
 }

@@ -43,7 +43,9 @@ def _plan(idg_mod, L, fov, x, n_bl=12, wide=4, n_t=12, flags=0):
 
 VALUES = (1.0, 0.5j, -1.0, -1j)   # of the correlations
 GEOMETRIES = [(32, 0.35, 5.0), (32, 0.35, 35.0), (64, 0.5, 1.5), (64, 0.5, 8.0), (96, 0.5, 3.9), (96, 0.5, 5.7),
-              (96, 0.5, 11.0), (96, 0.35, 40.0), (128, 0.5, 4.5), (128, 0.5, 11.0)]
+              (96, 0.5, 11.0), (96, 0.35, 40.0), (128, 0.5, 4.5), (128, 0.5, 11.0),
+              # small fields: long w ranges in wavelengths, tables far below the range of half precision
+              (96, 0.2, 110.0), (64, 0.1, 700.0), (96, 0.05, 3000.0), (32, 0.02, 12000.0), (128, 0.005, 250000.0)]
 
 
 @pytest.mark.parametrize("L,fov,x", GEOMETRIES)
