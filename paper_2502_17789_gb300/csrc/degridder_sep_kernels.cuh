@@ -67,7 +67,7 @@ struct alignas(128) DsepShared {
   float out[kDsepMaxVis][8];
   // the producers' part of an item, by item parity
   struct Info {
-    float scale;   // of Z, a power of two
+    float scale[4];  // of each correlation's Z, a power of two
     int sg, diag;
   } info[2];
   uint64_t ready[2];        // item prepared (2 preparing warps)
@@ -226,7 +226,7 @@ struct Dsep {
       // an item without a piece of this group is passed over: its barriers may be phases ahead
       if (pg >= base + kItemPieces) continue;
       wait(&S.ready[n & 1], (n >> 1) & 1);
-      const float scale = S.info[n & 1].scale;
+      const float scale = S.info[n & 1].scale[(threadIdx.x >> 5) & 3];
       const bool diag = S.info[n & 1].diag != 0;
       const float4* samples = raw + (n & 1) * 4 * nodes * nodes;
 #pragma unroll 1
@@ -349,10 +349,21 @@ struct Dsep {
       fb = sep_fix(((r[1] * fs) * a.g.fov - double(sd.y0 + L / 2 - a.g.N / 2)) * inv_l);
       dl = float(r[2] * fs - (double(a.w_ref[item.sg].x) + subgrid_w0(a.g, sd)));
     }
-    // scale of Z from the largest components of Y and of the A-terms' nodes
-    float ym = 0.f;
-    for (int k = 0; k < a.g.npol; ++k) ym = fmaxf(ym, a.ymax[item.sg * 4 + k]);
-    const DsepShared::Info info = {sep_scale(ym * a.amax[sp] * a.amax[sq]), item.sg, a.adiag[sp] & a.adiag[sq]};
+    // scale of each correlation's Z = A_p Y A_q^H (thread = correlation (r, c)) from the largest components of Y and of
+    // the A-terms' nodes: a faint correlation keeps its bits beside a bright one
+    const int diag = a.adiag[sp] & a.adiag[sq];
+    float bound;
+    {
+      const float4 am = a.amax[sp], bm = a.amax[sq], y = *reinterpret_cast<const float4*>(a.ymax + item.sg * 4);
+      const int r = (tid >> 1) & 1, c = tid & 1;
+      const float p0 = r ? am.z : am.x, p1 = r ? am.w : am.y, q0 = c ? bm.z : bm.x, q1 = c ? bm.w : bm.y;
+      if (a.g.npol == 1)
+        bound = diag ? (r == c ? (r ? p1 * q1 : p0 * q0) * y.x : 0.f) : (p0 * q0 + p1 * q1) * y.x;
+      else if (diag)
+        bound = (r ? p1 : p0) * (r ? (c ? y.w : y.z) : (c ? y.y : y.x)) * (c ? q1 : q0);
+      else
+        bound = p0 * (y.x * q0 + y.y * q1) + p1 * (y.z * q0 + y.w * q1);
+    }
     if (n >= 2) wait<100>(&S.done[b], ((n >> 1) - 1) & 1);  // the buffers' previous item (two back) is done
     {
       const float4* src = reinterpret_cast<const float4*>(a.aterms);
@@ -366,7 +377,11 @@ struct Dsep {
       S.fix_b[b][tid] = __int_as_float(fb);
       S.delta[b][tid] = dl;
     }
-    if (tid == 0) S.info[b] = info;
+    if (tid < 4) S.info[b].scale[tid] = sep_scale(bound);
+    if (tid == 0) {
+      S.info[b].sg = item.sg;
+      S.info[b].diag = diag;
+    }
     asm volatile("bar.sync %0, %1;" ::"n"(kDsepPreparerBar), "n"(kDsepPreparers) : "memory");
     const uint32_t block = uint32_t(n_pad) * 16, group = 2 * block, chunk = 2 * group, level = kPieces * chunk;
     const uint32_t base = smem_u32(fside) + b * uint32_t(a.kv) * L * 12;
@@ -420,7 +435,7 @@ struct Dsep {
       const DegridItem item = a.items[idx];
       const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
       wait(&S.ready[b], (n >> 1) & 1);
-      const float inv = sep_unbias(kPieces) / S.info[b].scale;
+      const float inv = sep_unbias(kPieces) / S.info[b].scale[pol];
       float sum[kDsepMaxVis / 16];  // component lane & 1 of visibility 16 h + lane / 2
 #pragma unroll
       for (int h = 0; h < kDsepMaxVis / 16; ++h) sum[h] = 0.f;

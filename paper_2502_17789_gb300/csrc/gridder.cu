@@ -115,8 +115,8 @@ __global__ void __launch_bounds__(256) stage_records_kernel(const StageArgs a, i
 
 // Staging for the separable-phasor gridder: one block per subgrid writes its segments' records, 16 visibilities per
 // chunk (the last padded with zeros; kGsepChunkFloat4): a fix, b fix, delta, 1 / scale and the 4 values times the
-// segment's scale, a power of two that puts the largest component in [512, 1024) so that hi + lo halves keep 22 bits
-// down to 2^-9 of it.  Bound by latency, not bytes: a pass over a segment's values for the scale, then one that reads
+// scale of the segment and correlation (sep_scale; of each correlation by itself, so that a faint one keeps its bits and
+// an infinity in one leaves the others alone).  Bound by latency, not bytes: a pass over a segment's values for the scale, then one that reads
 // them again (from L1 or L2) and writes.
 __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const SegmentDesc* seg, const float2* w_ref,
                                                         int L) {
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
   const double inv_l = 1.0 / double(L), sgn = subgrid_sign(sd);
   const double off_x = double(sd.x0 + L / 2 - a.g.N / 2), off_y = double(sd.y0 + L / 2 - a.g.N / 2);
   float4* base = a.records + size_t(sd.rec_offset) * kRecordFloat4;
-  __shared__ float s_max[8];
+  __shared__ float4 s_max[8];
   // a warp per segment where there are enough segments, else the whole block per segment
   const bool by_warp = sd.seg_count >= 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -141,26 +141,35 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
         const int row = k / nc;
         return (size_t(sd.b) * a.g.n_t + sd.t0 + row) * a.g.n_ch + sd.c0 + (k - row * nc);
       };
-      float m = 0.f;
+      float4 m = make_float4(0.f, 0.f, 0.f, 0.f);  // per correlation
+      const auto take = [&m](float x, float y, float z, float w) {
+        m = make_float4(fmaxf(m.x, x), fmaxf(m.y, y), fmaxf(m.z, z), fmaxf(m.w, w));
+      };
       for (int k = sg.k_begin + t0; k < sg.k_end; k += nt) {
         const size_t v = vis_index(k);
         const float4 v0 = a.vis[2 * v], v1 = a.vis[2 * v + 1];
-        m = fmaxf(fmaxf(fmaxf(fmaxf(m, fabsf(v0.x)), fmaxf(fabsf(v0.y), fabsf(v0.z))), fmaxf(fabsf(v0.w), fabsf(v1.x))),
-                  fmaxf(fmaxf(fabsf(v1.y), fabsf(v1.z)), fabsf(v1.w)));
+        take(fmaxf(fabsf(v0.x), fabsf(v0.y)), fmaxf(fabsf(v0.z), fabsf(v0.w)), fmaxf(fabsf(v1.x), fabsf(v1.y)),
+             fmaxf(fabsf(v1.z), fabsf(v1.w)));
       }
 #pragma unroll
-      for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      for (int o = 16; o; o >>= 1)
+        take(__shfl_xor_sync(0xffffffffu, m.x, o), __shfl_xor_sync(0xffffffffu, m.y, o),
+             __shfl_xor_sync(0xffffffffu, m.z, o), __shfl_xor_sync(0xffffffffu, m.w, o));
       if (!by_warp) {
         if (lane == 0) s_max[warp] = m;
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < 8; ++w) m = fmaxf(m, s_max[w]);
+        for (int w = 0; w < 8; ++w) take(s_max[w].x, s_max[w].y, s_max[w].z, s_max[w].w);
         __syncthreads();
       }
-      const float scale = sep_scale(m), inv = 1.f / scale;  // powers of two: exact
+      // powers of two: exact.  Mirroring swaps XY and YX
+      const float4 scale = make_float4(sep_scale(m.x), sep_scale(mirror ? m.z : m.y), sep_scale(mirror ? m.y : m.z),
+                                       sep_scale(m.w));
       float4* dst = base + size_t(chunk0) * kGsepChunkFloat4;
       for (int k = t0; k < chunks * kSepK; k += nt) {
         float* c = reinterpret_cast<float*>(dst + size_t(k / kSepK) * kGsepChunkFloat4) + (k & (kSepK - 1));
+        const int kc = k & (kSepK - 1);
+        const float inv = kc > 3 ? 0.f : 1.f / (kc == 0 ? scale.x : kc == 1 ? scale.y : kc == 2 ? scale.z : scale.w);
         float4 prm = make_float4(0.f, 0.f, 0.f, inv), v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
         if (k < n) {
           const int row = (sg.k_begin + k) / nc, ch = sd.c0 + (sg.k_begin + k - row * nc);
@@ -173,8 +182,8 @@ __global__ void __launch_bounds__(256) stage_sep_kernel(const StageArgs a, const
           v0 = a.vis[2 * v];
           v1 = a.vis[2 * v + 1];
           if (mirror) mirror_values(v0, v1);
-          v0 = make_float4(v0.x * scale, v0.y * scale, v0.z * scale, v0.w * scale);
-          v1 = make_float4(v1.x * scale, v1.y * scale, v1.z * scale, v1.w * scale);
+          v0 = make_float4(v0.x * scale.x, v0.y * scale.x, v0.z * scale.y, v0.w * scale.y);
+          v1 = make_float4(v1.x * scale.z, v1.y * scale.z, v1.z * scale.w, v1.w * scale.w);
         }
         c[0] = prm.x;
         c[16] = prm.y;
@@ -199,30 +208,37 @@ int launch_stage_sep(int L, const StageArgs& a, const SegmentDesc* seg, const fl
   return int(cudaGetLastError());
 }
 
-// one warp per (interval, station): are all off-diagonal node entries zero, and the largest component
-__global__ void aterm_flags_kernel(const float2* aterms, uint8_t* flags, float* amax, int n_pairs, int nodes) {
+// one warp per (interval, station): are all off-diagonal node entries zero, and each entry's largest component
+__global__ void aterm_flags_kernel(const float2* aterms, uint8_t* flags, float4* amax, int n_pairs, int nodes) {
   const int pair = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (pair >= n_pairs) return;
   const float4* A = reinterpret_cast<const float4*>(aterms + size_t(pair) * nodes * nodes * 4);
   bool diag = true;
-  float m = 0.f;
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int n = lane; n < nodes * nodes; n += 32) {
     const float4 a = A[2 * n], b = A[2 * n + 1];  // (00, 01) (10, 11)
     diag = diag && a.z == 0.f && a.w == 0.f && b.x == 0.f && b.y == 0.f;
-    m = fmaxf(fmaxf(fmaxf(m, fabsf(a.x)), fmaxf(fabsf(a.y), fabsf(a.z))),
-              fmaxf(fmaxf(fabsf(a.w), fabsf(b.x)), fmaxf(fmaxf(fabsf(b.y), fabsf(b.z)), fabsf(b.w))));
+    m.x = fmaxf(fmaxf(m.x, fabsf(a.x)), fabsf(a.y));
+    m.y = fmaxf(fmaxf(m.y, fabsf(a.z)), fabsf(a.w));
+    m.z = fmaxf(fmaxf(m.z, fabsf(b.x)), fabsf(b.y));
+    m.w = fmaxf(fmaxf(m.w, fabsf(b.z)), fabsf(b.w));
   }
   diag = __all_sync(0xffffffffu, diag);
 #pragma unroll
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int o = 16; o; o >>= 1) {
+    m.x = fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, o));
+    m.y = fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
+    m.z = fmaxf(m.z, __shfl_xor_sync(0xffffffffu, m.z, o));
+    m.w = fmaxf(m.w, __shfl_xor_sync(0xffffffffu, m.w, o));
+  }
   if (lane == 0) {
     flags[pair] = diag ? 1 : 0;
     if (amax) amax[pair] = m;
   }
 }
 
-int launch_aterm_flags(const float2* aterms, uint8_t* flags, float* amax, int n_int, int n_st, int nodes, void* stream) {
+int launch_aterm_flags(const float2* aterms, uint8_t* flags, float4* amax, int n_int, int n_st, int nodes, void* stream) {
   const int n = n_int * n_st;
   if (n <= 0) return 0;
   aterm_flags_kernel<<<(n + 7) / 8, 256, 0, cudaStream_t(stream)>>>(aterms, flags, amax, n, nodes);

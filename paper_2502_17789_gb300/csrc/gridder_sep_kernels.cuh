@@ -248,7 +248,8 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
     const int2 org = gsep_origin<L>(item);
     const int i = org.x + lane, j0 = org.y + warp * C::kSpan;
     const NodeWeight wx = node_weight(i, nodes, L);
-    const float4* rec = a.records + size_t(sd.rec_offset) * kRecordFloat4;  // first chunk of the next segment
+    // 1 / scale of the next segment's first chunk, for the correlation that the warp takes from tensor memory
+    const float* rec = reinterpret_cast<const float*>(a.records + size_t(sd.rec_offset) * kRecordFloat4) + 48 + (warp & 3);
     cf acc[C::kSpan][4];
 #pragma unroll
     for (int r = 0; r < C::kSpan; ++r)
@@ -273,9 +274,9 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
       if (left == 0) left = gsep_chunks(seg);
       const int n = gsep_part(left);
       diag_next = a.adiag[sp] & a.adiag[sq];
-      // 1 / scale of the segment's values (undone on the p side) and the accumulation's bias
-      inv_next = __ldg(&rec[12].x) * sep_unbias(n);
-      rec += size_t(n) * kGsepChunkFloat4;
+      // the scale of the segment's values and the accumulation's bias, undone on the way to S.x
+      inv_next = __ldg(rec) * sep_unbias(n);
+      rec += size_t(n) * kGsepChunkFloat4 * 4;
       left -= n;
       if (left == 0 && ++s < sd.seg_count) seg = a.seg[sd.seg_begin + s];
     };
@@ -301,8 +302,8 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
           tmem_wait_ld();
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            S.x[pol][0][(r0 + b) / 2 + e][lane] = make_float2(re[2 * e], re[2 * e + 1]);
-            S.x[pol][1][(r0 + b) / 2 + e][lane] = make_float2(im[2 * e], im[2 * e + 1]);
+            S.x[pol][0][(r0 + b) / 2 + e][lane] = make_float2(re[2 * e] * inv, re[2 * e + 1] * inv);
+            S.x[pol][1][(r0 + b) / 2 + e][lane] = make_float2(im[2 * e] * inv, im[2 * e + 1] * inv);
           }
         }
         tc_fence_before();
@@ -322,7 +323,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
         constexpr bool DIAG = decltype(dtag)::value;
         const int st = DIAG ? w : w >> 1;
         const float4* n0 = smp + st * n4 + r * nodes * 2;
-        const float k1 = st ? wx.f : wx.f * inv, k0 = st ? 1.f - wx.f : (1.f - wx.f) * inv;
+        const float k1 = wx.f, k0 = 1.f - wx.f;
         if constexpr (DIAG) {
           const float4 x0 = n0[0], x1 = n0[1], y0 = n0[2], y1 = n0[3];
           return make_float4(k0 * x0.x + k1 * y0.x, k0 * x0.y + k1 * y0.y, k0 * x1.z + k1 * y1.z, k0 * x1.w + k1 * y1.w);

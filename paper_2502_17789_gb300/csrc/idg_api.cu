@@ -93,7 +93,7 @@ struct idg_plan {
   float sep_p_scale = 1.f;      // of p (SepTables)
   float2* d_n1 = nullptr;       // [L*L] n' as two floats
   float2* d_wref = nullptr;     // [exec subgrids] reference w, a quarter of the largest squared distance from it
-  float* d_amax = nullptr;      // [n_int][n_st] largest A-term component of the current call (degrid_sep)
+  float4* d_amax = nullptr;     // [n_int][n_st] largest component of each A-term entry of the current call (degrid_sep)
   float* d_ymax = nullptr;      // [batch capacity][4] largest component of the split subgrid planes (degrid_sep)
   double* d_aweights = nullptr; // [L*L + 1] A-term power weights (IDG_NORMALIZE_ATERM)
   // image-domain wrapper, made at its first use
@@ -817,9 +817,9 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   if (!e) e = upload(p, &p->d_twiddle, tw.data(), tw.size());
   if (!e && p->degrid_sep) {
     const size_t na = size_t(n_intervals) * std::max(1, n_stations), ny = size_t(4) * p->batch_cap;
-    e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_amax), na * sizeof(float), p->stream));
+    e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_amax), na * sizeof(float4), p->stream));
     if (!e) e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_ymax), ny * sizeof(float), p->stream));
-    if (!e) p->device_bytes += int64_t((na + ny) * sizeof(float));
+    if (!e) p->device_bytes += int64_t(na * sizeof(float4) + ny * sizeof(float));
   }
   if (!e && (p->grid_sep || p->degrid_sep)) {
     e = upload(p, &p->d_sep, sep.tab.data(), sep.tab.size());

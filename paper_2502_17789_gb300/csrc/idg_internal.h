@@ -133,8 +133,9 @@ __host__ __device__ inline int64_t tc_records(int n_groups, int nc) {
 
 // Separable-phasor kernels (sep_common.cuh): the staged records of a subgrid
 // are chunks of 16 visibilities of one segment (the last chunk of a segment
-// padded with zeros): 16 floats each of a fix, b fix, delta (sep_common.cuh) and
-// 1 / scale, then per correlation 16 each of Re and Im (48 bytes a visibility)
+// padded with zeros): 16 floats each of a fix, b fix, delta (sep_common.cuh), 16
+// of which the first 4 are the correlations' 1 / scale, then per correlation 16
+// each of Re and Im (48 bytes a visibility)
 constexpr int kGsepChunkVis = 16;
 constexpr int kGsepChunkFloat4 = 48;
 // gridder work item: 32 pixel columns x gsep_rows(L) rows
@@ -274,7 +275,7 @@ struct DegridArgs {
   const float2* scratch;      // [batch][4][L][L] subgrid images Y
   // separable-phasor degridder
   int* status = nullptr;          // device status word (kStatusTimeout)
-  const float* amax = nullptr;    // [n_int][n_st] largest component of the A-term's nodes
+  const float4* amax = nullptr;   // [n_int][n_st] largest component of each entry of the A-term's nodes
   const float* ymax = nullptr;    // [batch subgrids][4] largest component of the subgrid's planes
   const float2* w_ref = nullptr;  // [batch subgrids] reference w, a quarter of the largest squared distance from it
   int kv = 0;                     // visibilities per item
@@ -328,8 +329,8 @@ int launch_image_pass(int npol, const double2* in, double2* out, const double* w
 // one warp waits, bounded by limit_ns, on an mbarrier nothing completes; sets kStatusTimeout bit in *status
 int launch_wait_selftest(int* status, int64_t limit_ns, void* stream);
 // flags[i][s] = 1 when every node of A-term (interval i, station s) has zero off-diagonal entries;
-// amax[i][s] (may be null) its largest component
-int launch_aterm_flags(const float2* aterms, uint8_t* flags, float* amax, int n_int, int n_st, int nodes, void* stream);
+// amax[i][s] (may be null) the largest component of each of its entries
+int launch_aterm_flags(const float2* aterms, uint8_t* flags, float4* amax, int n_int, int n_st, int nodes, void* stream);
 // split: the items are of at most kSplitLanes lanes and run in the kernel that spreads each
 // visibility's pixels over several lanes (one block per item; persistent_blocks is ignored)
 int launch_degridder(int L, int channels, const DegridArgs& a, int n_items, int persistent_blocks, void* stream,

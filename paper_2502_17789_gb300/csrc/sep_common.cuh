@@ -220,10 +220,12 @@ __device__ __forceinline__ float sep_phase(int fix, int off, float delta, float 
 // slope in turns per pixel as a multiple of 2^-32 (whole turns wrap away)
 __device__ __forceinline__ int sep_fix(double turns) { return int(unsigned(__double2ll_rn(turns * 4294967296.0))); }
 
-// power of two that brings `m` into [512, 1024); 1 for 0, infinity and NaN
+// power of two that brings `m` into [8192, 16384); 1 for 0, infinity and NaN.  A complex product of values whose
+// components are bounded by `m` stays below 2^1.5 m = 46341 of a half's 65504, so that hi + lo halves keep 22 bits of
+// values down to 2^-13 of the largest, and an absolute 2^-38 of it below.
 __device__ __forceinline__ float sep_scale(float m) {
-  if (!(m > 0.f) || m > 3.4e38f) return 1.f;
-  const int e = 9 - ilogbf(m);
+  if (!(m > 0.f) || isinf(m)) return 1.f;
+  const int e = 13 - ilogbf(m);
   return ldexpf(1.f, e > 126 ? 126 : e);
 }
 
