@@ -632,6 +632,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     }
     sep_ok = sep_parts(p->exec, sep.x_max, p->part.w_step, n_timesteps, uvw_m, freqs_hz, aterm_offsets, &p->segs, &parts,
                        &w_ref);
+    if (sep_ok && !host_only) {
+      // a build whose register counts are not those the kernels' roles divide runs the general kernels
+      int blocks = 0;
+      int e = configure_gridder_sep(L, &blocks);
+      if (!e) e = configure_degridder_sep(L, &blocks);
+      if (e == int(cudaErrorInvalidConfiguration)) sep_ok = false;
+    }
   }
   // the default: gridder and degridder on the tensor cores (the gridder falls back to FP32 below where it
   // cannot run); both on FP32 when channel groups were asked for, and for Stokes I without the separable form

@@ -104,7 +104,7 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 // The block's first 256 threads (producers) write operands and issue MMAs, the
 // others (consumers) read the accumulators; each half has its own barrier.
 constexpr int kSepHalf = 256;
-constexpr int kSepProducerBar = 1, kSepConsumerBar = 2;  // + 2 for a second producer group
+constexpr int kSepProducerBar = 1, kSepConsumerBar = 2;
 __device__ __forceinline__ void half_sync(int bar) {
   asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory");
 }
@@ -188,11 +188,6 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-
-// complex numbers of two pixels, for packed f32x2 arithmetic
-struct c2 {
-  float2 re, im;
-};
 
 // the thread's warp as a value the compiler knows to be the same for the whole warp, so that a role taken by one
 // warp is a branch for the others and not predicated through
