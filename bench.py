@@ -63,8 +63,9 @@ MAC_NAMES = {1: "FP32 pipe (gridder and degridder)", 2: "tensor cores (gridder a
 
 
 def ncu_traffic_command(kern: str) -> str:
-    mac = {"gridder": " --mac-unit 3", "gridder_tc": " --mac-unit 2", "gridder_sep": " --mac-unit 2",
-           "degridder": " --mac-unit 1"}.get(kern, "")
+    # the workload's default plans run the separable kernels; a flat taper leaves them no w range
+    mac = {"gridder": " --mac-unit 3", "gridder_tc": " --mac-unit 2 --flat-taper", "gridder_sep": " --mac-unit 2",
+           "degridder": " --mac-unit 1", "degridder_tc": " --flat-taper"}.get(kern, "")
     return (f'ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none '
             f'--kernel-name-base demangled -k regex:"idg::{kern}_kernel<" -c 2 --csv '
             f'--log-file traffic_{kern}.csv {BENCH_SHORT} --stations {TRAFFIC_STATIONS}{mac}')
@@ -135,6 +136,9 @@ def parse_args():
     ap.add_argument("--mac-unit", type=int, default=0, choices=[0, 1, 2, 3],
                     help="the multiply-accumulate unit of the main, uneven and small legs (idg_geometry.mac_unit: 0 the library's default, "
                          "1 FP32 pipe, 2 tensor cores for both kernels, 3 tensor-core degridder only)")
+    ap.add_argument("--flat-taper", action="store_true",
+                    help="plan the main leg with a taper of 1 everywhere, which takes it to the kernels of one phasor per "
+                         "visibility and pixel (profiling)")
     ap.add_argument("--aterms", choices=["beam", "full"], default="beam",
                     help="beam: the scalar beam x screen gain (diagonal Jones); full: the same plus 5%% "
                          "polarisation leakage, so every Jones matrix is full")
@@ -522,7 +526,8 @@ def run_native(args):
     obs_r, shard = parallel.shard_observation(obs, rank, world)
     vis_d = vis_full if world == 1 else vis_full[torch.as_tensor(shard, device=dev)].contiguous()
     del vis_full
-    plan = idg.Plan(obs_r, stream=stream.cuda_stream, mac_unit=args.mac_unit)
+    plan = idg.Plan(obs_r, stream=stream.cuda_stream, mac_unit=args.mac_unit,
+                    taper_user=np.ones(obs_r.subgrid_size) if args.flat_taper else None)
     st = plan.stats()
     N = obs.grid_size
     G_model = torch.zeros((4, N, N), dtype=torch.complex128, device=dev)
@@ -580,7 +585,7 @@ def run_native(args):
     peak_tflops = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     achieved_vispx = vispx / (k_ms * 1e-3)
     achieved = achieved_vispx * FLOP_PER_VISPX / 1e12
-    separable = plan.kernels()[0] == idg.IDG_KERNEL_FACTORED
+    separable = plan.kernels()[0 if kern == "gridder" else 1] == idg.IDG_KERNEL_FACTORED
     kern_name = kernel_of(kern, int(st.mac_unit), separable)
     traffic = recorded_traffic(kern_name, desc)
     roofline = {"bound": "alu", "kernel": kern_name, "achieved": round(achieved, 3), "peak": round(peak_tflops, 3),
@@ -588,14 +593,17 @@ def run_native(args):
                 "peak_basis": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 FMA lanes x 2 flop x {sm_max:.0f} MHz (max SM clock)",
                 "achieved_vispx_per_s": achieved_vispx, "flop_per_vispx": FLOP_PER_VISPX,
                 "launches": k_launches, "avg_launch_ms": k_ms / max(k_launches, 1)}
-    if separable and peaks.get("bf16_tflops"):
-        # the separable kernels replace the direct sum's FP32 operations (`frac` above is against those and
-        # may pass 1) by f16 products on the tensor cores, at the measured rate of a 16-bit GEMM
-        t = achieved_vispx * SEP_FLOP_PER_VISPX / 1e12
-        roofline["tensor"] = {"achieved": round(t, 1), "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
-                              "frac": round(t / peaks["bf16_tflops"], 4), "flop_per_vispx": SEP_FLOP_PER_VISPX}
     if clocks.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = round(achieved / (peak_tflops * clocks["sm_mhz"] / sm_max), 4)
+    if separable and peaks.get("bf16_tflops"):
+        # the separable kernels take f16 products on the tensor cores in place of the direct sum's FP32 operations:
+        # the bound is the measured rate of a 16-bit GEMM; against the FP32 pipe the fraction may pass 1
+        direct = {k: roofline.pop(k) for k in ("achieved", "peak", "unit", "frac", "peak_basis", "flop_per_vispx")}
+        direct["frac_at_sampled_clock"] = roofline.pop("frac_at_sampled_clock", None)
+        t = achieved_vispx * SEP_FLOP_PER_VISPX / 1e12
+        roofline.update(bound="tensor", achieved=round(t, 1), peak=peaks["bf16_tflops"], unit="TFLOP/s",
+                        frac=round(t / peaks["bf16_tflops"], 4), peak_basis="measured 16-bit GEMM",
+                        flop_per_vispx=SEP_FLOP_PER_VISPX, direct_sum=direct)
     # the same fractions against the rates the library's probe kernels measure on this device (FP32
     # FMA and __sincosf throughput): R_vp = min(F_fma / 17, F_sincos), one sincos per visibility-pixel
     f_fma, f_sin = idg.idg_peak_rates(stream.cuda_stream)

@@ -8,7 +8,7 @@ tunable), the degridder's kind (tensor cores, or the FP32 pipe with 1, 2 or
 4 channels per lane: phasors of later channels by rotation) and whether the
 gridder also runs on the tensor cores, by timing a grid + degrid pass on the
 observation's own plans with CUDA events.  The search is staged: every (L,
-mode) with the library's defaults, then the chunk for the best (L, mode),
+mode) with the FP32 gridder and the tensor-core degridder, then the chunk for the best (L, mode),
 then the degridder's kind, then the gridder's unit.  The winner is cached in a JSON file keyed by the GPU and
 the observation's shape.  Changing L changes the partition and hence the
 numbers (legitimately: each L has its own oracle result); the other choices
@@ -30,7 +30,7 @@ MODES = ("blocks", "persistent")
 GRID_CHUNKS = (32, 48, 64)      # staged records per gridder chunk; 48 is the library's default
 DEGRID_CHANNELS = (1, 2, 4)     # channels per lane of the FP32 degridder
 # multiply-accumulate units (idg.h): 1 both kernels on FP32, 2 both on the tensor cores, 3 the degridder
-# on the tensor cores (the library's default)
+# on the tensor cores, the first stage's choice (the library's own default is 2 where that gridder runs)
 MAC_FP32, MAC_TENSOR, MAC_TENSOR_DEGRID = 1, 2, 3
 DEFAULT_CHUNK, DEFAULT_CHANNELS, DEFAULT_MAC = 48, 1, MAC_TENSOR_DEGRID
 
