@@ -283,14 +283,24 @@ constexpr double kSepFit[] = {0.12, 0.20, 0.28, 0.31, 0.32};
 
 struct SepFit {
   std::vector<float> tab;   // [4][L]: 2 pi A, 2 pi B, 2 pi p, q
-  std::vector<float2> n1;   // [j][i]
   float p_scale = 1.f;      // of 2 pi p (SepTables)
   double x_max = 0.0;       // largest |w - w_ref| (wavelengths) that meets kSepTolerance, kSepToleranceOuter and kSepPhase
 };
 
-SepFit sep_fit(int L, double fov, const std::vector<double>& taper, double h) {
+// n'(i,j) over the subgrid, [j][i]
+std::vector<double> pixel_n1(int L, double fov) {
+  std::vector<double> c(size_t(L) * L);
+  for (int j = 0; j < L; ++j)
+    for (int i = 0; i < L; ++i) {
+      const double l = double(i - L / 2) * fov / double(L), m = double(j - L / 2) * fov / double(L);
+      c[size_t(j) * L + i] = std::sqrt(1.0 - l * l - m * m) - 1.0;
+    }
+  return c;
+}
+
+SepFit sep_fit(int L, std::vector<double> c, const std::vector<double>& taper, double h) {
   SepFit f;
-  std::vector<double> w(L), c(size_t(L) * L), A(L), B(L), p(L), q(L, 1.0);
+  std::vector<double> w(L), A(L), B(L), p(L), q(L, 1.0);
   double tmax = 0.0, ww = 0.0;
   for (int i = 0; i < L; ++i) tmax = std::max(tmax, std::fabs(taper[i]));
   if (!(tmax > 0.0)) tmax = 1.0;
@@ -299,35 +309,25 @@ SepFit sep_fit(int L, double fov, const std::vector<double>& taper, double h) {
     w[i] = std::fabs(x) <= 1.0 ? 1.0 / std::sqrt(std::max(1.0 - x * x, 1.0 / (h * L))) : 0.0;
     ww += w[i];
   }
-  f.n1.resize(size_t(L) * L);
   for (int j = 0; j < L; ++j)
-    for (int i = 0; i < L; ++i) {
-      const double l = double(i - L / 2) * fov / double(L), m = double(j - L / 2) * fov / double(L);
-      const double n = std::sqrt(1.0 - l * l - m * m) - 1.0;
-      c[size_t(j) * L + i] = n;
-      f.n1[size_t(j) * L + i] = make_float2(float(n), float(n - double(float(n))));
-    }
-  for (int i = 0; i < L; ++i) {
-    for (int j = 0; j < L; ++j) A[i] += w[j] * c[size_t(j) * L + i];
-    A[i] /= ww;
-  }
+    for (int i = 0; i < L; ++i) A[i] += w[j] * c[size_t(j) * L + i];
+  for (double& v : A) v /= ww;
   for (int j = 0; j < L; ++j) {
     for (int i = 0; i < L; ++i) B[j] += w[i] * (c[size_t(j) * L + i] - A[i]);
     B[j] /= ww;
   }
   for (int j = 0; j < L; ++j)
     for (int i = 0; i < L; ++i) c[size_t(j) * L + i] -= A[i] + B[j];
-  // leading pair of the weighted remainder by alternating least squares
+  // leading pair of the weighted remainder by alternating least squares (the next pair is 1e-3 of it or less, so that an
+  // iteration gains six digits)
   for (int j = 0; j < L; ++j) q[j] = B[j] - B[L / 2];
-  for (int it = 0; it < 24; ++it) {
+  for (int it = 0; it < 3; ++it) {
     double qq = 0.0, pp = 0.0;
     for (int j = 0; j < L; ++j) qq += w[j] * q[j] * q[j];
-    for (int i = 0; i < L; ++i) {
-      p[i] = 0.0;
-      for (int j = 0; j < L; ++j) p[i] += w[j] * c[size_t(j) * L + i] * q[j];
-      p[i] = qq > 0.0 ? p[i] / qq : 0.0;
-      pp += w[i] * p[i] * p[i];
-    }
+    std::fill(p.begin(), p.end(), 0.0);
+    for (int j = 0; j < L && qq > 0.0; ++j)
+      for (int i = 0; i < L; ++i) p[i] += w[j] / qq * q[j] * c[size_t(j) * L + i];
+    for (int i = 0; i < L; ++i) pp += w[i] * p[i] * p[i];
     for (int j = 0; j < L; ++j) {
       q[j] = 0.0;
       for (int i = 0; i < L; ++i) q[j] += w[i] * c[size_t(j) * L + i] * p[i];
@@ -396,35 +396,41 @@ WRange w_range(const SubgridDesc& d, int t0, int t1, int c0, int c1, double w_st
 
 // The subgrids as the separable kernels work on them: one whose w range is
 // wider than 2 x_max is taken in parts of its timesteps or channels, each at
-// the subgrid's place with a reference w of its own and segments appended to
-// `seg` (subgrid images and visibilities add up, so only the order of
-// additions changes).  false when the parts would be more than twice the
-// subgrids (then the general kernels are the better ones), or for a NaN.
-bool sep_parts(const std::vector<SubgridDesc>& in, double x_max, double w_step, int n_t, const double* uvw_m,
-               const double* freqs_hz, const int32_t* aterm_offsets, std::vector<SegmentDesc>* seg,
-               std::vector<SubgridDesc>* out, std::vector<float2>* w_ref) {
+// the subgrid's place with a reference w and segments of its own (subgrid
+// images and visibilities add up, so only the order of additions changes).
+// false when the parts would be more than twice the subgrids (then the general
+// kernels are the better ones), or for a NaN.
+// `range` holds the subgrids' own ranges, `seg` their segments; those of parts go to `more` and are numbered behind `seg`.
+bool sep_parts(const std::vector<SubgridDesc>& in, const std::vector<WRange>& range, double x_max, double w_step, int n_t,
+               const double* uvw_m, const double* freqs_hz, const int32_t* aterm_offsets,
+               const std::vector<SegmentDesc>& seg, std::vector<SegmentDesc>* more, std::vector<SubgridDesc>* out,
+               std::vector<float2>* w_ref) {
   struct Part {
     int t0, t1, c0, c1;
   };
   std::vector<Part> todo;
-  out->reserve(in.size());
-  for (const SubgridDesc& d : in) {
+  out->reserve(in.size() + in.size() / 4);
+  w_ref->reserve(in.size() + in.size() / 4);
+  for (size_t o = 0; o < in.size(); ++o) {
+    const SubgridDesc& d = in[o];
     const int seg_begin = d.seg_begin, seg_count = d.seg_count;
+    bool whole = true;
     todo.assign(1, Part{d.t0, d.t1, d.c0, d.c1});
     while (!todo.empty()) {
       const Part s = todo.back();
       todo.pop_back();
-      const WRange w = w_range(d, s.t0, s.t1, s.c0, s.c1, w_step, n_t, uvw_m, freqs_hz);
+      const WRange w = whole ? range[o] : w_range(d, s.t0, s.t1, s.c0, s.c1, w_step, n_t, uvw_m, freqs_hz);
       const float mid = float(0.5 * (w.lo + w.hi));
       const double x = std::max(w.hi - double(mid), double(mid) - w.lo);
       if (!(x <= x_max)) {
+        whole = false;
         // halve what spreads w more; in time at the A-term interval nearest to the middle, if one is near, so that
         // no segment is cut
         const bool in_t = s.t1 - s.t0 > 1 && (w.t >= w.c || s.c1 - s.c0 == 1);
         const int half = (s.t0 + s.t1) / 2, cm = (s.c0 + s.c1) / 2;
         int tm = half, best = (s.t1 - s.t0) / 4 + 1;
         for (int k = seg_begin; k < seg_begin + seg_count; ++k) {
-          const int a = aterm_offsets[(*seg)[k].interval];
+          const int a = aterm_offsets[seg[k].interval];
           if (std::abs(a - half) < best && a > s.t0 && a < s.t1) {
             best = std::abs(a - half);
             tm = a;
@@ -438,7 +444,7 @@ bool sep_parts(const std::vector<SubgridDesc>& in, double x_max, double w_step, 
       }
       SubgridDesc e = d;
       e.rec_offset = int32_t(out->size());  // place in w_ref
-      if (s.t0 != d.t0 || s.t1 != d.t1 || s.c0 != d.c0 || s.c1 != d.c1) {
+      if (!whole) {
         e.t0 = s.t0;
         e.t1 = s.t1;
         e.c0 = s.c0;
@@ -446,13 +452,13 @@ bool sep_parts(const std::vector<SubgridDesc>& in, double x_max, double w_step, 
         const int width = s.c1 - s.c0;
         e.n_vis = (s.t1 - s.t0) * width;
         e.flags |= kSubgridPart;
-        e.seg_begin = int32_t(seg->size());
+        e.seg_begin = int32_t(seg.size() + more->size());
         for (int k = seg_begin; k < seg_begin + seg_count; ++k) {
-          const SegmentDesc g = (*seg)[k];
+          const SegmentDesc g = seg[k];
           const int a = std::max(aterm_offsets[g.interval], s.t0), b = std::min(aterm_offsets[g.interval + 1], s.t1);
-          if (a < b) seg->push_back(SegmentDesc{g.subgrid, g.interval, (a - s.t0) * width, (b - s.t0) * width});
+          if (a < b) more->push_back(SegmentDesc{g.subgrid, g.interval, (a - s.t0) * width, (b - s.t0) * width});
         }
-        e.seg_count = int32_t(seg->size()) - e.seg_begin;
+        e.seg_count = int32_t(seg.size() + more->size()) - e.seg_begin;
       }
       out->push_back(e);
       w_ref->push_back(make_float2(mid, float(0.25 * x * x)));
@@ -617,21 +623,25 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
   SepFit sep;
   std::vector<float2> w_ref;
   std::vector<SubgridDesc> parts;
+  std::vector<SegmentDesc> more;
+  std::vector<double> n1;
   bool sep_ok = false;
-  p->segs = p->part.segments;
   if (supported_subgrid_size(L)) {  // host-only plans take other sizes too
     double x = 0.0;  // largest half width of a subgrid's w range
+    std::vector<WRange> range;
+    range.reserve(p->exec.size());
     for (const SubgridDesc& d : p->exec) {
-      const WRange w = w_range(d, d.t0, d.t1, d.c0, d.c1, p->part.w_step, n_timesteps, uvw_m, freqs_hz);
-      x = std::max(x, 0.5001 * (w.hi - w.lo));  // and the rounding of w_ref
+      range.push_back(w_range(d, d.t0, d.t1, d.c0, d.c1, p->part.w_step, n_timesteps, uvw_m, freqs_hz));
+      x = std::max(x, 0.5001 * (range.back().hi - range.back().lo));  // and the rounding of w_ref
     }
+    n1 = pixel_n1(L, g->image_size);
     for (double h : kSepFit) {
-      const SepFit f = sep_fit(L, g->image_size, taper_d, h);
+      const SepFit f = sep_fit(L, n1, taper_d, h);
       if (sep.tab.empty() || f.x_max > sep.x_max) sep = f;
       if (sep.x_max >= x) break;
     }
-    sep_ok = sep_parts(p->exec, sep.x_max, p->part.w_step, n_timesteps, uvw_m, freqs_hz, aterm_offsets, &p->segs, &parts,
-                       &w_ref);
+    sep_ok = sep_parts(p->exec, range, sep.x_max, p->part.w_step, n_timesteps, uvw_m, freqs_hz, aterm_offsets,
+                       p->part.segments, &more, &parts, &w_ref);
     if (sep_ok && !host_only) {
       // a build whose register counts are not those the kernels' roles divide runs the general kernels
       int blocks = 0;
@@ -668,10 +678,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
   }
   p->sep_p_scale = sep.p_scale;
-  if (p->grid_sep || p->degrid_sep)
+  p->segs = p->part.segments;
+  if (p->grid_sep || p->degrid_sep) {
     p->exec = std::move(parts);
-  else
-    p->segs.resize(p->part.segments.size());
+    p->segs.insert(p->segs.end(), more.begin(), more.end());
+  }
   p->grid_chunk = g->grid_chunk > 0 ? g->grid_chunk : kDefaultGridChunk;
   for (SubgridDesc& d : p->exec) d.layer -= k_lo;  // device tables hold the grid plane set
   if (host_only) {
@@ -828,9 +839,11 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     if (!e) e = int(cudaMallocAsync(reinterpret_cast<void**>(&p->d_ymax), ny * sizeof(float), p->stream));
     if (!e) p->device_bytes += int64_t(na * sizeof(float4) + ny * sizeof(float));
   }
+  std::vector<float2> n1_f(n1.size());  // as two floats
+  for (size_t k = 0; k < n1.size(); ++k) n1_f[k] = make_float2(float(n1[k]), float(n1[k] - double(float(n1[k]))));
   if (!e && (p->grid_sep || p->degrid_sep)) {
     e = upload(p, &p->d_sep, sep.tab.data(), sep.tab.size());
-    if (!e) e = upload(p, &p->d_n1, sep.n1.data(), sep.n1.size());
+    if (!e) e = upload(p, &p->d_n1, n1_f.data(), n1_f.size());
     if (!e) e = upload(p, &p->d_wref, w_ref.data(), w_ref.size());
   }
   if (!e) e = upload(p, &p->d_sg, p->exec.data(), p->exec.size());
