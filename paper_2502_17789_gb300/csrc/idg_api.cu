@@ -1200,13 +1200,15 @@ namespace {
 
 // The plans of one grid_many / degrid_many call must share subgrid size,
 // planes per layer, normalisation, degridder channels per lane and the
-// multiply-accumulate unit: the one in use, or the one that is used where the
-// separable form does not hold.  Whether it holds follows from the uvw data, and
+// multiply-accumulate unit: all the one in use, or all the one that is used where
+// the separable form does not hold (the same answer for any order of the plans).
+// Whether it holds follows from the uvw data, and
 // neither a plan's neighbours nor the caller should have to know: plans of the
 // separable kernels and of the general ones run side by side, a launch each.
 idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, const void* const* b,
                       void* const* c, const char* an, const char* bn, const char* cn) {
   if (n < 1 || !plans || !a || !b || !c) return set_err(nullptr, IDG_ERR_INVALID_ARG, "NULL array or n < 1");
+  bool same_mac = true, same_general = true;
   for (int32_t k = 0; k < n; ++k) {
     idg_plan* p = plans[k];
     if (!p) return set_err(nullptr, IDG_ERR_INVALID_ARG, "a plan is NULL");
@@ -1215,9 +1217,11 @@ idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, c
     if ((st = check_buffer(p, a[k], an)) || (st = check_buffer(p, b[k], bn)) || (st = check_buffer(p, c[k], cn)))
       return st;
     const idg_plan* p0 = plans[0];
+    same_mac = same_mac && p->mac == p0->mac;
+    same_general = same_general && p->mac_general == p0->mac_general;
     if (p->L != p0->L || p->npol != p0->npol || (p->d_aweights != nullptr) != (p0->d_aweights != nullptr) ||
         p->degrid_channels != p0->degrid_channels || p->grid_chunk != p0->grid_chunk ||
-        (p->mac != p0->mac && p->mac_general != p0->mac_general))
+        !(same_mac || same_general))
       return set_err(p, IDG_ERR_INVALID_ARG,
                      "plans of one call must share subgrid size, Stokes-I mode, normalisation, grid_chunk, "
                      "degrid_channels and mac_unit");

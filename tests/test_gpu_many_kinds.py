@@ -1,6 +1,8 @@
 """grid_many / degrid_many over plans whose kernels differ: whether the
 phasors can be factored follows from each plan's own w range, so plans of one
 geometry may run different kernels and still share a call."""
+import itertools
+
 import numpy as np
 import pytest
 
@@ -117,6 +119,33 @@ def test_uniform_and_irregular_channels_share_a_call(idg_mod, cuda_device):
     try:
         assert plans[0].kernels() == plans[1].kernels() and plans[0].stats().mac_unit == plans[1].stats().mac_unit
         _same_as_alone(idg_mod, plans, obs_list)
+    finally:
+        for p in plans:
+            p.close()
+
+
+def test_answer_does_not_depend_on_the_order(idg_mod, cuda_device):
+    """Plans of uniform channels, of irregular ones inside the bound of the factored phasors and of irregular ones
+    outside share neither the unit in use nor the one without factored phasors, though each neighbour of the second
+    shares one with it: refused in every order.  Any two with the second in common are taken in both."""
+    obs_list = [_obs(seed=9), _obs(seed=10), _obs(seed=11, N=4096, **GENERAL)]
+    for o in obs_list[1:]:
+        o.freqs = o.freqs + np.linspace(0.0, 1.0, o.n_channels) ** 2 * 2e5
+    plans = [idg_mod.Plan(o, flags=idg_mod.IDG_W_LAYERS) for o in obs_list]
+    try:
+        F, T, P = idg_mod.IDG_KERNEL_FACTORED, idg_mod.IDG_KERNEL_TENSOR, idg_mod.IDG_KERNEL_FP32
+        assert [p.kernels() for p in plans] == [(F, F), (F, F), (P, T)]
+        A, V, G = _inputs(plans, obs_list)
+        for n in (2, 3):
+            for order in itertools.permutations(range(3), n):
+                p, v, a, g = ([x[k] for k in order] for x in (plans, V, A, G))
+                for call, args in ((idg_mod.grid_many, (p, v, a, g)), (idg_mod.degrid_many, (p, g, a, v))):
+                    if n == 2 and 1 in order:
+                        call(*args)
+                    else:
+                        with pytest.raises(idg_mod.IdgError) as e:
+                            call(*args)
+                        assert e.value.status == 1
     finally:
         for p in plans:
             p.close()
