@@ -72,14 +72,15 @@ int degridder_sep_vis_l(int nodes);
 template <int L>
 int configure_degridder_sep_l(int* persistent_blocks);
 template <int L>
-int launch_degridder_sep_l(const DegridArgs& a, int n_items, int blocks, void* stream);
+int launch_degridder_sep_l(const DegridArgs& a, int n_items, int blocks, bool few, void* stream);
 template <int L>
-int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* items, int n_items, int max_nodes, void* stream);
+int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* items, int n_items, int max_nodes, bool few,
+                                 void* stream);
 #define IDG_DEGRID_SEP_EXTERN(L)                                                                                 \
   extern template int degridder_sep_vis_l<L>(int);                                                              \
   extern template int configure_degridder_sep_l<L>(int*);                                                       \
-  extern template int launch_degridder_sep_l<L>(const DegridArgs&, int, int, void*);                            \
-  extern template int launch_degridder_sep_multi_l<L>(const DegridArgs*, const int2*, int, int, void*);
+  extern template int launch_degridder_sep_l<L>(const DegridArgs&, int, int, bool, void*);                      \
+  extern template int launch_degridder_sep_multi_l<L>(const DegridArgs*, const int2*, int, int, bool, void*);
 IDG_DEGRID_SEP_EXTERN(32)
 IDG_DEGRID_SEP_EXTERN(64)
 IDG_DEGRID_SEP_EXTERN(96)
@@ -105,14 +106,14 @@ int configure_degridder_sep(int L, int* persistent_blocks) {
   IDG_SWITCH_L(C_)
 #undef C_
 }
-int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int blocks, void* stream) {
-#define C_(X) launch_degridder_sep_l<X>(a, n_items, blocks, stream)
+int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int blocks, bool few, void* stream) {
+#define C_(X) launch_degridder_sep_l<X>(a, n_items, blocks, few, stream)
   IDG_SWITCH_L(C_)
 #undef C_
 }
 int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
-                               void* stream) {
-#define C_(X) launch_degridder_sep_multi_l<X>(args, blocks, n_blocks, max_nodes, stream)
+                               bool few, void* stream) {
+#define C_(X) launch_degridder_sep_multi_l<X>(args, blocks, n_blocks, max_nodes, few, stream)
   IDG_SWITCH_L(C_)
 #undef C_
 }

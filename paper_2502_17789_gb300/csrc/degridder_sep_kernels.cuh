@@ -58,6 +58,13 @@ static_assert(kDsepConsumer * kDsepProducerRegs + 128 * (kDsepConsumerRegs + kDs
               "registers");
 constexpr int kDsepColStride = 2 * kDsepMaxVis;       // between the two accumulators (re, im)
 constexpr int kDsepZCol = 2 * kDsepColStride;         // first column of the Z ring
+// Items of few visibilities have a kernel of their own (idg_plan_create says which), which keeps the accuracy of the FP32
+// kernels that take them elsewhere (errors of single-channel plans at L = 32 .. 128: 3.2 .. 5.0e-7 without it, 2.4 ..
+// 3.0e-7 with it, 2.3 .. 3.7e-7 on FP32): the corrections have accumulators of their own (sep_product) in the columns
+// that the visibilities leave, and the F side exact sines and cosines.  As branches of the one kernel they cost its
+// regular items 8 % (22.8 ms on the MWA-like workload).
+constexpr int kDsepFewCorr = kDsepMaxVis;   // columns from the sums to the corrections
+static_assert(kDsepFewVis % 16 == 0 && 2 * kDsepFewVis <= kDsepFewCorr, "corrections beside the sums");
 constexpr uint32_t kDsepTmemCols = 512;
 static_assert(kDsepZCol + kDsepRing * 48 <= int(kDsepTmemCols), "tensor memory");
 
@@ -96,7 +103,7 @@ int dsep_vis(int nodes) {
   return kv;
 }
 
-template <int L>
+template <int L, bool FEW>
 struct Dsep {
   const DegridArgs& a;
   DsepShared& S;
@@ -105,6 +112,7 @@ struct Dsep {
   const SepShare share;
 
   static constexpr int kBlocks = L / 32, kPieces = L / 16;
+  static constexpr int kGroups16 = (FEW ? kDsepFewVis : kDsepMaxVis) / 16;
 
   template <int SLEEP = 32>
   __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) {
@@ -316,8 +324,8 @@ struct Dsep {
           tc_fence_after();
           __syncwarp();
           if (elect_one()) {
-            sep_product(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48, f0 + jc * chunk, n_pad, block, group,
-                        level, jc == 0);
+            sep_product<FEW ? kDsepFewCorr : 0>(tm + (dg & 1) * kDsepColStride, tm + kDsepZCol + slot * 48,
+                                                f0 + jc * chunk, n_pad, block, group, level, jc == 0);
             sep_commit(&S.empty[slot]);
             if (jc + 1 == kPieces) sep_commit(&S.full[dg & 1]);
           }
@@ -400,8 +408,13 @@ struct Dsep {
           const int w = 2 * u + h, off = 8 * o + 2 * w - L / 2;
           const float2 fb = pair_of(b4, h), fq = pair_of(q4, h);
           float2 c, s;
-          __sincosf(sep_phase(fix, off, dl, fb.x), &s.x, &c.x);
-          __sincosf(sep_phase(fix, off + 1, dl, fb.y), &s.y, &c.y);
+          if (FEW) {
+            sep_sincos_exact(fix, off, dl, fb.x, &s.x, &c.x);
+            sep_sincos_exact(fix, off + 1, dl, fb.y, &s.y, &c.y);
+          } else {
+            __sincosf(sep_phase(fix, off, dl, fb.x), &s.x, &c.x);
+            __sincosf(sep_phase(fix, off + 1, dl, fb.y), &s.y, &c.y);
+          }
           const __half2 d2 = __floats2half2_rn(-dp * fq.x, -dp * fq.y);
           const __half2 hc = sep_split(c, f.r_hi[w], f.r_lo[w]);
           const __half2 hs = sep_split(s, f.i_hi[w], f.i_lo[w]);
@@ -435,10 +448,10 @@ struct Dsep {
       const DegridItem item = a.items[idx];
       const int nv = item.k_end - item.k_begin, n_pad = (nv + 15) & ~15, b = n & 1;
       wait(&S.ready[b], (n >> 1) & 1);
-      const float inv = sep_unbias(kPieces) / S.info[b].scale[pol];
-      float sum[kDsepMaxVis / 16];  // component lane & 1 of visibility 16 h + lane / 2
+      const float inv = sep_unbias(FEW ? 0.25f * kPieces : float(kPieces)) / S.info[b].scale[pol];
+      float sum[kGroups16];  // component lane & 1 of visibility 16 h + lane / 2
 #pragma unroll
-      for (int h = 0; h < kDsepMaxVis / 16; ++h) sum[h] = 0.f;
+      for (int h = 0; h < kGroups16; ++h) sum[h] = 0.f;
 #pragma unroll 1
       for (int ib = 0; ib < kBlocks; ++ib, ++dg) {
         const int i = ib * 32 + lane;
@@ -447,7 +460,7 @@ struct Dsep {
         tc_fence_after();
         const uint32_t d = S.tmem + (uint32_t(pol * 32) << 16) + (dg & 1) * kDsepColStride;
 #pragma unroll
-        for (int h = 0; h < kDsepMaxVis / 16; ++h) {
+        for (int h = 0; h < kGroups16; ++h) {
           const int k0 = 16 * h;
           if (k0 < n_pad) {
             float v[32];  // (re, im) of 16 visibilities
@@ -456,6 +469,17 @@ struct Dsep {
               tmem_ld16(dr, d + k0);
               tmem_ld16(di, d + n_pad + k0);
               tmem_wait_ld();
+              if (FEW) {
+                float cr[16], ci[16];
+                tmem_ld16(cr, d + kDsepFewCorr + k0);
+                tmem_ld16(ci, d + kDsepFewCorr + n_pad + k0);
+                tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                  dr[k] += cr[k];
+                  di[k] += ci[k];
+                }
+              }
               const float4* fx = reinterpret_cast<const float4*>(&S.fix_a[b][k0]);
               const float4* dl = reinterpret_cast<const float4*>(&S.delta[b][k0]);
 #pragma unroll
@@ -487,7 +511,7 @@ struct Dsep {
         if (lane == 0) mbar_arrive(&S.drained[dg & 1]);
       }
 #pragma unroll
-      for (int h = 0; h < kDsepMaxVis / 16; ++h)
+      for (int h = 0; h < kGroups16; ++h)
         if (16 * h < n_pad) S.out[16 * h + (lane >> 1)][2 * pol + (lane & 1)] = inv * sum[h];
       asm volatile("bar.sync %0, 128;" ::"n"(kSepConsumerBar) : "memory");
       if (tid < nv) {
@@ -506,7 +530,7 @@ struct Dsep {
   }
 };
 
-template <int L>
+template <int L, bool FEW = false>
 __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShare share, unsigned char* smem) {
   DsepShared& S = *reinterpret_cast<DsepShared*>(smem);
   unsigned char* fside = reinterpret_cast<unsigned char*>(&S + 1);
@@ -530,7 +554,7 @@ __device__ __forceinline__ void degridder_sep_block(const DegridArgs& a, SepShar
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  Dsep<L> it{a, S, fside, reinterpret_cast<float4*>(fside + size_t(2) * a.kv * L * 12), share};
+  Dsep<L, FEW> it{a, S, fside, reinterpret_cast<float4*>(fside + size_t(2) * a.kv * L * 12), share};
   if (threadIdx.x < kDsepConsumer) {
     regs_give<kDsepProducerRegs>();
     it.producer();
@@ -573,15 +597,38 @@ __global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_multi_kernel(co
   degridder_sep_block<L>(a, SepShare{it.y * a.run, a.n_items, a.stride, a.run}, sep_smem);
 }
 
+// The same two for items of at most kDsepFewVis visibilities
+template <int L>
+__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_few_kernel(const DegridArgs a) {
+  extern __shared__ __align__(128) unsigned char sep_smem[];
+  degridder_sep_block<L, true>(a, SepShare{int(blockIdx.x) * a.run, a.n_items, int(gridDim.x), a.run}, sep_smem);
+}
+
+template <int L>
+__global__ void __launch_bounds__(kDsepThreads, 1) degridder_sep_few_multi_kernel(const DegridArgs* args,
+                                                                                const int2* blocks) {
+  extern __shared__ __align__(128) unsigned char sep_smem[];
+  __shared__ __align__(16) unsigned char s_args_raw[sizeof(DegridArgs)];
+  const int2 it = blocks[blockIdx.x];
+  if (threadIdx.x == 0) memcpy(s_args_raw, args + it.x, sizeof(DegridArgs));
+  __syncthreads();
+  const DegridArgs& a = *reinterpret_cast<const DegridArgs*>(s_args_raw);
+  degridder_sep_block<L, true>(a, SepShare{it.y * a.run, a.n_items, a.stride, a.run}, sep_smem);
+}
+
 template <int L>
 int configure_degridder_sep_l(int* persistent_blocks) {
   // the roles' register split is of the registers the block is launched with
-  cudaError_t e = sep_check_regs(degridder_sep_kernel<L>, kDsepLaunchRegs);
-  if (e == cudaSuccess) e = sep_check_regs(degridder_sep_multi_kernel<L>, kDsepLaunchRegs);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(degridder_sep_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kSepSmemLimit);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(degridder_sep_multi_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSepSmemLimit);
+  cudaError_t e = cudaSuccess;
+  const auto configure = [&e](auto kernel) {
+    if (e == cudaSuccess) e = sep_check_regs(kernel, kDsepLaunchRegs);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSepSmemLimit);
+  };
+  configure(degridder_sep_kernel<L>);
+  configure(degridder_sep_multi_kernel<L>);
+  configure(degridder_sep_few_kernel<L>);
+  configure(degridder_sep_few_multi_kernel<L>);
   int dev = 0, sms = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -595,16 +642,20 @@ int degridder_sep_vis_l(int nodes) {
 }
 
 template <int L>
-int launch_degridder_sep_l(const DegridArgs& args, int n_items, int blocks, void* stream) {
+int launch_degridder_sep_l(const DegridArgs& args, int n_items, int blocks, bool few, void* stream) {
   if (n_items <= 0) return 0;
   DegridArgs a = args;
   a.n_items = n_items;
-  degridder_sep_kernel<L><<<blocks, kDsepThreads, dsep_smem<L>(a.kv, a.g.nodes), cudaStream_t(stream)>>>(a);
+  const size_t smem = dsep_smem<L>(a.kv, a.g.nodes);
+  if (few)
+    degridder_sep_few_kernel<L><<<blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(a);
+  else
+    degridder_sep_kernel<L><<<blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(a);
   return int(cudaGetLastError());
 }
 
 template <int L>
-int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
+int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes, bool few,
                                  void* stream) {
   if (n_blocks <= 0) return 0;
   size_t smem = 0;  // the largest layout of any plan of up to max_nodes (a plan's items are cut to its own)
@@ -612,7 +663,10 @@ int launch_degridder_sep_multi_l(const DegridArgs* args, const int2* blocks, int
     const size_t s = dsep_smem<L>(dsep_vis<L>(n), n);
     smem = s > smem ? s : smem;
   }
-  degridder_sep_multi_kernel<L><<<n_blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(args, blocks);
+  if (few)
+    degridder_sep_few_multi_kernel<L><<<n_blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(args, blocks);
+  else
+    degridder_sep_multi_kernel<L><<<n_blocks, kDsepThreads, smem, cudaStream_t(stream)>>>(args, blocks);
   return int(cudaGetLastError());
 }
 

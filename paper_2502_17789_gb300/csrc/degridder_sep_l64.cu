@@ -5,7 +5,7 @@ namespace idg {
 
 template int configure_degridder_sep_l<64>(int*);
 template int degridder_sep_vis_l<64>(int);
-template int launch_degridder_sep_l<64>(const DegridArgs&, int, int, void*);
-template int launch_degridder_sep_multi_l<64>(const DegridArgs*, const int2*, int, int, void*);
+template int launch_degridder_sep_l<64>(const DegridArgs&, int, int, bool, void*);
+template int launch_degridder_sep_multi_l<64>(const DegridArgs*, const int2*, int, int, bool, void*);
 
 }  // namespace idg

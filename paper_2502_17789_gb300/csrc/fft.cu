@@ -211,8 +211,9 @@ __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) f
 }
 
 // degrid-direction: copy the subgrid's footprint out of the master grid
-// (FP64 -> FP32, times (-1)^(x+y)) and inverse-transform it into scratch
-template <int L>
+// (FP64 -> FP32, times (-1)^(x+y)) and inverse-transform it into scratch; EXACT: FftArgs.exact (as a branch it costs
+// the others 2 % of a small call)
+template <int L, bool EXACT>
 __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) splitter_ifft_kernel(const FftArgs a) {
   constexpr int T = FftShape<L>::kThreads, P = L + 1;
   extern __shared__ float2 sbuf[];
@@ -247,8 +248,8 @@ __global__ void __launch_bounds__(FftShape<L>::kThreads, FftShape<L>::kBlocks) s
     const float2 v0 = buf[fft_place<L>(2 * jp) * P + ip], v1 = buf[fft_place<L>(2 * jp + 1) * P + ip];
     const float ti = a.taper[i] * ((i & 1) ? -1.f : 1.f), t0 = ti * a.taper[2 * jp], t1 = -ti * a.taper[2 * jp + 1];
     const float fit_p = __ldg(a.sep.p + i);
-    const float2 p0 = sep_pixel(w_ref, __ldg(a.sep.n1 + 2 * jp * L + i), fit_p * __ldg(a.sep.q + 2 * jp));
-    const float2 p1 = sep_pixel(w_ref, __ldg(a.sep.n1 + (2 * jp + 1) * L + i), fit_p * __ldg(a.sep.q + 2 * jp + 1));
+    const float2 p0 = sep_pixel(w_ref, __ldg(a.sep.n1 + 2 * jp * L + i), fit_p * __ldg(a.sep.q + 2 * jp), EXACT);
+    const float2 p1 = sep_pixel(w_ref, __ldg(a.sep.n1 + (2 * jp + 1) * L + i), fit_p * __ldg(a.sep.q + 2 * jp + 1), EXACT);
     const float2 re = make_float2(t0 * (v0.x * p0.x + v0.y * p0.y), t1 * (v1.x * p1.x + v1.y * p1.y));
     const float2 im = make_float2(t0 * (v0.y * p0.x - v0.x * p0.y), t1 * (v1.y * p1.x - v1.x * p1.y));
     m = fmaxf(fmaxf(fmaxf(m, fabsf(re.x)), fabsf(re.y)), fmaxf(fabsf(im.x), fabsf(im.y)));
@@ -300,11 +301,14 @@ static int configure_t() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(fft_adder_kernel<L, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(splitter_ifft_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = cudaFuncSetAttribute(splitter_ifft_kernel<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(splitter_ifft_kernel<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   // shared memory is what bounds these kernels' occupancy: ask for the largest carveout
-  const void* fns[3] = {reinterpret_cast<const void*>(fft_adder_kernel<L, 0>),
+  const void* fns[4] = {reinterpret_cast<const void*>(fft_adder_kernel<L, 0>),
                         reinterpret_cast<const void*>(fft_adder_kernel<L, 1>),
-                        reinterpret_cast<const void*>(splitter_ifft_kernel<L>)};
+                        reinterpret_cast<const void*>(splitter_ifft_kernel<L, false>),
+                        reinterpret_cast<const void*>(splitter_ifft_kernel<L, true>)};
   for (const void* fn : fns)
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
@@ -334,7 +338,10 @@ static int fft_adder_t(const FftArgs& a, int n, int mode, void* stream) {
 template <int L>
 static int splitter_t(const FftArgs& a, int n, void* stream) {
   if (n <= 0) return 0;
-  splitter_ifft_kernel<L><<<n * a.npol, FftShape<L>::kThreads, fft_smem<L>(), cudaStream_t(stream)>>>(a);
+  if (a.exact)
+    splitter_ifft_kernel<L, true><<<n * a.npol, FftShape<L>::kThreads, fft_smem<L>(), cudaStream_t(stream)>>>(a);
+  else
+    splitter_ifft_kernel<L, false><<<n * a.npol, FftShape<L>::kThreads, fft_smem<L>(), cudaStream_t(stream)>>>(a);
   return int(cudaGetLastError());
 }
 

@@ -275,7 +275,7 @@ __device__ __forceinline__ void gsep_consumer(const GridArgs& a, SepShare share,
       const int n = gsep_part(left);
       diag_next = a.adiag[sp] & a.adiag[sq];
       // the scale of the segment's values and the accumulation's bias, undone on the way to S.x
-      inv_next = __ldg(rec) * sep_unbias(n);
+      inv_next = __ldg(rec) * sep_unbias(float(n));
       rec += size_t(n) * kGsepChunkFloat4 * 4;
       left -= n;
       if (left == 0 && ++s < sd.seg_count) seg = a.seg[sd.seg_begin + s];

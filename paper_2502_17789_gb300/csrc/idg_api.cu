@@ -56,6 +56,7 @@ struct idg_plan {
   bool grid_sep = false;             // separable-phasor gridder (sep_common.cuh)
   bool degrid_sep = false;           // and degridder
   int32_t degrid_vis = 0;            // its visibilities per item
+  int32_t degrid_few = 0;            // items of up to this many are for its kernel for few visibilities
   int32_t sms = 1;
   bool grid_tc = false;              // gridder on the tensor cores without it (mac, uniform channels, no A-term normalisation)
   cudaStream_t stream = nullptr;
@@ -672,7 +673,13 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
     const bool tc_ok = uniform && !(g->flags & IDG_NORMALIZE_ATERM);
     p->mac_general = unit(false) == IDG_MAC_TENSOR && !tc_ok ? IDG_MAC_TENSOR_DEGRID : unit(false);
     p->degrid_sep = p->mac != IDG_MAC_FP32 && sep_ok;
-    if (p->degrid_sep) p->degrid_vis = degridder_sep_vis(L, g->aterm_nodes);
+    if (p->degrid_sep) {
+      p->degrid_vis = degridder_sep_vis(L, g->aterm_nodes);
+      // Stokes I has FP32 sums elsewhere, whose errors the regular separable kernel stays below up to L = 96 (3.0, 3.4,
+      // 3.8 against 3.6, 3.5, 3.8e-7) but not at 128 (4.5 against 4.0; the one for few visibilities 3.1)
+      p->degrid_few = kSplitLanes;
+      if (p->npol == 1 && L == 128) p->degrid_few = p->degrid_vis = std::min(p->degrid_vis, kDsepFewVis);
+    }
     p->grid_sep = p->mac == IDG_MAC_TENSOR && sep_ok && !(g->flags & IDG_NORMALIZE_ATERM);
     p->grid_tc = p->mac == IDG_MAC_TENSOR && !p->grid_sep && tc_ok;
     if (p->mac == IDG_MAC_TENSOR && !p->grid_sep && !p->grid_tc) p->mac = IDG_MAC_TENSOR_DEGRID;  // the units in use
@@ -778,10 +785,16 @@ idg_status idg_plan_create(idg_plan** out, const idg_geometry* g, int32_t n_stat
       }
     }
     // items of at most kSplitLanes lanes go last, for the kernel that spreads a visibility over
-    // several lanes; both parts keep the longest-first order
-    const auto few = [&](const DegridItem& it) { return !p->degrid_sep && it.k_end - it.k_begin <= kSplitLanes; };
-    std::stable_partition(ditems.begin() + d_first, ditems.end(), [&](const DegridItem& it) { return !few(it); });
-    const size_t n_small = size_t(std::count_if(ditems.begin() + d_first, ditems.end(), few));
+    // several lanes (or the separable one for few visibilities, kDsepFewVis); both parts keep the longest-first order
+    const int few_max = p->degrid_sep ? p->degrid_few : kSplitLanes;
+    const auto few = [&](const DegridItem& it) { return it.k_end - it.k_begin <= few_max; };
+    size_t n_small = size_t(std::count_if(ditems.begin() + d_first, ditems.end(), few));
+    // the separable kernels' items are told apart for accuracy only: few small ones among others take the others' (a
+    // second launch costs 6 % of a call on 64 stations)
+    if (p->degrid_sep && 2 * n_small < ditems.size() - d_first)
+      n_small = 0;
+    else
+      std::stable_partition(ditems.begin() + d_first, ditems.end(), [&](const DegridItem& it) { return !few(it); });
     b.gi_count = int32_t(gitems.size()) - b.gi_offset;
     b.ds_count = int32_t(n_small);
     b.di_count = int32_t(ditems.size()) - b.di_offset - b.ds_count;
@@ -1022,6 +1035,7 @@ static FftArgs splitter_args(const idg_plan* p, const Batch& b, const void* grid
     fa.w_ref = p->d_wref + b.sg_offset;
     fa.taper = p->d_taper;
     fa.sep = sep_tables(p);
+    fa.exact = p->npol == 1 || b.ds_count > 0;
   }
   return fa;
 }
@@ -1087,7 +1101,7 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
     da.run = sep_run(plan, b.di_count);
     e = timed(plan, kDegridder, [&] {
       if (plan->degrid_sep)
-        return launch_degridder_sep(L, da, b.di_count, sep_blocks(plan, b.di_count, da.run), plan->stream);
+        return launch_degridder_sep(L, da, b.di_count, sep_blocks(plan, b.di_count, da.run), false, plan->stream);
       if (plan->mac != IDG_MAC_FP32)
         return launch_degridder_tc(L, da, b.di_count, plan->persistent_degrid_blocks, plan->stream);
       return launch_degridder(L, plan->degrid_channels, da, b.di_count, plan->persistent_degrid_blocks,
@@ -1098,7 +1112,10 @@ idg_status idg_degrid(idg_plan* plan, const void* grid_c128, const void* aterms_
       DegridArgs ds = da;
       ds.items = plan->d_ditems + b.di_offset + b.di_count;
       ds.n_items = b.ds_count;
+      ds.run = sep_run(plan, b.ds_count);
       e = timed(plan, kDegridder, [&] {
+        if (plan->degrid_sep)
+          return launch_degridder_sep(L, ds, b.ds_count, sep_blocks(plan, b.ds_count, ds.run), true, plan->stream);
         return launch_degridder(L, plan->degrid_channels, ds, b.ds_count, 0, plan->stream, true);
       });
       if (e) return cuda_err(plan, e, "degridder launch (items of few lanes)");
@@ -1230,6 +1247,9 @@ idg_status check_many(int32_t n, idg_plan* const* plans, const void* const* a, c
   }
   return IDG_OK;
 }
+
+// beside IDG_KERNEL_*: the separable degridder for items of few visibilities
+constexpr int kFactoredFew = 4;
 
 // The counts of the slots whose kernel is `kind`, 0 for the others
 std::vector<int32_t> of_kind(const std::vector<int32_t>& count, const std::vector<int>& slot_kind, int kind) {
@@ -1401,13 +1421,25 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
       cost.push_back(p->dcost.data() + b.di_offset);
       count.push_back(b.di_count);
       cost_s.push_back(p->dcost.data() + b.di_offset + b.di_count);
-      count_s.push_back(b.ds_count);
+      count_s.push_back(p->degrid_sep ? 0 : b.ds_count);
+      if (p->degrid_sep && b.ds_count > 0) {  // a slot of their own: their blocks have a stride of their own
+        kind.push_back(kFactoredFew);
+        args.push_back(da);
+        args.back().items += b.di_count;
+        args.back().n_items = b.ds_count;
+        cost.push_back(cost_s.back());
+        count.push_back(b.ds_count);
+        cost_s.push_back(nullptr);
+        count_s.push_back(0);
+      }
     }
     // a launch per kernel that these plans use; then the items of few lanes (the general kernels' plans), which
     // index their plan's item table past the regular ones
-    std::vector<int32_t> strides;
+    std::vector<int32_t> strides, strides_few;
     std::vector<int2> items = share_blocks(plans[0], of_kind(count, kind, IDG_KERNEL_FACTORED), &strides);
-    for (size_t s = 0; s < args.size(); ++s) args[s].stride = strides[s];
+    const size_t n_wide = items.size();
+    for (int2 it : share_blocks(plans[0], of_kind(count, kind, kFactoredFew), &strides_few)) items.push_back(it);
+    for (size_t s = 0; s < args.size(); ++s) args[s].stride = kind[s] == kFactoredFew ? strides_few[s] : strides[s];
     const size_t n_sep = items.size();
     for (int2 it : merge_items(cost, of_kind(count, kind, IDG_KERNEL_TENSOR))) items.push_back(it);
     const size_t n_tc = items.size() - n_sep;
@@ -1417,7 +1449,8 @@ idg_status idg_degrid_many(int32_t n, idg_plan* const* plans, const void* const*
     DegridArgs* d_args = nullptr;
     int2* d_items = nullptr;
     int e = upload_wave(strm, args, items, &d_args, &d_items);
-    if (!e) e = launch_degridder_sep_multi(L, d_args, d_items, int(n_sep), max_nodes, strm);
+    if (!e) e = launch_degridder_sep_multi(L, d_args, d_items, int(n_wide), max_nodes, false, strm);
+    if (!e) e = launch_degridder_sep_multi(L, d_args, d_items + n_wide, int(n_sep - n_wide), max_nodes, true, strm);
     if (!e) e = launch_degridder_tc_multi(L, d_args, d_items + n_sep, int(n_tc), max_nodes, strm);
     if (!e)
       e = launch_degridder_multi(L, plans[0]->degrid_channels, false, d_args, d_items + n_sep + n_tc,

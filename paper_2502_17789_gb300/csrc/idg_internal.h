@@ -79,6 +79,8 @@ constexpr int kDegridSegs = 2;  // segments per degridder work item
 // degridder items of at most this many lanes run in the kernel that spreads a
 // visibility over several lanes (low occupancy)
 constexpr int kSplitLanes = 8;
+// the separable degridder's kernel for items of few visibilities takes up to this many
+constexpr int kDsepFewVis = 32;
 constexpr int kTcItemRows = 256;  // rows (16-row tiles) per item of the tensor-core degridder
 
 // channels per run of rotated phasors (one fresh evaluation per run bounds
@@ -298,6 +300,7 @@ struct FftArgs {
   const float2* w_ref = nullptr;
   const float* taper = nullptr;
   SepTables sep;
+  bool exact = false;      // sine and cosine of sep_pixel to a unit in the last place
 };
 
 // how long a device-side wait lasts before the kernel reports a timeout (idg_set_wait_limit)
@@ -353,11 +356,12 @@ int launch_gridder_sep_multi(int L, const GridArgs* args, const int2* blocks, in
 int configure_degridder_tc(int L, int nodes, int* persistent_blocks);
 int launch_degridder_tc_multi(int L, const DegridArgs* args, const int2* items, int n_items, int max_nodes,
                               void* stream);
-// the separable-phasor degridder: items of up to degridder_sep_vis visibilities of one segment
+// the separable-phasor degridder: items of up to degridder_sep_vis visibilities of one segment; few: of at most
+// kDsepFewVis
 int degridder_sep_vis(int L, int nodes);
 int configure_degridder_sep(int L, int* persistent_blocks);
-int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int blocks, void* stream);
-int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes,
+int launch_degridder_sep(int L, const DegridArgs& a, int n_items, int blocks, bool few, void* stream);
+int launch_degridder_sep_multi(int L, const DegridArgs* args, const int2* blocks, int n_blocks, int max_nodes, bool few,
                                void* stream);
 // mode 0: FFT + add into grid; mode 1: FFT in place in scratch (inspection)
 int launch_fft_adder(int L, const FftArgs& a, int n_subgrids, int mode, void* stream);

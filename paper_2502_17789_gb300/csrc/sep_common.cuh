@@ -61,7 +61,7 @@ __device__ __forceinline__ void sep_mma(uint32_t d, uint32_t a, uint64_t b, uint
 // mean, and chains are kept short (kSepMaxChain chunks of 8 MMAs in the gridder, L / 16 in the degridder): the grid's
 // error against 64 bits at L = 96 falls from 9.7e-7 to 5e-7, and does not grow with the length of a segment.
 constexpr int kSepMaxChain = 8;
-__device__ __forceinline__ float sep_unbias(int chunks) { return fmaf(1.7e-8f * 8.f, float(chunks), 1.f); }
+__device__ __forceinline__ float sep_unbias(float chunks) { return fmaf(1.7e-8f * 8.f, chunks, 1.f); }
 
 // arrive on `bar` when every MMA issued so far by this thread has completed
 __device__ __forceinline__ void sep_commit(uint64_t* bar) {
@@ -212,6 +212,12 @@ __device__ __forceinline__ float sep_phase(int fix, int off, float delta, float 
   return fmaf(float(int(unsigned(fix) * unsigned(off))), kTurnsToRad, delta * fit);
 }
 
+// the same phase's sine and cosine to a unit in the last place (half turns, sincospif): __sincosf's absolute error of 2^-21
+// is the largest of the factored form, which takes three of them where one phasor per visibility and pixel takes one
+__device__ __forceinline__ void sep_sincos_exact(int fix, int off, float delta, float fit, float* s, float* c) {
+  sincospif(fmaf(float(int(unsigned(fix) * unsigned(off))), 4.656612873077393e-10f, delta * fit * 0.3183098861837907f), s, c);
+}
+
 // slope in turns per pixel as a multiple of 2^-32 (whole turns wrap away)
 __device__ __forceinline__ int sep_fix(double turns) { return int(unsigned(__double2ll_rn(turns * 4294967296.0))); }
 
@@ -265,29 +271,37 @@ __device__ __forceinline__ void sep_store_f(const SepF& f, uint32_t dst, uint32_
 // Re first order, Im first order) of 8 columns each, the F side in shared memory (sep_store_f, k groups `group`
 // bytes apart), D = re at column d and im at d + n, n columns each.  Products lo hi, hi lo, first order, hi hi; all
 // MMAs on one accumulator have the same shape, so they run in the order of issue.
+// CORR: columns from d to an accumulator of its own for all but hi hi, or 0: the truncations then happen at the
+// corrections' magnitude, and 2 of 8 MMAs a chunk truncate the sum itself.
+template <uint32_t CORR = 0>
 __device__ __forceinline__ void sep_product(uint32_t d, uint32_t e, uint32_t f, int n, uint32_t block, uint32_t group,
                                             uint32_t level, bool first) {
   const uint32_t add = sep_idesc(n), sub = sep_idesc(n, true);
   const uint32_t el[4] = {1, 0, 2, 0}, fl[4] = {0, 1, 2, 0};
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
-    const uint32_t ea = e + el[t] * 16, fa = f + fl[t] * level, acc = (first && t == 0) ? 0u : 1u;
+    const uint32_t ea = e + el[t] * 16, fa = f + fl[t] * level;
+    const uint32_t acc = first && (t == 0 || (t == 3 && CORR)) ? 0u : 1u, dt = t < 3 ? d + CORR : d;
     const uint64_t fr = sep_desc(fa, group), fi = sep_desc(fa + block, group);
-    sep_mma(d, ea, fr, add, acc);           // re += Re E Re F
-    sep_mma(d + n, ea, fi, add, acc);       // im += Re E Im F
-    sep_mma(d, ea + 8, fi, sub, 1u);        // re -= Im E Im F
-    sep_mma(d + n, ea + 8, fr, add, 1u);    // im += Im E Re F
+    sep_mma(dt, ea, fr, add, acc);           // re += Re E Re F
+    sep_mma(dt + n, ea, fi, add, acc);       // im += Re E Im F
+    sep_mma(dt, ea + 8, fi, sub, 1u);        // re -= Im E Im F
+    sep_mma(dt + n, ea + 8, fr, add, 1u);    // im += Im E Re F
   }
 }
 
-// P of a pixel: w = (w_ref, x^2 / 4), the two-float n' (exact range reduction), 2 pi p_i q_j
-__device__ __forceinline__ float2 sep_pixel(float2 w, float2 n1, float pq) {
+// P of a pixel: w = (w_ref, x^2 / 4), the two-float n' (exact range reduction), 2 pi p_i q_j; exact: sine and cosine to
+// a unit in the last place (sep_sincos_exact)
+__device__ __forceinline__ float2 sep_pixel(float2 w, float2 n1, float pq, bool exact = false) {
   const float t = w.x * n1.x;
   const float lo = fmaf(w.x, n1.y, fmaf(w.x, n1.x, -t));
-  const float ang = ((t - rintf(t)) + lo) * kTwoPiF;
+  const float turns = (t - rintf(t)) + lo;
   const float k = fmaf(-w.y * pq, pq, 1.f);
   float s, c;
-  __sincosf(ang, &s, &c);
+  if (exact)
+    sincospif(2.f * turns, &s, &c);
+  else
+    __sincosf(turns * kTwoPiF, &s, &c);
   return make_float2(k * c, k * s);
 }
 
