@@ -24,14 +24,16 @@
 // warp.  Preparing warps write the next item's phase slopes, F side of all L
 // rows and A-term samples (double buffers) while one runs.
 //
-// What bounds it: the producers' issue slots and instruction supply.  With all threads
+// What bounds it: the producers' issue slots and instruction supply (81 % of the slots, tensor pipe 31 %;
+// profiles/degridder_sep_mwa_like_90st.md).  With all threads
 // doing each step in turn and Z in shared memory it took 46.8 ms (MWA-like workload, 96 x
 // 96 subgrids, segments of about 60 visibilities, per degrid call on GB300), with a half
 // of producers in step and a half of consumers 31.4 ms, with roles and a thread's 8 rows
 // of a piece written out 19.7 ms; 16 rows per thread pay a piece's waits and set-up for
 // twice the rows, and four rows at a time in a loop keep the code small (18.2 ms; full
 // Jones matrices, 64 stations: 1.43 -> 1.16; written out 16 times 20.6 and 1.65).  The
-// kernel with one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.
+// kernel with one phasor per visibility and pixel (degridder_tc_kernels.cuh) takes 78.4 ms.  With subgrids of a wide w range
+// in parts it is 18.8 ms.
 #pragma once
 
 #include "sep_common.cuh"

@@ -25,13 +25,13 @@
 //
 // What bounds it: the latency of a chunk's chain (phasors, splits, the stores to
 // tensor memory, a barrier) at 4 warps a scheduler, which the pixel sums'
-// registers allow: about 60 % of the issue slots, tensor pipe 37 % and shared
-// memory 59 % busy.  With the E side in shared memory too, operands, their reads by the MMAs
+// registers allow: 61 % of the issue slots, tensor pipe 38 % and shared-memory
+// loads and stores 46 % busy (profiles/gridder_sep_mwa_like_90st.md).  With the E side in shared memory too, operands, their reads by the MMAs
 // and a transpose per 16 rows kept shared memory 80 % busy (21.2 ms where that took
 // 17.6); the E side in tensor memory costs none.  E's phasors computed once for the
 // 4 correlations and passed through shared memory lengthen the chain (16.0 ms).
 // Measured (GB300, MWA-like workload, 96 x 96 subgrids, segments of about 60
-// visibilities, per grid call): 15.2 ms, against 81.7 ms of the kernel with one
+// visibilities, per grid call): 15.3 ms, against 81.7 ms of the kernel with one
 // phasor per visibility and pixel (gridder_tc_kernels.cuh); grid error 5e-7
 // against 2.2e-6.
 #pragma once
